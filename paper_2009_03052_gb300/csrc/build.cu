@@ -98,208 +98,158 @@ __global__ void hub_reduce_kernel(CT *__restrict__ partial, CT *__restrict__ dst
 }
 
 // ---------------------------------------------------------------------------
-// merge of level h: one thread per (node, output entry).  Output o of level
-// h carries (|T'|, |T''|, beta, #terms) and a list of (index into the
-// c_{|T'|} row, index into the S_{|T''|} row) pairs, one per split of the
-// colour set; c_1 is the constant 1.
-// ---------------------------------------------------------------------------
-struct MergeArgs {
+// merge of level h.  Output o carries (beta, #terms) and a list of (index
+// into the c_{|T'|} row, index into the S_{|T''|} row) pairs, one per split of
+// the colour set; c_1 is the constant 1.
+//
+// The merge by tiles of TN nodes, TN = 8 .. 128.  Each lower level pairs with
+// one other level only -- c_{h1} with S_{h - h1} -- so a block stages the
+// rows of one such pair at a time (cp.async, rows padded to an odd stride),
+// computes the outputs of that pair, and goes on to the next; the output rows
+// gather in shared memory and leave in one coalesced pass.  A thread keeps
+// one node (tid mod TN) and takes every (threads / TN)-th output, so the
+// threads that share an output run one program and read one entry of
+// neighbouring rows: no divergence, no bank conflicts, and every lower row
+// crosses the memory bus once.  Bound by the bytes of the rows (and, at
+// k = 8, by the latency of a stage: two blocks per SM).  Against a thread per
+// (node, output) reading its operands through L1, ms per level 5 / 6 / 7 on
+// R-MAT scale 22, k = 7, 128-bit counts: 10.6 / 15.0 / 12.5 before, 4.1 / 5.8
+// / 5.1 now; level 5 / 6 on a 994k-node grid, k = 6, 64-bit counts: 0.69 /
+// 0.47 before, 0.44 / 0.40 now.
+struct TilePair {
+    int h1, h2;         // sizes of T' and T''
+    int wa, wb;         // row widths of c_{h1} (0 for h1 = 1: implicit) and S_{h2}
+    int sa, sb;         // their strides in shared memory (odd), in counts
+    uint32_t ma, mb;    // ceil(2^32 / w): division by the row width
+    int rec0, rec1;     // the pair's outputs in the record list
+};
+struct MergeTileArgs {
     const void *c[MAXK + 1];
     const void *S[MAXK + 1];
     int Wc[MAXK + 1], Ws[MAXK + 1];
     ExactDiv div[MAXK + 1];
-    const int32_t *info, *off;
-    const uint32_t *terms;
+    TilePair pair[MAXK];
+    int npair;
+    const uint2 *rec;       // output records: (o | beta << 16 | nterms << 24, first term)
+    const uint32_t *terms;  // byte offsets in the pair's rows: c_{h1} | S_{h2} << 16
+    int nrec, nterms;
+    const uint32_t *order;  // the nodes to do, NULL: 0 .. n_do - 1
+    int64_t n_do;
     void *out;
-    int64_t n;
-    int W, Bc, R;                     // row width, colour sets and shapes of the level
-    const MergeLevel *program;        // host copy of the program (schedule planning only)
-    const uint8_t *zero_root_colors;  // set: only colour-0 nodes get counts
+    int W, so;              // output row width and its stride in shared memory
+    uint32_t mw;
+    int log_tn, in_counts;  // log2 TN; counts of the staging area
+    const uint8_t *zero_root_colors;
     int *err;
 };
 
-template <typename CT, int MINB>
-__global__ void __launch_bounds__(256, MINB) merge_kernel(const __grid_constant__ MergeArgs a)
-{
-    bool ovf = false, inexact = false;
-    const int64_t total = a.n * a.W;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        // node and output entry; 32-bit division when the level fits 2^32
-        // entries.  Threads walk a row in (shape, set) order, so the threads
-        // of a warp mostly share one shape and one program length, and write
-        // entry (set, shape) at its set-major position.
-        const int64_t v = total <= 0xffffffffll ? (int64_t)((uint32_t)t / (uint32_t)a.W) : t / a.W;
-        const int q = (int)(t - v * a.W);
-        const int sh = q / a.Bc;
-        const int o = (q - sh * a.Bc) * a.R + sh;
-        if (a.zero_root_colors && a.zero_root_colors[v] != 0) {
-            ((CT *)a.out)[v * a.W + o] = 0;
-            continue;
-        }
-        const int info = a.info[o];
-        const int h1 = info & 15, h2 = (info >> 4) & 15, beta = (info >> 8) & 255, nt = info >> 16;
-        const uint32_t *term = a.terms + a.off[o];
-        const CT *B = (const CT *)a.S[h2] + v * a.Ws[h2];
-        CT sum = 0;
-        if (h1 == 1) {
-            for (int i = 0; i < nt; ++i) ovf |= add_ovf(sum, B[term[i] >> 16]);
-        } else {
-            const CT *A = (const CT *)a.c[h1] + v * a.Wc[h1];
-            for (int i = 0; i < nt; ++i) {
-                const uint32_t tm = term[i];
-                CT p;
-                ovf |= mul_ovf(A[tm & 0xffffu], B[tm >> 16], p);
-                ovf |= add_ovf(sum, p);
-            }
-        }
-        CT qt;
-        if (!exact_div(sum, a.div[beta], qt)) inexact = true;
-        ((CT *)a.out)[v * a.W + o] = qt;
-    }
-    if (ovf) atomicOr(a.err, ERR_OVERFLOW);
-    if (inexact) atomicOr(a.err, ERR_INEXACT);
-}
-
-// The merge with its operands streamed through shared memory: a block takes
-// tiles of NB consecutive nodes; while it computes the outputs of one tile
-// from one buffer, cp.async copies the next tile's rows (every lower level
-// the program reads; rows of consecutive nodes are contiguous) into the
-// other, 16 bytes per copy.  Waiting is cp.async.wait_group on the thread's
-// own copies, followed by a block barrier.
-struct MergeStage {
-    int nlev;
-    int is_s[2 * MAXK];
-    int lev[2 * MAXK];
-    int off[2 * MAXK];        // offset of the level's NB rows inside one buffer, in counts
-    int soff_c[MAXK + 1];     // the same per c level (-1: not staged)
-    int soff_s[MAXK + 1];
-    int NB;
-    int buf;                  // counts per buffer
-};
-
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
+// 8- or 16-byte asynchronous copy to shared memory
+template <typename CT> __device__ __forceinline__ void cp_async_count(CT *smem, const CT *gmem)
 {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+    if constexpr (sizeof(CT) == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+
+// i / w for i < 2^16 by the precomputed m = ceil(2^32 / w)
+__device__ __forceinline__ int div_width(int i, int w, uint32_t m) { return w == 1 ? i : (int)__umulhi((uint32_t)i, m); }
 
 template <typename CT>
-__device__ __forceinline__ void merge_stage_copy(const MergeArgs &a, const MergeStage &st, int64_t tile, CT *buf)
+__device__ __forceinline__ void stage_rows(CT *dst, const CT *src, int w, int stride, uint32_t m, int tn,
+                                           const uint32_t *node, int nthreads)
 {
-    const int64_t v0 = tile * st.NB;
-    if (v0 >= a.n) return;
-    const int nv = (int)min((int64_t)st.NB, a.n - v0);
-    for (int l = 0; l < st.nlev; ++l) {
-        const int h = st.lev[l];
-        const int W = st.is_s[l] ? a.Ws[h] : a.Wc[h];
-        const char *g = (const char *)((const CT *)(st.is_s[l] ? a.S[h] : a.c[h]) + v0 * W);
-        char *d = (char *)(buf + st.off[l]);
-        const int chunks = (int)(((int64_t)nv * W * (int64_t)sizeof(CT)) >> 4);
-        for (int i = threadIdx.x; i < chunks; i += blockDim.x) cp_async16(d + 16 * i, g + 16 * i);
+    for (int i = threadIdx.x; i < tn * w; i += nthreads) {
+        const int r = div_width(i, w, m), e = i - r * w;
+        const uint32_t v = node[r];
+        if (v != 0xffffffffu) cp_async_count(dst + r * stride + e, src + (int64_t)v * w + e);
     }
 }
 
-template <typename CT>
-__global__ void __launch_bounds__(256) merge_pipe_kernel(const __grid_constant__ MergeArgs a,
-                                                         const __grid_constant__ MergeStage st)
+template <typename CT, int THREADS>
+__global__ void __launch_bounds__(THREADS) merge_tile_kernel(const __grid_constant__ MergeTileArgs a)
 {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    CT *bufs = (CT *)s_raw;
+    const int tn = 1 << a.log_tn;
+    CT *s_in = (CT *)s_raw;
+    CT *s_out = s_in + a.in_counts;
+    uint2 *s_rec = (uint2 *)(s_out + (tn * a.so + 1) / 2 * 2);
+    uint32_t *s_terms = (uint32_t *)(s_rec + a.nrec);
+    uint32_t *s_src = s_terms + a.nterms;  // nodes whose rows are read (0xffffffff: none)
+    uint32_t *s_dst = s_src + tn;          // nodes whose row is written
+    for (int i = threadIdx.x; i < a.nrec; i += THREADS) s_rec[i] = a.rec[i];
+    for (int i = threadIdx.x; i < a.nterms; i += THREADS) s_terms[i] = a.terms[i];
+    const int node = threadIdx.x & (tn - 1), grp = threadIdx.x >> a.log_tn, ngrp = THREADS >> a.log_tn;
     bool ovf = false, inexact = false;
-    const int64_t ntiles = (a.n + st.NB - 1) / st.NB;
-    int64_t tile = blockIdx.x;
-    merge_stage_copy<CT>(a, st, tile, bufs);
-    cp_async_commit();
-    for (int it = 0; tile < ntiles; ++it, tile += gridDim.x) {
-        CT *cur = bufs + (int64_t)(it & 1) * st.buf;
-        merge_stage_copy<CT>(a, st, tile + gridDim.x, bufs + (int64_t)((it + 1) & 1) * st.buf);
-        cp_async_commit();
-        cp_async_wait1();   // this thread's copies of `tile` have landed
-        __syncthreads();    // and every other thread's
-        const int64_t v0 = tile * st.NB;
-        const int nv = (int)min((int64_t)st.NB, a.n - v0);
-        const int nout = nv * a.W;
-        for (int t = threadIdx.x; t < nout; t += blockDim.x) {
-            const int vl = t / a.W;
-            const int q = t - vl * a.W;
-            const int sh = q / a.Bc;
-            const int o = (q - sh * a.Bc) * a.R + sh;
-            const int64_t v = v0 + vl;
-            CT *dst = (CT *)a.out + v * a.W + o;
-            if (a.zero_root_colors && a.zero_root_colors[v] != 0) {
-                *dst = 0;
-                continue;
-            }
-            const int info = a.info[o];
-            const int h1 = info & 15, h2 = (info >> 4) & 15, beta = (info >> 8) & 255, nt = info >> 16;
-            const uint32_t *term = a.terms + a.off[o];
-            CT sum = 0;
-            if (nt > 0) {
-                const CT *B = cur + st.soff_s[h2] + vl * a.Ws[h2];
-                if (h1 == 1) {
-                    for (int i = 0; i < nt; ++i) ovf |= add_ovf(sum, B[term[i] >> 16]);
-                } else {
-                    const CT *A = cur + st.soff_c[h1] + vl * a.Wc[h1];
-                    for (int i = 0; i < nt; ++i) {
-                        const uint32_t tm = term[i];
-                        CT p;
-                        ovf |= mul_ovf(A[tm & 0xffffu], B[tm >> 16], p);
-                        ovf |= add_ovf(sum, p);
+    const int64_t ntiles = (a.n_do + tn - 1) >> a.log_tn;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t i0 = tile << a.log_tn;
+        if (threadIdx.x < tn) {
+            const int64_t i = i0 + threadIdx.x;
+            const uint32_t v = i < a.n_do ? (a.order ? a.order[i] : (uint32_t)i) : 0xffffffffu;
+            s_dst[threadIdx.x] = v;
+            s_src[threadIdx.x] = (v != 0xffffffffu && a.zero_root_colors && a.zero_root_colors[v] != 0) ? 0xffffffffu : v;
+        }
+        __syncthreads();
+        const bool live = s_src[node] != 0xffffffffu;
+        for (int p = 0; p < a.npair; ++p) {
+            const TilePair &P = a.pair[p];
+            CT *s_b = s_in + tn * P.sa;
+            if (P.wa) stage_rows<CT>(s_in, (const CT *)a.c[P.h1], P.wa, P.sa, P.ma, tn, s_src, THREADS);
+            stage_rows<CT>(s_b, (const CT *)a.S[P.h2], P.wb, P.sb, P.mb, tn, s_src, THREADS);
+            asm volatile("cp.async.wait_all;\n" ::: "memory");
+            __syncthreads();
+            const char *A = (const char *)(s_in + node * P.sa);
+            const char *B = (const char *)(s_b + node * P.sb);
+            for (int r = P.rec0 + grp; r < P.rec1; r += ngrp) {
+                const uint2 rc = s_rec[r];
+                const uint32_t *term = s_terms + rc.y;
+                const int beta = (rc.x >> 16) & 255, nt = rc.x >> 24;
+                CT sum = 0;
+                if (live) {
+                    if (P.wa == 0) {
+                        for (int i = 0; i < nt; ++i) ovf |= add_ovf(sum, *(const CT *)(B + (term[i] >> 16)));
+                    } else {
+#pragma unroll 2
+                        for (int i = 0; i < nt; ++i) {
+                            const uint32_t tm = term[i];
+                            CT q;
+                            ovf |= mul_ovf(*(const CT *)(A + (tm & 0xffffu)), *(const CT *)(B + (tm >> 16)), q);
+                            ovf |= add_ovf(sum, q);
+                        }
+                    }
+                    if (beta != 1) {
+                        CT q = 0;
+                        if (!exact_div(sum, a.div[beta], q)) inexact = true;
+                        sum = q;
                     }
                 }
+                s_out[node * a.so + (rc.x & 0xffffu)] = sum;
             }
-            CT qt;
-            if (!exact_div(sum, a.div[beta], qt)) inexact = true;
-            *dst = qt;
+            __syncthreads();
         }
-        __syncthreads();    // the buffer is free for the copy two tiles ahead
+        for (int i = threadIdx.x; i < tn * a.W; i += THREADS) {
+            const int r = div_width(i, a.W, a.mw), e = i - r * a.W;
+            const uint32_t v = s_dst[r];
+            if (v != 0xffffffffu) ((CT *)a.out)[(int64_t)v * a.W + e] = s_out[r * a.so + e];
+        }
+        __syncthreads();
     }
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
     if (ovf) atomicOr(a.err, ERR_OVERFLOW);
     if (inexact) atomicOr(a.err, ERR_INEXACT);
 }
 
-// The same merge with a thread per node walking all W outputs of its row in
-// (shape, set) order: every lane of a warp runs the same output program at
-// the same time (no divergence; the program's loads are uniform), reading
-// its own node's rows.
-template <typename CT, int MINB>
-__global__ void __launch_bounds__(256, MINB) merge_node_kernel(const __grid_constant__ MergeArgs a)
+// Rows of the nodes in list[0 .. cnt) set to zero, a warp per row.
+template <typename CT>
+__global__ void __launch_bounds__(256) zero_rows_kernel(CT *__restrict__ out, const uint32_t *__restrict__ list,
+                                                        int64_t cnt, int W)
 {
-    bool ovf = false, inexact = false;
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < a.n; v += (int64_t)gridDim.x * blockDim.x) {
-        CT *row = (CT *)a.out + v * a.W;
-        const bool zero = a.zero_root_colors && a.zero_root_colors[v] != 0;
-        for (int sh = 0; sh < a.R; ++sh)
-            for (int rho = 0; rho < a.Bc; ++rho) {
-                const int o = rho * a.R + sh;
-                if (zero) { row[o] = 0; continue; }
-                const int info = a.info[o];
-                const int h1 = info & 15, h2 = (info >> 4) & 15, beta = (info >> 8) & 255, nt = info >> 16;
-                const uint32_t *term = a.terms + a.off[o];
-                const CT *B = (const CT *)a.S[h2] + v * a.Ws[h2];
-                CT sum = 0;
-                if (h1 == 1) {
-                    for (int i = 0; i < nt; ++i) ovf |= add_ovf(sum, B[term[i] >> 16]);
-                } else {
-                    const CT *A = (const CT *)a.c[h1] + v * a.Wc[h1];
-                    for (int i = 0; i < nt; ++i) {
-                        const uint32_t tm = term[i];
-                        CT p;
-                        ovf |= mul_ovf(A[tm & 0xffffu], B[tm >> 16], p);
-                        ovf |= add_ovf(sum, p);
-                    }
-                }
-                CT qt;
-                if (!exact_div(sum, a.div[beta], qt)) inexact = true;
-                row[o] = qt;
-            }
-    }
-    if (ovf) atomicOr(a.err, ERR_OVERFLOW);
-    if (inexact) atomicOr(a.err, ERR_INEXACT);
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = warp; i < cnt; i += nwarps)
+        for (int e = lane; e < W; e += 32) out[(int64_t)list[i] * W + e] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -863,75 +813,78 @@ template <typename CT> static bool launch_gather(GatherArgs &ga, int r, int h, i
     return launch_gather_ub<uint64_t, 8>(ga, h, cand, s);
 }
 
-// The pipelined merge's staging plan for level h: the lower levels its
-// program reads, NB nodes per tile with two tiles of at most 96 KB of rows
-// per block; false when rows cannot be copied in 16-byte pieces.
-template <typename CT>
-static bool merge_stage_plan(const MergeArgs &ma, const MergeLevel &M, int h, MergeStage &st)
+// The tiled merge's plan: TN nodes per tile, the largest power of two up to
+// 128 whose rows fit 72 KB of shared memory (three blocks per SM) and that
+// leaves two tiles per SM, at least 8; shifted by `shift` (the tuner's
+// neighbours: twice the tile is 1.4x faster at level 6 of k = 6, half of it
+// with 128 threads up to 10% at levels 3-5 of k = 7).  False when the plan
+// does not exist.
+template <typename CT> static bool plan_merge_tile(MergeTileArgs &ta, const MergePairs &Q, int shift, size_t &smem)
 {
-    bool use_c[MAXK + 1] = {false}, use_s[MAXK + 1] = {false};
-    for (int32_t info : M.info) {
-        if ((info >> 16) == 0) continue;
-        const int h1 = info & 15, h2 = (info >> 4) & 15;
-        if (h1 >= 2) use_c[h1] = true;
-        use_s[h2] = true;
+    auto odd = [](int w) { return w | 1; };
+    auto magic = [](int w) { return w > 1 ? (uint32_t)((((uint64_t)1 << 32) + w - 1) / w) : 0u; };
+    ta.npair = Q.n;
+    int widest = 0;
+    for (int p = 0; p < Q.n; ++p) {
+        TilePair &P = ta.pair[p];
+        P.h1 = Q.h1[p];
+        P.h2 = Q.h2[p];
+        P.wa = P.h1 == 1 ? 0 : ta.Wc[P.h1];
+        P.wb = ta.Ws[P.h2];
+        P.sa = P.wa ? odd(P.wa) : 0;
+        P.sb = odd(P.wb);
+        P.ma = magic(P.wa);
+        P.mb = magic(P.wb);
+        P.rec0 = Q.rec0[p];
+        P.rec1 = Q.rec0[p + 1];
+        widest = std::max(widest, P.sa + P.sb);
     }
-    int per_node = 0;
-    for (int x = 1; x < h; ++x) per_node += (use_c[x] ? ma.Wc[x] : 0) + (use_s[x] ? ma.Ws[x] : 0);
-    if (per_node == 0) return false;
-    const int cb = (int)sizeof(CT);
-    int NB = (int)std::min<int64_t>(64, (48 * 1024) / ((int64_t)per_node * cb));
-    if (cb == 8) NB &= ~1;  // u64 rows: an even count of rows per level is 16-byte aligned
-    if (NB < 1) return false;
-    st = MergeStage{};
-    st.NB = NB;
-    for (int x = 0; x <= MAXK; ++x) st.soff_c[x] = st.soff_s[x] = -1;
-    int off = 0;
-    for (int pass = 0; pass < 2; ++pass)
-        for (int x = 1; x < h; ++x) {
-            if (!(pass ? use_s[x] : use_c[x])) continue;
-            const int W = pass ? ma.Ws[x] : ma.Wc[x];
-            st.is_s[st.nlev] = pass;
-            st.lev[st.nlev] = x;
-            st.off[st.nlev] = off;
-            (pass ? st.soff_s : st.soff_c)[x] = off;
-            off += NB * W;
-            ++st.nlev;
-        }
-    st.buf = off;
+    ta.so = odd(ta.W);
+    ta.mw = magic(ta.W);
+    ta.nrec = (int)Q.rec.size() / 2;
+    ta.nterms = (int)Q.terms.size();
+    const size_t fixed = (size_t)ta.nrec * 8 + (size_t)ta.nterms * 4 + 64;
+    const size_t node = (size_t)(widest + ta.so) * sizeof(CT) + 8;
+    int lt = 7;
+    while (lt > 3 && (fixed + (node << lt) > 72 * 1024 || (ta.n_do >> lt) < 2 * (int64_t)sm_count())) --lt;
+    lt += shift;
+    if (lt < 3 || lt > 7) return false;
+    ta.log_tn = lt;
+    ta.in_counts = widest << lt;
+    smem = fixed + (node << lt);
+    return smem <= 220 * 1024;
+}
+
+// Merge candidates (threads per block, tile size): 256 threads at the plan's
+// tile, half and twice that; 512 threads at the plan's tile; 128 threads at
+// the plan's tile and half of it.
+constexpr int MERGE_CANDIDATES = 6;
+
+template <typename CT, int THREADS>
+static bool launch_merge_tile(const MergeTileArgs &base, const MergePairs &Q, int h, int shift, cudaStream_t s)
+{
+    MergeTileArgs ta = base;
+    size_t smem = 0;
+    if (!plan_merge_tile<CT>(ta, Q, shift, smem)) return false;
+    if (smem > 48 * 1024)
+        MC_CUDA(cudaFuncSetAttribute(merge_tile_kernel<CT, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int64_t ntiles = (ta.n_do + (1 << ta.log_tn) - 1) >> ta.log_tn;
+    const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(2048 / THREADS, (int64_t)(227 * 1024 / (smem + 1024))));
+    const int g = (int)std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)sm_count() * per_sm));
+    MC_LAUNCH(kMergeName[h], s, merge_tile_kernel<CT, THREADS><<<g, THREADS, smem, s>>>(ta));
     return true;
 }
 
-// Merge candidates: a thread per output entry with occupancy targets of 1
-// (no register cap), 6 and 8 blocks of 256 threads per SM; a thread per node
-// (all of its outputs) at 6 and 8 blocks per SM; the pipelined merge through
-// shared memory.
-constexpr int MERGE_CANDIDATES = 6;
-
-template <typename CT> static bool launch_merge(const MergeArgs &ma, int h, int cand, cudaStream_t s)
+template <typename CT>
+static bool launch_merge(const MergeTileArgs &ta, const MergePairs &Q, int h, int cand, cudaStream_t s)
 {
-    const int grid = grid_for(ma.n * ma.W, 256);
-    const int gnode = grid_for(ma.n, 256);
     switch (cand) {
-    case 0: MC_LAUNCH(kMergeName[h], s, merge_kernel<CT, 1><<<grid, 256, 0, s>>>(ma)); return true;
-    case 1: MC_LAUNCH(kMergeName[h], s, merge_kernel<CT, 6><<<grid, 256, 0, s>>>(ma)); return true;
-    case 2: MC_LAUNCH(kMergeName[h], s, merge_kernel<CT, 8><<<grid, 256, 0, s>>>(ma)); return true;
-    case 3: MC_LAUNCH(kMergeName[h], s, merge_node_kernel<CT, 6><<<gnode, 256, 0, s>>>(ma)); return true;
-    case 4: MC_LAUNCH(kMergeName[h], s, merge_node_kernel<CT, 8><<<gnode, 256, 0, s>>>(ma)); return true;
-    case 5: {
-        MergeStage st;
-        if (!ma.program || !merge_stage_plan<CT>(ma, *ma.program, h, st)) return false;
-        // the last partial tile of u64 rows may be an odd count: 16-byte
-        // copies need even tiles throughout
-        if (sizeof(CT) == 8 && (ma.n % st.NB) != 0 && ((ma.n % st.NB) & 1)) return false;
-        const size_t smem = 2 * (size_t)st.buf * sizeof(CT);
-        if (smem > 48 * 1024)
-            MC_CUDA(cudaFuncSetAttribute(merge_pipe_kernel<CT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        const int64_t ntiles = (ma.n + st.NB - 1) / st.NB;
-        const int g = (int)std::min<int64_t>(ntiles, (int64_t)sm_count() * 4);
-        MC_LAUNCH(kMergeName[h], s, merge_pipe_kernel<CT><<<g, 256, smem, s>>>(ma, st));
-        return true;
-    }
+    case 0: return launch_merge_tile<CT, 256>(ta, Q, h, 0, s);
+    case 1: return launch_merge_tile<CT, 256>(ta, Q, h, -1, s);
+    case 2: return launch_merge_tile<CT, 256>(ta, Q, h, 1, s);
+    case 3: return launch_merge_tile<CT, 512>(ta, Q, h, 0, s);
+    case 4: return launch_merge_tile<CT, 128>(ta, Q, h, 0, s);
+    case 5: return launch_merge_tile<CT, 128>(ta, Q, h, -1, s);
     default: return false;
     }
 }
@@ -1084,29 +1037,29 @@ template <typename CT> static void build_levels(mc_tables *t, int *err, cudaStre
                                               g->col, t->ecol, g->row_ptr, g->chunk_node, g->chunk_e0, g->chunk_e1,
                                               g->n_chunks, k, ccnt, t->coff, t->scol));
     }
-    MergeArgs ma{};
+    MergeTileArgs ta{};
     for (int h = 1; h <= k; ++h) {
-        ma.c[h] = t->c[h];
-        ma.S[h] = t->S[h];
-        ma.Wc[h] = G.Wc[h];
-        ma.Ws[h] = G.Ws[h];
-        if (h <= MAXK) ma.div[h] = make_div(h);
+        ta.c[h] = t->c[h];
+        ta.S[h] = t->S[h];
+        ta.Wc[h] = G.Wc[h];
+        ta.Ws[h] = G.Ws[h];
     }
-    ma.n = n;
-    ma.err = err;
+    for (int b = 1; b <= MAXK; ++b) ta.div[b] = make_div(b);
+    ta.order = g->order;
+    ta.n_do = g->n_do;
+    ta.err = err;
     for (int h = 2; h <= k; ++h) {
         if (t->skip_round && h == k - 1) continue;  // round k-1 skipped: nothing reads it
-        ma.info = t->m_info[h];
-        ma.off = t->m_off[h];
-        ma.terms = t->m_terms[h];
-        ma.out = t->c[h];
-        ma.W = G.Wc[h];
-        ma.Bc = G.Bc[h];
-        ma.R = shape_catalog().r[h];
-        ma.program = &programs(k, t->skip_round).merge[h];
-        ma.zero_root_colors = (t->zero_root && h == k) ? t->colors : nullptr;
+        ta.rec = t->p_rec[h];
+        ta.terms = t->p_terms[h];
+        ta.out = t->c[h];
+        ta.W = G.Wc[h];
+        ta.zero_root_colors = (t->zero_root && h == k) ? t->colors : nullptr;
+        if (g->order)
+            MC_LAUNCH("zero_rows", s, zero_rows_kernel<CT><<<grid_for((n - g->n_do) * 32, 256), 256, 0, s>>>(
+                                          (CT *)t->c[h], g->order + g->n_do, n - g->n_do, G.Wc[h]));
         const TuneKey mkey = tune_key(1, k, (int)sizeof(CT) * 8, h, n, g->nnz, g->max_degree);
-        run_tuned(mkey, MERGE_CANDIDATES, allow_tune, s, [&](int c) { return launch_merge<CT>(ma, h, c, s); });
+        run_tuned(mkey, MERGE_CANDIDATES, allow_tune, s, [&](int c) { return launch_merge<CT>(ta, programs(k, t->skip_round).pairs[h], h, c, s); });
         if (h <= k - 1) {
             GatherArgs ga{};
             ga.row_ptr = g->row_ptr;
@@ -1245,13 +1198,13 @@ extern "C" mc_status mc_build_tables(const mc_graph *g, const uint8_t *colors, i
         for (int j = 0; j < 32; ++j) t->copies_k[j] = P.copies[j];
         for (int h = 2; h <= k; ++h) {
             if (t->level_missing(h)) continue;
-            const MergeLevel &M = P.merge[h];
-            t->m_info[h] = t->arena.get<int32_t>(M.info.size());
-            t->m_off[h] = t->arena.get<int32_t>(M.offset.size());
-            t->m_terms[h] = t->arena.get<uint32_t>(M.terms.size());
-            MC_CUDA(cudaMemcpyAsync(t->m_info[h], M.info.data(), M.info.size() * 4, cudaMemcpyHostToDevice, s));
-            MC_CUDA(cudaMemcpyAsync(t->m_off[h], M.offset.data(), M.offset.size() * 4, cudaMemcpyHostToDevice, s));
-            MC_CUDA(cudaMemcpyAsync(t->m_terms[h], M.terms.data(), M.terms.size() * 4, cudaMemcpyHostToDevice, s));
+            const MergePairs &Q = P.pairs[h];
+            std::vector<uint32_t> bt(Q.terms);
+            for (uint32_t &x : bt) x = (x & 0xffffu) * (uint32_t)cb | ((x >> 16) * (uint32_t)cb) << 16;
+            t->p_rec[h] = t->arena.get<uint2>(Q.rec.size() / 2);
+            t->p_terms[h] = t->arena.get<uint32_t>(bt.size());
+            MC_CUDA(cudaMemcpyAsync(t->p_rec[h], Q.rec.data(), Q.rec.size() * 4, cudaMemcpyHostToDevice, s));
+            MC_CUDA(cudaMemcpyAsync(t->p_terms[h], bt.data(), bt.size() * 4, cudaMemcpyHostToDevice, s));
         }
         for (int h = 1; h <= k - 1; ++h) {
             if (t->level_missing(h)) continue;

@@ -276,6 +276,31 @@ static Programs build_programs(int k, bool skip)
             }
         }
     }
+    for (int h = 2; h <= k; ++h) {
+        if (skip && h == k - 1) continue;
+        const MergeLevel &M = P.merge[h];
+        MergePairs &Q = P.pairs[h];
+        const int W = (int)M.info.size(), r = cat.r[h];
+        auto add = [&](int o) {
+            const int info = M.info[o], nt = info >> 16;
+            Q.rec.push_back((uint32_t)o | (uint32_t)((info >> 8) & 255) << 16 | (uint32_t)nt << 24);
+            Q.rec.push_back((uint32_t)Q.terms.size());
+            Q.terms.insert(Q.terms.end(), M.terms.begin() + M.offset[o], M.terms.begin() + M.offset[o] + nt);
+        };
+        for (int h1 = h - 1; h1 >= 1; --h1) {
+            const size_t before = Q.rec.size();
+            for (int s = 0; s < r; ++s)
+                for (int o = s; o < W; o += r)
+                    if ((M.info[o] >> 16) > 0 && (M.info[o] & 15) == h1) add(o);
+            if (Q.rec.size() == before) continue;
+            if (Q.n == 0)  // uncounted outputs (no terms) go with the first pair
+                for (int o = 0; o < W; ++o)
+                    if ((M.info[o] >> 16) == 0) add(o);
+            Q.h1[Q.n] = h1;
+            Q.h2[Q.n] = h - h1;
+            Q.rec0[++Q.n] = (int)Q.rec.size() / 2;
+        }
+    }
     for (int h = 1; h <= k - 1; ++h) {
         if (skip && h == k - 1) continue;
         GatherLevel &L = P.gather[h];

@@ -61,6 +61,18 @@ struct MergeLevel {
     std::vector<uint32_t> terms;  // ia | ib << 16
 };
 
+// The same program by pairs (h1, h2) = (|T'|, |T''|): the outputs of one pair
+// read only the rows of c_{h1} and S_{h2}, and every lower level is in one
+// pair.  Outputs of a pair keep the shapes together, so neighbouring records
+// have programs of one length.
+struct MergePairs {
+    int n = 0;
+    int h1[MAXK] = {0}, h2[MAXK] = {0};
+    int rec0[MAXK + 1] = {0};      // first record of each pair
+    std::vector<uint32_t> rec;     // per record: o | beta << 16 | nterms << 24, first term
+    std::vector<uint32_t> terms;   // ia | ib << 16
+};
+
 // Gather map of level h: S_h(v)[rho'', s] accumulates c_h(u)[src, s] over
 // neighbours u and every shape s, src = map[(c_v * k + c_u) * Bs[h] + rho'']
 // (-1: no contribution because c_u is not in the set).
@@ -76,6 +88,7 @@ struct GatherLevel {
 struct Programs {
     Geometry geo;
     MergeLevel merge[MAXK + 1];
+    MergePairs pairs[MAXK + 1];
     GatherLevel gather[MAXK + 1];
     bool skip = false;
     int bal_left[MAX_SHAPES], bal_right[MAX_SHAPES], bal_beta[MAX_SHAPES];  // per level-k shape (global

@@ -191,6 +191,37 @@ __global__ void degree_order_kernel(const int64_t *__restrict__ row_ptr, int64_t
     }
 }
 
+// The nodes with neighbours first, then those without: a block takes a tile
+// of blockDim nodes and reserves a run of each part; ascending inside a run.
+__global__ void __launch_bounds__(256) active_order_kernel(const int64_t *__restrict__ row_ptr, int64_t n,
+                                                           unsigned *cursor, uint32_t *__restrict__ order)
+{
+    __shared__ unsigned wcnt[8], base[2];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x; t0 < n; t0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = t0 + threadIdx.x;
+        const bool in = v < n, act = in && row_ptr[v + 1] > row_ptr[v];
+        const unsigned ba = __ballot_sync(0xffffffffu, act), bi = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) wcnt[w] = (unsigned)__popc(ba);
+        __syncthreads();
+        unsigned before = 0, all = 0;
+        for (int i = 0; i < 8; ++i) {
+            if (i < w) before += wcnt[i];
+            all += wcnt[i];
+        }
+        if (threadIdx.x == 0) {
+            const unsigned tile = (unsigned)min((int64_t)blockDim.x, n - t0);
+            base[0] = atomicAdd(&cursor[0], all);
+            base[1] = atomicAdd(&cursor[1], tile - all);
+        }
+        __syncthreads();
+        const unsigned lt = (1u << lane) - 1u, pa = before + (unsigned)__popc(ba & lt);
+        const unsigned pi = (unsigned)(w * 32) + (unsigned)__popc(bi & lt) - pa;
+        if (in) order[act ? base[0] + pa : base[1] + pi] = (uint32_t)v;
+        __syncthreads();  // wcnt and base are reused by the next tile
+    }
+}
+
 // Hubs of more than HUB_SERIAL chunks (their chunk sums get a warp each).
 __global__ void big_hubs_kernel(const int64_t *__restrict__ hub_chunk0, int64_t n_hubs, unsigned *count,
                                 uint32_t *__restrict__ big)
@@ -525,7 +556,8 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
         // the schedule of the neighbour sums: the other nodes by descending degree
         g->n_small = n - g->n_hubs;
         g->sched = g->arena.get<uint4>((size_t)std::max<int64_t>(g->n_small, 1));
-        unsigned hh[HUB_CHUNK + 1], cur[HUB_CHUNK + 1];  // live until the synchronisation below
+        unsigned hh[HUB_CHUNK + 1], cur[HUB_CHUNK + 1], oc[2] = {0, 0};  // live until the synchronisation below
+        g->n_do = n;
         if (g->n_small > 0) {
             unsigned *dh = scratch.get<unsigned>(2 * (HUB_CHUNK + 1));
             MC_CUDA(cudaMemsetAsync(dh, 0, (HUB_CHUNK + 1) * sizeof(unsigned), s));
@@ -539,6 +571,18 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
             MC_CUDA(cudaMemcpyAsync(dh + HUB_CHUNK + 1, cur, sizeof(cur), cudaMemcpyHostToDevice, s));
             MC_LAUNCH("degree_order", s, degree_order_kernel<<<grid_for(n, 256), 256, 0, s>>>(
                                              g->row_ptr, n, dh + HUB_CHUNK + 1, g->sched));
+            // the merges skip neighbourless nodes when at least an eighth are
+            // (below that, reading 4 bytes per node for the list and losing
+            // the runs of consecutive rows costs what the skipped rows give)
+            if ((int64_t)hh[0] * 8 >= n) {
+                g->order = g->arena.get<uint32_t>((size_t)n);
+                g->n_do = n - hh[0];
+                oc[1] = (unsigned)g->n_do;
+                unsigned *dc = scratch.get<unsigned>(2);
+                MC_CUDA(cudaMemcpyAsync(dc, oc, sizeof(oc), cudaMemcpyHostToDevice, s));
+                MC_LAUNCH("active_order", s, active_order_kernel<<<grid_for(n, 256), 256, 0, s>>>(g->row_ptr, n, dc,
+                                                                                                  g->order));
+            }
         }
         if (side.done) MC_CUDA(cudaStreamWaitEvent(s, side.done, 0));  // the ids are in place
         MC_CUDA(cudaStreamSynchronize(s));

@@ -165,6 +165,10 @@ struct mc_graph {
     int64_t n_small = 0;
     uint32_t *big_hub = nullptr;  // hubs (indices into hub_node) of more than HUB_SERIAL chunks
     int64_t n_big_hubs = 0;
+    // when many nodes have no neighbour: the others in order[0 .. n_do), the
+    // neighbourless in order[n_do .. n); else NULL and n_do = n
+    uint32_t *order = nullptr;
+    int64_t n_do = 0;
     mc::Arena arena;
     // uncoloured h-star index, built on first use: inclusive prefix over v of
     // C(d_v, h-1) and its total
@@ -205,9 +209,8 @@ struct mc_tables {
     mc::u128 bucketD[mc::MAXK + 1] = {0};
     int64_t nbucket = 0;
     // merge and gather programs (device)
-    int32_t *m_info[mc::MAXK + 1] = {nullptr};
-    int32_t *m_off[mc::MAXK + 1] = {nullptr};
-    uint32_t *m_terms[mc::MAXK + 1] = {nullptr};
+    uint2 *p_rec[mc::MAXK + 1] = {nullptr};
+    uint32_t *p_terms[mc::MAXK + 1] = {nullptr};
     int16_t *g_map[mc::MAXK + 1] = {nullptr};
     // kept for in-place rebuilds (mc_rebuild_tables): error flags, hub colour
     // counts, scan tile sums and the bucket width of level k, all on the device
