@@ -16,15 +16,17 @@
 #include <map>
 #include <set>
 #include <tuple>
+#include <type_traits>
 
 #include "gather.cuh"
 
 namespace mc {
 
-GatherKernel gather_kernel_ptr(size_t count_bytes, int UB, int G, int NU, int U, int MB)
+GatherKernel gather_kernel_ptr(size_t count_bytes, int N, int UB, int G, int NU, int P, int U, int MB)
 {
-    if (count_bytes == 16) return gather_kernel_ptr_u128_16(G, NU, U, MB);
-    return UB == 16 ? gather_kernel_ptr_u64_16(G, NU, U, MB) : gather_kernel_ptr_u64_8(G, NU, U, MB);
+    if (count_bytes == 16)
+        return N == 4 ? gather_kernel_ptr_u128_4(UB, G, NU, P, U, MB) : gather_kernel_ptr_u128_8(UB, G, NU, P, U, MB);
+    return N == 4 ? gather_kernel_ptr_u64_4(UB, G, NU, P, U, MB) : gather_kernel_ptr_u64_8(UB, G, NU, P, U, MB);
 }
 
 // The neighbour-sum kernel and its instantiations live in gather.cuh and
@@ -33,17 +35,30 @@ GatherKernel gather_kernel_ptr(size_t count_bytes, int UB, int G, int NU, int U,
 // (hub, S entry) pair are contiguous; they become their inclusive prefix
 // (the sampler binary-searches it) and the last prefix is the hub's
 // neighbour sum.  Any overflowing partial sum means the total overflows too.
+// A hub's S row is written in both planes; it is marked wide when an entry
+// needs its upper part.
 // Hubs of at most HUB_SERIAL chunks: a thread per (hub, entry) scans them in
 // order (the threads of a warp take consecutive entries of one hub, whose
 // chunk sums are adjacent); larger hubs: a warp per (hub, entry), 32 chunks
 // per warp scan.
 
 template <typename CT>
-__global__ void hub_reduce_small_kernel(CT *__restrict__ partial, CT *__restrict__ dst,
+__device__ __forceinline__ void store_hub_entry(const Rows &dst, uint32_t v, int e, CT x, bool &wide)
+{
+    store_low<1, CT>(dst.low(v) + e * dst.N, &x, dst.N);
+    store_rest<CT>(dst.high(v), dst.W, dst.N, e, x);
+    if (above<CT>(x, dst.N)) {
+        atomicOr(dst.wide + v, dst.bit);
+        wide = true;
+    }
+}
+
+template <typename CT>
+__global__ void hub_reduce_small_kernel(CT *__restrict__ partial, Rows dst, uint32_t *levels,
                                         const uint32_t *__restrict__ hub_node,
                                         const int64_t *__restrict__ hub_chunk0, int64_t n_hubs, int Ws, int *err)
 {
-    bool ovf = false;
+    bool ovf = false, wide = false;
     const int64_t total = n_hubs * Ws;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -57,18 +72,19 @@ __global__ void hub_reduce_small_kernel(CT *__restrict__ partial, CT *__restrict
             ovf |= add_ovf(run, p[c]);
             p[c] = run;
         }
-        dst[(int64_t)hub_node[hub] * Ws + e] = run;
+        store_hub_entry<CT>(dst, hub_node[hub], e, run, wide);
     }
     if (ovf) atomicOr(err, ERR_OVERFLOW);
+    if (wide) atomicOr(levels, dst.bit);
 }
 
 template <typename CT>
-__global__ void hub_reduce_kernel(CT *__restrict__ partial, CT *__restrict__ dst,
+__global__ void hub_reduce_kernel(CT *__restrict__ partial, Rows dst, uint32_t *levels,
                                   const uint32_t *__restrict__ hub_node,
                                   const int64_t *__restrict__ hub_chunk0, const uint32_t *__restrict__ big_hub,
                                   int64_t n_big, int Ws, int *err)
 {
-    bool ovf = false;
+    bool ovf = false, wide = false;
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -92,9 +108,10 @@ __global__ void hub_reduce_kernel(CT *__restrict__ partial, CT *__restrict__ dst
             if (c < nch) p[c] = x;
             carry = shfl(x, 31);
         }
-        if (lane == 0) dst[(int64_t)hub_node[hub] * Ws + e] = carry;
+        if (lane == 0) store_hub_entry<CT>(dst, hub_node[hub], e, carry, wide);
     }
     if (ovf) atomicOr(err, ERR_OVERFLOW);
+    if (wide) atomicOr(levels, dst.bit);
 }
 
 // ---------------------------------------------------------------------------
@@ -116,72 +133,129 @@ __global__ void hub_reduce_kernel(CT *__restrict__ partial, CT *__restrict__ dst
 // R-MAT scale 22, k = 7, 128-bit counts: 10.6 / 15.0 / 12.5 before, 4.1 / 5.8
 // / 5.1 now; level 5 / 6 on a 994k-node grid, k = 6, 64-bit counts: 0.69 /
 // 0.47 before, 0.44 / 0.40 now.
+// Rows are read and written by their first planes (common.cuh): operands of 4
+// or 8 bytes, with products of 64 to 128 bits.  A node with a wide row among a
+// pair's operands reads that pair's operands from memory instead, in full;
+// an output that exceeds its first plane writes its upper part at once, and
+// the rest of such a row is zeroed when the tile leaves.
 struct TilePair {
     int h1, h2;         // sizes of T' and T''
     int wa, wb;         // row widths of c_{h1} (0 for h1 = 1: implicit) and S_{h2}
-    int sa, sb;         // their strides in shared memory (odd), in counts
-    uint32_t ma, mb;    // ceil(2^32 / w): division by the row width
+    int ca, cb;         // 8-byte pieces of their first planes
+    int sa, sb;         // strides in shared memory (odd), in 8-byte pieces
+    uint32_t ma, mb;    // ceil(2^32 / pieces): division by the row's pieces
+    uint32_t bits;      // the pair's bits in the nodes' wide words
     int rec0, rec1;     // the pair's outputs in the record list
 };
 struct MergeTileArgs {
-    const void *c[MAXK + 1];
-    const void *S[MAXK + 1];
-    int Wc[MAXK + 1], Ws[MAXK + 1];
+    Rows c[MAXK + 1], S[MAXK + 1];
     ExactDiv div[MAXK + 1];
     TilePair pair[MAXK];
     int npair;
     const uint2 *rec;       // output records: (o | beta << 16 | nterms << 24, first term)
-    const uint32_t *terms;  // byte offsets in the pair's rows: c_{h1} | S_{h2} << 16
+    const uint32_t *terms;  // entries of the pair's rows: c_{h1} | S_{h2} << 16
     int nrec, nterms;
     const uint32_t *order;  // the nodes to do, NULL: 0 .. n_do - 1
     int64_t n_do;
-    void *out;
-    int W, so;              // output row width and its stride in shared memory
-    uint32_t mw;
-    int log_tn, in_counts;  // log2 TN; counts of the staging area
+    Rows out;
+    int so, cw;             // output row: stride in shared memory and pieces of its first plane
+    uint32_t mw;            // ceil(2^32 / cw)
+    int log_tn, in_pieces;  // log2 TN; 8-byte pieces of the staging area
+    uint32_t *levels;       // the levels that have a wide row
     const uint8_t *zero_root_colors;
     int *err;
 };
 
-// 8- or 16-byte asynchronous copy to shared memory
-template <typename CT> __device__ __forceinline__ void cp_async_count(CT *smem, const CT *gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    if constexpr (sizeof(CT) == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-
 // i / w for i < 2^16 by the precomputed m = ceil(2^32 / w)
 __device__ __forceinline__ int div_width(int i, int w, uint32_t m) { return w == 1 ? i : (int)__umulhi((uint32_t)i, m); }
 
-template <typename CT>
-__device__ __forceinline__ void stage_rows(CT *dst, const CT *src, int w, int stride, uint32_t m, int tn,
+// The first-plane rows of a tile's nodes, in 8-byte pieces.
+__device__ __forceinline__ void stage_rows(uint64_t *dst, const Rows &src, int pieces, int stride, uint32_t m, int tn,
                                            const uint32_t *node, int nthreads)
 {
-    for (int i = threadIdx.x; i < tn * w; i += nthreads) {
-        const int r = div_width(i, w, m), e = i - r * w;
+    for (int i = threadIdx.x; i < tn * pieces; i += nthreads) {
+        const int r = div_width(i, pieces, m), e = i - r * pieces;
         const uint32_t v = node[r];
-        if (v != 0xffffffffu) cp_async_count(dst + r * stride + e, src + (int64_t)v * w + e);
+        if (v == 0xffffffffu) continue;
+        const unsigned sa = (unsigned)__cvta_generic_to_shared(dst + r * stride + e);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(src.low(v) + 8 * e) : "memory");
     }
+}
+
+// sum over the terms of A[ia] * B[ib] (HA = false: of B[ib]), the operands
+// first-plane counts of NA and NB bytes.  Exact: `ovf` is set when the sum
+// does not fit CT.
+template <typename CT, bool HA, int NA, int NB>
+__device__ __forceinline__ CT merge_sum(const uint8_t *A, const uint8_t *B, const uint32_t *term, int nt, bool &ovf)
+{
+    typedef typename std::conditional<NA == 4, uint32_t, uint64_t>::type TA;
+    typedef typename std::conditional<NB == 4, uint32_t, uint64_t>::type TB;
+    const TA *a = (const TA *)A;
+    const TB *b = (const TB *)B;
+    if constexpr (!HA || (NA == 4 && NB == 4)) {
+        // at most 35 terms below 2^64: 64 bits and a carry count
+        uint64_t lo = 0;
+        uint32_t hi = 0;
+#pragma unroll 2
+        for (int i = 0; i < nt; ++i) {
+            const uint32_t tm = term[i];
+            uint64_t p = b[tm >> 16];
+            if constexpr (HA) p *= a[tm & 0xffffu];
+            lo += p;
+            hi += lo < p;
+        }
+        if constexpr (sizeof(CT) == 16) return ((CT)hi << 64) | lo;
+        ovf |= hi != 0;
+        return (CT)lo;
+    } else {
+        CT sum = 0;
+#pragma unroll 2
+        for (int i = 0; i < nt; ++i) {
+            const uint32_t tm = term[i];
+            const uint64_t x = a[tm & 0xffffu], y = b[tm >> 16];
+            CT p;
+            if constexpr (sizeof(CT) == 16) p = (CT)x * y;
+            else ovf |= mul_ovf(x, y, p);
+            ovf |= add_ovf(sum, p);
+        }
+        return sum;
+    }
+}
+
+// The same from the rows in memory, upper parts included.
+template <typename CT>
+__device__ __noinline__ CT merge_sum_wide(const Rows &A, const Rows &B, bool has_a, int64_t v, const uint32_t *term, int nt,
+                                          bool &ovf)
+{
+    CT sum = 0;
+    for (int i = 0; i < nt; ++i) {
+        CT p = entry_at<CT>(B, v, term[i] >> 16);
+        if (has_a) {
+            CT q;
+            ovf |= mul_ovf(entry_at<CT>(A, v, term[i] & 0xffffu), p, q);
+            p = q;
+        }
+        ovf |= add_ovf(sum, p);
+    }
+    return sum;
 }
 
 template <typename CT, int THREADS>
 __global__ void __launch_bounds__(THREADS) merge_tile_kernel(const __grid_constant__ MergeTileArgs a)
 {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    const int tn = 1 << a.log_tn;
-    CT *s_in = (CT *)s_raw;
-    CT *s_out = s_in + a.in_counts;
-    uint2 *s_rec = (uint2 *)(s_out + (tn * a.so + 1) / 2 * 2);
+    const int tn = 1 << a.log_tn, W = a.out.W, N = a.out.N, wpn = (W + 31) >> 5;
+    uint64_t *s_in = (uint64_t *)s_raw;
+    uint64_t *s_out = s_in + a.in_pieces;
+    uint2 *s_rec = (uint2 *)(s_out + tn * a.so);
     uint32_t *s_terms = (uint32_t *)(s_rec + a.nrec);
     uint32_t *s_src = s_terms + a.nterms;  // nodes whose rows are read (0xffffffff: none)
     uint32_t *s_dst = s_src + tn;          // nodes whose row is written
+    uint32_t *s_big = s_dst + tn;          // per node, a bit per output above its first plane
     for (int i = threadIdx.x; i < a.nrec; i += THREADS) s_rec[i] = a.rec[i];
     for (int i = threadIdx.x; i < a.nterms; i += THREADS) s_terms[i] = a.terms[i];
     const int node = threadIdx.x & (tn - 1), grp = threadIdx.x >> a.log_tn, ngrp = THREADS >> a.log_tn;
-    bool ovf = false, inexact = false;
+    bool ovf = false, inexact = false, any_wide = false;
     const int64_t ntiles = (a.n_do + tn - 1) >> a.log_tn;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int64_t i0 = tile << a.log_tn;
@@ -191,65 +265,94 @@ __global__ void __launch_bounds__(THREADS) merge_tile_kernel(const __grid_consta
             s_dst[threadIdx.x] = v;
             s_src[threadIdx.x] = (v != 0xffffffffu && a.zero_root_colors && a.zero_root_colors[v] != 0) ? 0xffffffffu : v;
         }
+        for (int i = threadIdx.x; i < tn * wpn; i += THREADS) s_big[i] = 0;
         __syncthreads();
-        const bool live = s_src[node] != 0xffffffffu;
+        const uint32_t v = s_src[node];
+        const bool live = v != 0xffffffffu;
+        const uint32_t wide = live ? a.out.wide[v] : 0u;
+        bool big = false;
         for (int p = 0; p < a.npair; ++p) {
             const TilePair &P = a.pair[p];
-            CT *s_b = s_in + tn * P.sa;
-            if (P.wa) stage_rows<CT>(s_in, (const CT *)a.c[P.h1], P.wa, P.sa, P.ma, tn, s_src, THREADS);
-            stage_rows<CT>(s_b, (const CT *)a.S[P.h2], P.wb, P.sb, P.mb, tn, s_src, THREADS);
+            uint64_t *s_b = s_in + tn * P.sa;
+            if (P.wa) stage_rows(s_in, a.c[P.h1], P.ca, P.sa, P.ma, tn, s_src, THREADS);
+            stage_rows(s_b, a.S[P.h2], P.cb, P.sb, P.mb, tn, s_src, THREADS);
             asm volatile("cp.async.wait_all;\n" ::: "memory");
             __syncthreads();
-            const char *A = (const char *)(s_in + node * P.sa);
-            const char *B = (const char *)(s_b + node * P.sb);
-            for (int r = P.rec0 + grp; r < P.rec1; r += ngrp) {
-                const uint2 rc = s_rec[r];
-                const uint32_t *term = s_terms + rc.y;
-                const int beta = (rc.x >> 16) & 255, nt = rc.x >> 24;
-                CT sum = 0;
-                if (live) {
-                    if (P.wa == 0) {
-                        for (int i = 0; i < nt; ++i) ovf |= add_ovf(sum, *(const CT *)(B + (term[i] >> 16)));
-                    } else {
-#pragma unroll 2
-                        for (int i = 0; i < nt; ++i) {
-                            const uint32_t tm = term[i];
-                            CT q;
-                            ovf |= mul_ovf(*(const CT *)(A + (tm & 0xffffu)), *(const CT *)(B + (tm >> 16)), q);
-                            ovf |= add_ovf(sum, q);
+            const uint8_t *A = (const uint8_t *)(s_in + node * P.sa);
+            const uint8_t *B = (const uint8_t *)(s_b + node * P.sb);
+            const int na = a.c[P.h1].N, nb = a.S[P.h2].N;
+            const bool full = (wide & P.bits) != 0;
+            auto outputs = [&](auto sum_of) {
+                for (int r = P.rec0 + grp; r < P.rec1; r += ngrp) {
+                    const uint2 rc = s_rec[r];
+                    const uint32_t *term = s_terms + rc.y;
+                    const int o = rc.x & 0xffffu, beta = (rc.x >> 16) & 255, nt = rc.x >> 24;
+                    CT sum = 0;
+                    if (live) {
+                        if (!full)
+                            sum = sum_of(term, nt);
+                        else
+                            sum = merge_sum_wide<CT>(a.c[P.h1], a.S[P.h2], P.wa != 0, v, term, nt, ovf);
+                        if (beta != 1) {
+                            CT q = 0;
+                            if (!exact_div(sum, a.div[beta], q)) inexact = true;
+                            sum = q;
+                        }
+                        if (above<CT>(sum, N)) {
+                            store_rest<CT>(a.out.high(v), W, N, o, sum);
+                            atomicOr(&s_big[node * wpn + (o >> 5)], 1u << (o & 31));
+                            big = true;
                         }
                     }
-                    if (beta != 1) {
-                        CT q = 0;
-                        if (!exact_div(sum, a.div[beta], q)) inexact = true;
-                        sum = q;
-                    }
+                    uint8_t *row = (uint8_t *)(s_out + node * a.so);
+                    if (N == 4) ((uint32_t *)row)[o] = (uint32_t)sum;
+                    else ((uint64_t *)row)[o] = (uint64_t)sum;
                 }
-                s_out[node * a.so + (rc.x & 0xffffu)] = sum;
+            };
+            if (!P.wa) {
+                if (nb == 4) outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, false, 4, 4>(A, B, t, nt, ovf); });
+                else outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, false, 4, 8>(A, B, t, nt, ovf); });
+            } else if (na == 4) {
+                if (nb == 4) outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, true, 4, 4>(A, B, t, nt, ovf); });
+                else outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, true, 4, 8>(A, B, t, nt, ovf); });
+            } else {
+                if (nb == 4) outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, true, 8, 4>(A, B, t, nt, ovf); });
+                else outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, true, 8, 8>(A, B, t, nt, ovf); });
             }
             __syncthreads();
         }
-        for (int i = threadIdx.x; i < tn * a.W; i += THREADS) {
-            const int r = div_width(i, a.W, a.mw), e = i - r * a.W;
-            const uint32_t v = s_dst[r];
-            if (v != 0xffffffffu) ((CT *)a.out)[(int64_t)v * a.W + e] = s_out[r * a.so + e];
+        for (int i = threadIdx.x; i < tn * a.cw; i += THREADS) {
+            const int r = div_width(i, a.cw, a.mw), e = i - r * a.cw;
+            const uint32_t u = s_dst[r];
+            if (u != 0xffffffffu) ((uint64_t *)a.out.low(u))[e] = s_out[r * a.so + e];
         }
-        __syncthreads();
+        if (__syncthreads_or(big)) {
+            any_wide = true;
+            for (int r = 0; r < tn; ++r) {
+                bool has = false;
+                for (int w = 0; w < wpn; ++w) has |= s_big[r * wpn + w] != 0;
+                if (!has) continue;
+                uint8_t *high = a.out.high(s_dst[r]);
+                for (int e = threadIdx.x; e < W; e += THREADS)
+                    if (!((s_big[r * wpn + (e >> 5)] >> (e & 31)) & 1u)) store_rest<CT>(high, W, N, e, (CT)0);
+                if (threadIdx.x == 0) atomicOr(a.out.wide + s_dst[r], a.out.bit);
+            }
+            __syncthreads();
+        }
     }
     if (ovf) atomicOr(a.err, ERR_OVERFLOW);
     if (inexact) atomicOr(a.err, ERR_INEXACT);
+    if (any_wide && threadIdx.x == 0) atomicOr(a.levels, a.out.bit);
 }
 
-// Rows of the nodes in list[0 .. cnt) set to zero, a warp per row.
-template <typename CT>
-__global__ void __launch_bounds__(256) zero_rows_kernel(CT *__restrict__ out, const uint32_t *__restrict__ list,
-                                                        int64_t cnt, int W)
+// First-plane rows of the nodes in list[0 .. cnt) set to zero, a warp per row.
+__global__ void __launch_bounds__(256) zero_rows_kernel(Rows out, const uint32_t *__restrict__ list, int64_t cnt)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = warp; i < cnt; i += nwarps)
-        for (int e = lane; e < W; e += 32) out[(int64_t)list[i] * W + e] = 0;
+        for (int e = lane; e < out.s0 / 8; e += 32) ((uint64_t *)out.low(list[i]))[e] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -258,7 +361,7 @@ __global__ void __launch_bounds__(256) zero_rows_kernel(CT *__restrict__ out, co
 // nodes for the root draw).
 // ---------------------------------------------------------------------------
 template <typename CT, int G>
-__global__ void __launch_bounds__(256) row_totals_kernel(const CT *__restrict__ c, int64_t n, int W, int R,
+__global__ void __launch_bounds__(256) row_totals_kernel(Rows c, int64_t n, int W, int R,
                                                          uint64_t allow0, uint64_t allow1,
                                                          u128 *__restrict__ tot, int *err)
 {
@@ -272,6 +375,7 @@ __global__ void __launch_bounds__(256) row_totals_kernel(const CT *__restrict__ 
     for (int64_t v0 = warp * NG; v0 < n; v0 += nwarps * NG) {
         const int64_t v = v0 + grp;
         u128 s = 0;
+        const bool wide = v < n && (c.wide[v] & c.bit);
         if (v < n)
             for (int eb = j; eb < W; eb += 8 * G) {  // up to 8 loads in flight per lane
                 CT x[8];
@@ -280,7 +384,8 @@ __global__ void __launch_bounds__(256) row_totals_kernel(const CT *__restrict__ 
                     const int e = eb + i * G;
                     const int sh = e % R;  // set-major row: entry e is (set e / R, shape e % R)
                     const bool ok = e < W && (sh < 64 ? (allow0 >> sh) & 1 : (allow1 >> (sh - 64)) & 1);
-                    x[i] = ok ? c[v * W + e] : (CT)0;
+                    x[i] = ok ? row_low<CT>(c.low(v), c.N, e) : (CT)0;
+                    if (ok && wide) x[i] |= row_rest<CT>(c.high(v), W, c.N, e);
                 }
 #pragma unroll
                 for (int i = 0; i < 8; ++i) ovf |= add_ovf(s, widen(x[i]));
@@ -307,7 +412,7 @@ struct TreeletShapes {
 // thread per (node, treelet), treelet fastest, so a warp reads a few whole
 // rows.  Overflow of a sum is flagged.
 template <typename CT>
-__global__ void __launch_bounds__(256) treelet_totals_kernel(const CT *__restrict__ c, int64_t n, int W, int R, int Bc,
+__global__ void __launch_bounds__(256) treelet_totals_kernel(Rows c, int64_t n, int R, int Bc,
                                                              int nu, const __grid_constant__ TreeletShapes ts,
                                                              u128 *__restrict__ tot, int *err)
 {
@@ -317,11 +422,10 @@ __global__ void __launch_bounds__(256) treelet_totals_kernel(const CT *__restric
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = i / nu;
         const int j = (int)(i - v * nu);
-        const CT *row = c + v * W;
         u128 s = 0;
         for (int q = ts.off[j]; q < ts.off[j + 1]; ++q) {
             const int sh = ts.shape[q];
-            for (int b = 0; b < Bc; ++b) ovf |= add_ovf(s, widen(row[b * R + sh]));
+            for (int b = 0; b < Bc; ++b) ovf |= add_ovf(s, widen(entry_at<CT>(c, v, b * R + sh)));
         }
         tot[(int64_t)j * n + v] = s;
     }
@@ -422,12 +526,12 @@ __global__ void edge_colours_kernel(const uint32_t *__restrict__ col, const uint
 // Nodes of degree <= HUB_CHUNK: one thread each, per-colour counts and
 // cursors packed one byte per colour.
 // The per-colour counts are also the level-1 neighbour sums S_1(v)[{a}]
-// (c of a single node is 1 at its own colour), written here too.
-template <typename CT>
+// (c of a single node is 1 at its own colour), written here too: rows of
+// 4-byte first-plane counts (a degree is below 2^32), never wide.
 __global__ void colour_blocks_kernel(const int64_t *__restrict__ row_ptr, const uint32_t *__restrict__ col,
                                      const uint8_t *__restrict__ ecol, const uint8_t *__restrict__ colors,
                                      int64_t n, int k, uint32_t *__restrict__ scol, int32_t *__restrict__ coff,
-                                     CT *__restrict__ S1)
+                                     Rows S1)
 {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
@@ -446,7 +550,7 @@ __global__ void colour_blocks_kernel(const int64_t *__restrict__ row_ptr, const 
         const int cv = colors[v];
         for (int a = 0; a < k - 1; ++a) {
             const int abs_a = a < cv ? a : a + 1;
-            S1[v * (k - 1) + a] = (CT)((cnt >> (8 * abs_a)) & 0xffu);
+            ((uint32_t *)S1.low(v))[a] = (uint32_t)((cnt >> (8 * abs_a)) & 0xffu);
         }
         for (int64_t e = e0; e < e1; ++e) {
             const int c = ecol[e];
@@ -488,11 +592,10 @@ __global__ void hub_chunk_counts_kernel(const uint8_t *__restrict__ ecol, const 
     }
 }
 
-template <typename CT>
 __global__ void hub_chunk_prefix_kernel(const uint8_t *__restrict__ colors, const uint32_t *__restrict__ hub_node,
                                         const int64_t *__restrict__ hub_chunk0, int64_t n_hubs, int k,
                                         uint32_t *__restrict__ ccnt, int32_t *__restrict__ coff,
-                                        CT *__restrict__ S1)
+                                        Rows S1)
 {
     // one warp per hub: lanes take 32 chunks at a time; a warp scan per
     // colour turns the counts, in place, into each chunk's start inside that
@@ -534,7 +637,7 @@ __global__ void hub_chunk_prefix_kernel(const uint8_t *__restrict__ colors, cons
             const int cv = colors[v];
 #pragma unroll
             for (int a = 0; a < MAXK - 1; ++a)
-                if (a < k - 1) S1[v * (k - 1) + a] = (CT)tot[a < cv ? a : a + 1];
+                if (a < k - 1) ((uint32_t *)S1.low(v))[a] = tot[a < cv ? a : a + 1];
         }
     }
 }
@@ -620,15 +723,17 @@ int64_t bucket_count(int64_t n) { return std::max<int64_t>(1, std::min<int64_t>(
 
 // A colour >= k is reported and replaced by 0 in the tables' own copy, so
 // the kernels after this one never index past a colour's slot; the build
-// then fails when its error flags are read.
-__global__ void check_colours_kernel(uint8_t *colors, int64_t n, int k, int *err)
+// then fails when its error flags are read.  No row is wide yet.
+__global__ void check_colours_kernel(uint8_t *colors, int64_t n, int k, uint32_t *wide, int *err)
 {
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
-         v += (int64_t)gridDim.x * blockDim.x)
+         v += (int64_t)gridDim.x * blockDim.x) {
+        wide[v] = 0;
         if (colors[v] >= k) {
             atomicOr(err, ERR_COLOUR);
             colors[v] = 0;
         }
+    }
 }
 
 __global__ void fill_ones_kernel(void *dst, int64_t n, int bytes)
@@ -683,7 +788,7 @@ ExactDiv make_div(int beta)
 template <typename CT> size_t bytes_of() { return sizeof(CT); }
 
 template <typename CT>
-static void launch_row_totals_t(const CT *c, int64_t n, int W, int R, uint64_t allow0, uint64_t allow1, u128 *tot,
+static void launch_row_totals_t(const Rows &c, int64_t n, int W, int R, uint64_t allow0, uint64_t allow1, u128 *tot,
                                 int *err, cudaStream_t s)
 {
     int G = 1;  // lanes per node: each covers up to 8 entries
@@ -710,9 +815,9 @@ void launch_row_totals(const mc_tables *t, int h, uint64_t allow0, uint64_t allo
     }
     const int W = t->geo.Wc[h], R = shape_catalog().r[h];
     if (t->bits == 64)
-        launch_row_totals_t<uint64_t>((const uint64_t *)t->c[h], n, W, R, allow0, allow1, tot, err, s);
+        launch_row_totals_t<uint64_t>(t->rows(h, 0), n, W, R, allow0, allow1, tot, err, s);
     else
-        launch_row_totals_t<u128>((const u128 *)t->c[h], n, W, R, allow0, allow1, tot, err, s);
+        launch_row_totals_t<u128>(t->rows(h, 0), n, W, R, allow0, allow1, tot, err, s);
 }
 
 // Dense tables: tot[j * n + v] for every unrooted treelet j of level h in
@@ -732,14 +837,14 @@ void launch_treelet_totals(const mc_tables *t, int h, u128 *tot, int *err, cudaS
             if (cat.shapes[cat.gid(h, i)].unrooted == j) ts.shape[q++] = (uint8_t)i;
     }
     ts.off[nu] = (int16_t)q;
-    const int W = t->geo.Wc[h], Bc = t->geo.Bc[h];
+    const int Bc = t->geo.Bc[h];
     const int grid = grid_for(n * nu, 256);
     if (t->bits == 64)
         MC_LAUNCH("treelet_totals", s, treelet_totals_kernel<uint64_t><<<grid, 256, 0, s>>>(
-                                           (const uint64_t *)t->c[h], n, W, R, Bc, nu, ts, tot, err));
+                                           t->rows(h, 0), n, R, Bc, nu, ts, tot, err));
     else
         MC_LAUNCH("treelet_totals", s, treelet_totals_kernel<u128><<<grid, 256, 0, s>>>(
-                                           (const u128 *)t->c[h], n, W, R, Bc, nu, ts, tot, err));
+                                           t->rows(h, 0), n, R, Bc, nu, ts, tot, err));
 }
 
 static const char *const kGatherName[MAXK + 1] = {"gather_h0", "gather_h1", "gather_h2", "gather_h3",
@@ -748,69 +853,42 @@ static const char *const kGatherName[MAXK + 1] = {"gather_h0", "gather_h1", "gat
 static const char *const kMergeName[MAXK + 1] = {"merge_h0", "merge_h1", "merge_h2", "merge_h3", "merge_h4",
                                                  "merge_h5", "merge_h6", "merge_h7", "merge_h8"};
 
-static int rows_in_flight(int NU) { return NU >= 16 ? 1 : NU >= 8 ? 2 : NU >= 4 ? 4 : 8; }
-
-// Schedule candidates of the neighbour sums (the autotuner's choices), on
-// G0 lanes per node (the smallest power of two covering the row's units, at
-// most 32) and NU0 units per lane, with R0 = the standard rows in flight:
-//   0: R0 rows in flight, no register cap
-//   1: R0 / 2,  2: R0 / 4 (fewer registers, more warps per SM)
-//   3: R0 / 2 with at most 40 registers (6 blocks of 256 per SM)
-//   4: R0 / 4 with at most 32 registers (8 blocks of 256 per SM)
-//   5: one row in flight, 8 blocks per SM
-//   6: G0 / 2 lanes per node with two units each (twice the nodes per warp),
-//      a quarter of their rows in flight, 8 blocks per SM (2 <= G0 <= 16)
+// Schedules of the neighbour sums (the autotuner's choices): rows in flight
+// and blocks of 256 threads per SM (4: at most 64 registers, 6: 40, 8: 32).
 constexpr int GATHER_CANDIDATES = 7;
+static const int kGatherU[GATHER_CANDIDATES] = {4, 2, 1, 2, 1, 2, 4};
+static const int kGatherMB[GATHER_CANDIDATES] = {4, 4, 4, 6, 6, 8, 8};
 
-template <typename CT, int UB>
-static bool launch_gather_ub(const GatherArgs &ga, int h, int cand, cudaStream_t s)
+// G lanes for a row: the smallest power of two that covers its units, at most
+// 32, then NU units per lane.  Rows of fewer than 8 units take P neighbours
+// of the node at once, 8 lanes per node (4 when the average degree is below
+// 8: most of 8 would idle), so that the ids and colours of 8 neighbours are
+// one coalesced read.
+template <typename CT> static bool launch_gather(const GatherArgs &base, int r, int h, int cand, cudaStream_t s)
 {
+    if (cand < 0 || cand >= GATHER_CANDIDATES) return false;
+    GatherArgs ga = base;
+    const int N = ga.src.N, set_bytes = r * N;
+    const int UB = set_bytes % 16 == 0 ? 16 : set_bytes % 8 == 0 ? 8 : 4;  // a unit never straddles two colour sets
+    ga.ups = set_bytes / UB;
+    ga.ws_units = ga.dst.W * N / UB;
     int G = 1;
     while (G < ga.ws_units && G < 32) G <<= 1;
-    int NU = 1;
-    while (NU * 32 < ga.ws_units) NU <<= 1;
-    if (NU > 16) throw Error(MC_E_INTERNAL, "gather: S row too wide");
-    const int R0 = rows_in_flight(NU);
-    int U = R0, MB = 1;
-    switch (cand) {
-    case 0: break;
-    case 1: U = std::max(1, R0 / 2); break;
-    case 2: U = std::max(1, R0 / 4); break;
-    case 3: U = std::max(1, R0 / 2); MB = 6; break;
-    case 4: U = std::max(1, R0 / 4); MB = 8; break;
-    case 5: U = 1; MB = 8; break;
-    case 6:
-        if (G < 2 || G > 16) return false;
-        G /= 2;
-        NU *= 2;
-        U = std::max(1, rows_in_flight(NU) / 4);
-        MB = 8;
-        break;
-    default: return false;
-    }
-    auto kern = gather_kernel_ptr(sizeof(CT), UB, G, NU, U, MB);
-    if (!kern) return false;
-    const int NG = 32 / G;
+    int NU = (ga.ws_units + 31) / 32;
+    if (NU > 3) NU = 6;
+    if (NU * 32 < ga.ws_units) throw Error(MC_E_INTERNAL, "gather: S row too wide");
+    const int lanes = ga.nnz >= 8 * ga.n ? 8 : 4, P = G < lanes ? lanes / G : 1;
+    auto kern = gather_kernel_ptr(sizeof(CT), N, UB, G, NU, P, kGatherU[cand], kGatherMB[cand]);
+    if (!kern) throw Error(MC_E_INTERNAL, "gather: no kernel for this row layout");
+    const int NG = 32 / (G * P);
     const int wpb = 256 / 32;
-    GatherArgs g2 = ga;
     const int64_t cap = (int64_t)sm_count() * 32;
-    g2.chunk_blocks = (int)std::min<int64_t>((ga.n_chunks + wpb - 1) / wpb, cap);
+    ga.chunk_blocks = (int)std::min<int64_t>((ga.n_chunks + wpb - 1) / wpb, cap);
     const int64_t node_blocks = std::max<int64_t>(1, std::min<int64_t>((ga.n_small + NG * wpb - 1) / (NG * wpb), cap));
-    const int grid = (int)(g2.chunk_blocks + node_blocks);
-    const size_t smem = (size_t)ga.k * ga.k * ga.Bs * sizeof(int16_t);
-    MC_LAUNCH(kGatherName[h], s, kern<<<grid, 256, smem, s>>>(g2));
+    const int grid = (int)(ga.chunk_blocks + node_blocks);
+    const size_t smem = (size_t)ga.k * ga.k * NU * G * sizeof(int16_t);
+    MC_LAUNCH(kGatherName[h], s, kern<<<grid, 256, smem, s>>>(ga));
     return true;
-}
-
-template <typename CT> static bool launch_gather(GatherArgs &ga, int r, int h, int cand, cudaStream_t s)
-{
-    const int B = (int)sizeof(CT);
-    const int UB = (r * B) % 16 == 0 ? 16 : 8;  // a unit never straddles two colour sets
-    ga.ups = r * B / UB;
-    ga.wc_units = ga.Wc * B / UB;
-    ga.ws_units = ga.Ws * B / UB;
-    if (UB == 16) return launch_gather_ub<CT, 16>(ga, h, cand, s);
-    return launch_gather_ub<uint64_t, 8>(ga, h, cand, s);
 }
 
 // The tiled merge's plan: TN nodes per tile, the largest power of two up to
@@ -819,9 +897,8 @@ template <typename CT> static bool launch_gather(GatherArgs &ga, int r, int h, i
 // neighbours: twice the tile is 1.4x faster at level 6 of k = 6, half of it
 // with 128 threads up to 10% at levels 3-5 of k = 7).  False when the plan
 // does not exist.
-template <typename CT> static bool plan_merge_tile(MergeTileArgs &ta, const MergePairs &Q, int shift, size_t &smem)
+static bool plan_merge_tile(MergeTileArgs &ta, const MergePairs &Q, int shift, size_t &smem)
 {
-    auto odd = [](int w) { return w | 1; };
     auto magic = [](int w) { return w > 1 ? (uint32_t)((((uint64_t)1 << 32) + w - 1) / w) : 0u; };
     ta.npair = Q.n;
     int widest = 0;
@@ -829,28 +906,32 @@ template <typename CT> static bool plan_merge_tile(MergeTileArgs &ta, const Merg
         TilePair &P = ta.pair[p];
         P.h1 = Q.h1[p];
         P.h2 = Q.h2[p];
-        P.wa = P.h1 == 1 ? 0 : ta.Wc[P.h1];
-        P.wb = ta.Ws[P.h2];
-        P.sa = P.wa ? odd(P.wa) : 0;
-        P.sb = odd(P.wb);
-        P.ma = magic(P.wa);
-        P.mb = magic(P.wb);
+        P.wa = P.h1 == 1 ? 0 : ta.c[P.h1].W;
+        P.wb = ta.S[P.h2].W;
+        P.ca = P.wa ? ta.c[P.h1].s0 / 8 : 0;
+        P.cb = ta.S[P.h2].s0 / 8;
+        P.sa = P.wa ? P.ca | 1 : 0;
+        P.sb = P.cb | 1;
+        P.ma = magic(P.ca);
+        P.mb = magic(P.cb);
+        P.bits = (P.wa ? 1u << P.h1 : 0u) | 1u << (16 + P.h2);
         P.rec0 = Q.rec0[p];
         P.rec1 = Q.rec0[p + 1];
         widest = std::max(widest, P.sa + P.sb);
     }
-    ta.so = odd(ta.W);
-    ta.mw = magic(ta.W);
+    ta.cw = ta.out.s0 / 8;
+    ta.so = ta.cw | 1;
+    ta.mw = magic(ta.cw);
     ta.nrec = (int)Q.rec.size() / 2;
     ta.nterms = (int)Q.terms.size();
-    const size_t fixed = (size_t)ta.nrec * 8 + (size_t)ta.nterms * 4 + 64;
-    const size_t node = (size_t)(widest + ta.so) * sizeof(CT) + 8;
+    const size_t fixed = (size_t)ta.nrec * 8 + (size_t)ta.nterms * 4;
+    const size_t node = (size_t)(widest + ta.so) * 8 + 8 + (size_t)(ta.out.W + 31) / 32 * 4;
     int lt = 7;
     while (lt > 3 && (fixed + (node << lt) > 72 * 1024 || (ta.n_do >> lt) < 2 * (int64_t)sm_count())) --lt;
     lt += shift;
     if (lt < 3 || lt > 7) return false;
     ta.log_tn = lt;
-    ta.in_counts = widest << lt;
+    ta.in_pieces = widest << lt;
     smem = fixed + (node << lt);
     return smem <= 220 * 1024;
 }
@@ -865,7 +946,7 @@ static bool launch_merge_tile(const MergeTileArgs &base, const MergePairs &Q, in
 {
     MergeTileArgs ta = base;
     size_t smem = 0;
-    if (!plan_merge_tile<CT>(ta, Q, shift, smem)) return false;
+    if (!plan_merge_tile(ta, Q, shift, smem)) return false;
     if (smem > 48 * 1024)
         MC_CUDA(cudaFuncSetAttribute(merge_tile_kernel<CT, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int64_t ntiles = (ta.n_do + (1 << ta.log_tn) - 1) >> ta.log_tn;
@@ -1021,43 +1102,42 @@ template <typename CT> static void build_levels(mc_tables *t, int *err, cudaStre
     const int k = t->k;
     const int64_t n = g->n;
     if (n == 0) return;
+    uint32_t *levels = (uint32_t *)err + 1;  // the levels with a wide row
     // level 1 neighbour sums
     // colour blocks of every adjacency list, and the level-1 neighbour sums
-    MC_LAUNCH("colour_blocks", s, colour_blocks_kernel<CT><<<grid_for(n, 256), 256, 0, s>>>(
+    MC_LAUNCH("colour_blocks", s, colour_blocks_kernel<<<grid_for(n, 256), 256, 0, s>>>(
                                       g->row_ptr, g->col, t->ecol, t->colors, n, k, t->scol, t->coff,
-                                      (CT *)t->S[1]));
+                                      t->rows(1, 1)));
     if (g->n_hubs) {
         uint32_t *ccnt = t->ccnt;
         MC_LAUNCH("colour_blocks_hub", s, hub_chunk_counts_kernel<<<grid_for(g->n_chunks * 32, 256), 256, 0, s>>>(
                                               t->ecol, g->chunk_e0, g->chunk_e1, g->n_chunks, k, ccnt));
-        MC_LAUNCH("colour_blocks_hub", s, hub_chunk_prefix_kernel<CT><<<grid_for(g->n_hubs * 32, 256), 256, 0, s>>>(
+        MC_LAUNCH("colour_blocks_hub", s, hub_chunk_prefix_kernel<<<grid_for(g->n_hubs * 32, 256), 256, 0, s>>>(
                                               t->colors, g->hub_node, g->hub_chunk0, g->n_hubs, k, ccnt, t->coff,
-                                              (CT *)t->S[1]));
+                                              t->rows(1, 1)));
         MC_LAUNCH("colour_blocks_hub", s, hub_chunk_scatter_kernel<<<grid_for(g->n_chunks * 32, 256), 256, 0, s>>>(
                                               g->col, t->ecol, g->row_ptr, g->chunk_node, g->chunk_e0, g->chunk_e1,
                                               g->n_chunks, k, ccnt, t->coff, t->scol));
     }
     MergeTileArgs ta{};
     for (int h = 1; h <= k; ++h) {
-        ta.c[h] = t->c[h];
-        ta.S[h] = t->S[h];
-        ta.Wc[h] = G.Wc[h];
-        ta.Ws[h] = G.Ws[h];
+        ta.c[h] = t->rows(h, 0);
+        ta.S[h] = t->rows(h, 1);
     }
     for (int b = 1; b <= MAXK; ++b) ta.div[b] = make_div(b);
     ta.order = g->order;
     ta.n_do = g->n_do;
+    ta.levels = levels;
     ta.err = err;
     for (int h = 2; h <= k; ++h) {
         if (t->skip_round && h == k - 1) continue;  // round k-1 skipped: nothing reads it
         ta.rec = t->p_rec[h];
         ta.terms = t->p_terms[h];
-        ta.out = t->c[h];
-        ta.W = G.Wc[h];
+        ta.out = t->rows(h, 0);
         ta.zero_root_colors = (t->zero_root && h == k) ? t->colors : nullptr;
         if (g->order)
-            MC_LAUNCH("zero_rows", s, zero_rows_kernel<CT><<<grid_for((n - g->n_do) * 32, 256), 256, 0, s>>>(
-                                          (CT *)t->c[h], g->order + g->n_do, n - g->n_do, G.Wc[h]));
+            MC_LAUNCH("zero_rows", s, zero_rows_kernel<<<grid_for((n - g->n_do) * 32, 256), 256, 0, s>>>(
+                                          ta.out, g->order + g->n_do, n - g->n_do));
         const TuneKey mkey = tune_key(1, k, (int)sizeof(CT) * 8, h, n, g->nnz, g->max_degree);
         run_tuned(mkey, MERGE_CANDIDATES, allow_tune, s, [&](int c) { return launch_merge<CT>(ta, programs(k, t->skip_round).pairs[h], h, c, s); });
         if (h <= k - 1) {
@@ -1067,19 +1147,19 @@ template <typename CT> static void build_levels(mc_tables *t, int *err, cudaStre
             ga.colors = t->colors;
             ga.ecol = t->ecol;
             ga.node_chunk0 = g->node_chunk0;
-            ga.src = t->c[h];
-            ga.dst = t->S[h];
+            ga.src = t->rows(h, 0);
+            ga.dst = t->rows(h, 1);
+            ga.levels = levels;
             ga.partial = t->Sp[h];
             ga.chunk_node = g->chunk_node;
             ga.chunk_e0 = g->chunk_e0;
             ga.chunk_e1 = g->chunk_e1;
             ga.gmap = t->g_map[h];
             ga.n = n;
+            ga.nnz = g->nnz;
             ga.n_chunks = g->n_chunks;
             ga.k = k;
             ga.Bs = G.Bs[h];
-            ga.Wc = G.Wc[h];
-            ga.Ws = G.Ws[h];
             ga.err = err;
             ga.sched = g->sched;
             ga.n_small = g->n_small;
@@ -1088,10 +1168,10 @@ template <typename CT> static void build_levels(mc_tables *t, int *err, cudaStre
             run_tuned(gkey, GATHER_CANDIDATES, allow_tune, s, [&](int c) { return launch_gather<CT>(ga, rh, h, c, s); });
             if (g->n_hubs) {
                 MC_LAUNCH("hub_reduce", s, hub_reduce_small_kernel<CT><<<grid_for(g->n_hubs * G.Ws[h], 256), 256, 0, s>>>(
-                    (CT *)t->Sp[h], (CT *)t->S[h], g->hub_node, g->hub_chunk0, g->n_hubs, G.Ws[h], err));
+                    (CT *)t->Sp[h], t->rows(h, 1), levels, g->hub_node, g->hub_chunk0, g->n_hubs, G.Ws[h], err));
                 if (g->n_big_hubs)
                     MC_LAUNCH("hub_reduce", s, hub_reduce_kernel<CT><<<grid_for(g->n_big_hubs * G.Ws[h] * 32, 256), 256, 0, s>>>(
-                        (CT *)t->Sp[h], (CT *)t->S[h], g->hub_node, g->hub_chunk0, g->big_hub, g->n_big_hubs,
+                        (CT *)t->Sp[h], t->rows(h, 1), levels, g->hub_node, g->hub_chunk0, g->big_hub, g->n_big_hubs,
                         G.Ws[h], err));
             }
         }
@@ -1101,6 +1181,29 @@ template <typename CT> static void build_levels(mc_tables *t, int *err, cudaStre
 }  // namespace mc
 
 using namespace mc;
+
+// Bytes of the first-plane counts of each level: 4 where the counts of the
+// level are expected below 2^30, so that (almost) no row is wide, else 8.
+// Expected largest count: the star of the largest degree, (d_max / k)^(h-1),
+// and the trees at the end of a random edge, (h-1)! (g / k)^(h-1) with g the
+// sum of squared degrees / nnz.  S_h counts like c_{h+1}.  A level with some
+// wide rows is exact but costs its readers a look at the node's word: with
+// 0.3% wide rows at level 4 the sampler of the 1M-node, k = 5 workload was
+// 20% slower than with none.
+static void plan_widths(mc_tables *t)
+{
+    const double star = std::log2(std::max((double)t->g->max_degree / t->k, 1.0));
+    const double walk = std::log2(std::max(t->g->walk_growth / t->k, 1e-3));
+    auto width = [&](int h) {
+        double fact = 0;
+        for (int i = 2; i < h; ++i) fact += std::log2((double)i);
+        return h <= 2 || ((h - 1) * star <= 30 && (h - 1) * walk + fact <= 30) ? 4 : 8;
+    };
+    for (int h = 1; h <= t->k; ++h) {
+        t->Nc[h] = width(h);
+        t->Ns[h] = h == 1 ? 4 : width(h + 1);
+    }
+}
 
 // Every launch of a build for the colours in `colors`, on stream s, into the
 // buffers of t: no allocation, no host read, no synchronisation (so a
@@ -1116,7 +1219,7 @@ static void enqueue_build(mc_tables *t, const uint8_t *colors, cudaStream_t s, b
         // the tables' own copy of the colours, checked before any kernel reads them
         if (colors != t->colors)
             MC_CUDA(cudaMemcpyAsync(t->colors, colors, (size_t)n, cudaMemcpyDefault, s));
-        MC_LAUNCH("check_colours", s, check_colours_kernel<<<grid_for(n, 256), 256, 0, s>>>(t->colors, n, k, err));
+        MC_LAUNCH("check_colours", s, check_colours_kernel<<<grid_for(n, 256), 256, 0, s>>>(t->colors, n, k, t->wide, err));
     }
     if (g->nnz)
         MC_LAUNCH("edge_colours", s, edge_colours_kernel<<<grid_for(g->nnz, 256), 256, 0, s>>>(
@@ -1136,14 +1239,16 @@ static void enqueue_build(mc_tables *t, const uint8_t *colors, cudaStream_t s, b
 static void finish_build(mc_tables *t, cudaStream_t s)
 {
     const int64_t n = t->g->n;
-    int herr = 0;
+    int flags[2] = {0, 0};
     u128 R = 0, D = 1;
-    MC_CUDA(cudaMemcpyAsync(&herr, t->dev_err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    MC_CUDA(cudaMemcpyAsync(flags, t->dev_err, sizeof(flags), cudaMemcpyDeviceToHost, s));
     if (n) {
         MC_CUDA(cudaMemcpyAsync(&R, t->prefix[t->k] + (n - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
         MC_CUDA(cudaMemcpyAsync(&D, t->dev_D, sizeof(u128), cudaMemcpyDeviceToHost, s));
     }
     MC_CUDA(cudaStreamSynchronize(s));
+    const int herr = flags[0];
+    t->wide_levels = (uint32_t)flags[1];
     if (herr & ERR_COLOUR) throw Error(MC_E_INVALID, "a colour is >= k");
     if (herr & ERR_OVERFLOW)
         throw Error(MC_E_OVERFLOW, "a count does not fit in " + std::to_string(t->bits) + " bits");
@@ -1190,6 +1295,8 @@ extern "C" mc_status mc_build_tables(const mc_graph *g, const uint8_t *colors, i
         t->scan_tmp = t->arena.get<u128>((size_t)std::max<int64_t>(scan_tiles(n), 1));
         if (g->n_hubs) t->ccnt = t->arena.get<uint32_t>((size_t)g->n_chunks * k);
         t->colors = t->arena.get<uint8_t>((size_t)n);
+        t->wide = t->arena.get<uint32_t>((size_t)n);
+        plan_widths(t);
         t->ecol = t->arena.get<uint8_t>((size_t)g->nnz);
         t->scol = t->arena.get<uint32_t>((size_t)g->nnz);
         t->coff = t->arena.get<int32_t>((size_t)n * (k + 1));
@@ -1199,12 +1306,10 @@ extern "C" mc_status mc_build_tables(const mc_graph *g, const uint8_t *colors, i
         for (int h = 2; h <= k; ++h) {
             if (t->level_missing(h)) continue;
             const MergePairs &Q = P.pairs[h];
-            std::vector<uint32_t> bt(Q.terms);
-            for (uint32_t &x : bt) x = (x & 0xffffu) * (uint32_t)cb | ((x >> 16) * (uint32_t)cb) << 16;
             t->p_rec[h] = t->arena.get<uint2>(Q.rec.size() / 2);
-            t->p_terms[h] = t->arena.get<uint32_t>(bt.size());
+            t->p_terms[h] = t->arena.get<uint32_t>(Q.terms.size());
             MC_CUDA(cudaMemcpyAsync(t->p_rec[h], Q.rec.data(), Q.rec.size() * 4, cudaMemcpyHostToDevice, s));
-            MC_CUDA(cudaMemcpyAsync(t->p_terms[h], bt.data(), bt.size() * 4, cudaMemcpyHostToDevice, s));
+            MC_CUDA(cudaMemcpyAsync(t->p_terms[h], Q.terms.data(), Q.terms.size() * 4, cudaMemcpyHostToDevice, s));
         }
         for (int h = 1; h <= k - 1; ++h) {
             if (t->level_missing(h)) continue;
@@ -1214,9 +1319,9 @@ extern "C" mc_status mc_build_tables(const mc_graph *g, const uint8_t *colors, i
         }
         // tables
         for (int h = 2; h <= k; ++h)
-            if (!t->level_missing(h)) t->c[h] = t->arena.get<uint8_t>((size_t)n * G.Wc[h] * cb);
+            if (!t->level_missing(h)) t->c[h] = t->arena.get<uint8_t>(t->level_bytes(h, 0, n));
         for (int h = 1; h <= k - 1; ++h)
-            if (!t->level_missing(h)) t->S[h] = t->arena.get<uint8_t>((size_t)n * G.Ws[h] * cb);
+            if (!t->level_missing(h)) t->S[h] = t->arena.get<uint8_t>(t->level_bytes(h, 1, n));
         for (int h = 2; h <= k - 1; ++h)
             if (!t->level_missing(h)) t->Sp[h] = t->arena.get<uint8_t>((size_t)g->n_chunks * G.Ws[h] * cb);
         t->nbucket = bucket_count(n);
@@ -1483,13 +1588,12 @@ extern "C" mc_status mc_build_tables_batch(int count, const mc_graph *const *gra
     return MC_OK;
 }
 
-// number of non-zero entries among n words (or pairs of words for u128)
-template <typename CT>
-__global__ void nonzeros_kernel(const CT *__restrict__ x, int64_t n, unsigned long long *count)
+// number of non-zero entries among the n entries of a level
+template <typename CT> __global__ void nonzeros_kernel(Rows x, int64_t n, unsigned long long *count)
 {
     unsigned long long c = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        c += x[i] != 0;
+        c += entry_at<CT>(x, i / x.W, (int)(i % x.W)) != 0;
     for (int o = 16; o >= 1; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
 }
@@ -1521,12 +1625,12 @@ extern "C" mc_status mc_table_nonzeros(const mc_tables *t, int h, int which, int
         scratch.stream = s;
         unsigned long long *d = scratch.get<unsigned long long>(1), hc = 0;
         MC_CUDA(cudaMemsetAsync(d, 0, sizeof(*d), s));
-        const void *src = which ? t->S[h] : t->c[h];
+        const Rows src = t->rows(h, which);
         if (m > 0) {
             if (t->bits == 64)
-                MC_LAUNCH("nonzeros", s, nonzeros_kernel<uint64_t><<<grid_for(m, 256), 256, 0, s>>>((const uint64_t *)src, m, d));
+                MC_LAUNCH("nonzeros", s, nonzeros_kernel<uint64_t><<<grid_for(m, 256), 256, 0, s>>>(src, m, d));
             else
-                MC_LAUNCH("nonzeros", s, nonzeros_kernel<u128><<<grid_for(m, 256), 256, 0, s>>>((const u128 *)src, m, d));
+                MC_LAUNCH("nonzeros", s, nonzeros_kernel<u128><<<grid_for(m, 256), 256, 0, s>>>(src, m, d));
         }
         MC_CUDA(cudaMemcpyAsync(&hc, d, sizeof(hc), cudaMemcpyDeviceToHost, s));
         MC_CUDA(cudaStreamSynchronize(s));
@@ -1545,6 +1649,27 @@ extern "C" mc_status mc_table_layout(const mc_tables *t, int h, int which, int64
         if (row_entries) *row_entries = which ? t->geo.Ws[h] : t->geo.Wc[h];
         if (entry_bytes) *entry_bytes = t->bits / 8;
     });
+}
+
+// Rows v0 .. v0 + cnt of a dense level as plain counts.
+template <typename CT>
+__global__ void __launch_bounds__(256) expand_kernel(Rows x, int64_t v0, int64_t total, CT *__restrict__ dst)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = total <= 0xffffffffll ? (int64_t)((uint32_t)i / (uint32_t)x.W) : i / x.W;
+        dst[i] = entry_at<CT>(x, v0 + v, (int)(i - v * x.W));
+    }
+}
+
+static void launch_expand(const mc_tables *t, int h, int which, int64_t v0, int64_t cnt, void *dst, cudaStream_t s)
+{
+    const Rows x = t->rows(h, which);
+    const int64_t total = cnt * x.W;
+    if (total == 0) return;
+    if (t->bits == 64)
+        MC_LAUNCH("expand", s, expand_kernel<uint64_t><<<grid_for(total, 256), 256, 0, s>>>(x, v0, total, (uint64_t *)dst));
+    else
+        MC_LAUNCH("expand", s, expand_kernel<u128><<<grid_for(total, 256), 256, 0, s>>>(x, v0, total, (u128 *)dst));
 }
 
 extern "C" mc_status mc_read_table(const mc_tables *t, int h, int which, void *dst, size_t dst_bytes,
@@ -1580,9 +1705,21 @@ extern "C" mc_status mc_read_table(const mc_tables *t, int h, int which, void *d
                 MC_CUDA(cudaMemcpyAsync(dst, tmp, bytes, cudaMemcpyDeviceToHost, s));
                 MC_CUDA(cudaStreamSynchronize(s));
             }
-        } else {
-            const void *src = which ? t->S[h] : t->c[h];
-            MC_CUDA(cudaMemcpyAsync(dst, src, bytes, dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s));
+        } else if (dst_on_device) {
+            launch_expand(t, h, which, 0, t->g->n, dst, s);
+        } else {  // through a scratch buffer of some rows
+            const int64_t row = W * (t->bits / 8), n = t->g->n;
+            const int64_t step = std::max<int64_t>(1, std::min<int64_t>(n, ((int64_t)64 << 20) / row));
+            Arena scratch(true);
+            scratch.alloc = t->arena.alloc;
+            scratch.stream = s;
+            void *tmp = scratch.get<uint8_t>((size_t)(step * row));
+            for (int64_t v = 0; v < n; v += step) {
+                const int64_t cnt = std::min(step, n - v);
+                launch_expand(t, h, which, v, cnt, tmp, s);
+                MC_CUDA(cudaMemcpyAsync((uint8_t *)dst + v * row, tmp, (size_t)(cnt * row), cudaMemcpyDeviceToHost, s));
+            }
+            MC_CUDA(cudaStreamSynchronize(s));
         }
         MC_CUDA(cudaStreamSynchronize(s));
     });

@@ -213,6 +213,83 @@ __host__ __device__ __forceinline__ unsigned insert_colour_gap(unsigned rel, int
 }
 
 // ---------------------------------------------------------------------------
+// Dense table levels, in two planes.  The first holds the low N bytes (4 or 8)
+// of every count, row after row; when a count of a row does not fit N bytes
+// the row is wide -- the level's bit is set in the node's word of `wide` -- and
+// its row of the second plane holds the upper parts: for 64-bit counts
+// (N = 4) the high words; for 128-bit counts the high 64 bits and, for N = 4,
+// bits 32..63 after them.  Rows of the second plane that are not wide are
+// never read or written.  Most counts are far below their width, so the build
+// moves a quarter to a half of the tables' bytes, and whole rows of narrow
+// counts stay in L2.  N is chosen per level when the tables are made.
+// ---------------------------------------------------------------------------
+struct Rows {
+    uint8_t *p0 = nullptr, *p1 = nullptr;  // the planes
+    int s0 = 0, s1 = 0;                    // their row strides, multiples of 8 bytes
+    int W = 0, N = 8;                      // counts per row, bytes of a first-plane count
+    uint32_t *wide = nullptr;
+    uint32_t bit = 0;
+    __host__ __device__ __forceinline__ uint8_t *low(int64_t v) const { return p0 + v * s0; }
+    __host__ __device__ __forceinline__ uint8_t *high(int64_t v) const { return p1 + v * s1; }
+};
+__host__ __device__ __forceinline__ int plane0_stride(int W, int N) { return (W * N + 7) / 8 * 8; }
+__host__ __device__ __forceinline__ int plane1_stride(int W, int N, int count_bytes)
+{
+    return (W * (count_bytes - N) + 7) / 8 * 8;
+}
+
+// entry e of a first-plane row
+template <typename CT> __device__ __forceinline__ CT row_low(const uint8_t *low, int N, int e)
+{
+    return N == 4 ? (CT)((const uint32_t *)low)[e] : (CT)((const uint64_t *)low)[e];
+}
+
+// the same without a branch, for lanes whose rows differ in N: one 8-byte
+// load (rows are padded to 8 bytes) and a select
+template <typename CT> __device__ __forceinline__ CT row_low_any(const uint8_t *low, int N, int e)
+{
+    const int at = e * N;
+    const uint64_t x = *(const uint64_t *)(low + (at & ~7));
+    return (CT)(N == 8 ? x : (uint64_t)(uint32_t)(x >> (8 * (at & 4))));
+}
+
+// the part of entry e above its low N bytes, in place (a wide row's)
+template <typename CT> __device__ __forceinline__ CT row_rest(const uint8_t *high, int W, int N, int e)
+{
+    if constexpr (sizeof(CT) == 8) {
+        return N == 4 ? (CT)((const uint32_t *)high)[e] << 32 : (CT)0;
+    } else {
+        CT x = (CT)((const uint64_t *)high)[e] << 64;
+        if (N == 4) x |= (CT)((const uint32_t *)(high + 8 * W))[e] << 32;
+        return x;
+    }
+}
+
+template <typename CT> __device__ __forceinline__ void store_rest(uint8_t *high, int W, int N, int e, CT x)
+{
+    if constexpr (sizeof(CT) == 8) {
+        if (N == 4) ((uint32_t *)high)[e] = (uint32_t)(x >> 32);
+    } else {
+        ((uint64_t *)high)[e] = (uint64_t)(x >> 64);
+        if (N == 4) ((uint32_t *)(high + 8 * W))[e] = (uint32_t)(x >> 32);
+    }
+}
+
+// x does not fit N bytes
+template <typename CT> __device__ __forceinline__ bool above(CT x, int N)
+{
+    if constexpr (sizeof(CT) == 8) return N == 4 && (x >> 32) != 0;
+    else return N == 4 ? (x >> 32) != 0 : (x >> 64) != 0;
+}
+
+template <typename CT> __device__ __forceinline__ CT entry_at(const Rows &r, int64_t v, int e)
+{
+    CT x = row_low<CT>(r.low(v), r.N, e);
+    if (r.wide[v] & r.bit) x |= row_rest<CT>(r.high(v), r.W, r.N, e);
+    return x;
+}
+
+// ---------------------------------------------------------------------------
 // Packed (zero-suppressed) table levels, Section 3.2.1: per node row only the
 // non-zero entries, in row order, each as a key (the entry's index in the
 // dense row) and a count.  Counts are stored at `width` bytes each when

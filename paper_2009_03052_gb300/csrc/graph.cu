@@ -98,23 +98,29 @@ __global__ void validate_offsets(const int64_t *row_ptr, int64_t n, int64_t nnz,
 }
 
 // per node: number of hub chunks (0 unless degree > HUB_CHUNK) and whether
-// it is a hub; the largest degree
-__global__ void degree_stats(const int64_t *row_ptr, int64_t n, u128 *nch, u128 *nhub, unsigned long long *maxdeg)
+// it is a hub; the largest degree (stat[0]) and the sum of the squared
+// degrees (stat[1])
+__global__ void degree_stats(const int64_t *row_ptr, int64_t n, u128 *nch, u128 *nhub, unsigned long long *stat)
 {
-    unsigned long long md = 0;
+    unsigned long long md = 0, sq = 0;
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t d = row_ptr[v + 1] - row_ptr[v];
         nch[v] = d > HUB_CHUNK ? (u128)((d + HUB_CHUNK - 1) / HUB_CHUNK) : (u128)0;
         nhub[v] = d > HUB_CHUNK ? 1 : 0;
         if ((unsigned long long)d > md) md = (unsigned long long)d;
+        sq += (unsigned long long)d * (unsigned long long)d;
     }
     // one atomic per warp, not per thread (a single address serialises them)
     for (int o = 16; o >= 1; o >>= 1) {
         const unsigned long long x = __shfl_xor_sync(0xffffffffu, md, o);
         if (x > md) md = x;
+        sq += __shfl_xor_sync(0xffffffffu, sq, o);
     }
-    if ((threadIdx.x & 31) == 0 && md) atomicMax(maxdeg, md);
+    if ((threadIdx.x & 31) == 0 && md) {
+        atomicMax(stat, md);
+        atomicAdd(stat + 1, sq);
+    }
 }
 
 // from the inclusive prefixes of chunk and hub counts: every hub writes its
@@ -453,7 +459,7 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
         Arena scratch(true);
         scratch.alloc = g->arena.alloc;
         scratch.stream = s;
-        int64_t *dstat = scratch.get<int64_t>(4);  // flags, max degree, #chunks, #hubs
+        int64_t *dstat = scratch.get<int64_t>(4);  // flags, max degree, sum of squared degrees
         MC_CUDA(cudaMemsetAsync(dstat, 0, 4 * sizeof(int64_t), s));
         g->row_ptr = g->arena.get<int64_t>((size_t)n + 1);
         g->col = g->arena.get<uint32_t>((size_t)(nnz > 0 ? nnz : 1));
@@ -529,6 +535,7 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
                                              std::to_string(((int *)hst)[0]) +
                                              ": 1 range, 2 loop, 4 order/duplicate, 8 asymmetric)");
         g->max_degree = hst[1];
+        g->walk_growth = nnz ? (double)(uint64_t)hst[2] / (double)nnz : 0.0;
         g->n_chunks = (int64_t)tails[0];
         g->n_hubs = (int64_t)tails[1];
         MC_REQUIRE(g->n_chunks < (int64_t)0x7fffffff, "too many hub chunks");

@@ -149,6 +149,7 @@ constexpr int HUB_SERIAL = 32;
 struct mc_tables;
 struct mc_graph {
     int64_t n = 0, nnz = 0, max_degree = 0;
+    double walk_growth = 0;      // sum of squared degrees / nnz: neighbours of a random edge's end
     int64_t *row_ptr = nullptr;  // device int64[n+1]
     uint32_t *col = nullptr;     // device uint32[nnz]
     // hub chunks (device): node, first edge, end edge; per hub, its first chunk
@@ -196,8 +197,11 @@ struct mc_tables {
                                                // by colour, ascending ids inside a colour
     int32_t *coff = nullptr;                   // device int32[n*(k+1)]: start of colour a's block in
                                                // v's row of scol, relative to row_ptr[v]
-    void *c[mc::MAXK + 1] = {nullptr};         // level h >= 2: n x Wc[h] counts
-    void *S[mc::MAXK + 1] = {nullptr};         // level h <= k-1: n x Ws[h] counts
+    void *c[mc::MAXK + 1] = {nullptr};         // level h >= 2: the planes of n x Wc[h] counts (Rows, common.cuh)
+    void *S[mc::MAXK + 1] = {nullptr};         // level h <= k-1: the planes of n x Ws[h] counts
+    int Nc[mc::MAXK + 1] = {0}, Ns[mc::MAXK + 1] = {0};  // bytes of their first-plane counts
+    uint32_t *wide = nullptr;                  // device uint32[n]: bit h row c_h is wide, bit 16 + h row S_h
+    uint32_t wide_levels = 0;                  // the levels with a wide row (of dev_err[1])
     void *Sp[mc::MAXK + 1] = {nullptr};        // level h <= k-1: per hub and S entry, the inclusive
                                                // prefix of its chunk sums, n_chunks x Ws[h]
     mc::u128 *prefix[mc::MAXK + 1] = {nullptr};  // inclusive node prefix of level totals
@@ -226,5 +230,28 @@ struct mc_tables {
     bool stale = false;                         // rebuilt since R[k], bucketD[k] were read back
     bool level_stale[mc::MAXK + 1] = {false};   // root index of level h from an older colouring
     std::string broken;                         // set when a rebuild failed its checks
+    // bytes of a level's first plane, the second after it
+    size_t plane0_bytes(int h, int which, int64_t n) const
+    {
+        return ((size_t)n * mc::plane0_stride(which ? geo.Ws[h] : geo.Wc[h], which ? Ns[h] : Nc[h]) + 255) & ~(size_t)255;
+    }
+    size_t level_bytes(int h, int which, int64_t n) const
+    {
+        return plane0_bytes(h, which, n) +
+               (size_t)n * mc::plane1_stride(which ? geo.Ws[h] : geo.Wc[h], which ? Ns[h] : Nc[h], bits / 8);
+    }
+    mc::Rows rows(int h, int which) const
+    {
+        mc::Rows r;
+        r.W = which ? geo.Ws[h] : geo.Wc[h];
+        r.N = which ? Ns[h] : Nc[h];
+        r.s0 = mc::plane0_stride(r.W, r.N);
+        r.s1 = mc::plane1_stride(r.W, r.N, bits / 8);
+        r.p0 = (uint8_t *)(which ? S[h] : c[h]);
+        r.p1 = r.p0 ? r.p0 + plane0_bytes(h, which, g->n) : nullptr;
+        r.wide = wide;
+        r.bit = which ? 1u << (16 + h) : 1u << h;
+        return r;
+    }
     mc::Arena arena;
 };

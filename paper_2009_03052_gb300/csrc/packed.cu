@@ -47,7 +47,7 @@ __device__ __forceinline__ u128 warp_max(u128 x)
 // (varlen: the row's own width, else the table's) and the row's count bytes
 // rounded up to 8.
 template <typename CT>
-__global__ void pack_count_kernel(const CT *__restrict__ D, int64_t n, int W, int varlen, u128 *cnt,
+__global__ void pack_count_kernel(Rows D, int64_t n, int W, int varlen, u128 *cnt,
                                   u128 *bytes, uint8_t *wid)
 {
     const int lane = threadIdx.x & 31;
@@ -57,7 +57,7 @@ __global__ void pack_count_kernel(const CT *__restrict__ D, int64_t n, int W, in
         unsigned nz = 0;
         u128 mx = 0;
         for (int e = lane; e < W; e += 32) {
-            const u128 x = widen(D[v * W + e]);
+            const u128 x = widen(entry_at<CT>(D, v, e));
             nz += x != 0;
             if (x > mx) mx = x;
         }
@@ -82,7 +82,7 @@ __global__ void offsets_kernel(const u128 *__restrict__ inc, int64_t n, int64_t 
 // Pass 2, a warp per node: keys and counts of the non-zero entries, in row
 // order.
 template <typename CT>
-__global__ void pack_fill_kernel(const CT *__restrict__ D, int64_t n, int W, PackedView p, uint16_t *__restrict__ key,
+__global__ void pack_fill_kernel(Rows D, int64_t n, int W, PackedView p, uint16_t *__restrict__ key,
                                  uint8_t *__restrict__ val)
 {
     const int lane = threadIdx.x & 31;
@@ -96,7 +96,7 @@ __global__ void pack_fill_kernel(const CT *__restrict__ D, int64_t n, int W, Pac
         int64_t base = 0;
         for (int e0 = 0; e0 < W; e0 += 32) {
             const int e = e0 + lane;
-            const u128 x = e < W ? widen(D[v * W + e]) : (u128)0;
+            const u128 x = e < W ? widen(entry_at<CT>(D, v, e)) : (u128)0;
             const unsigned m = __ballot_sync(0xffffffffu, x != 0);
             if (x != 0) {
                 const int64_t j = base + __popc(m & lt);
@@ -152,7 +152,7 @@ __global__ void unpack_kernel(PackedView p, int64_t n, int W, CT *__restrict__ d
 }
 
 template <typename CT>
-static PackedView pack_level(mc_tables *t, const void *dense, int W, cudaStream_t s, int64_t &stored)
+static PackedView pack_level(mc_tables *t, const Rows &dense, int W, cudaStream_t s, int64_t &stored)
 {
     const int64_t n = t->g->n;
     Arena scratch(true);
@@ -166,7 +166,7 @@ static PackedView pack_level(mc_tables *t, const void *dense, int W, cudaStream_
     p.width = (int)sizeof(CT);
     uint8_t *wid = t->varlen ? t->arena.get<uint8_t>((size_t)n) : nullptr;
     const int grid = grid_for(n * 32, 256);
-    MC_LAUNCH("pack", s, pack_count_kernel<CT><<<grid, 256, 0, s>>>((const CT *)dense, n, W, t->varlen ? 1 : 0, cnt,
+    MC_LAUNCH("pack", s, pack_count_kernel<CT><<<grid, 256, 0, s>>>(dense, n, W, t->varlen ? 1 : 0, cnt,
                                                                       bytes, wid));
     inclusive_scan_u128(cnt, n, err, scratch, s);
     inclusive_scan_u128(bytes, n, err, scratch, s);
@@ -188,7 +188,7 @@ static PackedView pack_level(mc_tables *t, const void *dense, int W, cudaStream_
     p.wid = wid;
     p.key = key;
     p.val = val;
-    MC_LAUNCH("pack", s, pack_fill_kernel<CT><<<grid, 256, 0, s>>>((const CT *)dense, n, W, p, key, val));
+    MC_LAUNCH("pack", s, pack_fill_kernel<CT><<<grid, 256, 0, s>>>(dense, n, W, p, key, val));
     stored += tail[0] * 2 + tail[1] + 16 * (n + 1) + (wid ? n : 0);
     return p;
 }
@@ -205,8 +205,9 @@ void pack_tables(mc_tables *t, cudaStream_t s)
             const int W = which ? t->geo.Ws[h] : t->geo.Wc[h];
             dense += n * W * (int64_t)cb;
             if (n == 0) continue;
-            PackedView p = t->bits == 64 ? pack_level<uint64_t>(t, D, W, s, stored)
-                                         : pack_level<u128>(t, D, W, s, stored);
+            const Rows R = t->rows(h, which);
+            PackedView p = t->bits == 64 ? pack_level<uint64_t>(t, R, W, s, stored)
+                                         : pack_level<u128>(t, R, W, s, stored);
             (which ? t->ps : t->pc)[h] = p;
             MC_CUDA(cudaStreamSynchronize(s));
             t->arena.release(D);

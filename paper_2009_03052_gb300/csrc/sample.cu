@@ -186,14 +186,14 @@ ClassCatalog *class_catalog(int h)
 // class graph with each node its own colour; the colourful h-treelets are
 // then exactly the spanning trees.  All classes go through one build, as a
 // disjoint union.
-__global__ void sigma_kernel(const uint64_t *c, int64_t n, int h, int W, const int8_t *unrooted_of,
+__global__ void sigma_kernel(Rows c, int64_t n, int h, int W, const int8_t *unrooted_of,
                              int nu, unsigned long long *acc)
 {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n * W;
          t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = t / W;
         const int s = (int)(t - v * W);  // one colour set (all colours) per shape
-        const uint64_t x = c[t];
+        const uint64_t x = entry_at<uint64_t>(c, v, s);
         if (x) atomicAdd(&acc[(v / h) * nu + unrooted_of[s]], (unsigned long long)x);
     }
 }
@@ -249,7 +249,7 @@ static void ensure_sigma(ClassCatalog *cc)
     MC_CUDA(cudaMemcpy(duo, uo.data(), uo.size(), cudaMemcpyHostToDevice));
     MC_CUDA(cudaMemset(dacc, 0, (size_t)ncls * nu * 8));
     const int W = t->geo.Wc[h];  // = r_h: one colour set
-    MC_LAUNCH("sigma", nullptr, sigma_kernel<<<grid_for(n * W, 256), 256>>>((const uint64_t *)t->c[h], n, h, W, duo, nu, dacc));
+    MC_LAUNCH("sigma", nullptr, sigma_kernel<<<grid_for(n * W, 256), 256>>>(t->rows(h, 0), n, h, W, duo, nu, dacc));
     std::vector<unsigned long long> acc((size_t)ncls * nu);
     MC_CUDA(cudaMemcpy(acc.data(), dacc, acc.size() * 8, cudaMemcpyDeviceToHost));
     cudaFree(duo);
@@ -275,11 +275,10 @@ ClassCatalog *class_catalog_sigma(int h)
 }
 
 // ---------------------------------------------------------------------------
-// Sampler: one warp per sample.
-//   step 0  X = uniform(R); v = first node whose inclusive prefix exceeds X
-//           (32-ary warp search); (T, C) = first entry of v's level-h row,
-//           in (shape id, colour mask) order, whose running sum exceeds the
-//           remainder (warp scan);
+// Sampler.
+//   step 0  X = uniform(R); v = first node whose inclusive prefix exceeds X;
+//           (T, C) = first entry of v's level-h row, in (shape id, colour
+//           mask) order, whose running sum exceeds the remainder;
 //   step s  for each decomposition node (T, C, x) in pre-order (T' before
 //           T''): Y = uniform(beta_T c(T_C, x)); the block of colour sets
 //           C'' (ascending mask) is found from the block weights
@@ -346,8 +345,8 @@ struct SampleArgs {
     const uint32_t *scol;
     const int32_t *coff;
     int64_t n;
-    const void *c[MAXK + 1];
-    const void *S[MAXK + 1];
+    Rows c[MAXK + 1], S[MAXK + 1];  // the levels of dense tables
+    uint32_t levels;            // the levels that have wide rows
     PackedView pc[MAXK + 1], ps[MAXK + 1];  // the levels of packed (succinct) tables
     const void *Sp[MAXK + 1];   // per level: inclusive prefix of each hub's chunk sums
     const int32_t *node_chunk0; // first chunk of a hub, -1 for other nodes
@@ -377,36 +376,54 @@ struct SampleArgs {
     unsigned long long *next;   // when set: warps take batches of 32 samples from this counter
                                 // (zero at launch) as they finish; else a fixed grid stride
     int ncls;
+    bool long_rows;             // adjacency offsets beyond 32 bits
     int *err;
 };
 
+// What the descent looks up by shape and by level, in shared memory: the
+// lanes of a warp are at different shapes and levels, and constant memory
+// serves one address at a time.
 struct SampleSmem {
     uint8_t crank[1 << (MAXK - 1)];
     uint8_t unrank[MAXK][36];
+    uint8_t pair[32];                   // per bit of the adjacency word: i | j << 4
+    uint2 shape[MAX_SHAPES];            // size | local id << 8 | beta << 16; T' | T'' << 8
+    uint4 level[2][MAXK + 1];           // c, S: first-plane base, row stride, N | has wide rows << 8
+    int r[MAXK + 1];                    // rooted shapes per size
 };
 
-// Entry idx of node x's level-h row of c or S: dense rows, or (PK) a binary
-// search of the packed row's keys.
-template <typename CT, bool PK>
-__device__ __forceinline__ CT c_at(const SampleArgs &a, int h, int64_t x, int idx)
-{
-    if constexpr (PK) return (CT)packed_get(a.pc[h], x, idx);
-    else return ((const CT *)a.c[h])[x * a.Wc[h] + idx];
-}
-template <typename CT, bool PK>
-__device__ __forceinline__ CT s_at(const SampleArgs &a, int h, int64_t x, int idx)
-{
-    if constexpr (PK) return (CT)packed_get(a.ps[h], x, idx);
-    else return ((const CT *)a.S[h])[x * a.Ws[h] + idx];
-}
+// Row x of level h of c (which = 0) or S (1): entry get(idx) of dense rows, or
+// (PK) by a binary search of the packed row's keys.
+template <typename CT, bool PK> struct RowRef {
+    const SampleArgs &a;
+    const uint8_t *low;
+    int64_t x;
+    int h, N, which;
+    bool wide;
+    __device__ __forceinline__ RowRef(const SampleArgs &a_, const SampleSmem &sm, int which_, int h_, int64_t x_)
+        : a(a_), low(nullptr), x(x_), h(h_), N(8), which(which_), wide(false)
+    {
+        if constexpr (!PK) {
+            const uint4 l = sm.level[which][h];
+            low = (const uint8_t *)(((uint64_t)l.y << 32) | l.x) + x * (uint64_t)l.z;
+            N = (int)(l.w & 255u);
+            if (l.w >> 8) wide = (rows().wide[x] & rows().bit) != 0;
+        }
+    }
+    __device__ __forceinline__ const Rows &rows() const { return which ? a.S[h] : a.c[h]; }
+    // entry idx of a row that is not wide
+    __device__ __forceinline__ CT get(int idx) const
+    {
+        if constexpr (PK) return (CT)packed_get(which ? a.ps[h] : a.pc[h], x, idx);
+        else return row_low_any<CT>(low, N, idx);
+    }
+};
 
-template <typename CT, typename V, bool PK>
-__device__ __forceinline__ V count_at(const SampleArgs &a, const SampleSmem &sm, int g, unsigned C, uint32_t x, int cx)
+// Entries of rows that may be wide (dense tables), out of line: few levels of
+// few tables have any, and the sampler is large for the instruction cache.
+template <typename CT> __device__ __noinline__ CT entry_wide(const SampleArgs &a, int which, int h, int64_t x, int idx)
 {
-    const int hg = a.sz[g];
-    if (hg == 1) return 1;
-    const unsigned rel = drop_colour(C & ~(1u << cx), cx);
-    return (V)c_at<CT, PK>(a, hg, x, sm.crank[rel] * a.R_[hg] + a.loc[g]);
+    return entry_at<CT>(which ? a.S[h] : a.c[h], x, idx);
 }
 
 __device__ __forceinline__ uint64_t quotient(uint64_t a, uint64_t b) { return a / b; }
@@ -415,16 +432,18 @@ __device__ __forceinline__ u128 quotient(u128 a, u128 b)
     return ((a >> 64) == 0 && (b >> 64) == 0) ? (u128)((uint64_t)a / (uint64_t)b) : a / b;
 }
 
-// the set bits of `rest` selected by index mask `im` (i-th bit of im picks
-// the i-th lowest set bit of rest)
-__device__ __forceinline__ unsigned deposit(unsigned im, unsigned rest)
+// The positions of a mask's set bits, four bits each, and the set bits that an
+// index mask selects (bit i of im: the i-th lowest).
+__device__ __forceinline__ uint32_t bit_positions(unsigned m)
+{
+    uint32_t p = 0;
+    for (int i = 0; m; ++i, m &= m - 1) p |= (uint32_t)(__ffs(m) - 1) << (4 * i);
+    return p;
+}
+__device__ __forceinline__ unsigned select_bits(unsigned im, uint32_t pos)
 {
     unsigned out = 0;
-    for (int i = 0; rest; ++i) {
-        const unsigned low = rest & (0u - rest);
-        if ((im >> i) & 1u) out |= low;
-        rest &= rest - 1;
-    }
+    for (; im; im &= im - 1) out |= 1u << ((pos >> (4 * (__ffs(im) - 1))) & 15u);
     return out;
 }
 
@@ -540,46 +559,6 @@ __device__ __forceinline__ void adjacent4(const int64_t *row_ptr, const uint32_t
     for (int i = 0; i < NQ; ++i) out[i] = i < nq && lo[i] < end[i] && col[lo[i]] == key[i];
 }
 
-// The same tests for pairs of a sample's nodes whose adjacency offsets
-// (rlo, degree rdg) were loaded once per node: qa, qb index nodes[].
-template <int NQ, bool CNT>
-__device__ __forceinline__ void adjacent_nodes(const uint32_t *col, const int64_t *rlo, const uint32_t *rdg,
-                                               const uint32_t *nodes, const uint32_t *qa, const uint32_t *qb,
-                                               int nq, bool *out, uint64_t &rb, uint64_t &rs)
-{
-    int64_t lo[NQ], hi[NQ], end[NQ];
-    uint32_t key[NQ];
-#pragma unroll
-    for (int i = 0; i < NQ; ++i) {
-        if (i < nq) {
-            uint32_t x = qa[i], y = qb[i];
-            if (rdg[y] < rdg[x]) { const uint32_t t = x; x = y; y = t; }
-            lo[i] = rlo[x];
-            hi[i] = lo[i] + rdg[x];
-            end[i] = hi[i];
-            key[i] = nodes[y];
-            MC_COUNT(4, 32);  // the final probe
-        } else {
-            lo[i] = hi[i] = end[i] = 0;
-            key[i] = 0;
-        }
-    }
-    bool more = true;
-    while (more) {
-        more = false;
-#pragma unroll
-        for (int i = 0; i < NQ; ++i)
-            if (lo[i] < hi[i]) {
-                const int64_t mid = (lo[i] + hi[i]) >> 1;
-                if (col[mid] < key[i]) lo[i] = mid + 1; else hi[i] = mid;
-                MC_COUNT(4, 32);
-                more |= lo[i] < hi[i];
-            }
-    }
-#pragma unroll
-    for (int i = 0; i < NQ; ++i) out[i] = i < nq && lo[i] < end[i] && col[lo[i]] == key[i];
-}
-
 // Lane-per-sample sampler: the 32 lanes of a warp draw 32 samples and walk
 // their h-1 decomposition steps in lockstep (every h-treelet has h-1 internal
 // decomposition nodes).  A lane does its own scalar work, short scans and
@@ -587,32 +566,63 @@ __device__ __forceinline__ void adjacent_nodes(const uint32_t *col, const int64_
 // tables' count type; V: the type of the descent's weights, draws and
 // running sums (64 bits when every level total leaves room for beta, else
 // 128 bits).
+//
+// A sample's node list, its stack of decomposition nodes (one word each:
+// shape, colour set, root colour, root's place in the node list) and the
+// adjacency offsets of its nodes live in shared memory, one column per
+// thread: indexed per lane, they would be local memory, whose 464 bytes per
+// thread times 1536 threads per SM passed through L1 and L2 beside the
+// tables (half a gigabyte of DRAM writes per million samples).
+//
+// Bound by the latency of dependent random reads.  Occupancy target: 3 blocks
+// of 512 per SM, 2 for 128-bit counts in dense tables (a wider state: 15.7
+// against 22.7 ms for the launches of a 2M-sample adaptive run at k = 7 on
+// R-MAT 19; packed rows 0.94 against 1.15 ms the other way, 200k samples,
+// k = 6); 4 items in flight (8: 1.19-1.46 against 1.09 ms per 1M samples of
+// Chung-Lu 1M, k = 5).  LAT (launches too
+// small to fill the GPU, e.g. the batches of AGS): no register cap, 16 items
+// of a scan and 8 adjacency searches in flight per lane, so each sample's
+// chain of dependent loads is shorter.  The samples are the same in both
+// modes.
+constexpr int SAMPLE_WORDS = 3 * MAXK;  // shared words per thread
+constexpr int SAMPLE_BLOCK = 512, SAMPLE_BLOCK_LAT = 64;
 
-// Occupancy target: 6 blocks of 256 per SM for 64-bit counts, 4 for 128-bit
-// ones (their wider state spills less; measured faster on both workloads).
-// LAT (launches too small to fill the GPU, e.g. the batches of AGS): no
-// register cap, 16 items of a scan and 8 adjacency searches in flight per
-// lane, so each sample's chain of dependent loads is shorter.  The samples
-// are the same in both modes.
 template <typename CT, typename V, bool PK, bool LAT, bool CNT>
-__global__ void __launch_bounds__(256, LAT ? 1 : (sizeof(CT) == 16 ? 4 : 6))
+__global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1 : (sizeof(CT) == 16 && !PK ? 2 : 3))
     sample_kernel(const __grid_constant__ SampleArgs a)
 {
     constexpr int NW = LAT ? 16 : 4;  // items of a scan in flight
     constexpr int NQ = LAT ? 8 : 4;   // adjacency searches in flight
     constexpr int KS = LAT ? 8 : 1;   // probes per round of the root and hub chunk searches
-    extern __shared__ unsigned int s_hist[];
+    constexpr int T = LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
+    extern __shared__ uint32_t s_dyn[];
+    uint32_t *const stk = s_dyn + threadIdx.x;             // entry i at i * T; after the descent the degrees
+    uint32_t *const nod = s_dyn + MAXK * T + threadIdx.x;  // the nodes, in order of discovery
+    uint32_t *const off = s_dyn + 2 * MAXK * T + threadIdx.x;  // their adjacency offsets (low words)
+    unsigned int *const s_hist = s_dyn + SAMPLE_WORDS * T;
     __shared__ SampleSmem sm;
-    for (int i = threadIdx.x; i < (1 << (MAXK - 1)); i += blockDim.x) sm.crank[i] = a.crank[i];
-    for (int i = threadIdx.x; i < MAXK * 36; i += blockDim.x) (&sm.unrank[0][0])[i] = (&a.unrank[0][0])[i];
+    for (int i = threadIdx.x; i < (1 << (MAXK - 1)); i += T) sm.crank[i] = a.crank[i];
+    for (int i = threadIdx.x; i < MAXK * 36; i += T) (&sm.unrank[0][0])[i] = (&a.unrank[0][0])[i];
+    for (int i = threadIdx.x; i < MAX_SHAPES; i += T)
+        sm.shape[i] = make_uint2((uint32_t)a.sz[i] | (uint32_t)a.loc[i] << 8 | (uint32_t)a.beta[i] << 16,
+                                 (uint32_t)a.lft[i] | (uint32_t)a.rgt[i] << 8);
+    for (int i = threadIdx.x; i < 2 * (MAXK + 1); i += T) {
+        const int l = i % (MAXK + 1);
+        const Rows &r = i > MAXK ? a.S[l] : a.c[l];
+        sm.level[i / (MAXK + 1)][l] = make_uint4((uint32_t)(uint64_t)r.p0, (uint32_t)((uint64_t)r.p0 >> 32), (uint32_t)r.s0,
+                                                 (uint32_t)r.N | ((a.levels & r.bit) ? 256u : 0u));
+        if (i <= MAXK) sm.r[l] = a.R_[l];
+    }
+    const int h = a.h, P = h * (h - 1) / 2;
+    if (threadIdx.x < P)
+        sm.pair[pair_pos(h, a.pi[threadIdx.x], a.pj[threadIdx.x])] = (uint8_t)(a.pi[threadIdx.x] | a.pj[threadIdx.x] << 4);
     if (a.hist)
-        for (int i = threadIdx.x; i < a.ncls; i += blockDim.x) s_hist[i] = 0;
+        for (int i = threadIdx.x; i < a.ncls; i += T) s_hist[i] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int h = a.h;
-    const int CB = (int)sizeof(CT);
+    const int64_t warp = (blockIdx.x * (int64_t)T + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * T) >> 5;
+    constexpr int CB = (int)sizeof(CT);
     bool bad = false;
     uint64_t rb = 0, rs = 0;  // byte counts (CNT): data items, 32-byte sectors
     // a warp's next batch of 32 samples: from the shared counter (the warps
@@ -624,247 +634,325 @@ __global__ void __launch_bounds__(256, LAT ? 1 : (sizeof(CT) == 16 ? 4 : 6))
         if (lane == 0) b = atomicAdd(a.next, 32ull);
         return (int64_t)__shfl_sync(0xffffffffu, b, 0);
     };
+    auto entry = [](int g, unsigned C, int cx, int at) {
+        return (uint32_t)g | C << 8 | (uint32_t)cx << 16 | (uint32_t)at << 20;
+    };
     for (int64_t base = take(-1); base < a.count; base = take(base)) {
         const int64_t sid = base + lane;
         bool ok = sid < a.count;
         uint64_t index = a.first_index + (uint64_t)sid;
-        const u128 *prefix = a.prefix;
-        const uint32_t *bucket = a.bucket;
-        u128 R = a.R, Xbase = a.Xbase, D = a.D;
-        uint64_t allow0 = a.allow0, allow1 = a.allow1;
-        if (a.nseg > 0 && ok) {  // the part this sample falls in
-            int g = 0;
-            while (g + 1 < a.nseg && sid >= a.seg[g].end) ++g;
-            const SampleSeg &sg = a.seg[g];
-            index = sg.first_index + (uint64_t)(sid - (g ? a.seg[g - 1].end : 0));
-            prefix = sg.prefix;
-            bucket = sg.bucket;
-            R = sg.R;
-            Xbase = sg.Xbase;
-            D = sg.D;
-            allow0 = sg.allow0;
-            allow1 = sg.allow1;
-        }
-        // ---- root: X = uniform(R); v = first node with prefix[v] > X, found
-        // by binary search inside the bucket of X
-        V X = 0;
         uint32_t v = 0;
-        if (ok && !draw_below(a.seed, index, 0, (V)R, X)) { ok = false; bad = true; }
-        X += (V)Xbase;  // a node range: the draw lands inside its part of the prefix
-        if (ok) {
-            const uint64_t bk = (uint64_t)(X / (V)D);
-            const int64_t blo = bucket[bk], bhi = bucket[bk + 1];
-            MC_COUNT(8, 32);
-            const int64_t lo = first_true<KS>(
-                blo, bhi, [&](int64_t i) { return prefix[i] > (u128)X; }, [&] { MC_COUNT(16, 32); });
-            MC_COUNT(32, 32);  // the check below and prefix[v - 1]
-            v = (uint32_t)lo;
-            if (!(prefix[v] > (u128)X)) { ok = false; bad = true; }
-        }
-        // ---- entry of v's level-h row, in (shape id, colour mask) order
-        int s0 = 0, cv0 = 0;
-        unsigned C0 = 0;
-        if (ok) {
-            const V rem = X - (v ? (V)prefix[v - 1] : (V)0);
-            const int Bc = a.Bc[h], Rh = a.R_[h];
-            V bf;
-            // e runs in (shape id, colour mask) order; the row is set-major
-            const int found = lane_first_exceeding<NW, V>(a.Wc[h], rem, [&](int e) -> V {
-                const int sh = e / Bc;
-                const bool al = sh < 64 ? (allow0 >> sh) & 1 : (allow1 >> (sh - 64)) & 1;
-                MC_COUNT(al ? CB : 0, al ? CB : 0);  // one contiguous row
-                return al ? (V)c_at<CT, PK>(a, h, v, (e - sh * Bc) * Rh + sh) : (V)0;
-            }, bf);
-            if (found < 0) { ok = false; bad = true; }
-            else {
-                cv0 = a.colors[v];
-                s0 = found / Bc;
-                C0 = (1u << cv0) | insert_colour_gap(sm.unrank[h - 1][found % Bc], cv0);
+        int s0 = 0, sp = 0, nn = 0;
+        uint32_t par = 0;  // per node, four bits: its parent's place in the node list
+        {
+            const u128 *prefix = a.prefix;
+            const uint32_t *bucket = a.bucket;
+            u128 R = a.R, Xbase = a.Xbase, D = a.D;
+            uint64_t allow0 = a.allow0, allow1 = a.allow1;
+            if (a.nseg > 0 && ok) {  // the part this sample falls in
+                int g = 0;
+                while (g + 1 < a.nseg && sid >= a.seg[g].end) ++g;
+                const SampleSeg &sg = a.seg[g];
+                index = sg.first_index + (uint64_t)(sid - (g ? a.seg[g - 1].end : 0));
+                prefix = sg.prefix;
+                bucket = sg.bucket;
+                R = sg.R;
+                Xbase = sg.Xbase;
+                D = sg.D;
+                allow0 = sg.allow0;
+                allow1 = sg.allow1;
+            }
+            // ---- root: X = uniform(R); v = first node with prefix[v] > X, found
+            // by binary search inside the bucket of X
+            V X = 0;
+            if (ok && !draw_below(a.seed, index, 0, (V)R, X)) { ok = false; bad = true; }
+            X += (V)Xbase;  // a node range: the draw lands inside its part of the prefix
+            if (ok) {
+                const uint64_t bk = (uint64_t)(X / (V)D);
+                const int64_t blo = bucket[bk], bhi = bucket[bk + 1];
+                MC_COUNT(8, 32);
+                const int64_t lo = first_true<KS>(
+                    blo, bhi, [&](int64_t i) { return prefix[i] > (u128)X; }, [&] { MC_COUNT(16, 32); });
+                MC_COUNT(32, 32);  // the check below and prefix[v - 1]
+                v = (uint32_t)lo;
+                if (!(prefix[v] > (u128)X)) { ok = false; bad = true; }
+            }
+            // ---- entry of v's level-h row, in (shape id, colour mask) order
+            if (ok) {
+                const V rem = X - (v ? (V)prefix[v - 1] : (V)0);
+                const int Bc = a.Bc[h], Rh = a.R_[h];
+                const RowRef<CT, PK> row(a, sm, 0, h, v);
+                V bf;
+                // e runs in (shape id, colour mask) order; the row is set-major
+                auto scan = [&](auto at) {
+                    return lane_first_exceeding<NW, V>(a.Wc[h], rem, [&](int e) -> V {
+                        const int sh = e / Bc;
+                        const bool al = sh < 64 ? (allow0 >> sh) & 1 : (allow1 >> (sh - 64)) & 1;
+                        MC_COUNT(al ? CB : 0, al ? CB : 0);  // one contiguous row
+                        return al ? (V)at((e - sh * Bc) * Rh + sh) : (V)0;
+                    }, bf);
+                };
+                const int found = !PK && row.wide ? scan([&](int i) { return entry_wide<CT>(a, 0, h, v, i); })
+                                                  : scan([&](int i) { return row.get(i); });
+                if (found < 0) { ok = false; bad = true; }
+                else {
+                    const int cv = a.colors[v];
+                    s0 = found / Bc;
+                    const unsigned C = (1u << cv) | insert_colour_gap(sm.unrank[h - 1][found % Bc], cv);
+                    stk[0] = entry(a.first[h] + s0, C, cv, 0);
+                    nod[0] = v;
+                    sp = nn = 1;
+                }
             }
         }
         // ---- descent: decomposition nodes in pre-order (T' before T'')
-        int stg[MAXK], stc[MAXK], sp = 0, nn = 0, ne = 0;
-        unsigned stC[MAXK];
-        uint32_t stx[MAXK], nodes[MAXK], ea[MAXK], eb[MAXK];
-        if (ok) { stg[0] = a.first[h] + s0; stC[0] = C0; stx[0] = v; stc[0] = cv0; sp = 1; }
         for (uint32_t step = 1; step < (uint32_t)h; ++step) {
-            int g = 0, cx = 0;
-            unsigned C = 0;
-            uint32_t x = 0;
-            if (ok) {  // leaves on top of the stack are sample nodes
+            uint2 sg = make_uint2(0, 0);
+            uint32_t en = 0, x = 0;
+            if (ok) {  // leaves on top of the stack are done
                 for (;;) {
                     if (sp <= 0 || nn >= MAXK) { ok = false; bad = true; break; }
-                    --sp;
-                    g = stg[sp]; C = stC[sp]; x = stx[sp]; cx = stc[sp];
-                    if (a.sz[g] > 1) break;
-                    nodes[nn++] = x;
+                    en = stk[--sp * T];
+                    sg = sm.shape[en & 255u];
+                    if ((sg.x & 255u) > 1) break;
                 }
             }
-            int ga = 0, gb = 0, hb = 1, sbase = 0, sidx = 0, chunk0 = -1;
-            unsigned C1 = 0, C2 = 0;
-            int64_t e0 = 0, e1 = 0, nch = 0;
+            const int cx = (int)(en >> 16 & 15u), at = (int)(en >> 20);
+            const unsigned C = en >> 8 & 255u;
+            int ga = 0, gb = 0, hb = 1, lb = 0, sidx = 0, chunk0 = -1;
+            unsigned C2 = 0;
+            int64_t e0 = 0, deg = 0;
             CT q = 0;
             if (ok) {
-                ga = a.lft[g]; gb = a.rgt[g]; hb = a.sz[gb];
+                x = nod[at * T];
+                ga = (int)(sg.y & 255u);
+                gb = (int)(sg.y >> 8 & 255u);
+                const uint32_t sa = sm.shape[ga].x, sb = sm.shape[gb].x;
+                const int hg = (int)(sg.x & 255u), ha = (int)(sa & 255u), la = (int)(sa >> 8 & 255u);
+                hb = (int)(sb & 255u);
+                lb = (int)(sb >> 8 & 255u);
                 MC_COUNT(16 + 4 + CB, 96);  // row offsets, first chunk, c(T_C, x)
                 e0 = a.row_ptr[x];
-                e1 = a.row_ptr[x + 1];
+                deg = a.row_ptr[x + 1] - e0;
                 chunk0 = a.node_chunk0[x];
-                const V W = (V)a.beta[g] * count_at<CT, V, PK>(a, sm, g, C, x, cx);
+                // colour sets relative to x: c_x deleted from the palette
+                const unsigned rest = drop_colour(C & ~(1u << cx), cx);
                 V Y = 0;
+                const RowRef<CT, PK> rg(a, sm, 0, hg, x);
+                const int ig = sm.crank[rest] * sm.r[hg] + (int)(sg.x >> 8 & 255u);
+                const V W = (V)(sg.x >> 16 & 255u) * (V)(!PK && rg.wide ? entry_wide<CT>(a, 0, hg, x, ig) : rg.get(ig));
                 if (!draw_below(a.seed, index, step, W, Y)) { ok = false; bad = true; }
                 if (ok) {
                     // block of C'' (ascending mask), weights c(T'_{C\C''}, x) S(T'', C'', x)
-                    const unsigned rest = C & ~(1u << cx);
+                    const uint32_t pos = bit_positions(rest);
                     const int nr = __popc(rest);
                     int nsub = 1;
                     for (int i = 1; i <= hb; ++i) nsub = nsub * (nr - hb + i) / i;
-                    sbase = a.loc[gb];
-                    const int Rb = a.R_[hb];
+                    const int Ra = sm.r[ha], Rb = sm.r[hb];
+                    const RowRef<CT, PK> ra(a, sm, 0, ha, x), rb_(a, sm, 1, hb, x);
+                    const bool wide = !PK && (ra.wide || rb_.wide);
+                    auto index_a = [&](unsigned c2) { return sm.crank[rest & ~c2] * Ra + la; };
                     V before;
-                    const int blk = lane_first_exceeding<NW, V>(nsub, Y, [&](int i) -> V {
-                        const unsigned c2 = deposit(sm.unrank[hb][i], rest);
-                        MC_COUNT(2 * CB, 64);
-                        return count_at<CT, V, PK>(a, sm, ga, C & ~c2, x, cx) *
-                               (V)s_at<CT, PK>(a, hb, x, sm.crank[drop_colour(c2, cx)] * Rb + sbase);
-                    }, before);
+                    auto scan = [&](auto at_a, auto at_b) {
+                        return lane_first_exceeding<NW, V>(nsub, Y, [&](int i) -> V {
+                            const unsigned c2 = select_bits(sm.unrank[hb][i], pos);
+                            MC_COUNT(2 * CB, 64);
+                            return (ha == 1 ? (V)1 : (V)at_a(index_a(c2))) * (V)at_b(sm.crank[c2] * Rb + lb);
+                        }, before);
+                    };
+                    const int blk = wide ? scan([&](int i) { return entry_wide<CT>(a, 0, ha, x, i); },
+                                                [&](int i) { return entry_wide<CT>(a, 1, hb, x, i); })
+                                         : scan([&](int i) { return ra.get(i); }, [&](int i) { return rb_.get(i); });
                     if (blk < 0) { ok = false; bad = true; }
                     else {
-                        C2 = deposit(sm.unrank[hb][blk], rest);
-                        C1 = C & ~C2;
-                        const V x1 = count_at<CT, V, PK>(a, sm, ga, C1, x, cx);
+                        const unsigned c2 = select_bits(sm.unrank[hb][blk], pos);
+                        C2 = insert_colour_gap(c2, cx);
+                        const V x1 = ha == 1 ? (V)1
+                                             : (V)(wide ? entry_wide<CT>(a, 0, ha, x, index_a(c2)) : ra.get(index_a(c2)));
                         q = (CT)quotient(Y - before, x1);  // < S(T'', C'', x): fits CT
-                        sidx = sm.crank[drop_colour(C2, cx)] * a.R_[hb] + sbase;
-                        if (chunk0 >= 0) nch = (e1 - e0 + HUB_CHUNK - 1) / HUB_CHUNK;
+                        sidx = sm.crank[c2] * Rb + lb;
                     }
                 }
             }
-            // ---- hub: the 64-neighbour chunk holding the answer, from the
-            // inclusive prefix of its chunk sums (contiguous per hub and entry)
-            // T'' one node: c(T''_{C''}, u) is 1 for the neighbours of the one
-            // colour of C'' and 0 otherwise, so the answer is the (q+1)-th
-            // neighbour of that colour in ascending id order: position q of
-            // that colour's block in the colour-sorted adjacency
-            const bool single = ok && hb == 1;
-            const bool chunked = ok && !single && chunk0 >= 0;
-            const CT *spp = nullptr;
-            if (chunked) spp = (const CT *)a.Sp[hb] + (int64_t)chunk0 * a.Ws[hb] + (int64_t)sidx * nch;
-            int64_t ci = -1;
-            CT bc = 0;
-            if (chunked) {
-                // the first chunk whose inclusive prefix exceeds q: a binary
-                // search of the hub's chunk prefix sums for this S entry
-                const int64_t lo = first_true<KS>(
-                    0, nch - 1, [&](int64_t i) { return spp[i] > q; }, [&] { MC_COUNT(CB, 32); });
-                MC_COUNT(2 * CB, 32);
-                if (spp[lo] > q) { ci = lo; bc = lo ? spp[lo - 1] : (CT)0; }
-            }
-            int64_t lo_e = e0, hi_e = e1;
-            CT qq = q;
-            if (chunked) {
-                if (ci < 0) { ok = false; bad = true; }
-                else {
-                    lo_e = e0 + ci * HUB_CHUNK;
-                    hi_e = min(e1, lo_e + HUB_CHUNK);
-                    qq = q - bc;
-                }
-            }
-            // ---- neighbour: first u (ascending) whose running sum of
-            // c(T''_{C''}, u) exceeds qq (at most HUB_CHUNK neighbours)
-            if (single) {
-                const int col2 = __ffs(C2) - 1;
-                const int32_t b0 = a.coff[(int64_t)x * (a.k + 1) + col2];
-                const int32_t b1 = a.coff[(int64_t)x * (a.k + 1) + col2 + 1];
+            uint32_t u = 0;
+            int cu = 0;
+            if (ok && hb == 1) {
+                // T'' one node: c(T''_{C''}, u) is 1 for the neighbours of the one
+                // colour of C'' and 0 otherwise, so the answer is the (q+1)-th
+                // neighbour of that colour in ascending id order: position q of
+                // that colour's block in the colour-sorted adjacency
+                cu = __ffs(C2) - 1;
+                const int32_t b0 = a.coff[(int64_t)x * (a.k + 1) + cu];
+                const int32_t b1 = a.coff[(int64_t)x * (a.k + 1) + cu + 1];
                 MC_COUNT(8 + 4, 64);
-                if ((uint64_t)q >= (uint64_t)(b1 - b0) || sp + 2 > MAXK || ne >= MAXK) { ok = false; bad = true; }
-                else {
-                    const uint32_t u = a.scol[e0 + b0 + (int64_t)q];
-                    ea[ne] = x; eb[ne] = u; ++ne;
-                    stg[sp] = gb; stC[sp] = C2; stx[sp] = u; stc[sp] = col2; ++sp;
-                    stg[sp] = ga; stC[sp] = C1; stx[sp] = x; stc[sp] = cx; ++sp;
-                }
+                if ((uint64_t)q >= (uint64_t)(b1 - b0)) { ok = false; bad = true; }
+                else u = a.scol[e0 + b0 + (int64_t)q];
             } else if (ok) {
-                int64_t sel = -1;
-                {
-                    const int lb = a.loc[gb];
-                    const int rcb = a.R_[hb];
-                    CT bn;
-                    const int r = lane_first_exceeding<NW, CT>((int)(hi_e - lo_e), qq, [&](int i) -> CT {
-                        const int cu = a.ecol[lo_e + i];
-                        MC_COUNT(1, 1);  // contiguous edge colours
-                        if (!((C2 >> cu) & 1u)) return (CT)0;
-                        MC_COUNT(4 + CB, 4 + 32);  // contiguous ids; the neighbour's row entry
-                        const uint32_t u = a.col[lo_e + i];
-                        return c_at<CT, PK>(a, hb, u, sm.crank[drop_colour(C2 & ~(1u << cu), cu)] * rcb + lb);
-                    }, bn);
-                    if (r >= 0) sel = lo_e + r;
+                // ---- hub: the 64-neighbour chunk holding the answer, from the
+                // inclusive prefix of its chunk sums (contiguous per hub and entry):
+                // the first chunk whose prefix exceeds q
+                int64_t lo_e = e0;
+                int64_t len = deg;
+                if (chunk0 >= 0) {
+                    const int64_t nch = (deg + HUB_CHUNK - 1) / HUB_CHUNK;
+                    const CT *spp = (const CT *)a.Sp[hb] + (int64_t)chunk0 * a.Ws[hb] + (int64_t)sidx * nch;
+                    const int64_t ci = first_true<KS>(
+                        0, nch - 1, [&](int64_t i) { return spp[i] > q; }, [&] { MC_COUNT(CB, 32); });
+                    MC_COUNT(2 * CB, 32);
+                    if (!(spp[ci] > q)) { ok = false; bad = true; }
+                    else {
+                        lo_e = e0 + ci * HUB_CHUNK;
+                        len = min((int64_t)HUB_CHUNK, deg - ci * HUB_CHUNK);
+                        q -= ci ? spp[ci - 1] : (CT)0;
+                    }
                 }
-                if (sel < 0 || sp + 2 > MAXK || ne >= MAXK) { ok = false; bad = true; }
+                // ---- neighbour: first u (ascending) whose running sum of
+                // c(T''_{C''}, u) exceeds q (at most HUB_CHUNK neighbours)
+                int r = -1;
+                if (ok) {
+                    const int rcb = sm.r[hb];
+                    const uint32_t *ids = a.col + lo_e;
+                    const uint8_t *cols = a.ecol + lo_e;
+                    auto index_of = [&](int ci) { return sm.crank[drop_colour(C2 & ~(1u << ci), ci)] * rcb + lb; };
+                    CT bn;
+                    if constexpr (PK) {
+                        r = lane_first_exceeding<NW, CT>((int)len, q, [&](int i) -> CT {
+                            const int ci = cols[i];
+                            return ((C2 >> ci) & 1u) ? RowRef<CT, PK>(a, sm, 0, hb, ids[i]).get(index_of(ci)) : (CT)0;
+                        }, bn);
+                    } else if (sm.level[0][hb].w >> 8) {  // the level has wide rows
+                        r = lane_first_exceeding<NW, CT>((int)len, q, [&](int i) -> CT {
+                            const int ci = cols[i];
+                            return ((C2 >> ci) & 1u) ? entry_wide<CT>(a, 0, hb, ids[i], index_of(ci)) : (CT)0;
+                        }, bn);
+                    } else {
+                        // ids and colours of NW neighbours together, then the entries of
+                        // those whose colour is in C'', all in flight
+                        const uint4 lv = sm.level[0][hb];
+                        const uint8_t *p0 = (const uint8_t *)(((uint64_t)lv.y << 32) | lv.x);
+                        const int n = (int)len, N = (int)lv.w;
+                        CT run = 0;
+                        for (int b = 0; b < n && r < 0; b += NW) {
+                            uint32_t id[NW];
+                            int ci[NW];
+                            CT y[NW];
+#pragma unroll
+                            for (int i = 0; i < NW; ++i) {
+                                const int k2 = min(b + i, n - 1);
+                                ci[i] = cols[k2];
+                                id[i] = ids[k2];
+                            }
+#pragma unroll
+                            for (int i = 0; i < NW; ++i) {
+                                const bool in = b + i < n && ((C2 >> ci[i]) & 1u);
+                                MC_COUNT(5, 5);  // contiguous edge colours and ids
+                                if (in) MC_COUNT(CB, 32);  // the neighbour's row entry
+                                y[i] = in ? row_low_any<CT>(p0 + id[i] * (uint64_t)lv.z, N, index_of(ci[i])) : (CT)0;
+                            }
+#pragma unroll
+                            for (int i = 0; i < NW; ++i)
+                                if (r < 0) {
+                                    if (run + y[i] > q) { r = b + i; u = id[i]; cu = ci[i]; }
+                                    else run += y[i];
+                                }
+                        }
+                    }
+                }
+                if (r < 0) { ok = false; bad = true; }
+                else if (PK || (sm.level[0][hb].w >> 8)) {
+                    u = a.col[lo_e + r];
+                    cu = a.ecol[lo_e + r];
+                }
+            }
+            if (ok) {
+                if (sp + 2 > MAXK) { ok = false; bad = true; }
                 else {
-                    const uint32_t u = a.col[sel];
-                    const int cu = a.ecol[sel];
-                    ea[ne] = x; eb[ne] = u; ++ne;   // a treelet edge: adjacent for sure
-                    stg[sp] = gb; stC[sp] = C2; stx[sp] = u; stc[sp] = cu; ++sp;
-                    stg[sp] = ga; stC[sp] = C1; stx[sp] = x; stc[sp] = cx; ++sp;
+                    nod[nn * T] = u;
+                    par |= (uint32_t)at << (4 * nn);
+                    stk[sp * T] = entry(gb, C2, cu, nn);
+                    stk[(sp + 1) * T] = entry(ga, C & ~C2, cx, at);
+                    sp += 2;
+                    ++nn;
                 }
             }
         }
-        if (ok) {  // remaining leaves
-            while (sp > 0 && nn < MAXK) { --sp; nodes[nn++] = stx[sp]; }
-            if (nn != h || sp != 0) { ok = false; bad = true; }
-        }
+        if (ok && nn != h) { ok = false; bad = true; }
         int cls = -1;
         if (ok) {
-            for (int i = 1; i < h; ++i)
-                for (int j = i; j > 0 && nodes[j - 1] > nodes[j]; --j) {
-                    const uint32_t tmp = nodes[j]; nodes[j] = nodes[j - 1]; nodes[j - 1] = tmp;
-                }
-            // induced subgraph: the treelet's edges are known; the other pairs
-            // are tested against the adjacency lists, four at a time
-            const int P = h * (h - 1) / 2;
-            uint32_t word = 0, known = 0;
-            for (int t = 0; t < ne; ++t) {
-                int i = 0, j = 0;
-                for (int p = 0; p < h; ++p) {
-                    if (nodes[p] == ea[t]) i = p;
-                    if (nodes[p] == eb[t]) j = p;
-                }
-                if (i > j) { const int tmp = i; i = j; j = tmp; }
-                known |= 1u << pair_pos(h, i, j);
-            }
-            word = known;
-            int64_t rlo[MAXK];  // adjacency offsets and degrees, loaded once per node
-            uint32_t rdg[MAXK];
+            // induced subgraph, its nodes in order of discovery (the class does
+            // not depend on the labels): the treelet's edges are known; the other
+            // pairs are searched in the shorter adjacency list, NQ at a time
+            uint32_t word = 0;
+            for (int i = 1; i < h; ++i) word |= 1u << pair_pos(h, (int)(par >> (4 * i) & 15u), i);
             for (int i = 0; i < h; ++i) {
-                rlo[i] = a.row_ptr[nodes[i]];
-                rdg[i] = (uint32_t)(a.row_ptr[nodes[i] + 1] - rlo[i]);
+                const uint32_t x = nod[i * T];
+                const int64_t lo = a.row_ptr[x];
+                off[i * T] = (uint32_t)lo;
+                stk[i * T] = (uint32_t)(a.row_ptr[x + 1] - lo);
                 MC_COUNT(16, 32);
             }
-            uint32_t qa[NQ], qb[NQ];
-            int qp[NQ], nq = 0;
-            for (int p = 0; p < P; ++p) {
-                const int i = a.pi[p], j = a.pj[p];
-                const int bit = pair_pos(h, i, j);
-                if ((known >> bit) & 1u) continue;
-                qa[nq] = i; qb[nq] = j; qp[nq] = bit; ++nq;
-                if (nq == NQ || p == P - 1) {
-                    bool r4[NQ];
-                    adjacent_nodes<NQ, CNT>(a.col, rlo, rdg, nodes, qa, qb, nq, r4, rb, rs);
-                    for (int t = 0; t < nq; ++t)
-                        if (r4[t]) word |= 1u << qp[t];
-                    nq = 0;
+            uint32_t todo = ((1u << P) - 1u) & ~word;
+            while (todo) {
+                const uint32_t *row[NQ];
+                uint32_t lo[NQ], hi[NQ], key[NQ], bit[NQ];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    lo[q] = hi[q] = key[q] = 0;
+                    row[q] = a.col;
+                    bit[q] = todo & (0u - todo);
+                    if (!bit[q]) continue;
+                    todo &= todo - 1;
+                    const unsigned ij = sm.pair[__ffs(bit[q]) - 1];
+                    int x = (int)(ij & 15u), y = (int)(ij >> 4);
+                    uint32_t dx = stk[x * T];
+                    const uint32_t dy = stk[y * T];
+                    if (dy < dx) { const int t = x; x = y; y = t; dx = dy; }
+                    hi[q] = dx;
+                    key[q] = nod[y * T];
+                    row[q] = a.col + (a.long_rows ? a.row_ptr[nod[x * T]] : (int64_t)off[x * T]);
                 }
-            }
-            if (nq) {
-                bool r4[NQ];
-                adjacent_nodes<NQ, CNT>(a.col, rlo, rdg, nodes, qa, qb, nq, r4, rb, rs);
-                for (int t = 0; t < nq; ++t)
-                    if (r4[t]) word |= 1u << qp[t];
+                bool more = true;
+                while (more) {
+                    more = false;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q)
+                        if (lo[q] < hi[q]) {
+                            const uint32_t mid = (lo[q] + hi[q]) >> 1;
+                            const uint32_t w = row[q][mid];
+                            MC_COUNT(4, 32);
+                            if (w == key[q]) { word |= bit[q]; hi[q] = lo[q]; }
+                            else if (w < key[q]) lo[q] = mid + 1;
+                            else hi[q] = mid;
+                            more |= lo[q] < hi[q];
+                        }
+                }
             }
             cls = a.lut[word];
             MC_COUNT(2, 32);
             if (cls == 0xffff) { cls = -1; bad = true; }
-            if (a.nodes) for (int i = 0; i < h; ++i) a.nodes[sid * h + i] = nodes[i];
+            if (a.nodes) {
+                // ascending: an odd-even merge sort of 8, absent nodes last
+                uint32_t n_[MAXK];
+#pragma unroll
+                for (int i = 0; i < MAXK; ++i) n_[i] = i < h ? nod[i * T] : 0xffffffffu;
+                auto order = [&](int i, int j) {
+                    const uint32_t lo = min(n_[i], n_[j]), hi = max(n_[i], n_[j]);
+                    n_[i] = lo;
+                    n_[j] = hi;
+                };
+#pragma unroll
+                for (int p = 1; p < MAXK; p <<= 1)
+#pragma unroll
+                    for (int k2 = p; k2 >= 1; k2 >>= 1)
+#pragma unroll
+                        for (int j = k2 % p; j + k2 < MAXK; j += 2 * k2)
+#pragma unroll
+                            for (int i = 0; i < k2; ++i)
+                                if (i + j + k2 < MAXK && (i + j) / (2 * p) == (i + j + k2) / (2 * p)) order(i + j, i + j + k2);
+#pragma unroll
+                for (int i = 0; i < MAXK; ++i)
+                    if (i < h) a.nodes[sid * h + i] = n_[i];
+            }
             if (a.roots) a.roots[sid] = v;
             if (a.shapes) a.shapes[sid] = s0;
             {
@@ -889,7 +977,7 @@ __global__ void __launch_bounds__(256, LAT ? 1 : (sizeof(CT) == 16 ? 4 : 6))
     }
     if (a.hist) {
         __syncthreads();
-        for (int i = threadIdx.x; i < a.ncls; i += blockDim.x)
+        for (int i = threadIdx.x; i < a.ncls; i += T)
             if (s_hist[i]) atomicAdd(&a.hist[i], (unsigned long long)s_hist[i]);
     }
 }
@@ -1058,10 +1146,11 @@ static void fill_sample_args(SampleArgs &a, const mc_tables *t, int h)
     a.scol = t->scol;
     a.coff = t->coff;
     a.n = g->n;
+    a.long_rows = g->nnz > 0xffffffffll;
     a.node_chunk0 = g->node_chunk0;
     for (int i = 1; i <= t->k; ++i) {
-        a.c[i] = t->c[i];
-        a.S[i] = t->S[i];
+        a.c[i] = t->rows(i, 0);
+        a.S[i] = t->rows(i, 1);
         a.pc[i] = t->pc[i];
         a.ps[i] = t->ps[i];
         a.Sp[i] = t->Sp[i];
@@ -1071,6 +1160,7 @@ static void fill_sample_args(SampleArgs &a, const mc_tables *t, int h)
         a.Ws[i] = t->geo.Ws[i];
         a.R_[i] = cat.r[i];
     }
+    a.levels = t->wide_levels;
     a.k = t->k;
     a.h = h;
     for (int i = 0; i <= MAXK + 1; ++i) a.first[i] = cat.first[std::min(i, MAXK + 1)];
@@ -1212,8 +1302,8 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, cudaStream_t s)
     // a launch that leaves most SMs idle runs the latency mode (dense tables)
     // in blocks of 64, spread over more SMs
     const bool lat = !t->packed && a.count <= (int64_t)sm_count() * 256;
-    const int block = lat ? 64 : 256;
-    const size_t smem = a.hist ? (size_t)a.ncls * sizeof(unsigned int) : 0;
+    const int block = lat ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
+    const size_t smem = ((size_t)SAMPLE_WORDS * block + (a.hist ? (size_t)a.ncls : 0)) * sizeof(uint32_t);
     // one wave of resident blocks: the grid-stride loop then keeps every
     // warp busy until the samples run out
     // 64-bit descent arithmetic is exact when 8 R < 2^64: every weight is at
@@ -1236,15 +1326,16 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, cudaStream_t s)
                     : (t->bits == 64 ? (narrow ? sample_kernel<uint64_t, uint64_t, false, false, false>
                                                : sample_kernel<uint64_t, u128, false, false, false>)
                                      : sample_kernel<u128, u128, false, false, false>);
+    if (smem > 40 * 1024)  // beside the static tables
+        MC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     MC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem));
     if (per_sm < 1) per_sm = 1;
     int64_t grid = (a.count + block - 1) / block;  // one sample per thread
     const int64_t cap = (int64_t)sm_count() * per_sm;
+    if (grid > sm_count()) grid = (grid + sm_count() - 1) / sm_count() * sm_count();  // the same number on every SM
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
-    if (smem > 48 * 1024)
-        MC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     MC_LAUNCH("sample", s, kern<<<(unsigned)grid, block, smem, s>>>(a));
 }
 
