@@ -68,9 +68,15 @@ __global__ void hub_reduce_small_kernel(CT *__restrict__ partial, Rows dst, uint
         if (nch > HUB_SERIAL) continue;
         CT *p = partial + c0 * Ws + e * nch;
         CT run = 0;
-        for (int64_t c = 0; c < nch; ++c) {
-            ovf |= add_ovf(run, p[c]);
-            p[c] = run;
+        for (int64_t c = 0; c < nch; c += 4) {  // four loads in flight
+            CT x[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[i] = c + i < nch ? p[c + i] : (CT)0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                ovf |= add_ovf(run, x[i]);
+                if (c + i < nch) p[c + i] = run;
+            }
         }
         store_hub_entry<CT>(dst, hub_node[hub], e, run, wide);
     }
@@ -127,12 +133,15 @@ __global__ void hub_reduce_kernel(CT *__restrict__ partial, Rows dst, uint32_t *
 // one node (tid mod TN) and takes every (threads / TN)-th output, so the
 // threads that share an output run one program and read one entry of
 // neighbouring rows: no divergence, no bank conflicts, and every lower row
-// crosses the memory bus once.  Bound by the bytes of the rows (and, at
-// k = 8, by the latency of a stage: two blocks per SM).  Against a thread per
-// (node, output) reading its operands through L1, ms per level 5 / 6 / 7 on
-// R-MAT scale 22, k = 7, 128-bit counts: 10.6 / 15.0 / 12.5 before, 4.1 / 5.8
-// / 5.1 now; level 5 / 6 on a 994k-node grid, k = 6, 64-bit counts: 0.69 /
-// 0.47 before, 0.44 / 0.40 now.
+// crosses the memory bus once.  Bound by instruction issue (60%, a third of
+// it the integer multiplies) at 36% of the warps, which shared memory allows;
+// staging the next pair while one is computed needs more of it and was slower
+// (k = 7 levels 6 / 7: 4.8 / 5.5 against 3.9 / 4.8 ms), two nodes per thread
+// gave nothing.  Against a thread per (node, output) reading whole counts
+// through L1, ms per level 5 / 6 / 7 on R-MAT 22, k = 7, 128-bit counts: 10.6 /
+// 15.0 / 12.5 before, 2.8 / 3.9 / 4.8 now; levels 6 / 7 / 8 on Chung-Lu 2M,
+// k = 8: 20.8 / 27.8 / 21.1 before, 10.9 / 14.3 / 11.9 now; level 5 / 6 on a
+// 994k-node grid, k = 6, 64-bit counts: 0.69 / 0.47 before, 0.30 / 0.25 now.
 // Rows are read and written by their first planes (common.cuh): operands of 4
 // or 8 bytes, with products of 64 to 128 bits.  A node with a wide row among a
 // pair's operands reads that pair's operands from memory instead, in full;
@@ -160,7 +169,7 @@ struct MergeTileArgs {
     Rows out;
     int so, cw;             // output row: stride in shared memory and pieces of its first plane
     uint32_t mw;            // ceil(2^32 / cw)
-    int log_tn, in_pieces;  // log2 TN; 8-byte pieces of the staging area
+    int log_tn, in_pieces;  // log2 TN; staging room of a node in 8-byte pieces
     uint32_t *levels;       // the levels that have a wide row
     const uint8_t *zero_root_colors;
     int *err;
@@ -182,43 +191,88 @@ __device__ __forceinline__ void stage_rows(uint64_t *dst, const Rows &src, int p
     }
 }
 
-// sum over the terms of A[ia] * B[ib] (HA = false: of B[ib]), the operands
-// first-plane counts of NA and NB bytes.  Exact: `ovf` is set when the sum
-// does not fit CT.
+// Exact sums of products, as limbs with an explicit carry: no comparison per
+// term.  `ovf` is set when the sum does not fit CT.
+//   4 x 4 bytes: 64-bit products, 64 bits and a carry count;
+//   4 x 8: the two 64-bit partial products on sums of their own;
+//   8 x 8: 128-bit products, 128 bits and a carry count.
+// At most 35 terms.  (With a 128-bit sum compared after each addition: 16.9
+// against 14.3 ms at level 7 of Chung-Lu 2M, k = 8.)
+template <typename CT, int NA, int NB> struct ProductSum {
+    uint64_t lo = 0, hi = 0;
+    uint32_t c = 0, c2 = 0;
+    __device__ __forceinline__ void add(uint64_t x, uint64_t y)
+    {
+        if constexpr (NA == 8 && NB == 8) {
+            asm("mad.lo.cc.u64 %0, %3, %4, %0;\n\tmadc.hi.cc.u64 %1, %3, %4, %1;\n\taddc.u32 %2, %2, 0;"
+                : "+l"(lo), "+l"(hi), "+r"(c)
+                : "l"(x), "l"(y));
+        } else if constexpr (NA == 4 && NB == 4) {
+            add1(lo, c, (uint64_t)(uint32_t)x * (uint32_t)y);
+        } else {
+            const uint32_t s = (uint32_t)(NA == 4 ? x : y);  // the 4-byte operand
+            const uint64_t w = NA == 4 ? y : x;
+            add1(lo, c, (uint64_t)s * (uint32_t)w);
+            add1(hi, c2, (uint64_t)s * (uint32_t)(w >> 32));  // at 2^32
+        }
+    }
+    static __device__ __forceinline__ void add1(uint64_t &l, uint32_t &carry, uint64_t p)
+    {
+        asm("add.cc.u64 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+l"(l), "+r"(carry) : "l"(p));
+    }
+    __device__ __forceinline__ CT value(bool &ovf) const
+    {
+        if constexpr (sizeof(CT) == 16) {
+            if constexpr (NA == 8 && NB == 8) {
+                ovf |= c != 0;
+                return ((CT)hi << 64) | lo;
+            } else if constexpr (NA == 4 && NB == 4) {
+                return ((CT)c << 64) | lo;
+            } else {
+                return (((CT)c << 64) | lo) + ((((CT)c2 << 64) | hi) << 32);
+            }
+        } else {
+            if constexpr (NA == 8 && NB == 8) {
+                ovf |= (hi | c) != 0;
+                return lo;
+            } else if constexpr (NA == 4 && NB == 4) {
+                ovf |= c != 0;
+                return lo;
+            } else {
+                const u128 t = (((u128)c << 64) | lo) + ((((u128)c2 << 64) | hi) << 32);
+                ovf |= (uint64_t)(t >> 64) != 0;
+                return (uint64_t)t;
+            }
+        }
+    }
+};
+
+// Sum over the terms of A[ia] * B[ib] (HA = false: of B[ib]), the operands
+// first-plane counts of NA and NB bytes.
 template <typename CT, bool HA, int NA, int NB>
 __device__ __forceinline__ CT merge_sum(const uint8_t *A, const uint8_t *B, const uint32_t *term, int nt, bool &ovf)
 {
     typedef typename std::conditional<NA == 4, uint32_t, uint64_t>::type TA;
     typedef typename std::conditional<NB == 4, uint32_t, uint64_t>::type TB;
-    const TA *a = (const TA *)A;
-    const TB *b = (const TB *)B;
-    if constexpr (!HA || (NA == 4 && NB == 4)) {
-        // at most 35 terms below 2^64: 64 bits and a carry count
-        uint64_t lo = 0;
-        uint32_t hi = 0;
+    if constexpr (HA) {
+        ProductSum<CT, NA, NB> s;
 #pragma unroll 2
         for (int i = 0; i < nt; ++i) {
             const uint32_t tm = term[i];
-            uint64_t p = b[tm >> 16];
-            if constexpr (HA) p *= a[tm & 0xffffu];
-            lo += p;
-            hi += lo < p;
+            s.add(((const TA *)A)[tm & 0xffffu], ((const TB *)B)[tm >> 16]);
+        }
+        return s.value(ovf);
+    } else {
+        uint64_t lo = 0;
+        uint32_t hi = 0;
+        for (int i = 0; i < nt; ++i) {
+            const uint64_t x = ((const TB *)B)[term[i] >> 16];
+            lo += x;
+            hi += lo < x;
         }
         if constexpr (sizeof(CT) == 16) return ((CT)hi << 64) | lo;
         ovf |= hi != 0;
         return (CT)lo;
-    } else {
-        CT sum = 0;
-#pragma unroll 2
-        for (int i = 0; i < nt; ++i) {
-            const uint32_t tm = term[i];
-            const uint64_t x = a[tm & 0xffffu], y = b[tm >> 16];
-            CT p;
-            if constexpr (sizeof(CT) == 16) p = (CT)x * y;
-            else ovf |= mul_ovf(x, y, p);
-            ovf |= add_ovf(sum, p);
-        }
-        return sum;
     }
 }
 
@@ -246,7 +300,7 @@ __global__ void __launch_bounds__(THREADS) merge_tile_kernel(const __grid_consta
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int tn = 1 << a.log_tn, W = a.out.W, N = a.out.N, wpn = (W + 31) >> 5;
     uint64_t *s_in = (uint64_t *)s_raw;
-    uint64_t *s_out = s_in + a.in_pieces;
+    uint64_t *s_out = s_in + tn * a.in_pieces;
     uint2 *s_rec = (uint2 *)(s_out + tn * a.so);
     uint32_t *s_terms = (uint32_t *)(s_rec + a.nrec);
     uint32_t *s_src = s_terms + a.nterms;  // nodes whose rows are read (0xffffffff: none)
@@ -258,12 +312,11 @@ __global__ void __launch_bounds__(THREADS) merge_tile_kernel(const __grid_consta
     bool ovf = false, inexact = false, any_wide = false;
     const int64_t ntiles = (a.n_do + tn - 1) >> a.log_tn;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t i0 = tile << a.log_tn;
         if (threadIdx.x < tn) {
-            const int64_t i = i0 + threadIdx.x;
-            const uint32_t v = i < a.n_do ? (a.order ? a.order[i] : (uint32_t)i) : 0xffffffffu;
-            s_dst[threadIdx.x] = v;
-            s_src[threadIdx.x] = (v != 0xffffffffu && a.zero_root_colors && a.zero_root_colors[v] != 0) ? 0xffffffffu : v;
+            const int64_t i = (tile << a.log_tn) + threadIdx.x;
+            const uint32_t u = i < a.n_do ? (a.order ? a.order[i] : (uint32_t)i) : 0xffffffffu;
+            s_dst[threadIdx.x] = u;
+            s_src[threadIdx.x] = (u != 0xffffffffu && a.zero_root_colors && a.zero_root_colors[u] != 0) ? 0xffffffffu : u;
         }
         for (int i = threadIdx.x; i < tn * wpn; i += THREADS) s_big[i] = 0;
         __syncthreads();
@@ -289,10 +342,8 @@ __global__ void __launch_bounds__(THREADS) merge_tile_kernel(const __grid_consta
                     const int o = rc.x & 0xffffu, beta = (rc.x >> 16) & 255, nt = rc.x >> 24;
                     CT sum = 0;
                     if (live) {
-                        if (!full)
-                            sum = sum_of(term, nt);
-                        else
-                            sum = merge_sum_wide<CT>(a.c[P.h1], a.S[P.h2], P.wa != 0, v, term, nt, ovf);
+                        if (!full) sum = sum_of(term, nt);
+                        else sum = merge_sum_wide<CT>(a.c[P.h1], a.S[P.h2], P.wa != 0, v, term, nt, ovf);
                         if (beta != 1) {
                             CT q = 0;
                             if (!exact_div(sum, a.div[beta], q)) inexact = true;
@@ -309,16 +360,19 @@ __global__ void __launch_bounds__(THREADS) merge_tile_kernel(const __grid_consta
                     else ((uint64_t *)row)[o] = (uint64_t)sum;
                 }
             };
+#define MC_MERGE(HA, NA, NB) \
+    outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, HA, NA, NB>(A, B, t, nt, ovf); })
             if (!P.wa) {
-                if (nb == 4) outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, false, 4, 4>(A, B, t, nt, ovf); });
-                else outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, false, 4, 8>(A, B, t, nt, ovf); });
+                if (nb == 4) MC_MERGE(false, 4, 4);
+                else MC_MERGE(false, 4, 8);
             } else if (na == 4) {
-                if (nb == 4) outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, true, 4, 4>(A, B, t, nt, ovf); });
-                else outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, true, 4, 8>(A, B, t, nt, ovf); });
+                if (nb == 4) MC_MERGE(true, 4, 4);
+                else MC_MERGE(true, 4, 8);
             } else {
-                if (nb == 4) outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, true, 8, 4>(A, B, t, nt, ovf); });
-                else outputs([&](const uint32_t *t, int nt) { return merge_sum<CT, true, 8, 8>(A, B, t, nt, ovf); });
+                if (nb == 4) MC_MERGE(true, 8, 4);
+                else MC_MERGE(true, 8, 8);
             }
+#undef MC_MERGE
             __syncthreads();
         }
         for (int i = threadIdx.x; i < tn * a.cw; i += THREADS) {
@@ -901,7 +955,7 @@ static bool plan_merge_tile(MergeTileArgs &ta, const MergePairs &Q, int shift, s
 {
     auto magic = [](int w) { return w > 1 ? (uint32_t)((((uint64_t)1 << 32) + w - 1) / w) : 0u; };
     ta.npair = Q.n;
-    int widest = 0;
+    ta.in_pieces = 0;
     for (int p = 0; p < Q.n; ++p) {
         TilePair &P = ta.pair[p];
         P.h1 = Q.h1[p];
@@ -917,7 +971,7 @@ static bool plan_merge_tile(MergeTileArgs &ta, const MergePairs &Q, int shift, s
         P.bits = (P.wa ? 1u << P.h1 : 0u) | 1u << (16 + P.h2);
         P.rec0 = Q.rec0[p];
         P.rec1 = Q.rec0[p + 1];
-        widest = std::max(widest, P.sa + P.sb);
+        ta.in_pieces = std::max(ta.in_pieces, P.sa + P.sb);
     }
     ta.cw = ta.out.s0 / 8;
     ta.so = ta.cw | 1;
@@ -925,20 +979,18 @@ static bool plan_merge_tile(MergeTileArgs &ta, const MergePairs &Q, int shift, s
     ta.nrec = (int)Q.rec.size() / 2;
     ta.nterms = (int)Q.terms.size();
     const size_t fixed = (size_t)ta.nrec * 8 + (size_t)ta.nterms * 4;
-    const size_t node = (size_t)(widest + ta.so) * 8 + 8 + (size_t)(ta.out.W + 31) / 32 * 4;
+    const size_t node = (size_t)(ta.in_pieces + ta.so) * 8 + 8 + (size_t)(ta.out.W + 31) / 32 * 4;
     int lt = 7;
     while (lt > 3 && (fixed + (node << lt) > 72 * 1024 || (ta.n_do >> lt) < 2 * (int64_t)sm_count())) --lt;
     lt += shift;
     if (lt < 3 || lt > 7) return false;
     ta.log_tn = lt;
-    ta.in_pieces = widest << lt;
     smem = fixed + (node << lt);
     return smem <= 220 * 1024;
 }
 
-// Merge candidates (threads per block, tile size): 256 threads at the plan's
-// tile, half and twice that; 512 threads at the plan's tile; 128 threads at
-// the plan's tile and half of it.
+// Merge candidates: threads per block and the tile against the plan's (as a
+// power of two).
 constexpr int MERGE_CANDIDATES = 6;
 
 template <typename CT, int THREADS>
