@@ -53,68 +53,61 @@ __device__ __forceinline__ void store_hub_entry(const Rows &dst, uint32_t v, int
     }
 }
 
+// One launch: the first `big_blocks` blocks take the larger hubs.
 template <typename CT>
-__global__ void hub_reduce_small_kernel(CT *__restrict__ partial, Rows dst, uint32_t *levels,
-                                        const uint32_t *__restrict__ hub_node,
-                                        const int64_t *__restrict__ hub_chunk0, int64_t n_hubs, int Ws, int *err)
+__global__ void __launch_bounds__(256) hub_reduce_kernel(CT *__restrict__ partial, Rows dst, uint32_t *levels,
+                                                         const uint32_t *__restrict__ hub_node,
+                                                         const int64_t *__restrict__ hub_chunk0, int64_t n_hubs,
+                                                         const uint32_t *__restrict__ big_hub, int64_t n_big, int big_blocks,
+                                                         int *err)
 {
     bool ovf = false, wide = false;
-    const int64_t total = n_hubs * Ws;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t hub = i / Ws;
-        const int e = (int)(i - hub * Ws);
-        const int64_t c0 = hub_chunk0[hub], nch = hub_chunk0[hub + 1] - c0;
-        if (nch > HUB_SERIAL) continue;
-        CT *p = partial + c0 * Ws + e * nch;
-        CT run = 0;
-        for (int64_t c = 0; c < nch; c += 4) {  // four loads in flight
-            CT x[4];
+    const int Ws = dst.W;
+    if ((int)blockIdx.x < big_blocks) {
+        const int lane = threadIdx.x & 31;
+        const int64_t nwarps = ((int64_t)big_blocks * blockDim.x) >> 5;
+        for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < n_big * Ws; i += nwarps) {
+            const int64_t bi = i / Ws;
+            const int e = (int)(i - bi * Ws);
+            const int64_t hub = big_hub[bi];
+            const int64_t c0 = hub_chunk0[hub], nch = hub_chunk0[hub + 1] - c0;
+            CT *p = partial + c0 * Ws + e * nch;
+            CT carry = 0;
+            for (int64_t b = 0; b < nch; b += 32) {
+                const int64_t c = b + lane;
+                CT x = c < nch ? p[c] : (CT)0;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) x[i] = c + i < nch ? p[c + i] : (CT)0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                ovf |= add_ovf(run, x[i]);
-                if (c + i < nch) p[c + i] = run;
+                for (int d = 1; d < 32; d <<= 1) {
+                    const CT y = shfl_up(x, d);
+                    if (lane >= d) ovf |= add_ovf(x, y);
+                }
+                ovf |= add_ovf(x, carry);
+                if (c < nch) p[c] = x;
+                carry = shfl(x, 31);
             }
+            if (lane == 0) store_hub_entry<CT>(dst, hub_node[hub], e, carry, wide);
         }
-        store_hub_entry<CT>(dst, hub_node[hub], e, run, wide);
-    }
-    if (ovf) atomicOr(err, ERR_OVERFLOW);
-    if (wide) atomicOr(levels, dst.bit);
-}
-
-template <typename CT>
-__global__ void hub_reduce_kernel(CT *__restrict__ partial, Rows dst, uint32_t *levels,
-                                  const uint32_t *__restrict__ hub_node,
-                                  const int64_t *__restrict__ hub_chunk0, const uint32_t *__restrict__ big_hub,
-                                  int64_t n_big, int Ws, int *err)
-{
-    bool ovf = false, wide = false;
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t total = n_big * Ws;
-    for (int64_t i = warp; i < total; i += nwarps) {
-        const int64_t bi = i / Ws;
-        const int e = (int)(i - bi * Ws);
-        const int64_t hub = big_hub[bi];
-        const int64_t c0 = hub_chunk0[hub], nch = hub_chunk0[hub + 1] - c0;
-        CT *p = partial + c0 * Ws + e * nch;
-        CT carry = 0;
-        for (int64_t b = 0; b < nch; b += 32) {
-            const int64_t c = b + lane;
-            CT x = c < nch ? p[c] : (CT)0;
+    } else {
+        const int64_t step = (int64_t)(gridDim.x - big_blocks) * blockDim.x;
+        for (int64_t i = (int64_t)(blockIdx.x - big_blocks) * blockDim.x + threadIdx.x; i < n_hubs * Ws; i += step) {
+            const int64_t hub = i / Ws;
+            const int e = (int)(i - hub * Ws);
+            const int64_t c0 = hub_chunk0[hub], nch = hub_chunk0[hub + 1] - c0;
+            if (nch > HUB_SERIAL) continue;
+            CT *p = partial + c0 * Ws + e * nch;
+            CT run = 0;
+            for (int64_t c = 0; c < nch; c += 4) {  // four loads in flight
+                CT x[4];
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const CT y = shfl_up(x, d);
-                if (lane >= d) ovf |= add_ovf(x, y);
+                for (int q = 0; q < 4; ++q) x[q] = c + q < nch ? p[c + q] : (CT)0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    ovf |= add_ovf(run, x[q]);
+                    if (c + q < nch) p[c + q] = run;
+                }
             }
-            ovf |= add_ovf(x, carry);
-            if (c < nch) p[c] = x;
-            carry = shfl(x, 31);
+            store_hub_entry<CT>(dst, hub_node[hub], e, run, wide);
         }
-        if (lane == 0) store_hub_entry<CT>(dst, hub_node[hub], e, carry, wide);
     }
     if (ovf) atomicOr(err, ERR_OVERFLOW);
     if (wide) atomicOr(levels, dst.bit);
@@ -507,10 +500,19 @@ __device__ __forceinline__ u128 block_exclusive_scan(u128 x, u128 *smem, u128 &b
     return before + inc - x;
 }
 
-__global__ void __launch_bounds__(SCAN_THREADS) scan_tiles_kernel(const u128 *__restrict__ x, int64_t n,
+// Inclusive u128 prefix of m arrays of n entries, `stride` entries apart
+// (blockIdx.y picks one): tile sums, then each block adds up the sums of the
+// tiles before its own and scans its tile.  One tile (n <= 4096) needs the
+// second kernel only; beyond SCAN_DIRECT tiles the sums are scanned by a
+// kernel of their own first, since every block would read all of them (at
+// most 32 KB here; a tile is 64 KB).  Launches 3 -> 2 (1 for small arrays).
+constexpr int64_t SCAN_DIRECT = 2048;
+
+__global__ void __launch_bounds__(SCAN_THREADS) scan_tiles_kernel(const u128 *__restrict__ x, int64_t n, int64_t stride,
                                                                   u128 *__restrict__ tile_sum, int *err)
 {
     __shared__ u128 smem[32];
+    x += blockIdx.y * stride;
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
     u128 s = 0;
     bool ovf = false;
@@ -520,13 +522,14 @@ __global__ void __launch_bounds__(SCAN_THREADS) scan_tiles_kernel(const u128 *__
     const u128 ex = block_exclusive_scan(s, smem, tot);
     // the block total is exact iff no prefix wrapped
     if (ex + s < ex) ovf = true;
-    if (threadIdx.x == blockDim.x - 1) tile_sum[blockIdx.x] = tot;
+    if (threadIdx.x == blockDim.x - 1) tile_sum[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = tot;
     if (ovf) atomicOr(err, ERR_OVERFLOW);
 }
 
 __global__ void __launch_bounds__(1024) scan_tile_sums_kernel(u128 *tile_sum, int64_t ntiles, int *err)
 {
     __shared__ u128 smem[32];
+    tile_sum += blockIdx.y * ntiles;
     u128 carry = 0;
     bool ovf = false;
     for (int64_t b = 0; b < ntiles; b += blockDim.x) {
@@ -544,25 +547,74 @@ __global__ void __launch_bounds__(1024) scan_tile_sums_kernel(u128 *tile_sum, in
     if (ovf) atomicOr(err, ERR_OVERFLOW);
 }
 
-__global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(u128 *__restrict__ x, int64_t n,
-                                                                  const u128 *__restrict__ tile_ex)
+// `scanned`: tile_sum holds the sums before each tile, else the tiles' own
+__global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(u128 *__restrict__ x, int64_t n, int64_t stride,
+                                                                  const u128 *__restrict__ tile_sum, bool scanned, int *err)
 {
     __shared__ u128 smem[32];
+    bool ovf = false;
+    x += blockIdx.y * stride;
+    u128 before = 0;
+    if (scanned) {
+        before = tile_sum[(int64_t)blockIdx.y * gridDim.x + blockIdx.x];
+    } else if (blockIdx.x > 0) {
+        tile_sum += (int64_t)blockIdx.y * gridDim.x;
+        u128 s = 0;
+        for (int t = threadIdx.x; t < (int)blockIdx.x; t += SCAN_THREADS) ovf |= add_ovf(s, tile_sum[t]);
+        const u128 ex = block_exclusive_scan(s, smem, before);
+        if (ex + s < ex) ovf = true;
+    }
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
     u128 v[SCAN_ITEMS];
     u128 s = 0;
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; ++i) {
         v[i] = base + i < n ? x[base + i] : 0;
-        s += v[i];
+        ovf |= add_ovf(s, v[i]);
     }
     u128 tot;
-    u128 run = block_exclusive_scan(s, smem, tot) + tile_ex[blockIdx.x];
+    const u128 ex = block_exclusive_scan(s, smem, tot);
+    u128 run = before + ex;
+    if (run < before || run + s < run) ovf = true;
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; ++i) {
         run += v[i];
         if (base + i < n) x[base + i] = run;
     }
+    if (ovf) atomicOr(err, ERR_OVERFLOW);
+}
+
+// Sum over the nodes [lo, hi) of the level-h counts of unrooted treelet
+// first + blockIdx.y: per block its part, then the parts added up.
+template <typename CT>
+__global__ void __launch_bounds__(256) treelet_sum_kernel(Rows c, int64_t lo, int64_t hi, int R, int Bc, int first,
+                                                          const __grid_constant__ TreeletShapes ts, u128 *__restrict__ part,
+                                                          int *err)
+{
+    __shared__ u128 smem[32];
+    bool ovf = false;
+    u128 s = 0;
+    const int j = first + blockIdx.y;
+    for (int64_t v = lo + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < hi; v += (int64_t)gridDim.x * blockDim.x)
+        for (int q = ts.off[j]; q < ts.off[j + 1]; ++q)
+            for (int b = 0; b < Bc; ++b) ovf |= add_ovf(s, widen(entry_at<CT>(c, v, b * R + ts.shape[q])));
+    u128 tot;
+    const u128 ex = block_exclusive_scan(s, smem, tot);
+    if (ex + s < ex) ovf = true;
+    if (threadIdx.x == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = tot;
+    if (ovf) atomicOr(err, ERR_OVERFLOW);
+}
+__global__ void __launch_bounds__(256) part_sum_kernel(const u128 *__restrict__ part, int np, u128 *__restrict__ out, int *err)
+{
+    __shared__ u128 smem[32];
+    bool ovf = false;
+    u128 s = 0;
+    for (int i = threadIdx.x; i < np; i += blockDim.x) ovf |= add_ovf(s, part[(int64_t)blockIdx.x * np + i]);
+    u128 tot;
+    const u128 ex = block_exclusive_scan(s, smem, tot);
+    if (ex + s < ex) ovf = true;
+    if (threadIdx.x == 0) out[blockIdx.x] = tot;
+    if (ovf) atomicOr(err, ERR_OVERFLOW);
 }
 
 // Colour of every edge's far end, so that neighbour loops read colours
@@ -741,36 +793,54 @@ __global__ void hub_chunk_scatter_kernel(const uint32_t *__restrict__ col, const
 // Root-search buckets: X in [0, R) falls in bucket b = floor(X / D), D =
 // ceil(R / nb); start[b] is the first node whose inclusive prefix exceeds
 // b * D, so the node drawn for X lies in [start[b], start[b + 1]].
-__global__ void bucket_width_kernel(const u128 *prefix, int64_t n, int64_t nb, u128 *D)
+// (For m prefixes at once: blockIdx.y.)  A block's first and last bucket are
+// searched over all nodes, the others between those two.
+__global__ void __launch_bounds__(256) bucket_kernel(const u128 *__restrict__ prefix, int64_t n, int64_t nb, u128 *D_out,
+                                                     uint32_t *__restrict__ start, int64_t pstride, int64_t bstride)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        const u128 R = n > 0 ? prefix[n - 1] : 0;
-        u128 d = R / (u128)nb + ((R % (u128)nb) != 0 ? 1 : 0);
-        *D = d ? d : 1;
+    __shared__ u128 s_D;
+    __shared__ int64_t s_end[2];
+    prefix += blockIdx.y * pstride;
+    start += blockIdx.y * bstride;
+    if (threadIdx.x == 0) {
+        const u128 R = prefix[n - 1];
+        const u128 d = (R >> 64) == 0 ? (u128)(((uint64_t)R + (uint64_t)nb - 1 >= (uint64_t)R)
+                                                   ? ((uint64_t)R + (uint64_t)nb - 1) / (uint64_t)nb
+                                                   : (uint64_t)R / (uint64_t)nb + ((uint64_t)R % (uint64_t)nb != 0))
+                                      : R / (u128)nb + ((R % (u128)nb) != 0 ? 1 : 0);
+        s_D = d ? d : 1;
+        if (blockIdx.x == 0) D_out[blockIdx.y] = s_D;
     }
-}
-
-__global__ void bucket_kernel(const u128 *__restrict__ prefix, int64_t n, int64_t nb, const u128 *Dp,
-                              uint32_t *__restrict__ start)
-{
-    const u128 D = *Dp;
-    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b <= nb;
-         b += (int64_t)gridDim.x * blockDim.x) {
+    __syncthreads();
+    const u128 D = s_D;
+    auto search = [&](int64_t b, int64_t lo, int64_t hi) {
         const u128 X = (u128)b * D;
-        int64_t lo = 0, hi = n;  // first v with prefix[v] > X, else n - 1
-        while (lo < hi) {
+        while (lo < hi) {  // first v with prefix[v] > X, else n
             const int64_t mid = (lo + hi) >> 1;
             if (prefix[mid] > X) hi = mid; else lo = mid + 1;
         }
-        start[b] = (uint32_t)(lo < n ? lo : n - 1);
+        return lo;
+    };
+    for (int64_t b0 = blockIdx.x * (int64_t)blockDim.x; b0 <= nb; b0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b1 = min(nb, b0 + blockDim.x - 1);
+        if (threadIdx.x == 0) s_end[0] = search(b0, 0, n);
+        if (threadIdx.x == 32) s_end[1] = search(b1, 0, n);
+        __syncthreads();
+        const int64_t b = b0 + threadIdx.x;
+        if (b <= b1) {
+            const int64_t v = search(b, s_end[0], s_end[1]);
+            start[b] = (uint32_t)(v < n ? v : n - 1);
+        }
+        __syncthreads();
     }
 }
 
-void build_buckets(const u128 *prefix, int64_t n, int64_t nb, u128 *dD, uint32_t *start, cudaStream_t s)
+void build_buckets(const u128 *prefix, int64_t n, int64_t nb, u128 *dD, uint32_t *start, cudaStream_t s, int m,
+                   int64_t bstride)
 {
     if (n <= 0) return;
-    MC_LAUNCH("bucket_width", s, bucket_width_kernel<<<1, 32, 0, s>>>(prefix, n, nb, dD));
-    MC_LAUNCH("buckets", s, bucket_kernel<<<grid_for(nb + 1, 256), 256, 0, s>>>(prefix, n, nb, dD, start));
+    MC_LAUNCH("buckets", s, bucket_kernel<<<dim3((unsigned)grid_for(nb + 1, 256), (unsigned)m), 256, 0, s>>>(
+                                prefix, n, nb, dD, start, n, bstride));
 }
 
 int64_t bucket_count(int64_t n) { return std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)1 << 22)); }
@@ -804,20 +874,23 @@ __global__ void fill_ones_kernel(void *dst, int64_t n, int bytes)
 // ---------------------------------------------------------------------------
 static int64_t scan_tiles(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
 
-// the scan with a caller-provided tile-sum buffer of scan_tiles(n) entries
-static void inclusive_scan_u128_buf(u128 *x, int64_t n, int *err, u128 *ts, cudaStream_t s)
+// the scan with a caller-provided tile-sum buffer of m * scan_tiles(n) entries
+static void inclusive_scan_u128_buf(u128 *x, int64_t n, int *err, u128 *ts, cudaStream_t s, int m = 1)
 {
     if (n <= 0) return;
     const int64_t ntiles = scan_tiles(n);
-    MC_LAUNCH("scan_tiles", s, scan_tiles_kernel<<<(unsigned)ntiles, SCAN_THREADS, 0, s>>>(x, n, ts, err));
-    MC_LAUNCH("scan_tile_sums", s, scan_tile_sums_kernel<<<1, 1024, 0, s>>>(ts, ntiles, err));
-    MC_LAUNCH("scan_apply", s, scan_apply_kernel<<<(unsigned)ntiles, SCAN_THREADS, 0, s>>>(x, n, ts));
+    const dim3 grid((unsigned)ntiles, (unsigned)m);
+    const bool scanned = ntiles > SCAN_DIRECT;
+    if (ntiles > 1) MC_LAUNCH("scan_tiles", s, scan_tiles_kernel<<<grid, SCAN_THREADS, 0, s>>>(x, n, n, ts, err));
+    if (scanned)
+        MC_LAUNCH("scan_tile_sums", s, scan_tile_sums_kernel<<<dim3(1, (unsigned)m), 1024, 0, s>>>(ts, ntiles, err));
+    MC_LAUNCH("scan_apply", s, scan_apply_kernel<<<grid, SCAN_THREADS, 0, s>>>(x, n, n, ts, scanned, err));
 }
 
-void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s)
+void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s, int m)
 {
     if (n <= 0) return;
-    inclusive_scan_u128_buf(x, n, err, scratch.get<u128>((size_t)scan_tiles(n)), s);
+    inclusive_scan_u128_buf(x, n, err, scratch.get<u128>((size_t)scan_tiles(n) * m), s, m);
 }
 
 ExactDiv make_div(int beta)
@@ -874,6 +947,20 @@ void launch_row_totals(const mc_tables *t, int h, uint64_t allow0, uint64_t allo
         launch_row_totals_t<u128>(t->rows(h, 0), n, W, R, allow0, allow1, tot, err, s);
 }
 
+static TreeletShapes treelet_shapes(int h)
+{
+    const ShapeCatalog &cat = shape_catalog();
+    TreeletShapes ts{};
+    int q = 0;
+    for (int j = 0; j < cat.n_unrooted[h]; ++j) {
+        ts.off[j] = (int16_t)q;
+        for (int i = 0; i < cat.r[h]; ++i)
+            if (cat.shapes[cat.gid(h, i)].unrooted == j) ts.shape[q++] = (uint8_t)i;
+    }
+    ts.off[cat.n_unrooted[h]] = (int16_t)q;
+    return ts;
+}
+
 // Dense tables: tot[j * n + v] for every unrooted treelet j of level h in
 // one pass over the level's c rows.
 void launch_treelet_totals(const mc_tables *t, int h, u128 *tot, int *err, cudaStream_t s)
@@ -883,14 +970,7 @@ void launch_treelet_totals(const mc_tables *t, int h, u128 *tot, int *err, cudaS
     const int nu = cat.n_unrooted[h], R = cat.r[h];
     if (n == 0 || nu == 0) return;
     MC_REQUIRE(!t->packed, "treelet totals read dense tables");
-    TreeletShapes ts{};
-    int q = 0;
-    for (int j = 0; j < nu; ++j) {
-        ts.off[j] = (int16_t)q;
-        for (int i = 0; i < R; ++i)
-            if (cat.shapes[cat.gid(h, i)].unrooted == j) ts.shape[q++] = (uint8_t)i;
-    }
-    ts.off[nu] = (int16_t)q;
+    const TreeletShapes ts = treelet_shapes(h);
     const int Bc = t->geo.Bc[h];
     const int grid = grid_for(n * nu, 256);
     if (t->bits == 64)
@@ -1219,12 +1299,10 @@ template <typename CT> static void build_levels(mc_tables *t, int *err, cudaStre
             const int rh = shape_catalog().r[h];
             run_tuned(gkey, GATHER_CANDIDATES, allow_tune, s, [&](int c) { return launch_gather<CT>(ga, rh, h, c, s); });
             if (g->n_hubs) {
-                MC_LAUNCH("hub_reduce", s, hub_reduce_small_kernel<CT><<<grid_for(g->n_hubs * G.Ws[h], 256), 256, 0, s>>>(
-                    (CT *)t->Sp[h], t->rows(h, 1), levels, g->hub_node, g->hub_chunk0, g->n_hubs, G.Ws[h], err));
-                if (g->n_big_hubs)
-                    MC_LAUNCH("hub_reduce", s, hub_reduce_kernel<CT><<<grid_for(g->n_big_hubs * G.Ws[h] * 32, 256), 256, 0, s>>>(
-                        (CT *)t->Sp[h], t->rows(h, 1), levels, g->hub_node, g->hub_chunk0, g->big_hub, g->n_big_hubs,
-                        G.Ws[h], err));
+                const int big = g->n_big_hubs ? grid_for(g->n_big_hubs * G.Ws[h] * 32, 256) : 0;
+                MC_LAUNCH("hub_reduce", s, hub_reduce_kernel<CT><<<big + grid_for(g->n_hubs * G.Ws[h], 256), 256, 0, s>>>(
+                    (CT *)t->Sp[h], t->rows(h, 1), levels, g->hub_node, g->hub_chunk0, g->n_hubs, g->big_hub, g->n_big_hubs,
+                    big, err));
             }
         }
     }
@@ -1478,43 +1556,71 @@ extern "C" void mc_free_tables(mc_tables *t)
     mc_free_graph(owned);
 }
 
-// Rooted total R of level h over the nodes [lo, hi): all shapes (j < 0,
-// from the cached root index) or the rootings of unrooted shape j.
-static u128 level_rooted_total(const mc_tables *t, int h, int j, int64_t lo, int64_t hi, cudaStream_t s)
+// Rooted totals of level h over the nodes [lo, hi): of all shapes (j0 < 0, one
+// value, from the cached root index) or of the rootings of the unrooted
+// shapes j0 .. j0 + nj.
+static std::vector<u128> level_rooted_totals(const mc_tables *t, int h, int j0, int nj, int64_t lo, int64_t hi,
+                                             cudaStream_t s)
 {
     const ShapeCatalog &cat = shape_catalog();
     const int64_t n = t->g->n;
-    if (h == 1) return j > 0 ? 0 : (u128)(hi - lo);
-    if (hi <= lo) return 0;
-    // the level's node prefix, read at the range's ends
-    const u128 *pre = nullptr;
+    std::vector<u128> out((size_t)nj, 0);
+    if (h == 1) {
+        if (j0 <= 0) out[0] = (u128)(hi - lo);
+        return out;
+    }
+    if (hi <= lo) return out;
     Arena scratch(true);
     scratch.alloc = t->arena.alloc;
     scratch.stream = s;
     int *err = scratch.get<int>(1);
     MC_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    if (j < 0) {
-        ensure_level_index(t, h, s);
-        pre = t->prefix[h];
-    } else {
-        uint64_t a0 = 0, a1 = 0;
-        for (int i = 0; i < cat.r[h]; ++i)
-            if (cat.shapes[cat.gid(h, i)].unrooted == j) {
-                if (i < 64) a0 |= 1ull << i; else a1 |= 1ull << (i - 64);
-            }
-        u128 *tot = scratch.get<u128>((size_t)n);
-        launch_row_totals(t, h, a0, a1, tot, err, s);
-        inclusive_scan_u128(tot, n, err, scratch, s);
-        pre = tot;
-    }
-    u128 top = 0, base = 0;
     int herr = 0;
-    MC_CUDA(cudaMemcpyAsync(&top, pre + (hi - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
-    if (lo > 0) MC_CUDA(cudaMemcpyAsync(&base, pre + (lo - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
-    MC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
-    MC_CUDA(cudaStreamSynchronize(s));
-    if (herr) throw Error(MC_E_OVERFLOW, "level total does not fit in 128 bits");
-    return top - base;
+    if (j0 >= 0 && !t->packed) {
+        // one pass over the rows for all shapes, added up on the device
+        const int blocks = (int)std::min<int64_t>((hi - lo + 255) / 256, (int64_t)sm_count() * 4);
+        u128 *part = scratch.get<u128>((size_t)blocks * nj), *sum = scratch.get<u128>((size_t)nj);
+        const TreeletShapes ts = treelet_shapes(h);
+        const dim3 grid((unsigned)blocks, (unsigned)nj);
+        if (t->bits == 64)
+            MC_LAUNCH("treelet_sum", s, treelet_sum_kernel<uint64_t><<<grid, 256, 0, s>>>(
+                                            t->rows(h, 0), lo, hi, cat.r[h], t->geo.Bc[h], j0, ts, part, err));
+        else
+            MC_LAUNCH("treelet_sum", s, treelet_sum_kernel<u128><<<grid, 256, 0, s>>>(
+                                            t->rows(h, 0), lo, hi, cat.r[h], t->geo.Bc[h], j0, ts, part, err));
+        MC_LAUNCH("treelet_sum", s, part_sum_kernel<<<nj, 256, 0, s>>>(part, blocks, sum, err));
+        MC_CUDA(cudaMemcpyAsync(out.data(), sum, (size_t)nj * sizeof(u128), cudaMemcpyDeviceToHost, s));
+        MC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+        MC_CUDA(cudaStreamSynchronize(s));
+        if (herr) throw Error(MC_E_OVERFLOW, "level total does not fit in 128 bits");
+        return out;
+    }
+    // the level's node prefix, read at the range's ends
+    for (int i = 0; i < nj; ++i) {
+        const u128 *pre = nullptr;
+        if (j0 < 0) {
+            ensure_level_index(t, h, s);
+            pre = t->prefix[h];
+        } else {
+            uint64_t a0 = 0, a1 = 0;
+            for (int q = 0; q < cat.r[h]; ++q)
+                if (cat.shapes[cat.gid(h, q)].unrooted == j0 + i) {
+                    if (q < 64) a0 |= 1ull << q; else a1 |= 1ull << (q - 64);
+                }
+            u128 *tot = scratch.get<u128>((size_t)n);
+            launch_row_totals(t, h, a0, a1, tot, err, s);
+            inclusive_scan_u128(tot, n, err, scratch, s);
+            pre = tot;
+        }
+        u128 top = 0, base = 0;
+        MC_CUDA(cudaMemcpyAsync(&top, pre + (hi - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
+        if (lo > 0) MC_CUDA(cudaMemcpyAsync(&base, pre + (lo - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
+        MC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+        MC_CUDA(cudaStreamSynchronize(s));
+        if (herr) throw Error(MC_E_OVERFLOW, "level total does not fit in 128 bits");
+        out[(size_t)i] = top - base;
+    }
+    return out;
 }
 
 // Copies of unrooted shape j from its rooted total: R / h (one rooted copy
@@ -1550,14 +1656,14 @@ extern "C" mc_status mc_total_range(const mc_tables *t, int h, int32_t unrooted_
         if (hi <= 0) hi = n;
         MC_REQUIRE(lo >= 0 && lo <= hi && hi <= n, "node range out of bounds");
         cudaStream_t s = (cudaStream_t)stream;
-        const u128 R = level_rooted_total(t, h, unrooted_shape, lo, hi, s);
+        const u128 R = level_rooted_totals(t, h, unrooted_shape, 1, lo, hi, s)[0];
         u128 U = 0;
         if (unrooted_shape >= 0) {
             U = unrooted_from_rooted(t, h, unrooted_shape, R);
         } else if (t->skip_round && h == t->k) {
             // per-shape divisors differ: t = sum_j R_j / a_j
-            for (int j = 0; j < cat.n_unrooted[h]; ++j)
-                U += unrooted_from_rooted(t, h, j, level_rooted_total(t, h, j, lo, hi, s));
+            const std::vector<u128> Rj = level_rooted_totals(t, h, 0, cat.n_unrooted[h], lo, hi, s);
+            for (int j = 0; j < cat.n_unrooted[h]; ++j) U += unrooted_from_rooted(t, h, j, Rj[(size_t)j]);
         } else {
             const u128 div = (u128)t->copies_div(h);
             if (R % div != 0) throw Error(MC_E_INTERNAL, "rooted total not divisible by h");
@@ -1580,15 +1686,39 @@ extern "C" mc_status mc_total(const mc_tables *t, int h, int32_t unrooted_shape,
 // batches: several (graph, colouring) instances side by side as one disjoint
 // union, built in one pass (one launch per kernel for the whole batch)
 // ---------------------------------------------------------------------------
-__global__ void concat_csr_kernel(const int64_t *__restrict__ rp, const uint32_t *__restrict__ col, int64_t n,
-                                  int64_t nnz, int64_t noff, int64_t eoff, int64_t *__restrict__ urp,
-                                  uint32_t *__restrict__ ucol)
+struct ConcatPart {
+    const int64_t *row_ptr;
+    const uint32_t *col;
+    const uint8_t *colors;
+    int64_t noff, eoff;
+};
+
+// All instances in one launch (32 launches of 7 us each before, most of them
+// a few blocks): a thread finds its element's instance by a binary search of
+// the offsets.
+__global__ void __launch_bounds__(256) concat_kernel(const ConcatPart *__restrict__ part, int count, int64_t N, int64_t NNZ,
+                                                     int64_t *__restrict__ urp, uint32_t *__restrict__ ucol,
+                                                     uint8_t *__restrict__ ucolors)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nnz || i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (i < n) urp[noff + i] = eoff + rp[i];
-        if (i < nnz) ucol[eoff + i] = col[i] + (uint32_t)noff;
+    const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    auto find = [&](auto off, int64_t i) {  // the last instance that starts at or before i
+        int lo = 0, hi = count;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (off(part[mid]) <= i) lo = mid; else hi = mid;
+        }
+        return lo;
+    };
+    for (int64_t i = t0; i < NNZ; i += step) {
+        const ConcatPart p = part[find([](const ConcatPart &q) { return q.eoff; }, i)];
+        ucol[i] = p.col[i - p.eoff] + (uint32_t)p.noff;
     }
+    for (int64_t i = t0; i < N; i += step) {
+        const ConcatPart p = part[find([](const ConcatPart &q) { return q.noff; }, i)];
+        urp[i] = p.eoff + p.row_ptr[i - p.noff];
+        if (ucolors) ucolors[i] = p.colors[i - p.noff];
+    }
+    if (t0 == 0) urp[N] = NNZ;
 }
 
 extern "C" mc_status mc_build_tables_batch(int count, const mc_graph *const *graphs, const uint8_t *const *colors,
@@ -1615,14 +1745,23 @@ extern "C" mc_status mc_build_tables_batch(int count, const mc_graph *const *gra
         int64_t *urp = scratch.get<int64_t>((size_t)N + 1);
         uint32_t *ucol = scratch.get<uint32_t>((size_t)(NNZ > 0 ? NNZ : 1));
         uint8_t *ucolors = scratch.get<uint8_t>((size_t)(N > 0 ? N : 1));
+        std::vector<ConcatPart> parts((size_t)count);
+        bool on_device = true;  // colours in host memory are copied one by one
         for (int i = 0; i < count; ++i) {
-            const mc_graph *g = graphs[i];
-            if (g->n == 0) continue;
-            MC_LAUNCH("concat_csr", s, concat_csr_kernel<<<grid_for(std::max(g->n, g->nnz), 256), 256, 0, s>>>(
-                                           g->row_ptr, g->col, g->n, g->nnz, noff[i], eoff[i], urp, ucol));
-            MC_CUDA(cudaMemcpyAsync(ucolors + noff[i], colors[i], (size_t)g->n, cudaMemcpyDefault, s));
+            parts[(size_t)i] = {graphs[i]->row_ptr, graphs[i]->col, colors[i], noff[i], eoff[i]};
+            if (graphs[i]->n == 0) continue;
+            cudaPointerAttributes at{};
+            if (cudaPointerGetAttributes(&at, colors[i]) != cudaSuccess) cudaGetLastError();
+            on_device &= at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
         }
-        MC_CUDA(cudaMemcpyAsync(urp + N, &NNZ, sizeof(int64_t), cudaMemcpyHostToDevice, s));
+        ConcatPart *dparts = scratch.get<ConcatPart>((size_t)count);
+        MC_CUDA(cudaMemcpyAsync(dparts, parts.data(), (size_t)count * sizeof(ConcatPart), cudaMemcpyHostToDevice, s));
+        MC_LAUNCH("concat_csr", s, concat_kernel<<<grid_for(std::max(N, NNZ), 256), 256, 0, s>>>(
+                                       dparts, count, N, NNZ, urp, ucol, on_device ? ucolors : nullptr));
+        if (!on_device)
+            for (int i = 0; i < count; ++i)
+                if (graphs[i]->n)
+                    MC_CUDA(cudaMemcpyAsync(ucolors + noff[i], colors[i], (size_t)graphs[i]->n, cudaMemcpyDefault, s));
         mc_status s2 = mc_load_graph(N, NNZ, urp, ucol, MC_GRAPH_DEVICE_PTRS | MC_GRAPH_TRUSTED, alloc, stream, &ug);
         if (s2 != MC_OK) throw Error(s2, std::string("batch graph: ") + mc_last_error());
         s2 = mc_build_tables(ug, ucolors, k, count_bits, flags, alloc, stream, &t);

@@ -9,8 +9,6 @@
 
 namespace mc {
 
-void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s);
-
 static thread_local std::string g_last_error;
 
 void set_last_error(const std::string &msg) { g_last_error = msg; }
@@ -513,15 +511,13 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
         }
         // hub chunks, built on the device: chunk counts per node, their
         // prefix, then one thread per hub writes its chunks
-        u128 *nch = scratch.get<u128>((size_t)(n > 0 ? n : 1));
-        u128 *nhub = scratch.get<u128>((size_t)(n > 0 ? n : 1));
+        u128 *nch = scratch.get<u128>(2 * (size_t)(n > 0 ? n : 1)), *nhub = nch + n;
         int *serr = scratch.get<int>(1);
         MC_CUDA(cudaMemsetAsync(serr, 0, sizeof(int), s));
         if (n > 0) {
             MC_LAUNCH("degree_stats", s, degree_stats<<<grid_for(n, 256), 256, 0, s>>>(
                                              g->row_ptr, n, nch, nhub, (unsigned long long *)(dstat + 1)));
-            inclusive_scan_u128(nch, n, serr, scratch, s);
-            inclusive_scan_u128(nhub, n, serr, scratch, s);
+            inclusive_scan_u128(nch, n, serr, scratch, s, 2);
         }
         int64_t hst[4] = {0, 0, 0, 0};
         MC_CUDA(cudaMemcpyAsync(hst, dstat, sizeof(hst), cudaMemcpyDeviceToHost, s));

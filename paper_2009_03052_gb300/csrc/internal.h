@@ -93,6 +93,14 @@ template <typename F> mc_status guarded(F &&f)
     }
 }
 
+// Inclusive prefix, in place, of m arrays of n entries, one after the other;
+// overflow sets bit 0 of *err.
+void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s, int m = 1);
+// Bucket indexes (bstride entries apart) of m prefixes of n entries, and their
+// widths dD[m].
+void build_buckets(const u128 *prefix, int64_t n, int64_t nb, u128 *dD, uint32_t *start, cudaStream_t s, int m = 1,
+                   int64_t bstride = 0);
+
 int grid_for(int64_t work, int block);
 int sm_count();
 

@@ -8,8 +8,6 @@
 
 namespace mc {
 
-void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s);
-
 __device__ __forceinline__ int count_bytes(u128 x)
 {
     if ((x >> 64) != 0) return 16;
@@ -160,16 +158,14 @@ static PackedView pack_level(mc_tables *t, const Rows &dense, int W, cudaStream_
     scratch.stream = s;
     int *err = scratch.get<int>(1);
     MC_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    u128 *cnt = scratch.get<u128>((size_t)n);
-    u128 *bytes = scratch.get<u128>((size_t)n);
+    u128 *cnt = scratch.get<u128>(2 * (size_t)n), *bytes = cnt + n;
     PackedView p;
     p.width = (int)sizeof(CT);
     uint8_t *wid = t->varlen ? t->arena.get<uint8_t>((size_t)n) : nullptr;
     const int grid = grid_for(n * 32, 256);
     MC_LAUNCH("pack", s, pack_count_kernel<CT><<<grid, 256, 0, s>>>(dense, n, W, t->varlen ? 1 : 0, cnt,
                                                                       bytes, wid));
-    inclusive_scan_u128(cnt, n, err, scratch, s);
-    inclusive_scan_u128(bytes, n, err, scratch, s);
+    inclusive_scan_u128(cnt, n, err, scratch, s, 2);
     int64_t *off = t->arena.get<int64_t>((size_t)n + 1);
     int64_t *boff = t->arena.get<int64_t>((size_t)n + 1);
     MC_LAUNCH("pack", s, offsets_kernel<<<grid_for(n + 1, 256), 256, 0, s>>>(cnt, n, off));

@@ -11,8 +11,6 @@
 
 namespace mc {
 
-void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s);
-
 enum : int { SERR_SEARCH = 1, SERR_CLASS = 2 };
 
 // ---------------------------------------------------------------------------
@@ -1200,7 +1198,6 @@ struct RootIndex {
 void launch_row_totals(const mc_tables *t, int h, uint64_t allow0, uint64_t allow1, u128 *tot, int *err,
                        cudaStream_t s);
 void launch_treelet_totals(const mc_tables *t, int h, u128 *tot, int *err, cudaStream_t s);
-void build_buckets(const u128 *prefix, int64_t n, int64_t nb, u128 *dD, uint32_t *start, cudaStream_t s);
 int64_t bucket_count(int64_t n);
 
 // Restrict a root index to the nodes [lo, hi) (hi <= 0: all nodes).
@@ -1280,20 +1277,23 @@ static std::vector<RootIndex> treelet_root_indexes(const mc_tables *t, int h, Ar
     u128 *p = scratch.get<u128>((size_t)n * nu);
     u128 *dD = scratch.get<u128>((size_t)nu);
     launch_treelet_totals(t, h, p, err, s);
+    // all prefixes and bucket indexes in one launch per kernel
+    const int64_t bs = t->nbucket + 1;
+    uint32_t *bk = scratch.get<uint32_t>((size_t)bs * nu);
+    std::vector<u128> Dj((size_t)nu, 1);
+    inclusive_scan_u128(p, n, err, scratch, s, nu);
+    build_buckets(p, n, t->nbucket, dD, bk, s, nu, bs);
     for (int j = 0; j < nu; ++j) {
-        u128 *pj = p + (size_t)j * n;
-        uint32_t *bk = scratch.get<uint32_t>((size_t)t->nbucket + 1);
-        inclusive_scan_u128(pj, n, err, scratch, s);
-        build_buckets(pj, n, t->nbucket, dD + j, bk, s);
-        if (n) {
-            MC_CUDA(cudaMemcpyAsync(&ris[j].R, pj + (n - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
-            MC_CUDA(cudaMemcpyAsync(&ris[j].D, dD + j, sizeof(u128), cudaMemcpyDeviceToHost, s));
-        }
-        ris[j].prefix = pj;
-        ris[j].bucket = bk;
+        ris[j].prefix = p + (size_t)j * n;
+        ris[j].bucket = bk + j * bs;
+        if (n) MC_CUDA(cudaMemcpyAsync(&ris[j].R, ris[j].prefix + (n - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
     }
+    if (n) MC_CUDA(cudaMemcpyAsync(Dj.data(), dD, (size_t)nu * sizeof(u128), cudaMemcpyDeviceToHost, s));
     MC_CUDA(cudaStreamSynchronize(s));
-    for (int j = 0; j < nu; ++j) restrict_range(ris[j], n, lo, hi, s);
+    for (int j = 0; j < nu; ++j) {
+        ris[j].D = Dj[(size_t)j];
+        restrict_range(ris[j], n, lo, hi, s);
+    }
     return ris;
 }
 
