@@ -159,11 +159,18 @@ def _check(st: int):
 # torch plumbing: device memory and streams
 # ---------------------------------------------------------------------------
 
+_torch_module = None
+
+
 def _torch():
-    import torch
-    if not torch.cuda.is_available():
-        raise RuntimeError("libmotif needs a CUDA device")
-    return torch
+    # the availability check costs as much as a small call: once it has succeeded it holds
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        if not torch.cuda.is_available():
+            raise RuntimeError("libmotif needs a CUDA device")
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream_ptr(stream=None) -> int:

@@ -1433,19 +1433,12 @@ extern "C" mc_status mc_build_tables(const mc_graph *g, const uint8_t *colors, i
         // programs
         const Programs &P = programs(k, t->skip_round);
         for (int j = 0; j < 32; ++j) t->copies_k[j] = P.copies[j];
-        for (int h = 2; h <= k; ++h) {
-            if (t->level_missing(h)) continue;
-            const MergePairs &Q = P.pairs[h];
-            t->p_rec[h] = t->arena.get<uint2>(Q.rec.size() / 2);
-            t->p_terms[h] = t->arena.get<uint32_t>(Q.terms.size());
-            MC_CUDA(cudaMemcpyAsync(t->p_rec[h], Q.rec.data(), Q.rec.size() * 4, cudaMemcpyHostToDevice, s));
-            MC_CUDA(cudaMemcpyAsync(t->p_terms[h], Q.terms.data(), Q.terms.size() * 4, cudaMemcpyHostToDevice, s));
-        }
-        for (int h = 1; h <= k - 1; ++h) {
-            if (t->level_missing(h)) continue;
-            const GatherLevel &L = P.gather[h];
-            t->g_map[h] = t->arena.get<int16_t>(L.map.size());
-            MC_CUDA(cudaMemcpyAsync(t->g_map[h], L.map.data(), L.map.size() * 2, cudaMemcpyHostToDevice, s));
+        uint8_t *prog = t->arena.get<uint8_t>(P.blob.size());
+        MC_CUDA(cudaMemcpyAsync(prog, P.blob.data(), P.blob.size(), cudaMemcpyHostToDevice, s));
+        for (int h = 1; h <= k; ++h) {
+            t->p_rec[h] = (uint2 *)(prog + P.rec_at[h]);
+            t->p_terms[h] = (uint32_t *)(prog + P.terms_at[h]);
+            t->g_map[h] = (int16_t *)(prog + P.map_at[h]);
         }
         // tables
         for (int h = 2; h <= k; ++h)
@@ -1570,6 +1563,13 @@ static std::vector<u128> level_rooted_totals(const mc_tables *t, int h, int j0, 
         return out;
     }
     if (hi <= lo) return out;
+    if (j0 < 0) {
+        ensure_level_index(t, h, s);
+        if (lo == 0 && hi == n) {  // read back with the index
+            out[0] = t->R[h];
+            return out;
+        }
+    }
     Arena scratch(true);
     scratch.alloc = t->arena.alloc;
     scratch.stream = s;
@@ -1599,7 +1599,6 @@ static std::vector<u128> level_rooted_totals(const mc_tables *t, int h, int j0, 
     for (int i = 0; i < nj; ++i) {
         const u128 *pre = nullptr;
         if (j0 < 0) {
-            ensure_level_index(t, h, s);
             pre = t->prefix[h];
         } else {
             uint64_t a0 = 0, a1 = 0;

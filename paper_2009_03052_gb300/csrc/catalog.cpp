@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <map>
+#include <cstring>
 #include <mutex>
 
 namespace mc {
@@ -318,6 +319,17 @@ static Programs build_programs(int k, bool skip)
                     L.map[((size_t)cv * k + cu) * G.Bs[h] + rho] = (int16_t)colex_rank(relu);
                 }
             }
+    }
+    auto put = [&](const void *p, size_t bytes) {
+        const size_t at = P.blob.size();
+        P.blob.resize(at + (bytes + 15) / 16 * 16);
+        if (bytes) std::memcpy(P.blob.data() + at, p, bytes);
+        return at;
+    };
+    for (int h = 1; h <= k; ++h) {
+        P.rec_at[h] = put(P.pairs[h].rec.data(), P.pairs[h].rec.size() * 4);
+        P.terms_at[h] = put(P.pairs[h].terms.data(), P.pairs[h].terms.size() * 4);
+        P.map_at[h] = put(P.gather[h].map.data(), P.gather[h].map.size() * 2);
     }
     return P;
 }

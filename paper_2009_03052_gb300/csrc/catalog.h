@@ -90,6 +90,9 @@ struct Programs {
     MergeLevel merge[MAXK + 1];
     MergePairs pairs[MAXK + 1];
     GatherLevel gather[MAXK + 1];
+    // what the device needs of all levels in one buffer, 16-byte aligned parts
+    std::vector<uint8_t> blob;
+    size_t rec_at[MAXK + 1] = {0}, terms_at[MAXK + 1] = {0}, map_at[MAXK + 1] = {0};
     bool skip = false;
     int bal_left[MAX_SHAPES], bal_right[MAX_SHAPES], bal_beta[MAX_SHAPES];  // per level-k shape (global
                                                                              // ids; -1: not counted)

@@ -49,6 +49,9 @@ void Arena::release_all()
         else alloc.release(b.first, b.second, stream);
     }
     blocks.clear();
+    for (void *c : chunks) alloc.release(c, CHUNK, stream);
+    chunks.clear();
+    chunk_used = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -521,6 +524,13 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
         }
         int64_t hst[4] = {0, 0, 0, 0};
         MC_CUDA(cudaMemcpyAsync(hst, dstat, sizeof(hst), cudaMemcpyDeviceToHost, s));
+        unsigned hh[HUB_CHUNK + 1] = {0}, cur[HUB_CHUNK + 1], oc[2] = {0, 0};  // live until the last synchronisation
+        unsigned *dh = scratch.get<unsigned>(2 * (HUB_CHUNK + 1));
+        MC_CUDA(cudaMemsetAsync(dh, 0, (HUB_CHUNK + 1) * sizeof(unsigned), s));
+        if (n > 0) {
+            MC_LAUNCH("degree_order", s, degree_hist_kernel<<<grid_for(n, 256), 256, 0, s>>>(g->row_ptr, n, dh));
+            MC_CUDA(cudaMemcpyAsync(hh, dh, sizeof(hh), cudaMemcpyDeviceToHost, s));
+        }
         u128 tails[2] = {0, 0};
         if (n > 0) {
             MC_CUDA(cudaMemcpyAsync(&tails[0], nch + (n - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
@@ -559,15 +569,8 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
         // the schedule of the neighbour sums: the other nodes by descending degree
         g->n_small = n - g->n_hubs;
         g->sched = g->arena.get<uint4>((size_t)std::max<int64_t>(g->n_small, 1));
-        unsigned hh[HUB_CHUNK + 1], cur[HUB_CHUNK + 1], oc[2] = {0, 0};  // live until the synchronisation below
         g->n_do = n;
         if (g->n_small > 0) {
-            unsigned *dh = scratch.get<unsigned>(2 * (HUB_CHUNK + 1));
-            MC_CUDA(cudaMemsetAsync(dh, 0, (HUB_CHUNK + 1) * sizeof(unsigned), s));
-            MC_LAUNCH("degree_order", s, degree_hist_kernel<<<grid_for(n, 256), 256, 0, s>>>(g->row_ptr, n, dh));
-            MC_CUDA(cudaMemcpyAsync(hh, dh, sizeof(hh), cudaMemcpyDeviceToHost, s));
-            MC_CUDA(cudaStreamSynchronize(s));
-            g->n_big_hubs = nbig;
             unsigned run = 0;
             for (int d = HUB_CHUNK; d >= 0; --d) { cur[d] = run; run += hh[d]; }
             MC_REQUIRE((int64_t)run == g->n_small, "degree histogram does not match the hub count");

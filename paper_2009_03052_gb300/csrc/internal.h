@@ -48,12 +48,17 @@ struct Allocator {
 // A set of device buffers released together.  A scratch arena (buffers of
 // one call, used on its stream only) takes stream-ordered memory
 // (cudaMallocAsync) when no allocator is given, so concurrent calls on
-// different streams never synchronise the device to allocate.
+// different streams never synchronise the device to allocate.  Other arenas
+// carve buffers of up to 128 KB from chunks of 512 KB: an allocator callback
+// costs microseconds, and the tables of a small graph are some forty buffers.
 struct Arena {
+    static constexpr size_t SMALL = 128 << 10, CHUNK = 512 << 10;
     Allocator alloc;
     cudaStream_t stream = nullptr;
     bool scratch = false;
     std::vector<std::pair<void *, size_t>> blocks;
+    std::vector<void *> chunks;  // of CHUNK bytes; never in `blocks`
+    size_t chunk_used = 0;       // of the last one
     Arena() = default;
     explicit Arena(bool is_scratch) : scratch(is_scratch) {}
     template <typename T> T *get(size_t count)
@@ -61,6 +66,20 @@ struct Arena {
         size_t bytes = count * sizeof(T);
         if (bytes == 0) bytes = 256;
         void *p = nullptr;
+        if (bytes <= SMALL && !(scratch && !alloc.custom)) {
+            bytes = (bytes + 255) & ~(size_t)255;
+            if (chunks.empty() || chunk_used + bytes > CHUNK) {
+                if (void *c = alloc.alloc(CHUNK, stream)) {
+                    chunks.push_back(c);
+                    chunk_used = 0;
+                }
+            }
+            if (!chunks.empty() && chunk_used + bytes <= CHUNK) {
+                p = (char *)chunks.back() + chunk_used;
+                chunk_used += bytes;
+                return static_cast<T *>(p);
+            }
+        }
         if (scratch && !alloc.custom) {
             if (cudaMallocAsync(&p, bytes, stream) != cudaSuccess) { cudaGetLastError(); p = nullptr; }
         } else {
@@ -71,7 +90,7 @@ struct Arena {
         return static_cast<T *>(p);
     }
     void release_all();
-    void release(void *p);  // one block, by its pointer
+    void release(void *p);  // one block, by its pointer (a carved buffer stays)
     ~Arena() { release_all(); }
 };
 

@@ -1328,14 +1328,13 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, cudaStream_t s)
                                      : sample_kernel<u128, u128, false, false, false>);
     if (smem > 40 * 1024)  // beside the static tables
         MC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int per_sm = 0;
-    MC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem));
-    if (per_sm < 1) per_sm = 1;
     int64_t grid = (a.count + block - 1) / block;  // one sample per thread
-    const int64_t cap = (int64_t)sm_count() * per_sm;
-    if (grid > sm_count()) grid = (grid + sm_count() - 1) / sm_count() * sm_count();  // the same number on every SM
-    if (grid > cap) grid = cap;
-    if (grid < 1) grid = 1;
+    if (grid > sm_count()) {
+        int per_sm = 0;
+        MC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem));
+        const int64_t cap = (int64_t)sm_count() * std::max(per_sm, 1);
+        grid = std::min(cap, (grid + sm_count() - 1) / sm_count() * sm_count());  // the same number on every SM
+    }
     MC_LAUNCH("sample", s, kern<<<(unsigned)grid, block, smem, s>>>(a));
 }
 
