@@ -390,6 +390,25 @@ struct SampleSmem {
     int r[MAXK + 1];                    // rooted shapes per size
 };
 
+template <int T> __device__ __forceinline__ void fill_sample_smem(const SampleArgs &a, SampleSmem &sm)
+{
+    for (int i = threadIdx.x; i < (1 << (MAXK - 1)); i += T) sm.crank[i] = a.crank[i];
+    for (int i = threadIdx.x; i < MAXK * 36; i += T) (&sm.unrank[0][0])[i] = (&a.unrank[0][0])[i];
+    for (int i = threadIdx.x; i < MAX_SHAPES; i += T)
+        sm.shape[i] = make_uint2((uint32_t)a.sz[i] | (uint32_t)a.loc[i] << 8 | (uint32_t)a.beta[i] << 16,
+                                 (uint32_t)a.lft[i] | (uint32_t)a.rgt[i] << 8);
+    for (int i = threadIdx.x; i < 2 * (MAXK + 1); i += T) {
+        const int l = i % (MAXK + 1);
+        const Rows &r = i > MAXK ? a.S[l] : a.c[l];
+        sm.level[i / (MAXK + 1)][l] = make_uint4((uint32_t)(uint64_t)r.p0, (uint32_t)((uint64_t)r.p0 >> 32), (uint32_t)r.s0,
+                                                 (uint32_t)r.N | ((a.levels & r.bit) ? 256u : 0u));
+        if (i <= MAXK) sm.r[l] = a.R_[l];
+    }
+    const int h = a.h, P = h * (h - 1) / 2;
+    if (threadIdx.x < P)
+        sm.pair[pair_pos(h, a.pi[threadIdx.x], a.pj[threadIdx.x])] = (uint8_t)(a.pi[threadIdx.x] | a.pj[threadIdx.x] << 4);
+}
+
 // Row x of level h of c (which = 0) or S (1): entry get(idx) of dense rows, or
 // (PK) by a binary search of the packed row's keys.
 template <typename CT, bool PK> struct RowRef {
@@ -599,21 +618,8 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
     uint32_t *const off = s_dyn + 2 * MAXK * T + threadIdx.x;  // their adjacency offsets (low words)
     unsigned int *const s_hist = s_dyn + SAMPLE_WORDS * T;
     __shared__ SampleSmem sm;
-    for (int i = threadIdx.x; i < (1 << (MAXK - 1)); i += T) sm.crank[i] = a.crank[i];
-    for (int i = threadIdx.x; i < MAXK * 36; i += T) (&sm.unrank[0][0])[i] = (&a.unrank[0][0])[i];
-    for (int i = threadIdx.x; i < MAX_SHAPES; i += T)
-        sm.shape[i] = make_uint2((uint32_t)a.sz[i] | (uint32_t)a.loc[i] << 8 | (uint32_t)a.beta[i] << 16,
-                                 (uint32_t)a.lft[i] | (uint32_t)a.rgt[i] << 8);
-    for (int i = threadIdx.x; i < 2 * (MAXK + 1); i += T) {
-        const int l = i % (MAXK + 1);
-        const Rows &r = i > MAXK ? a.S[l] : a.c[l];
-        sm.level[i / (MAXK + 1)][l] = make_uint4((uint32_t)(uint64_t)r.p0, (uint32_t)((uint64_t)r.p0 >> 32), (uint32_t)r.s0,
-                                                 (uint32_t)r.N | ((a.levels & r.bit) ? 256u : 0u));
-        if (i <= MAXK) sm.r[l] = a.R_[l];
-    }
     const int h = a.h, P = h * (h - 1) / 2;
-    if (threadIdx.x < P)
-        sm.pair[pair_pos(h, a.pi[threadIdx.x], a.pj[threadIdx.x])] = (uint8_t)(a.pi[threadIdx.x] | a.pj[threadIdx.x] << 4);
+    fill_sample_smem<T>(a, sm);
     if (a.hist)
         for (int i = threadIdx.x; i < a.ncls; i += T) s_hist[i] = 0;
     __syncthreads();
@@ -980,6 +986,385 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
     }
 }
 
+// Warp-per-sample sampler, for requests of a few samples per resident warp: a
+// warp draws one sample at a time, so that its chain of dependent loads is as
+// short as it gets.  Lane i holds the sample's i-th node and i-th stack entry;
+// scans run 32 M items at a time (each lane M consecutive items, a prefix over
+// the lanes), searches probe 32 places at a time, the first random words of all
+// steps are drawn side by side, and the classification's pairs are one per
+// lane.  Bound by the latency of that chain: 1000 samples at k = 8 (Chung-Lu
+// 300k, 128-bit counts) 0.052 ms against 0.355 with a lane per sample.  For
+// large requests the lanes' repeated scalar work loses (1M samples at k = 5:
+// 7.6 against 1.1 ms; with 8 lanes per sample 3.5).
+template <typename T> __device__ __forceinline__ T warp_get(T x, int src)
+{
+    if constexpr (sizeof(T) == 16) return shfl(x, src);
+    else return __shfl_sync(0xffffffffu, x, src);
+}
+
+// Over items 0 .. len-1 in order, the first whose running sum of val(i)
+// exceeds q (-1 if none or !act), `before` the running sum before it.
+template <int M, typename V, typename F>
+__device__ __forceinline__ int warp_first_exceeding(bool act, int len, V q, F val, V &before)
+{
+    const int j = threadIdx.x & 31;
+    V run = 0;
+    int found = -1;
+    for (int b = 0; __any_sync(0xffffffffu, act && b < len); b += 32 * M) {
+        V x[M], s = 0;
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            const int i = b + j * M + m;
+            x[m] = act && i < len ? val(i) : (V)0;
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m) s += x[m];
+        V inc = s;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const V y = shfl_up(inc, d);
+            if (j >= d) inc += y;
+        }
+        V r = run + inc - s;
+        const unsigned hit = __ballot_sync(0xffffffffu, act && run + inc > q);
+        int mf = M - 1;
+#pragma unroll
+        for (int m = 0; m < M - 1; ++m)
+            if (mf == M - 1) {
+                if (r + x[m] > q) mf = m - M;  // found: stop adding
+                else r += x[m];
+            }
+        if (mf < 0) mf += M;
+        const int src = hit ? __ffs(hit) - 1 : 0;
+        const int at = warp_get(b + j * M + mf, src);
+        const V rb = warp_get(r, src);
+        if (hit && act) { found = at; before = rb; act = false; }
+        run += warp_get(inc, 31);
+    }
+    return found;
+}
+
+// The first i in [lo, hi) with pred(i), false then true along the range (hi if
+// never true): 32 evenly spaced probes per round.
+template <typename P>
+__device__ __forceinline__ int64_t warp_first_true(bool act, int64_t lo, int64_t hi, P pred)
+{
+    const int j = threadIdx.x & 31;
+    while (__any_sync(0xffffffffu, act && lo < hi)) {
+        const bool go = act && lo < hi;
+        const int64_t step = (hi - lo + 31) / 32, p = lo + (j + 1) * step - 1;
+        const bool t = go && (p >= hi || pred(p));
+        const unsigned b = __ballot_sync(0xffffffffu, t);
+        if (go) {
+            const int f = b ? __ffs(b) - 1 : 32;
+            const int64_t nlo = f ? lo + f * step : lo;
+            hi = f < 32 ? min(hi, lo + (f + 1) * step - 1) : hi;
+            lo = min(nlo, hi);
+            if (f == 32) lo = hi;
+        }
+    }
+    return lo;
+}
+
+template <typename CT, typename V, bool PK>
+__global__ void __launch_bounds__(256, 2) sample_warp_kernel(const __grid_constant__ SampleArgs a)
+{
+    constexpr int T = 256, M = 4;
+    extern __shared__ uint32_t s_dyn[];
+    unsigned int *const s_hist = s_dyn;
+    __shared__ SampleSmem sm;
+    const int h = a.h, P = h * (h - 1) / 2;
+    fill_sample_smem<T>(a, sm);
+    if (a.hist)
+        for (int i = threadIdx.x; i < a.ncls; i += T) s_hist[i] = 0;
+    __syncthreads();
+    const int j = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)T + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * T) >> 5;
+    bool bad = false;
+    auto full = [&](const RowRef<CT, PK> &r, int idx) -> CT {
+        return !PK && r.wide ? entry_wide<CT>(a, r.which, r.h, r.x, idx) : r.get(idx);
+    };
+    auto entry = [](int g, unsigned C, int cx, int at) {
+        return (uint32_t)g | C << 8 | (uint32_t)cx << 16 | (uint32_t)at << 20;
+    };
+    for (int64_t sid = warp; sid < a.count; sid += nwarps) {
+        bool ok = true;
+        uint64_t index = a.first_index + (uint64_t)sid;
+        const u128 *prefix = a.prefix;
+        const uint32_t *bucket = a.bucket;
+        u128 R = a.R, Xbase = a.Xbase, D = a.D;
+        uint64_t allow0 = a.allow0, allow1 = a.allow1;
+        if (a.nseg > 0) {  // the part this sample falls in
+            int g = 0;
+            while (g + 1 < a.nseg && sid >= a.seg[g].end) ++g;
+            const SampleSeg &sg = a.seg[g];
+            index = sg.first_index + (uint64_t)(sid - (g ? a.seg[g - 1].end : 0));
+            prefix = sg.prefix;
+            bucket = sg.bucket;
+            R = sg.R;
+            Xbase = sg.Xbase;
+            D = sg.D;
+            allow0 = sg.allow0;
+            allow1 = sg.allow1;
+        }
+        // the first attempt's words of every step, lane s for step s
+        uint32_t pw[4] = {(uint32_t)index, (uint32_t)(index >> 32), (uint32_t)j, 0u};
+        philox(pw, (uint32_t)a.seed, (uint32_t)(a.seed >> 32));
+        // uniform(W) of step `step` (the words of draw_below), false after 128 rejections
+        auto draw = [&](bool act, int step, V W, V &out) -> bool {
+            const V wm1 = W - 1;
+            V mask;
+            if constexpr (sizeof(V) == 16) {
+                const uint64_t hi = (uint64_t)(wm1 >> 64), lo = (uint64_t)wm1;
+                const int bits = hi ? 128 - __clzll(hi) : 64 - __clzll(lo);
+                mask = bits >= 128 ? ~(V)0 : (((V)1) << bits) - 1;
+            } else {
+                const int bits = 64 - __clzll(wm1);
+                mask = bits >= 64 ? ~0ull : (1ull << bits) - 1;
+            }
+            auto value = [&](const uint32_t *w) -> V {
+                V r = (V)w[0] | (V)((uint64_t)w[1] << 32);
+                if constexpr (sizeof(V) == 16) r |= (V)w[2] << 64 | (V)w[3] << 96;
+                return r & mask;
+            };
+            V r = warp_get(value(pw), step);
+            // (each lane masked its own words with this step's mask)
+            {
+                bool need = act && W != 0 && !(r < W);
+                for (uint32_t att = 1; att < 128 && __any_sync(0xffffffffu, need); att += 32) {
+                    uint32_t c[4] = {(uint32_t)index, (uint32_t)(index >> 32), (uint32_t)step, att + j};
+                    philox(c, (uint32_t)a.seed, (uint32_t)(a.seed >> 32));
+                    const V y = value(c);
+                    const unsigned b = __ballot_sync(0xffffffffu, y < W);
+                    const V z = warp_get(y, b ? __ffs(b) - 1 : 0);
+                    if (need && b) { r = z; need = false; }
+                }
+                out = r;
+                return act && W != 0 && !need;
+            }
+        };
+        // ---- root: X = uniform(R); v = first node with prefix[v] > X
+        V X = 0;
+        {
+            const bool d = draw(ok, 0, (V)R, X);
+            if (ok && !d) { ok = false; bad = true; }
+        }
+        X += (V)Xbase;  // a node range: the draw lands inside its part of the prefix
+        int64_t blo = 0, bhi = 0;
+        if (ok) {
+            const uint64_t bk = (uint64_t)(X / (V)D);
+            blo = bucket[bk];
+            bhi = bucket[bk + 1];
+        }
+        const uint32_t v = (uint32_t)warp_first_true(ok, blo, bhi, [&](int64_t i) { return prefix[i] > (u128)X; });
+        V rem = 0;
+        if (ok) {
+            if (!(prefix[v] > (u128)X)) { ok = false; bad = true; }
+            else rem = X - (v ? (V)prefix[v - 1] : (V)0);
+        }
+        // ---- entry of v's level-h row, in (shape id, colour mask) order
+        int s0 = 0, sp = 0, nn = 0;
+        uint32_t par = 0;  // per node, four bits: its parent's place in the node list
+        uint32_t mynode = 0, mystk = 0;
+        {
+            const int Bc = a.Bc[h], Rh = a.R_[h];
+            const RowRef<CT, PK> row(a, sm, 0, h, ok ? v : 0);
+            V bf;
+            const int found = warp_first_exceeding<M, V>(ok, a.Wc[h], rem, [&](int e) -> V {
+                const int sh = e / Bc;
+                const bool al = sh < 64 ? (allow0 >> sh) & 1 : (allow1 >> (sh - 64)) & 1;
+                return al ? (V)full(row, (e - sh * Bc) * Rh + sh) : (V)0;
+            }, bf);
+            if (ok && found < 0) { ok = false; bad = true; }
+            if (ok) {
+                const int cv = a.colors[v];
+                s0 = found / Bc;
+                const unsigned C = (1u << cv) | insert_colour_gap(sm.unrank[h - 1][found % Bc], cv);
+                if (j == 0) { mystk = entry(a.first[h] + s0, C, cv, 0); mynode = v; }
+                sp = nn = 1;
+            }
+        }
+        // ---- descent: decomposition nodes in pre-order (T' before T'')
+        for (int step = 1; step < h; ++step) {
+            uint2 sg = make_uint2(0, 0);
+            uint32_t en = 0;
+            bool look = ok;
+            while (__any_sync(0xffffffffu, look)) {  // leaves on top of the stack are done
+                if (look && (sp <= 0 || nn >= MAXK)) { ok = look = false; bad = true; }
+                if (look) --sp;
+                const uint32_t e = warp_get(mystk, sp & 31);
+                if (look) {
+                    en = e;
+                    sg = sm.shape[en & 255u];
+                    if ((sg.x & 255u) > 1) look = false;
+                }
+            }
+            const int cx = (int)(en >> 16 & 15u), at = (int)(en >> 20);
+            const unsigned C = en >> 8 & 255u;
+            const uint32_t x = warp_get(mynode, at & 31);
+            const int ga = (int)(sg.y & 255u), gb = (int)(sg.y >> 8 & 255u);
+            const uint32_t sa = sm.shape[ga].x, sb = sm.shape[gb].x;
+            const int hg = (int)(sg.x & 255u), ha = (int)(sa & 255u), la = (int)(sa >> 8 & 255u);
+            const int hb = (int)(sb & 255u), lb = (int)(sb >> 8 & 255u);
+            int64_t e0 = 0, deg = 0;
+            int chunk0 = -1;
+            // colour sets relative to x: c_x deleted from the palette
+            const unsigned rest = drop_colour(C & ~(1u << cx), cx);
+            V W = 0, Y = 0;
+            if (ok) {
+                e0 = a.row_ptr[x];
+                deg = a.row_ptr[x + 1] - e0;
+                chunk0 = a.node_chunk0[x];
+                W = (V)(sg.x >> 16 & 255u) *
+                    (V)full(RowRef<CT, PK>(a, sm, 0, hg, x), sm.crank[rest] * sm.r[hg] + (int)(sg.x >> 8 & 255u));
+            }
+            {
+                const bool d = draw(ok, step, W, Y);
+                if (ok && !d) { ok = false; bad = true; }
+            }
+            // block of C'' (ascending mask), weights c(T'_{C\C''}, x) S(T'', C'', x)
+            const uint32_t pos = bit_positions(rest);
+            const int nr = __popc(rest);
+            int nsub = 1;
+            for (int i = 1; i <= hb; ++i) nsub = nsub * (nr - hb + i) / i;
+            const int Ra = sm.r[ha], Rb = sm.r[hb];
+            unsigned c2 = 0;
+            CT q = 0;
+            {
+                const RowRef<CT, PK> ra(a, sm, 0, ha, ok ? x : 0), rb_(a, sm, 1, hb, ok ? x : 0);
+                auto count_a = [&](unsigned m) -> V {
+                    return ha == 1 ? (V)1 : (V)full(ra, sm.crank[rest & ~m] * Ra + la);
+                };
+                V before = 0;
+                const int blk = warp_first_exceeding<2, V>(ok, nsub, Y, [&](int i) -> V {
+                    const unsigned m = select_bits(sm.unrank[hb][i], pos);
+                    return count_a(m) * (V)full(rb_, sm.crank[m] * Rb + lb);
+                }, before);
+                if (ok && blk < 0) { ok = false; bad = true; }
+                if (ok) {
+                    c2 = select_bits(sm.unrank[hb][blk], pos);
+                    q = (CT)quotient(Y - before, count_a(c2));  // < S(T'', C'', x): fits CT
+                }
+            }
+            const unsigned C2 = insert_colour_gap(c2, cx);
+            uint32_t u = 0;
+            int cu = 0;
+            const bool single = ok && hb == 1, scan = ok && hb != 1;
+            if (single) {
+                // T'' one node: the (q+1)-th neighbour of the one colour of C'', at
+                // position q of that colour's block in the colour-sorted adjacency
+                cu = __ffs(C2) - 1;
+                const int32_t b0 = a.coff[(int64_t)x * (a.k + 1) + cu];
+                const int32_t b1 = a.coff[(int64_t)x * (a.k + 1) + cu + 1];
+                if ((uint64_t)q >= (uint64_t)(b1 - b0)) { ok = false; bad = true; }
+                else u = a.scol[e0 + b0 + (int64_t)q];
+            }
+            if (__any_sync(0xffffffffu, scan)) {
+                // ---- hub: the first 64-neighbour chunk whose prefix of the chunk sums
+                // (contiguous per hub and entry) exceeds q
+                int64_t lo_e = e0, len = deg;
+                bool act = scan;
+                const bool hub = scan && chunk0 >= 0;
+                const int64_t nch = (deg + HUB_CHUNK - 1) / HUB_CHUNK;
+                const CT *spp = nullptr;
+                if (hub)
+                    spp = (const CT *)a.Sp[hb] + (int64_t)chunk0 * a.Ws[hb] + (int64_t)(sm.crank[c2] * Rb + lb) * nch;
+                const int64_t ci = warp_first_true(hub, 0, nch - 1, [&](int64_t i) { return spp[i] > q; });
+                if (hub) {
+                    if (!(spp[ci] > q)) { ok = act = false; bad = true; }
+                    else {
+                        lo_e = e0 + ci * HUB_CHUNK;
+                        len = min((int64_t)HUB_CHUNK, deg - ci * HUB_CHUNK);
+                        q -= ci ? spp[ci - 1] : (CT)0;
+                    }
+                }
+                // ---- neighbour: first u (ascending) whose running sum of
+                // c(T''_{C''}, u) exceeds q (at most HUB_CHUNK neighbours)
+                CT bn;
+                const int r = warp_first_exceeding<2, CT>(act, (int)len, q, [&](int i) -> CT {
+                    const int ci2 = a.ecol[lo_e + i];
+                    if (!((C2 >> ci2) & 1u)) return (CT)0;
+                    const uint32_t w = a.col[lo_e + i];
+                    return full(RowRef<CT, PK>(a, sm, 0, hb, w), sm.crank[drop_colour(C2 & ~(1u << ci2), ci2)] * Rb + lb);
+                }, bn);
+                if (act) {
+                    if (r < 0) { ok = false; bad = true; }
+                    else {
+                        u = a.col[lo_e + r];
+                        cu = a.ecol[lo_e + r];
+                    }
+                }
+            }
+            if (ok) {
+                if (sp + 2 > MAXK) { ok = false; bad = true; }
+                else {
+                    if (j == nn) mynode = u;
+                    par |= (uint32_t)at << (4 * nn);
+                    if (j == sp) mystk = entry(gb, C2, cu, nn);
+                    if (j == sp + 1) mystk = entry(ga, C & ~C2, cx, at);
+                    sp += 2;
+                    ++nn;
+                }
+            }
+        }
+        if (ok && nn != h) { ok = false; bad = true; }
+        // induced subgraph, its nodes in order of discovery (the class does not
+        // depend on the labels): the treelet's edges are known; the other pairs
+        // are searched in the shorter adjacency list, spread over the lanes
+        uint32_t word = 0;
+        for (int i = 1; i < h; ++i) word |= 1u << pair_pos(h, (int)(par >> (4 * i) & 15u), i);
+        int64_t mylo = 0;
+        uint32_t mydeg = 0;
+        if (ok && j < h) {
+            mylo = a.row_ptr[mynode];
+            mydeg = (uint32_t)(a.row_ptr[mynode + 1] - mylo);
+        }
+        {
+            const unsigned ij = j < P ? sm.pair[j] : 0u;
+            const int x = (int)(ij & 15u), y = (int)(ij >> 4);
+            const uint32_t dx = warp_get(mydeg, x), dy = warp_get(mydeg, y);
+            const bool sw = dy < dx;
+            const uint32_t key = warp_get(mynode, sw ? x : y);
+            const uint32_t *row = a.col + warp_get(mylo, sw ? y : x);
+            uint32_t lo = 0, hi = (ok && j < P && !((word >> j) & 1u)) ? (sw ? dy : dx) : 0u;
+            bool mine = false;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1, w = row[mid];
+                if (w == key) { mine = true; hi = lo; }
+                else if (w < key) lo = mid + 1;
+                else hi = mid;
+            }
+            __syncwarp();
+            word |= __ballot_sync(0xffffffffu, mine);
+        }
+        int cls = -1;
+        if (ok) {
+            cls = a.lut[word];
+            if (cls == 0xffff) { cls = -1; bad = true; }
+        }
+        if (a.nodes) {  // ascending: a lane's node goes to its rank
+            int rank = 0;
+            for (int i = 0; i < h; ++i) rank += warp_get(mynode, i) < mynode;
+            if (ok && j < h) a.nodes[sid * h + rank] = mynode;
+        }
+        if (j == 0) {
+            if (ok) {
+                if (a.roots) a.roots[sid] = v;
+                if (a.shapes) a.shapes[sid] = s0;
+                if (a.hist && cls >= 0) atomicAdd(&s_hist[cls], 1u);
+            }
+            if (a.classes) a.classes[sid] = cls;
+        }
+    }
+    if (bad) atomicOr(a.err, SERR_SEARCH);
+    if (a.hist) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < a.ncls; i += T)
+            if (s_hist[i]) atomicAdd(&a.hist[i], (unsigned long long)s_hist[i]);
+    }
+}
+
 // Uniform estimator (Section 2.2): g_i = ((t * hits_i) / (sigma_i * N)) * (1/p),
 // one correctly rounded operation at a time.
 __global__ void uniform_estimate_kernel(const unsigned long long *hits, const int64_t *sigma, int ncls,
@@ -1302,8 +1687,13 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, cudaStream_t s)
     // a launch that leaves most SMs idle runs the latency mode (dense tables)
     // in blocks of 64, spread over more SMs
     const bool lat = !t->packed && a.count <= (int64_t)sm_count() * 256;
-    const int block = lat ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
-    const size_t smem = ((size_t)SAMPLE_WORDS * block + (a.hist ? (size_t)a.ncls : 0)) * sizeof(uint32_t);
+    // a warp per sample for at most two samples per resident warp (2 blocks of
+    // 256 per SM), four when h >= 5 (longer chains: us lane / warp at 4500 and
+    // 10000 samples 40 / 39 and 40 / 76 at k = 4, 159 / 63 and 159 / 126 at
+    // k = 5, 289 / 100 and 292 / 216 at k = 7, 373 / 105 and 375 / 236 at k = 8)
+    const bool warps = a.count <= (int64_t)sm_count() * (a.h >= 5 ? 64 : 32);
+    const int block = warps ? 256 : lat ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
+    const size_t smem = ((size_t)(warps ? 0 : SAMPLE_WORDS) * block + (a.hist ? (size_t)a.ncls : 0)) * sizeof(uint32_t);
     // one wave of resident blocks: the grid-stride loop then keeps every
     // warp busy until the samples run out
     // 64-bit descent arithmetic is exact when 8 R < 2^64: every weight is at
@@ -1312,9 +1702,15 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, cudaStream_t s)
     const bool narrow = t->bits == 64 && ((a.R + a.Xbase) >> 61) == 0;
     // byte counting (profiling) runs its own instantiation of the dense,
     // throughput-mode kernel, so uncounted launches carry none of its work
-    const bool cnt = a.bytes != nullptr && !t->packed && !lat;
+    const bool cnt = a.bytes != nullptr && !t->packed && !lat && !warps;
     if (!cnt) a.bytes = nullptr;
-    auto kern = t->packed ? (t->bits == 64 ? (narrow ? sample_kernel<uint64_t, uint64_t, true, false, false>
+    auto kern = warps ? (t->packed ? (t->bits == 64 ? (narrow ? sample_warp_kernel<uint64_t, uint64_t, true>
+                                                              : sample_warp_kernel<uint64_t, u128, true>)
+                                                    : sample_warp_kernel<u128, u128, true>)
+                                   : (t->bits == 64 ? (narrow ? sample_warp_kernel<uint64_t, uint64_t, false>
+                                                              : sample_warp_kernel<uint64_t, u128, false>)
+                                                    : sample_warp_kernel<u128, u128, false>))
+              : t->packed ? (t->bits == 64 ? (narrow ? sample_kernel<uint64_t, uint64_t, true, false, false>
                                                      : sample_kernel<uint64_t, u128, true, false, false>)
                                            : sample_kernel<u128, u128, true, false, false>)
               : lat ? (t->bits == 64 ? (narrow ? sample_kernel<uint64_t, uint64_t, false, true, false>
@@ -1328,7 +1724,7 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, cudaStream_t s)
                                      : sample_kernel<u128, u128, false, false, false>);
     if (smem > 40 * 1024)  // beside the static tables
         MC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int64_t grid = (a.count + block - 1) / block;  // one sample per thread
+    int64_t grid = warps ? (a.count + 7) / 8 : (a.count + block - 1) / block;  // one sample per warp or thread
     if (grid > sm_count()) {
         int per_sm = 0;
         MC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem));
