@@ -481,26 +481,37 @@ __global__ void __launch_bounds__(256) treelet_totals_kernel(Rows c, int64_t n, 
 
 constexpr int SCAN_THREADS = 512, SCAN_ITEMS = 8, SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 
-__device__ __forceinline__ u128 block_exclusive_scan(u128 x, u128 *smem, u128 &block_total)
+template <typename T> __device__ __forceinline__ T warp_prefix(T x)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const T y = shfl_up(x, d);
+        if (lane >= d) x += y;
+    }
+    return x;
+}
+
+template <typename T> __device__ __forceinline__ T block_exclusive_scan(T x, T *smem, T &block_total)
 {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const u128 inc = warp_inclusive_scan(x);
+    const T inc = warp_prefix(x);
     if (lane == 31) smem[w] = inc;
     __syncthreads();
     if (w == 0) {
         const int nw = blockDim.x >> 5;
-        u128 y = lane < nw ? smem[lane] : 0;
-        y = warp_inclusive_scan(y);
+        T y = lane < nw ? smem[lane] : (T)0;
+        y = warp_prefix(y);
         if (lane < nw) smem[lane] = y;
     }
     __syncthreads();
-    const u128 before = w > 0 ? smem[w - 1] : 0;
+    const T before = w > 0 ? smem[w - 1] : (T)0;
     block_total = smem[(blockDim.x >> 5) - 1];
     __syncthreads();
     return before + inc - x;
 }
 
-// Inclusive u128 prefix of m arrays of n entries, `stride` entries apart
+// Inclusive 64- or 128-bit prefix of m arrays of n entries, `stride` entries apart
 // (blockIdx.y picks one): tile sums, then each block adds up the sums of the
 // tiles before its own and scans its tile.  One tile (n <= 4096) needs the
 // second kernel only; beyond SCAN_DIRECT tiles the sums are scanned by a
@@ -508,39 +519,39 @@ __device__ __forceinline__ u128 block_exclusive_scan(u128 x, u128 *smem, u128 &b
 // most 32 KB here; a tile is 64 KB).  Launches 3 -> 2 (1 for small arrays).
 constexpr int64_t SCAN_DIRECT = 2048;
 
-__global__ void __launch_bounds__(SCAN_THREADS) scan_tiles_kernel(const u128 *__restrict__ x, int64_t n, int64_t stride,
-                                                                  u128 *__restrict__ tile_sum, int *err)
+template <typename T> __global__ void __launch_bounds__(SCAN_THREADS) scan_tiles_kernel(const T *__restrict__ x, int64_t n, int64_t stride,
+                                                                  T *__restrict__ tile_sum, int *err)
 {
-    __shared__ u128 smem[32];
+    __shared__ T smem[32];
     x += blockIdx.y * stride;
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-    u128 s = 0;
+    T s = 0;
     bool ovf = false;
     for (int i = 0; i < SCAN_ITEMS; ++i)
         if (base + i < n) ovf |= add_ovf(s, x[base + i]);
-    u128 tot;
-    const u128 ex = block_exclusive_scan(s, smem, tot);
+    T tot;
+    const T ex = block_exclusive_scan(s, smem, tot);
     // the block total is exact iff no prefix wrapped
     if (ex + s < ex) ovf = true;
     if (threadIdx.x == blockDim.x - 1) tile_sum[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = tot;
     if (ovf) atomicOr(err, ERR_OVERFLOW);
 }
 
-__global__ void __launch_bounds__(1024) scan_tile_sums_kernel(u128 *tile_sum, int64_t ntiles, int *err)
+template <typename T> __global__ void __launch_bounds__(1024) scan_tile_sums_kernel(T *tile_sum, int64_t ntiles, int *err)
 {
-    __shared__ u128 smem[32];
+    __shared__ T smem[32];
     tile_sum += blockIdx.y * ntiles;
-    u128 carry = 0;
+    T carry = 0;
     bool ovf = false;
     for (int64_t b = 0; b < ntiles; b += blockDim.x) {
         const int64_t i = b + threadIdx.x;
-        const u128 x = i < ntiles ? tile_sum[i] : 0;
-        u128 tot;
-        const u128 ex = block_exclusive_scan(x, smem, tot);
-        const u128 before = carry + ex;
+        const T x = i < ntiles ? tile_sum[i] : 0;
+        T tot;
+        const T ex = block_exclusive_scan(x, smem, tot);
+        const T before = carry + ex;
         if (before < carry || before + x < before) ovf = true;
         if (i < ntiles) tile_sum[i] = before;  // exclusive
-        const u128 nc = carry + tot;
+        const T nc = carry + tot;
         if (nc < carry) ovf = true;
         carry = nc;
     }
@@ -548,33 +559,33 @@ __global__ void __launch_bounds__(1024) scan_tile_sums_kernel(u128 *tile_sum, in
 }
 
 // `scanned`: tile_sum holds the sums before each tile, else the tiles' own
-__global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(u128 *__restrict__ x, int64_t n, int64_t stride,
-                                                                  const u128 *__restrict__ tile_sum, bool scanned, int *err)
+template <typename T> __global__ void __launch_bounds__(SCAN_THREADS) scan_apply_kernel(T *__restrict__ x, int64_t n, int64_t stride,
+                                                                  const T *__restrict__ tile_sum, bool scanned, int *err)
 {
-    __shared__ u128 smem[32];
+    __shared__ T smem[32];
     bool ovf = false;
     x += blockIdx.y * stride;
-    u128 before = 0;
+    T before = 0;
     if (scanned) {
         before = tile_sum[(int64_t)blockIdx.y * gridDim.x + blockIdx.x];
     } else if (blockIdx.x > 0) {
         tile_sum += (int64_t)blockIdx.y * gridDim.x;
-        u128 s = 0;
+        T s = 0;
         for (int t = threadIdx.x; t < (int)blockIdx.x; t += SCAN_THREADS) ovf |= add_ovf(s, tile_sum[t]);
-        const u128 ex = block_exclusive_scan(s, smem, before);
+        const T ex = block_exclusive_scan(s, smem, before);
         if (ex + s < ex) ovf = true;
     }
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-    u128 v[SCAN_ITEMS];
-    u128 s = 0;
+    T v[SCAN_ITEMS];
+    T s = 0;
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; ++i) {
         v[i] = base + i < n ? x[base + i] : 0;
         ovf |= add_ovf(s, v[i]);
     }
-    u128 tot;
-    const u128 ex = block_exclusive_scan(s, smem, tot);
-    u128 run = before + ex;
+    T tot;
+    const T ex = block_exclusive_scan(s, smem, tot);
+    T run = before + ex;
     if (run < before || run + s < run) ovf = true;
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; ++i) {
@@ -875,22 +886,27 @@ __global__ void fill_ones_kernel(void *dst, int64_t n, int bytes)
 static int64_t scan_tiles(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
 
 // the scan with a caller-provided tile-sum buffer of m * scan_tiles(n) entries
-static void inclusive_scan_u128_buf(u128 *x, int64_t n, int *err, u128 *ts, cudaStream_t s, int m = 1)
+template <typename T>
+static void inclusive_scan_buf(T *x, int64_t n, int64_t stride, int *err, T *ts, cudaStream_t s, int m)
 {
     if (n <= 0) return;
     const int64_t ntiles = scan_tiles(n);
     const dim3 grid((unsigned)ntiles, (unsigned)m);
     const bool scanned = ntiles > SCAN_DIRECT;
-    if (ntiles > 1) MC_LAUNCH("scan_tiles", s, scan_tiles_kernel<<<grid, SCAN_THREADS, 0, s>>>(x, n, n, ts, err));
+    if (ntiles > 1) MC_LAUNCH("scan_tiles", s, scan_tiles_kernel<T><<<grid, SCAN_THREADS, 0, s>>>(x, n, stride, ts, err));
     if (scanned)
-        MC_LAUNCH("scan_tile_sums", s, scan_tile_sums_kernel<<<dim3(1, (unsigned)m), 1024, 0, s>>>(ts, ntiles, err));
-    MC_LAUNCH("scan_apply", s, scan_apply_kernel<<<grid, SCAN_THREADS, 0, s>>>(x, n, n, ts, scanned, err));
+        MC_LAUNCH("scan_tile_sums", s, scan_tile_sums_kernel<T><<<dim3(1, (unsigned)m), 1024, 0, s>>>(ts, ntiles, err));
+    MC_LAUNCH("scan_apply", s, scan_apply_kernel<T><<<grid, SCAN_THREADS, 0, s>>>(x, n, stride, ts, scanned, err));
 }
 
 void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s, int m)
 {
-    if (n <= 0) return;
-    inclusive_scan_u128_buf(x, n, err, scratch.get<u128>((size_t)scan_tiles(n) * m), s, m);
+    if (n > 0) inclusive_scan_buf<u128>(x, n, n, err, scratch.get<u128>((size_t)scan_tiles(n) * m), s, m);
+}
+
+void inclusive_scan_u64(uint64_t *x, int64_t n, int64_t stride, int *err, Arena &scratch, cudaStream_t s, int m)
+{
+    if (n > 0) inclusive_scan_buf<uint64_t>(x, n, stride, err, scratch.get<uint64_t>((size_t)scan_tiles(n) * m), s, m);
 }
 
 ExactDiv make_div(int beta)
@@ -1360,7 +1376,7 @@ static void enqueue_build(mc_tables *t, const uint8_t *colors, cudaStream_t s, b
     // levels get theirs on first use
     if (n) {
         launch_row_totals(t, k, ~0ull, ~0ull, t->prefix[k], err, s);
-        inclusive_scan_u128_buf(t->prefix[k], n, err, t->scan_tmp, s);
+        inclusive_scan_buf<u128>(t->prefix[k], n, n, err, t->scan_tmp, s, 1);
         build_buckets(t->prefix[k], n, t->nbucket, t->dev_D, t->bucket[k], s);
     }
 }

@@ -101,13 +101,13 @@ __global__ void validate_offsets(const int64_t *row_ptr, int64_t n, int64_t nnz,
 // per node: number of hub chunks (0 unless degree > HUB_CHUNK) and whether
 // it is a hub; the largest degree (stat[0]) and the sum of the squared
 // degrees (stat[1])
-__global__ void degree_stats(const int64_t *row_ptr, int64_t n, u128 *nch, u128 *nhub, unsigned long long *stat)
+__global__ void degree_stats(const int64_t *row_ptr, int64_t n, uint64_t *nch, uint64_t *nhub, unsigned long long *stat)
 {
     unsigned long long md = 0, sq = 0;
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t d = row_ptr[v + 1] - row_ptr[v];
-        nch[v] = d > HUB_CHUNK ? (u128)((d + HUB_CHUNK - 1) / HUB_CHUNK) : (u128)0;
+        nch[v] = d > HUB_CHUNK ? (uint64_t)((d + HUB_CHUNK - 1) / HUB_CHUNK) : 0;
         nhub[v] = d > HUB_CHUNK ? 1 : 0;
         if ((unsigned long long)d > md) md = (unsigned long long)d;
         sq += (unsigned long long)d * (unsigned long long)d;
@@ -127,7 +127,7 @@ __global__ void degree_stats(const int64_t *row_ptr, int64_t n, u128 *nch, u128 
 // from the inclusive prefixes of chunk and hub counts: every hub writes its
 // chunks (node, first edge, end edge), its entry in the hub list and its
 // first chunk
-__global__ void hub_chunks(const int64_t *row_ptr, int64_t n, const u128 *nch, const u128 *nhub,
+__global__ void hub_chunks(const int64_t *row_ptr, int64_t n, const uint64_t *nch, const uint64_t *nhub,
                            uint32_t *chunk_node, int64_t *chunk_e0, int64_t *chunk_e1, uint32_t *hub_node,
                            int64_t *hub_chunk0, int32_t *node_chunk0, int64_t n_hubs, int64_t n_chunks)
 {
@@ -514,13 +514,13 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
         }
         // hub chunks, built on the device: chunk counts per node, their
         // prefix, then one thread per hub writes its chunks
-        u128 *nch = scratch.get<u128>(2 * (size_t)(n > 0 ? n : 1)), *nhub = nch + n;
+        uint64_t *nch = scratch.get<uint64_t>(2 * (size_t)(n > 0 ? n : 1)), *nhub = nch + n;
         int *serr = scratch.get<int>(1);
         MC_CUDA(cudaMemsetAsync(serr, 0, sizeof(int), s));
         if (n > 0) {
             MC_LAUNCH("degree_stats", s, degree_stats<<<grid_for(n, 256), 256, 0, s>>>(
                                              g->row_ptr, n, nch, nhub, (unsigned long long *)(dstat + 1)));
-            inclusive_scan_u128(nch, n, serr, scratch, s, 2);
+            inclusive_scan_u64(nch, n, n, serr, scratch, s, 2);
         }
         int64_t hst[4] = {0, 0, 0, 0};
         MC_CUDA(cudaMemcpyAsync(hst, dstat, sizeof(hst), cudaMemcpyDeviceToHost, s));
@@ -531,10 +531,10 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
             MC_LAUNCH("degree_order", s, degree_hist_kernel<<<grid_for(n, 256), 256, 0, s>>>(g->row_ptr, n, dh));
             MC_CUDA(cudaMemcpyAsync(hh, dh, sizeof(hh), cudaMemcpyDeviceToHost, s));
         }
-        u128 tails[2] = {0, 0};
+        uint64_t tails[2] = {0, 0};
         if (n > 0) {
-            MC_CUDA(cudaMemcpyAsync(&tails[0], nch + (n - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
-            MC_CUDA(cudaMemcpyAsync(&tails[1], nhub + (n - 1), sizeof(u128), cudaMemcpyDeviceToHost, s));
+            MC_CUDA(cudaMemcpyAsync(&tails[0], nch + (n - 1), sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
+            MC_CUDA(cudaMemcpyAsync(&tails[1], nhub + (n - 1), sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
         }
         MC_CUDA(cudaStreamSynchronize(s));
         MC_REQUIRE(((int *)hst)[0] == 0, "graph is not a canonical symmetric CSR (flags " +

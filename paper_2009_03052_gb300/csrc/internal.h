@@ -112,9 +112,10 @@ template <typename F> mc_status guarded(F &&f)
     }
 }
 
-// Inclusive prefix, in place, of m arrays of n entries, one after the other;
-// overflow sets bit 0 of *err.
+// Inclusive prefix, in place, of m arrays of n entries, one after the other
+// (or `stride` entries apart); overflow sets bit 0 of *err.
 void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s, int m = 1);
+void inclusive_scan_u64(uint64_t *x, int64_t n, int64_t stride, int *err, Arena &scratch, cudaStream_t s, int m = 1);
 // Bucket indexes (bstride entries apart) of m prefixes of n entries, and their
 // widths dD[m].
 void build_buckets(const u128 *prefix, int64_t n, int64_t nb, u128 *dD, uint32_t *start, cudaStream_t s, int m = 1,

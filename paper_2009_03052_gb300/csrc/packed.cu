@@ -31,77 +31,71 @@ __device__ __forceinline__ void store_count(uint8_t *q, u128 x, int w)
     }
 }
 
-__device__ __forceinline__ u128 warp_max(u128 x)
-{
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        const u128 y = shfl_xor(x, d);
-        if (y > x) x = y;
-    }
-    return x;
-}
+// Lanes per node of the packing passes: narrow rows share a warp.
+__host__ __device__ __forceinline__ int pack_lanes(int W) { return W <= 16 ? 8 : W <= 64 ? 16 : 32; }
 
-// Pass 1, a warp per node: the row's non-zero entries, the bytes per count
+// Pass 1, G lanes per node: the row's non-zero entries, the bytes per count
 // (varlen: the row's own width, else the table's) and the row's count bytes
-// rounded up to 8.
+// rounded up to 8, one place on: their inclusive prefix, in place, is the
+// row offsets.
 template <typename CT>
-__global__ void pack_count_kernel(Rows D, int64_t n, int W, int varlen, u128 *cnt,
-                                  u128 *bytes, uint8_t *wid)
+__global__ void pack_count_kernel(Rows D, int64_t n, int W, int varlen, int64_t *off, int64_t *boff, uint8_t *wid)
 {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, G = pack_lanes(W), NG = 32 / G, j = lane & (G - 1);
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = w0; v < n; v += nw) {
+    for (int64_t base = w0 * NG; base < n; base += nw * NG) {
+        const int64_t v = base + lane / G;
         unsigned nz = 0;
         u128 mx = 0;
-        for (int e = lane; e < W; e += 32) {
-            const u128 x = widen(entry_at<CT>(D, v, e));
-            nz += x != 0;
-            if (x > mx) mx = x;
+        if (v < n)
+            for (int e = j; e < W; e += G) {
+                const u128 x = widen(entry_at<CT>(D, v, e));
+                nz += x != 0;
+                if (x > mx) mx = x;
+            }
+        for (int d = G >> 1; d > 0; d >>= 1) {
+            nz += __shfl_xor_sync(0xffffffffu, nz, d);
+            const u128 y = shfl_xor(mx, d);
+            if (y > mx) mx = y;
         }
-        for (int d = 16; d > 0; d >>= 1) nz += __shfl_xor_sync(0xffffffffu, nz, d);
-        mx = warp_max(mx);
-        if (lane == 0) {
+        if (j == 0 && v < n) {
             const int w = varlen ? count_bytes(mx) : (int)sizeof(CT);
-            cnt[v] = nz;
-            bytes[v] = ((u128)nz * w + 7) & ~(u128)7;
+            off[v + 1] = nz;
+            boff[v + 1] = ((int64_t)nz * w + 7) & ~(int64_t)7;
+            if (v == 0) off[0] = boff[0] = 0;
             if (wid) wid[v] = (uint8_t)w;
         }
     }
 }
 
-// Exclusive int64 offsets (n + 1 of them) from an inclusive u128 prefix.
-__global__ void offsets_kernel(const u128 *__restrict__ inc, int64_t n, int64_t *__restrict__ off)
-{
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v <= n; v += (int64_t)gridDim.x * blockDim.x)
-        off[v] = v == 0 ? 0 : (int64_t)inc[v - 1];
-}
-
-// Pass 2, a warp per node: keys and counts of the non-zero entries, in row
+// Pass 2, G lanes per node: keys and counts of the non-zero entries, in row
 // order.
 template <typename CT>
 __global__ void pack_fill_kernel(Rows D, int64_t n, int W, PackedView p, uint16_t *__restrict__ key,
                                  uint8_t *__restrict__ val)
 {
-    const int lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
+    const int lane = threadIdx.x & 31, G = pack_lanes(W), NG = 32 / G, j = lane & (G - 1), g0 = lane - j;
+    const unsigned lt = (1u << j) - 1u, gm = G == 32 ? 0xffffffffu : (1u << G) - 1u;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = w0; v < n; v += nw) {
-        const int64_t o0 = p.off[v];
-        const int w = p.wid ? (int)p.wid[v] : p.width;
-        uint8_t *q0 = val + p.boff[v];
-        int64_t base = 0;
-        for (int e0 = 0; e0 < W; e0 += 32) {
-            const int e = e0 + lane;
-            const u128 x = e < W ? widen(entry_at<CT>(D, v, e)) : (u128)0;
-            const unsigned m = __ballot_sync(0xffffffffu, x != 0);
+    for (int64_t base = w0 * NG; base < n; base += nw * NG) {
+        const int64_t v = base + lane / G;
+        const bool in = v < n;
+        const int64_t o0 = in ? p.off[v] : 0;
+        const int w = !in ? 8 : p.wid ? (int)p.wid[v] : p.width;
+        uint8_t *q0 = val + (in ? p.boff[v] : 0);
+        int64_t done = 0;
+        for (int e0 = 0; e0 < W; e0 += G) {
+            const int e = e0 + j;
+            const u128 x = in && e < W ? widen(entry_at<CT>(D, v, e)) : (u128)0;
+            const unsigned m = (__ballot_sync(0xffffffffu, x != 0) >> g0) & gm;
             if (x != 0) {
-                const int64_t j = base + __popc(m & lt);
-                key[o0 + j] = (uint16_t)e;
-                store_count(q0 + j * w, x, w);
+                const int64_t at = done + __popc(m & lt);
+                key[o0 + at] = (uint16_t)e;
+                store_count(q0 + at * w, x, w);
             }
-            base += __popc(m);
+            done += __popc(m);
         }
     }
 }
@@ -149,8 +143,10 @@ __global__ void unpack_kernel(PackedView p, int64_t n, int W, CT *__restrict__ d
     }
 }
 
-template <typename CT>
-static PackedView pack_level(mc_tables *t, const Rows &dense, int W, cudaStream_t s, int64_t &stored)
+// Pack one level into p.  `done` runs once the stream is known to have passed
+// everything queued before this level (the previous level's fill).
+template <typename CT, typename F>
+static PackedView pack_level(mc_tables *t, const Rows &dense, int W, cudaStream_t s, int64_t &stored, F done)
 {
     const int64_t n = t->g->n;
     Arena scratch(true);
@@ -158,24 +154,21 @@ static PackedView pack_level(mc_tables *t, const Rows &dense, int W, cudaStream_
     scratch.stream = s;
     int *err = scratch.get<int>(1);
     MC_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    u128 *cnt = scratch.get<u128>(2 * (size_t)n), *bytes = cnt + n;
     PackedView p;
     p.width = (int)sizeof(CT);
     uint8_t *wid = t->varlen ? t->arena.get<uint8_t>((size_t)n) : nullptr;
-    const int grid = grid_for(n * 32, 256);
-    MC_LAUNCH("pack", s, pack_count_kernel<CT><<<grid, 256, 0, s>>>(dense, n, W, t->varlen ? 1 : 0, cnt,
-                                                                      bytes, wid));
-    inclusive_scan_u128(cnt, n, err, scratch, s, 2);
-    int64_t *off = t->arena.get<int64_t>((size_t)n + 1);
-    int64_t *boff = t->arena.get<int64_t>((size_t)n + 1);
-    MC_LAUNCH("pack", s, offsets_kernel<<<grid_for(n + 1, 256), 256, 0, s>>>(cnt, n, off));
-    MC_LAUNCH("pack", s, offsets_kernel<<<grid_for(n + 1, 256), 256, 0, s>>>(bytes, n, boff));
+    const int grid = grid_for(n * pack_lanes(W), 256);
+    const int64_t stride = (n + 32) / 32 * 32;  // both offset arrays in one buffer
+    int64_t *off = t->arena.get<int64_t>(2 * (size_t)stride), *boff = off + stride;
+    MC_LAUNCH("pack", s, pack_count_kernel<CT><<<grid, 256, 0, s>>>(dense, n, W, t->varlen ? 1 : 0, off, boff, wid));
+    inclusive_scan_u64((uint64_t *)off, n + 1, stride, err, scratch, s, 2);
     int64_t tail[2] = {0, 0};
     int herr = 0;
     MC_CUDA(cudaMemcpyAsync(&tail[0], off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     MC_CUDA(cudaMemcpyAsync(&tail[1], boff + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     MC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     MC_CUDA(cudaStreamSynchronize(s));
+    done();
     if (herr) throw Error(MC_E_INTERNAL, "packing: offset overflow");
     uint16_t *key = t->arena.get<uint16_t>((size_t)std::max<int64_t>(tail[0], 1));
     uint8_t *val = t->arena.get<uint8_t>((size_t)std::max<int64_t>(tail[1], 8));
@@ -194,6 +187,11 @@ void pack_tables(mc_tables *t, cudaStream_t s)
     const int64_t n = t->g->n;
     const size_t cb = t->bits / 8;
     int64_t dense = 0, stored = 0;
+    void *packed_last = nullptr;  // the dense level whose fill is queued: freed at the next level's synchronisation
+    auto done = [&] {
+        if (packed_last) t->arena.release(packed_last);
+        packed_last = nullptr;
+    };
     for (int which = 0; which < 2; ++which)
         for (int h = which ? 1 : 2; h <= (which ? t->k - 1 : t->k); ++h) {
             if (t->level_missing(h)) continue;
@@ -202,13 +200,14 @@ void pack_tables(mc_tables *t, cudaStream_t s)
             dense += n * W * (int64_t)cb;
             if (n == 0) continue;
             const Rows R = t->rows(h, which);
-            PackedView p = t->bits == 64 ? pack_level<uint64_t>(t, R, W, s, stored)
-                                         : pack_level<u128>(t, R, W, s, stored);
+            PackedView p = t->bits == 64 ? pack_level<uint64_t>(t, R, W, s, stored, done)
+                                         : pack_level<u128>(t, R, W, s, stored, done);
             (which ? t->ps : t->pc)[h] = p;
-            MC_CUDA(cudaStreamSynchronize(s));
-            t->arena.release(D);
+            packed_last = D;
             D = nullptr;
         }
+    MC_CUDA(cudaStreamSynchronize(s));
+    done();
     t->dense_bytes = dense;
     t->stored_bytes = stored;
 }
