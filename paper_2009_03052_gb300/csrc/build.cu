@@ -1022,11 +1022,19 @@ static const char *const kGatherName[MAXK + 1] = {"gather_h0", "gather_h1", "gat
 static const char *const kMergeName[MAXK + 1] = {"merge_h0", "merge_h1", "merge_h2", "merge_h3", "merge_h4",
                                                  "merge_h5", "merge_h6", "merge_h7", "merge_h8"};
 
-// Schedules of the neighbour sums (the autotuner's choices): rows in flight
-// and blocks of 256 threads per SM (4: at most 64 registers, 6: 40, 8: 32).
+// Schedules of the neighbour sums (the autotuner's choices): rows in flight,
+// blocks of 256 threads per SM (4: at most 64 registers, 6: 40, 8: 32) and, for
+// rows of 5 to 16 units, the lanes folded twice or four times: two or four
+// units per lane, so that a warp takes more nodes and hands fewer ids round.
+// Picked on GB300 (ms): folded four times at h = 2, 3, 5 of the grid, k = 6
+// (0.070 / 0.095 / 0.095; twice 0.097 / 0.137 / 0.117, not 0.131 / 0.164 /
+// 0.156) and at h = 2, 5 of the other k = 6 graphs (0.122 against 0.150, batch);
+// 4 blocks per SM at h = 4..6 of k = 8 (8.2 against 12.2 at h = 6 of Chung-Lu
+// 2M).
 constexpr int GATHER_CANDIDATES = 7;
-static const int kGatherU[GATHER_CANDIDATES] = {4, 2, 1, 2, 1, 2, 4};
-static const int kGatherMB[GATHER_CANDIDATES] = {4, 4, 4, 6, 6, 8, 8};
+static const int kGatherU[GATHER_CANDIDATES] = {2, 2, 1, 2, 2, 2, 4};
+static const int kGatherMB[GATHER_CANDIDATES] = {8, 4, 4, 6, 8, 8, 8};
+static const int kGatherFold[GATHER_CANDIDATES] = {1, 1, 1, 1, 2, 4, 1};
 
 // G lanes for a row: the smallest power of two that covers its units, at most
 // 32, then NU units per lane.  Rows of fewer than 8 units take P neighbours
@@ -1046,9 +1054,18 @@ template <typename CT> static bool launch_gather(const GatherArgs &base, int r, 
     int NU = (ga.ws_units + 31) / 32;
     if (NU > 3) NU = 6;
     if (NU * 32 < ga.ws_units) throw Error(MC_E_INTERNAL, "gather: S row too wide");
+    const int fold = kGatherFold[cand];
+    if (fold > 1) {
+        if (NU != 1 || G < 8 || G > 16 || (fold == 4 && UB == 16)) return false;
+        G /= fold;
+        NU = (ga.ws_units + G - 1) / G;
+    }
     const int lanes = ga.nnz >= 8 * ga.n ? 8 : 4, P = G < lanes ? lanes / G : 1;
     auto kern = gather_kernel_ptr(sizeof(CT), N, UB, G, NU, P, kGatherU[cand], kGatherMB[cand]);
-    if (!kern) throw Error(MC_E_INTERNAL, "gather: no kernel for this row layout");
+    if (!kern) {
+        if (fold > 1) return false;
+        throw Error(MC_E_INTERNAL, "gather: no kernel for this row layout");
+    }
     const int NG = 32 / (G * P);
     const int wpb = 256 / 32;
     const int64_t cap = (int64_t)sm_count() * 32;

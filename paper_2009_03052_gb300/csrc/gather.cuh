@@ -379,14 +379,16 @@ GatherKernel gather_kernel_ptr_u128_8(int UB, int G, int NU, int P, int U, int M
 // The schedules (rows in flight, blocks per SM) of one lane layout.
 #define MC_GATHER_LAYOUT(CT, N, UB_, G_, NU_, P_)                                               \
     if (UB == UB_ && G == G_ && NU == NU_ && P == P_) {                                         \
-        if (U == 4 && MB == 4) return gather_kernel<CT, N, UB_, G_, NU_, P_, 4, 4>;             \
+        if (U == 2 && MB == 8) return gather_kernel<CT, N, UB_, G_, NU_, P_, 2, 8>;             \
         if (U == 2 && MB == 4) return gather_kernel<CT, N, UB_, G_, NU_, P_, 2, 4>;             \
         if (U == 1 && MB == 4) return gather_kernel<CT, N, UB_, G_, NU_, P_, 1, 4>;             \
         if (U == 2 && MB == 6) return gather_kernel<CT, N, UB_, G_, NU_, P_, 2, 6>;             \
-        if (U == 1 && MB == 6) return gather_kernel<CT, N, UB_, G_, NU_, P_, 1, 6>;             \
-        if (U == 2 && MB == 8) return gather_kernel<CT, N, UB_, G_, NU_, P_, 2, 8>;             \
         if (U == 4 && MB == 8) return gather_kernel<CT, N, UB_, G_, NU_, P_, 4, 8>;             \
         return nullptr;                                                                         \
     }
+// A layout of fewer lanes than units (schedules 4 and 5).
+#define MC_GATHER_FOLDED(CT, N, UB_, G_, NU_, P_)                                               \
+    if (UB == UB_ && G == G_ && NU == NU_ && P == P_ && U == 2 && MB == 8)                      \
+        return gather_kernel<CT, N, UB_, G_, NU_, P_, 2, 8>;
 
 }  // namespace mc

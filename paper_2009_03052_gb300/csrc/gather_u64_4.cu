@@ -29,6 +29,21 @@ GatherKernel gather_kernel_ptr_u64_4(int UB, int G, int NU, int P, int U, int MB
     MC_GATHER_LAYOUT(uint64_t, 4, 16, 8, 1, 1)
     MC_GATHER_LAYOUT(uint64_t, 4, 16, 16, 1, 1)
     MC_GATHER_LAYOUT(uint64_t, 4, 16, 32, 2, 1)
+    MC_GATHER_FOLDED(uint64_t, 4, 4, 4, 2, 2)
+    MC_GATHER_FOLDED(uint64_t, 4, 4, 4, 2, 1)
+    MC_GATHER_FOLDED(uint64_t, 4, 4, 8, 2, 1)
+    MC_GATHER_FOLDED(uint64_t, 4, 8, 8, 2, 1)
+    MC_GATHER_FOLDED(uint64_t, 4, 16, 4, 2, 2)
+    MC_GATHER_FOLDED(uint64_t, 4, 16, 4, 2, 1)
+    MC_GATHER_FOLDED(uint64_t, 4, 16, 8, 2, 1)
+    MC_GATHER_FOLDED(uint64_t, 4, 4, 2, 3, 4)
+    MC_GATHER_FOLDED(uint64_t, 4, 4, 2, 3, 2)
+    MC_GATHER_FOLDED(uint64_t, 4, 4, 4, 3, 2)
+    MC_GATHER_FOLDED(uint64_t, 4, 4, 4, 3, 1)
+    MC_GATHER_FOLDED(uint64_t, 4, 4, 4, 4, 2)
+    MC_GATHER_FOLDED(uint64_t, 4, 4, 4, 4, 1)
+    MC_GATHER_FOLDED(uint64_t, 4, 8, 4, 3, 2)
+    MC_GATHER_FOLDED(uint64_t, 4, 8, 4, 3, 1)
     return nullptr;
 }
 

@@ -20,6 +20,10 @@ GatherKernel gather_kernel_ptr_u64_8(int UB, int G, int NU, int P, int U, int MB
     MC_GATHER_LAYOUT(uint64_t, 8, 16, 32, 1, 1)
     MC_GATHER_LAYOUT(uint64_t, 8, 16, 32, 2, 1)
     MC_GATHER_LAYOUT(uint64_t, 8, 16, 32, 3, 1)
+    MC_GATHER_FOLDED(uint64_t, 8, 8, 8, 2, 1)
+    MC_GATHER_FOLDED(uint64_t, 8, 16, 8, 2, 1)
+    MC_GATHER_FOLDED(uint64_t, 8, 8, 4, 3, 2)
+    MC_GATHER_FOLDED(uint64_t, 8, 8, 4, 3, 1)
     return nullptr;
 }
 
