@@ -1629,17 +1629,25 @@ static std::vector<u128> level_rooted_totals(const mc_tables *t, int h, int j0, 
     int herr = 0;
     if (j0 >= 0 && !t->packed) {
         // one pass over the rows for all shapes, added up on the device
-        const int blocks = (int)std::min<int64_t>((hi - lo + 255) / 256, (int64_t)sm_count() * 4);
-        u128 *part = scratch.get<u128>((size_t)blocks * nj), *sum = scratch.get<u128>((size_t)nj);
+        const int64_t cap = (int64_t)sm_count() * 4;
+        u128 *part = scratch.get<u128>((size_t)std::min<int64_t>((n + 255) / 256, cap) * nj);
+        u128 *sum = scratch.get<u128>((size_t)nj);
         const TreeletShapes ts = treelet_shapes(h);
-        const dim3 grid((unsigned)blocks, (unsigned)nj);
-        if (t->bits == 64)
-            MC_LAUNCH("treelet_sum", s, treelet_sum_kernel<uint64_t><<<grid, 256, 0, s>>>(
-                                            t->rows(h, 0), lo, hi, cat.r[h], t->geo.Bc[h], j0, ts, part, err));
-        else
-            MC_LAUNCH("treelet_sum", s, treelet_sum_kernel<u128><<<grid, 256, 0, s>>>(
-                                            t->rows(h, 0), lo, hi, cat.r[h], t->geo.Bc[h], j0, ts, part, err));
-        MC_LAUNCH("treelet_sum", s, part_sum_kernel<<<nj, 256, 0, s>>>(part, blocks, sum, err));
+        auto pass = [&](int64_t a, int64_t b) {
+            const int blocks = (int)std::min<int64_t>((b - a + 255) / 256, cap);
+            const dim3 grid((unsigned)blocks, (unsigned)nj);
+            if (t->bits == 64)
+                MC_LAUNCH("treelet_sum", s, treelet_sum_kernel<uint64_t><<<grid, 256, 0, s>>>(
+                                                t->rows(h, 0), a, b, cat.r[h], t->geo.Bc[h], j0, ts, part, err));
+            else
+                MC_LAUNCH("treelet_sum", s, treelet_sum_kernel<u128><<<grid, 256, 0, s>>>(
+                                                t->rows(h, 0), a, b, cat.r[h], t->geo.Bc[h], j0, ts, part, err));
+            MC_LAUNCH("treelet_sum", s, part_sum_kernel<<<nj, 256, 0, s>>>(part, blocks, sum, err));
+        };
+        // a total that does not fit is an error for its ranges too (the build
+        // has checked level k)
+        if (h < t->k && hi - lo < n) pass(0, n);
+        pass(lo, hi);
         MC_CUDA(cudaMemcpyAsync(out.data(), sum, (size_t)nj * sizeof(u128), cudaMemcpyDeviceToHost, s));
         MC_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));
         MC_CUDA(cudaStreamSynchronize(s));
@@ -1796,13 +1804,15 @@ extern "C" mc_status mc_build_tables_batch(int count, const mc_graph *const *gra
         uint32_t *ucol = scratch.get<uint32_t>((size_t)(NNZ > 0 ? NNZ : 1));
         uint8_t *ucolors = scratch.get<uint8_t>((size_t)(N > 0 ? N : 1));
         std::vector<ConcatPart> parts((size_t)count);
-        bool on_device = true;  // colours in host memory are copied one by one
+        bool on_device = true;  // colours elsewhere (host, another device) are copied one by one
+        int dev = 0;
+        MC_CUDA(cudaGetDevice(&dev));
         for (int i = 0; i < count; ++i) {
             parts[(size_t)i] = {graphs[i]->row_ptr, graphs[i]->col, colors[i], noff[i], eoff[i]};
             if (graphs[i]->n == 0) continue;
             cudaPointerAttributes at{};
             if (cudaPointerGetAttributes(&at, colors[i]) != cudaSuccess) cudaGetLastError();
-            on_device &= at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
+            on_device &= (at.type == cudaMemoryTypeDevice && at.device == dev) || at.type == cudaMemoryTypeManaged;
         }
         ConcatPart *dparts = scratch.get<ConcatPart>((size_t)count);
         MC_CUDA(cudaMemcpyAsync(dparts, parts.data(), (size_t)count * sizeof(ConcatPart), cudaMemcpyHostToDevice, s));
@@ -1913,6 +1923,36 @@ static void launch_expand(const mc_tables *t, int h, int which, int64_t v0, int6
         MC_LAUNCH("expand", s, expand_kernel<u128><<<grid_for(total, 256), 256, 0, s>>>(x, v0, total, (u128 *)dst));
 }
 
+// A dense level in host memory put together from its planes on the host.
+static void read_planes(const mc_tables *t, int h, int which, uint8_t *dst, cudaStream_t s)
+{
+    const Rows x = t->rows(h, which);
+    const int64_t n = t->g->n;
+    const int cb = t->bits / 8;
+    const int64_t step = std::max<int64_t>(1, ((int64_t)16 << 20) / (x.s0 + x.s1 + 4));
+    std::vector<uint8_t> low, high;
+    std::vector<uint32_t> wide;
+    for (int64_t v0 = 0; v0 < n; v0 += step) {
+        const int64_t cnt = std::min(step, n - v0);
+        low.resize((size_t)(cnt * x.s0));
+        high.resize((size_t)(cnt * x.s1) + 1);
+        wide.resize((size_t)cnt);
+        MC_CUDA(cudaMemcpyAsync(low.data(), x.low(v0), (size_t)(cnt * x.s0), cudaMemcpyDeviceToHost, s));
+        if (x.s1) MC_CUDA(cudaMemcpyAsync(high.data(), x.high(v0), (size_t)(cnt * x.s1), cudaMemcpyDeviceToHost, s));
+        MC_CUDA(cudaMemcpyAsync(wide.data(), x.wide + v0, (size_t)cnt * 4, cudaMemcpyDeviceToHost, s));
+        MC_CUDA(cudaStreamSynchronize(s));
+        for (int64_t v = 0; v < cnt; ++v)
+            for (int e = 0; e < x.W; ++e, dst += cb) {
+                const uint8_t *up = high.data() + v * x.s1;
+                std::memset(dst, 0, (size_t)cb);
+                std::memcpy(dst, low.data() + v * x.s0 + e * x.N, (size_t)x.N);
+                if (!(wide[(size_t)v] & x.bit) || x.N == cb) continue;
+                if (cb == 16) std::memcpy(dst + 8, up + 8 * e, 8);
+                if (x.N == 4) std::memcpy(dst + 4, up + (cb == 16 ? 8 * x.W : 0) + 4 * e, 4);
+            }
+    }
+}
+
 extern "C" mc_status mc_read_table(const mc_tables *t, int h, int which, void *dst, size_t dst_bytes,
                                    int dst_on_device, void *stream)
 {
@@ -1948,13 +1988,19 @@ extern "C" mc_status mc_read_table(const mc_tables *t, int h, int which, void *d
             }
         } else if (dst_on_device) {
             launch_expand(t, h, which, 0, t->g->n, dst, s);
-        } else {  // through a scratch buffer of some rows
+        } else {  // through a scratch buffer of some rows, without one from the planes as they are
             const int64_t row = W * (t->bits / 8), n = t->g->n;
             const int64_t step = std::max<int64_t>(1, std::min<int64_t>(n, ((int64_t)64 << 20) / row));
             Arena scratch(true);
             scratch.alloc = t->arena.alloc;
             scratch.stream = s;
-            void *tmp = scratch.get<uint8_t>((size_t)(step * row));
+            void *tmp = nullptr;
+            try {
+                tmp = scratch.get<uint8_t>((size_t)(step * row));
+            } catch (const Error &) {
+                read_planes(t, h, which, (uint8_t *)dst, s);
+                return;
+            }
             for (int64_t v = 0; v < n; v += step) {
                 const int64_t cnt = std::min(step, n - v);
                 launch_expand(t, h, which, v, cnt, tmp, s);

@@ -110,18 +110,6 @@ __device__ __forceinline__ u128 shfl(u128 x, int src)
     return ((u128)hi << 64) | lo;
 }
 
-// Inclusive warp scan of 128-bit values (sums never exceed a checked bound).
-__device__ __forceinline__ u128 warp_inclusive_scan(u128 x)
-{
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        u128 y = shfl_up(x, d);
-        if (lane >= d) x += y;
-    }
-    return x;
-}
-
 // u128 -> double, rounded to nearest even: the top 64 significant bits with
 // the lower bits folded into a sticky bit, then one correctly rounded
 // conversion and an exact scaling.

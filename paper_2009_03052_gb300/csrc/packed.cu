@@ -156,10 +156,22 @@ static PackedView pack_level(mc_tables *t, const Rows &dense, int W, cudaStream_
     MC_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     PackedView p;
     p.width = (int)sizeof(CT);
-    uint8_t *wid = t->varlen ? t->arena.get<uint8_t>((size_t)n) : nullptr;
     const int grid = grid_for(n * pack_lanes(W), 256);
     const int64_t stride = (n + 32) / 32 * 32;  // both offset arrays in one buffer
-    int64_t *off = t->arena.get<int64_t>(2 * (size_t)stride), *boff = off + stride;
+    uint8_t *wid = nullptr;
+    int64_t *off = nullptr;
+    auto arrays = [&] {
+        if (t->varlen && !wid) wid = t->arena.get<uint8_t>((size_t)n);
+        off = t->arena.get<int64_t>(2 * (size_t)stride);
+    };
+    try {
+        arrays();
+    } catch (const Error &) {  // no room beside the previous level's dense rows: free them first
+        MC_CUDA(cudaStreamSynchronize(s));
+        done();
+        arrays();
+    }
+    int64_t *boff = off + stride;
     MC_LAUNCH("pack", s, pack_count_kernel<CT><<<grid, 256, 0, s>>>(dense, n, W, t->varlen ? 1 : 0, off, boff, wid));
     inclusive_scan_u64((uint64_t *)off, n + 1, stride, err, scratch, s, 2);
     int64_t tail[2] = {0, 0};
