@@ -171,6 +171,9 @@ constexpr int HUB_CHUNK = 64;
 // Hubs of at most HUB_SERIAL chunks have their chunk sums added up by one
 // thread per S entry; larger ones (listed in big_hub) by a warp per entry.
 constexpr int HUB_SERIAL = 32;
+// Samples per launch of split sampling where the nodes or parents need scratch
+// (a power of two).
+constexpr int64_t SPLIT_CHUNK = (int64_t)1 << 20;
 
 }  // namespace mc
 

@@ -668,13 +668,15 @@ struct SplitScratch {
     {
         if (!arena) return false;
         try {
+            int64_t cap = 1;  // powers of two: launches of growing sizes take twice the largest at most
+            while (cap < n) cap *= 2;
             if (need_found && found_cap < n) {
-                found = arena->get<uint32_t>((size_t)n * h);
-                found_cap = n;
+                found = arena->get<uint32_t>((size_t)cap * h);
+                found_cap = cap;
             }
             if (need_par && par_cap < n) {
-                par = arena->get<uint32_t>((size_t)n);
-                par_cap = n;
+                par = arena->get<uint32_t>((size_t)cap);
+                par_cap = cap;
             }
         } catch (const Error &) {
             arena = nullptr;
@@ -683,7 +685,6 @@ struct SplitScratch {
         return true;
     }
 };
-constexpr int64_t SPLIT_CHUNK = (int64_t)1 << 20;  // samples per launch where the nodes need scratch
 
 static void launch_sampler(const mc_tables *t, SampleArgs &a, SplitScratch *split, cudaStream_t s)
 {

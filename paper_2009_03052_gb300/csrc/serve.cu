@@ -77,6 +77,12 @@ static size_t request_memory(const mc_tables *t, const mc_request &r)
     const int ncls = mc_num_classes(h);
     const size_t cls = (size_t)std::max(ncls, 1) * 8;
     size_t m = small + 3 * cls;                                           // histogram, sigma, estimates
+    auto split = [&](int64_t samples) {                                   // nodes and parents of split sampling
+        int64_t cap = 1;
+        while (cap < samples && cap < SPLIT_CHUNK) cap *= 2;
+        return (size_t)cap * ((size_t)h + 1) * 4;
+    };
+    if (p.mode != MC_EST_AGS) m += split(p.samples);
     if (!t->prefix[h]) m += index;
     if (p.mode == MC_EST_AGS) {
         // a root index per treelet shape it samples from (at most all of
@@ -86,7 +92,7 @@ static size_t request_memory(const mc_tables *t, const mc_request &r)
         const int64_t bmax = p.batch > 0 ? p.batch : (int64_t)1 << 22;
         const int64_t ahead = std::min<int64_t>(bmax, 4096);
         m += (size_t)std::max(nu, 1) * index + index + (size_t)(bmax + (int64_t)nu * ahead) * 4 +
-             (size_t)nu * 128;
+             (size_t)nu * 128 + 2 * split(bmax + (int64_t)nu * ahead);  // (grown by doubling)
     }
     if (p.star_samples > 0 && !t->g->star_prefix[h]) m += index + cls;
     return m;
