@@ -708,7 +708,11 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, SplitScratch *spli
     else if (split && split->room(!a.nodes, !a.classes, std::min(a.count, a.nodes && a.classes ? a.count : SPLIT_CHUNK), a.h))
         mode = SampleMode::Split;
     if (mode != SampleMode::Counted) a.bytes = nullptr;
-    auto kern = t->packed ? sample_kernel_packed(mode, t->bits, narrow) : sample_kernel_dense(mode, t->bits, narrow);
+    // rows below level h that carry upper parts
+    const uint32_t below = ((1u << a.h) - 1u) & ~3u;
+    const bool wide = mode == SampleMode::Split && !t->packed && t->bits == 128 && (a.levels & (below | below << 16 | 2u << 16));
+    auto kern = t->packed ? sample_kernel_packed(mode, t->bits, narrow)
+                          : sample_kernel_dense(wide ? SampleMode::SplitWide : mode, t->bits, narrow);
     const int block = mode == SampleMode::Warps ? 256 : mode == SampleMode::Latency ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
     const size_t hist = a.hist ? (size_t)a.ncls * sizeof(uint32_t) : 0;
     const size_t smem = (mode == SampleMode::Warps ? 0 : (size_t)SAMPLE_WORDS * block * sizeof(uint32_t)) +

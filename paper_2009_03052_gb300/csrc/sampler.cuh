@@ -153,6 +153,15 @@ template <typename CT> __device__ __noinline__ CT entry_wide(const SampleArgs &a
     return entry_at<CT>(which ? a.S[h] : a.c[h], x, idx);
 }
 
+// The same of a row that is (`wide`) or is not wide, in line, so that the
+// items of a scan are in flight together.
+template <typename CT> __device__ __forceinline__ CT entry_full(const Rows &r, int64_t x, bool wide, int idx)
+{
+    CT v = row_low_any<CT>(r.low(x), r.N, idx);
+    if (wide) v |= row_rest<CT>(r.high(x), r.W, r.N, idx);
+    return v;
+}
+
 __device__ __forceinline__ uint64_t quotient(uint64_t a, uint64_t b) { return a / b; }
 __device__ __forceinline__ u128 quotient(u128 a, u128 b)
 {
@@ -275,14 +284,22 @@ __device__ __forceinline__ int64_t first_true(int64_t lo, int64_t hi, P pred, F 
 // that the searches of the classification neither hold the sampler's registers
 // nor wait in the divergence of its warps (1M samples at k = 5: 0.75 + 0.16 ms
 // against 1.08 in one kernel; the code before both 1.11).
+// WD (split sampling from 128-bit tables with wide rows below level h): counts
+// above 64 bits carry most of the weight, so most samples pass through wide
+// rows; their entries are read in line, low and upper parts and the wide words
+// of 3 neighbours in flight, where the other kernels call entry_wide one at a
+// time (ms for 1M / 10M samples of R-MAT 22, k = 7: 2.71 / 24.6; by calls 3.25 /
+// 31.6; whole 16-byte counts 2.91 / 27.8; 2 in flight 2.70 / 23.6 but 0.88
+// against 0.85 for 200k, 4: 2.95 / 27.9).  Tables with wide rows at level h only
+// stay with the calls: 4.03 against 4.38 for 1M samples of Chung-Lu 2M, k = 8.
 constexpr int SAMPLE_WORDS = 3 * MAXK;  // shared words per thread
 constexpr int SAMPLE_BLOCK = 512, SAMPLE_BLOCK_LAT = 64;
 
-template <typename CT, typename V, bool PK, bool LAT, bool CNT, bool SPLIT>
+template <typename CT, typename V, bool PK, bool LAT, bool CNT, bool SPLIT, bool WD = false>
 __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1 : (sizeof(CT) == 16 && !PK ? 2 : 3))
     sample_kernel(const __grid_constant__ SampleArgs a)
 {
-    constexpr int NW = LAT ? 16 : sizeof(CT) == 16 && !PK ? 4 : 2;  // items of a scan in flight
+    constexpr int NW = LAT ? 16 : WD ? 3 : sizeof(CT) == 16 && !PK ? 4 : 2;  // items of a scan in flight
     constexpr int NQ = LAT ? 8 : 4;   // adjacency searches in flight
     constexpr int KS = LAT ? 8 : 1;   // probes per round of the root and hub chunk searches
     constexpr int T = LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
@@ -370,7 +387,10 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                         return al ? (V)at((e - sh * Bc) * Rh + sh) : (V)0;
                     }, bf);
                 };
-                const int found = !PK && row.wide ? scan([&](int i) { return entry_wide<CT>(a, 0, h, v, i); })
+                const int found = !PK && row.wide ? scan([&](int i) {
+                    if constexpr (CB == 16) return entry_full<CT>(a.c[h], v, true, i);
+                    else return entry_wide<CT>(a, 0, h, v, i);
+                })
                                                   : scan([&](int i) { return row.get(i); });
                 if (found < 0) { ok = false; bad = true; }
                 else {
@@ -438,8 +458,15 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                             return (ha == 1 ? (V)1 : (V)at_a(index_a(c2))) * (V)at_b(sm.crank[c2] * Rb + lb);
                         }, before);
                     };
-                    const int blk = wide ? scan([&](int i) { return entry_wide<CT>(a, 0, ha, x, i); },
-                                                [&](int i) { return entry_wide<CT>(a, 1, hb, x, i); })
+                    const int blk = wide ? scan(
+                                               [&](int i) {
+                                                   if constexpr (WD) return entry_full<CT>(a.c[ha], x, ra.wide, i);
+                                                   else return entry_wide<CT>(a, 0, ha, x, i);
+                                               },
+                                               [&](int i) {
+                                                   if constexpr (WD) return entry_full<CT>(a.S[hb], x, rb_.wide, i);
+                                                   else return entry_wide<CT>(a, 1, hb, x, i);
+                                               })
                                          : scan([&](int i) { return ra.get(i); }, [&](int i) { return rb_.get(i); });
                     if (blk < 0) { ok = false; bad = true; }
                     else {
@@ -498,7 +525,7 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                             const int ci = cols[i];
                             return ((C2 >> ci) & 1u) ? RowRef<CT, PK>(a, sm, 0, hb, ids[i]).get(index_of(ci)) : (CT)0;
                         }, bn);
-                    } else if (sm.level[0][hb].w >> 8) {  // the level has wide rows
+                    } else if (!WD && sm.level[0][hb].w >> 8) {  // the level has wide rows
                         r = lane_first_exceeding<NW, CT>((int)len, q, [&](int i) -> CT {
                             const int ci = cols[i];
                             return ((C2 >> ci) & 1u) ? entry_wide<CT>(a, 0, hb, ids[i], index_of(ci)) : (CT)0;
@@ -508,11 +535,12 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                         // those whose colour is in C'', all in flight
                         const uint4 lv = sm.level[0][hb];
                         const uint8_t *p0 = (const uint8_t *)(((uint64_t)lv.y << 32) | lv.x);
-                        const int n = (int)len, N = (int)lv.w;
+                        const int n = (int)len, N = (int)(lv.w & 255u);
                         CT run = 0;
                         for (int b = 0; b < n && r < 0; b += NW) {
                             uint32_t id[NW];
                             int ci[NW];
+                            uint32_t ww[NW];
                             CT y[NW];
 #pragma unroll
                             for (int i = 0; i < NW; ++i) {
@@ -526,6 +554,17 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                                 MC_COUNT(5, 5);  // contiguous edge colours and ids
                                 if (in) MC_COUNT(CB, 32);  // the neighbour's row entry
                                 y[i] = in ? row_low_any<CT>(p0 + id[i] * (uint64_t)lv.z, N, index_of(ci[i])) : (CT)0;
+                                if constexpr (WD) ww[i] = in && lv.w >> 8 ? a.c[hb].wide[id[i]] & a.c[hb].bit : 0u;
+                            }
+                            if constexpr (WD) {
+                                uint32_t any = 0;
+#pragma unroll
+                                for (int i = 0; i < NW; ++i) any |= ww[i];
+                                if (any) {
+#pragma unroll
+                                    for (int i = 0; i < NW; ++i)
+                                        if (ww[i]) y[i] |= row_rest<CT>(a.c[hb].high(id[i]), a.c[hb].W, N, index_of(ci[i]));
+                                }
                             }
 #pragma unroll
                             for (int i = 0; i < NW; ++i)
@@ -537,7 +576,7 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                     }
                 }
                 if (r < 0) { ok = false; bad = true; }
-                else if (PK || (sm.level[0][hb].w >> 8)) {
+                else if (PK || (!WD && sm.level[0][hb].w >> 8)) {
                     u = a.col[lo_e + r];
                     cu = a.ecol[lo_e + r];
                 }
@@ -1158,7 +1197,7 @@ static __global__ void __launch_bounds__(256) classify_kernel(const __grid_const
 }
 
 typedef void (*SampleKernel)(SampleArgs);
-enum class SampleMode { Lanes, Latency, Counted, Split, Warps };
+enum class SampleMode { Lanes, Latency, Counted, Split, Warps, SplitWide };
 // The kernel for tables of bits-bit counts with 64-bit descent arithmetic
 // (narrow) or 128-bit, dense (sampler_dense.cu; all modes) or packed
 // (sampler_packed.cu: Lanes, Split, Warps).

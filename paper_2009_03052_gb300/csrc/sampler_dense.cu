@@ -12,6 +12,9 @@ template <typename CT, typename V> static SampleKernel pick(SampleMode mode)
     case SampleMode::Counted: return sample_kernel<CT, V, false, false, true, false>;
     case SampleMode::Split: return sample_kernel<CT, V, false, false, false, true>;
     case SampleMode::Warps: return sample_warp_kernel<CT, V, false>;
+    case SampleMode::SplitWide:
+        if constexpr (sizeof(CT) == 16) return sample_kernel<CT, V, false, false, false, true, true>;
+        break;
     }
     return nullptr;
 }

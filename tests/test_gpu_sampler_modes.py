@@ -41,3 +41,20 @@ def test_sizes_draw_the_same_samples(M, k, h, bits, unrooted, packed):
     est = T.estimate(h, seed=5, samples=1500)[1]  # the class histogram of a small request
     cls = T.sample(h, 5, 0, 1500)[3].cpu().numpy()
     assert np.array_equal(est, np.bincount(cls, minlength=len(est)).astype(np.uint64))
+
+
+def test_wide_rows_below_the_sampled_level(M):
+    """Two joined centres with 16,000 leaves each, 128-bit counts, k = 8: rows of
+    level 7 are wide, so a large request takes the kernel that reads them in
+    line.  The same samples in requests of a warp per sample."""
+    i = np.arange(2, 32002)
+    g = synth.from_edges(32002, np.concatenate([[0], i]), np.concatenate([[1], i % 2]))
+    k = 8
+    T = M.Tables(M.Graph.from_csr(g), synth.balanced_colors(g.n, k, 6), k, 128)
+    assert int(T.read(k - 1)[:, :, 1].max()) > 0
+    count, part = 60000, 4000
+    big = [x.cpu().numpy() for x in T.sample(k, 11, 0, count)]
+    for lo in range(0, count, part):
+        small = T.sample(k, 11, lo, part)
+        for a, b in zip(big, small):
+            assert np.array_equal(a[lo:lo + part], b.cpu().numpy()), lo
