@@ -240,8 +240,11 @@ mc_status mc_table_layout(const mc_tables *t, int h, int which, int64_t *row_ent
 mc_status mc_table_nonzeros(const mc_tables *t, int h, int which, int64_t *count, void *stream);
 
 /* Copy a whole level (n * row_entries * entry_bytes bytes) into dst (host or
- * device as dst_on_device says).  Level 1 of c is all ones and is produced on
- * the fly.  Synchronises `stream`. */
+ * device as dst_on_device says; dst needs no alignment).  Level 1 of c is all
+ * ones and is produced on the fly.  Uses up to 64 MB of scratch unless dst is
+ * memory of the current device aligned to a count; without it, copies are put
+ * together on the host (packed tables: a whole dense level of scratch, else
+ * MC_E_NOMEM).  Synchronises `stream`. */
 mc_status mc_read_table(const mc_tables *t, int h, int which, void *dst, size_t dst_bytes,
                         int dst_on_device, void *stream);
 

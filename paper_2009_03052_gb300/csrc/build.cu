@@ -1923,17 +1923,17 @@ static void launch_expand(const mc_tables *t, int h, int which, int64_t v0, int6
         MC_LAUNCH("expand", s, expand_kernel<u128><<<grid_for(total, 256), 256, 0, s>>>(x, v0, total, (u128 *)dst));
 }
 
-// A dense level in host memory put together from its planes on the host.
-static void read_planes(const mc_tables *t, int h, int which, uint8_t *dst, cudaStream_t s)
+// Rows v0 .. v0 + rows of a dense level put together from their planes on the
+// host, into host memory.
+static void read_planes(const mc_tables *t, int h, int which, int64_t v0, int64_t rows, uint8_t *dst, cudaStream_t s)
 {
     const Rows x = t->rows(h, which);
-    const int64_t n = t->g->n;
     const int cb = t->bits / 8;
-    const int64_t step = std::max<int64_t>(1, ((int64_t)16 << 20) / (x.s0 + x.s1 + 4));
+    const int64_t end = v0 + rows, step = std::max<int64_t>(1, ((int64_t)16 << 20) / (x.s0 + x.s1 + 4));
     std::vector<uint8_t> low, high;
     std::vector<uint32_t> wide;
-    for (int64_t v0 = 0; v0 < n; v0 += step) {
-        const int64_t cnt = std::min(step, n - v0);
+    for (; v0 < end; v0 += step) {
+        const int64_t cnt = std::min(step, end - v0);
         low.resize((size_t)(cnt * x.s0));
         high.resize((size_t)(cnt * x.s1) + 1);
         wide.resize((size_t)cnt);
@@ -1953,6 +1953,22 @@ static void read_planes(const mc_tables *t, int h, int which, uint8_t *dst, cuda
     }
 }
 
+// Whether kernels may store whole counts at dst: memory of this device,
+// aligned to a count.  Other device destinations (any address, memory of
+// another device) are reached by copies.
+static bool stores_counts(const void *dst, size_t count_bytes)
+{
+    int dev = 0;
+    MC_CUDA(cudaGetDevice(&dev));
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return ((at.type == cudaMemoryTypeDevice && at.device == dev) || at.type == cudaMemoryTypeManaged) &&
+           (uintptr_t)dst % count_bytes == 0;
+}
+
 extern "C" mc_status mc_read_table(const mc_tables *t, int h, int which, void *dst, size_t dst_bytes,
                                    int dst_on_device, void *stream)
 {
@@ -1962,51 +1978,64 @@ extern "C" mc_status mc_read_table(const mc_tables *t, int h, int which, void *d
         MC_REQUIRE(which == 0 || which == 1, "which must be 0 (c) or 1 (S)");
         MC_REQUIRE(h >= 1 && h <= (which ? t->k - 1 : t->k), "h out of range");
         MC_REQUIRE(!t->level_missing(h), "level h was skipped (round skipping)");
-        const int64_t W = which ? t->geo.Ws[h] : t->geo.Wc[h];
-        const size_t bytes = (size_t)t->g->n * W * (t->bits / 8);
+        const int64_t W = which ? t->geo.Ws[h] : t->geo.Wc[h], n = t->g->n;
+        const size_t cb = t->bits / 8, bytes = (size_t)n * W * cb;
         MC_REQUIRE(dst_bytes >= bytes, "dst too small");
         cudaStream_t s = (cudaStream_t)stream;
         if (bytes == 0) return;
-        if (which == 0 && h == 1) {
-            if (dst_on_device) {
-                MC_LAUNCH("fill_ones", s, fill_ones_kernel<<<grid_for(t->g->n, 256), 256, 0, s>>>(dst, t->g->n, t->bits / 8));
-            } else {
-                std::memset(dst, 0, bytes);
-                for (int64_t v = 0; v < t->g->n; ++v) ((uint8_t *)dst)[v * (t->bits / 8)] = 1;
-            }
-        } else if (t->packed) {
-            if (dst_on_device) {
+        const bool ones = which == 0 && h == 1;
+        const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
+        Arena scratch(true);
+        scratch.alloc = t->arena.alloc;
+        scratch.stream = s;
+        if (dst_on_device && stores_counts(dst, cb)) {
+            if (ones)
+                MC_LAUNCH("fill_ones", s, fill_ones_kernel<<<grid_for(n, 256), 256, 0, s>>>(dst, n, (int)cb));
+            else if (t->packed)
                 launch_unpack(t, h, which, dst, s);
-            } else {
-                Arena scratch(true);
-                scratch.alloc = t->arena.alloc;
-                scratch.stream = s;
-                void *tmp = scratch.get<uint8_t>(bytes);
-                launch_unpack(t, h, which, tmp, s);
-                MC_CUDA(cudaMemcpyAsync(dst, tmp, bytes, cudaMemcpyDeviceToHost, s));
+            else
+                launch_expand(t, h, which, 0, n, dst, s);
+        } else if (ones) {
+            std::vector<uint8_t> one;
+            uint8_t *at = (uint8_t *)dst;
+            if (dst_on_device) {
+                one.resize(bytes);
+                at = one.data();
+            }
+            std::memset(at, 0, bytes);
+            for (int64_t v = 0; v < n; ++v) at[v * (int64_t)cb] = 1;
+            if (dst_on_device) {
+                MC_CUDA(cudaMemcpyAsync(dst, at, bytes, cudaMemcpyHostToDevice, s));
                 MC_CUDA(cudaStreamSynchronize(s));
             }
-        } else if (dst_on_device) {
-            launch_expand(t, h, which, 0, t->g->n, dst, s);
+        } else if (t->packed) {
+            void *tmp = scratch.get<uint8_t>(bytes);
+            launch_unpack(t, h, which, tmp, s);
+            MC_CUDA(cudaMemcpyAsync(dst, tmp, bytes, kind, s));
         } else {  // through a scratch buffer of some rows, without one from the planes as they are
-            const int64_t row = W * (t->bits / 8), n = t->g->n;
+            const int64_t row = W * (int64_t)cb;
             const int64_t step = std::max<int64_t>(1, std::min<int64_t>(n, ((int64_t)64 << 20) / row));
-            Arena scratch(true);
-            scratch.alloc = t->arena.alloc;
-            scratch.stream = s;
             void *tmp = nullptr;
+            std::vector<uint8_t> host;
             try {
                 tmp = scratch.get<uint8_t>((size_t)(step * row));
             } catch (const Error &) {
-                read_planes(t, h, which, (uint8_t *)dst, s);
-                return;
+                if (dst_on_device) host.resize((size_t)(step * row));
             }
             for (int64_t v = 0; v < n; v += step) {
                 const int64_t cnt = std::min(step, n - v);
-                launch_expand(t, h, which, v, cnt, tmp, s);
-                MC_CUDA(cudaMemcpyAsync((uint8_t *)dst + v * row, tmp, (size_t)(cnt * row), cudaMemcpyDeviceToHost, s));
+                uint8_t *at = (uint8_t *)dst + v * row;
+                if (tmp) {
+                    launch_expand(t, h, which, v, cnt, tmp, s);
+                    MC_CUDA(cudaMemcpyAsync(at, tmp, (size_t)(cnt * row), kind, s));
+                } else {
+                    read_planes(t, h, which, v, cnt, dst_on_device ? host.data() : at, s);
+                    if (dst_on_device) {
+                        MC_CUDA(cudaMemcpyAsync(at, host.data(), (size_t)(cnt * row), cudaMemcpyHostToDevice, s));
+                        MC_CUDA(cudaStreamSynchronize(s));
+                    }
+                }
             }
-            MC_CUDA(cudaStreamSynchronize(s));
         }
         MC_CUDA(cudaStreamSynchronize(s));
     });
