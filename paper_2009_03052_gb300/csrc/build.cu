@@ -1131,8 +1131,7 @@ static bool launch_merge_tile(const MergeTileArgs &base, const MergePairs &Q, in
     MergeTileArgs ta = base;
     size_t smem = 0;
     if (!plan_merge_tile(ta, Q, shift, smem)) return false;
-    if (smem > 48 * 1024)
-        MC_CUDA(cudaFuncSetAttribute(merge_tile_kernel<CT, THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 48 * 1024) allow_shared((const void *)merge_tile_kernel<CT, THREADS>);
     const int64_t ntiles = (ta.n_do + (1 << ta.log_tn) - 1) >> ta.log_tn;
     const int64_t per_sm = std::max<int64_t>(1, std::min<int64_t>(2048 / THREADS, (int64_t)(227 * 1024 / (smem + 1024))));
     const int g = (int)std::max<int64_t>(1, std::min<int64_t>(ntiles, (int64_t)sm_count() * per_sm));

@@ -4,6 +4,7 @@
 #include <atomic>
 #include <cstring>
 #include <mutex>
+#include <set>
 
 #include "internal.h"
 
@@ -371,6 +372,21 @@ int sm_count()
         if (sms <= 0) sms = 1;
     }
     return sms;
+}
+
+void allow_shared(const void *kernel)
+{
+    static std::mutex mu;
+    static std::set<std::pair<int, const void *>> raised;
+    int dev = 0, most = 0;
+    MC_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    if (raised.count({dev, kernel})) return;
+    cudaFuncAttributes at{};
+    MC_CUDA(cudaFuncGetAttributes(&at, kernel));
+    MC_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    MC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)at.sharedSizeBytes));
+    raised.insert({dev, kernel});
 }
 
 int grid_for(int64_t work, int block)

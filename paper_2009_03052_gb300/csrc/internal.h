@@ -123,6 +123,11 @@ void build_buckets(const u128 *prefix, int64_t n, int64_t nb, u128 *dD, uint32_t
 
 int grid_for(int64_t work, int block);
 int sm_count();
+// Lets `kernel` be launched with any dynamic shared memory the current device
+// has room for beside its static part.  The limit belongs to the kernel and is
+// shared by all host threads, so it is raised once per kernel and device and
+// never set to what one launch needs: another thread's larger launch would fail.
+void allow_shared(const void *kernel);
 
 // Kernel tracing: count every launch; when profiling is on, bracket it by
 // CUDA events on its stream, keyed by a kernel name.

@@ -717,8 +717,7 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, SplitScratch *spli
     const size_t hist = a.hist ? (size_t)a.ncls * sizeof(uint32_t) : 0;
     const size_t smem = (mode == SampleMode::Warps ? 0 : (size_t)SAMPLE_WORDS * block * sizeof(uint32_t)) +
                         (mode == SampleMode::Split ? 0 : hist);
-    if (smem > 40 * 1024)  // beside the static tables
-        MC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > 40 * 1024) allow_shared((const void *)kern);  // beside the static tables
     const int64_t total = a.count;
     const int64_t step = mode == SampleMode::Split && !(a.nodes && a.classes) ? SPLIT_CHUNK : total;
     for (int64_t b0 = 0; b0 < total; b0 += step) {
@@ -754,8 +753,7 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, SplitScratch *spli
             c.hist = a.hist;
             c.ncls = a.ncls;
             c.err = a.err;
-            if (hist > 32 * 1024)  // beside the static tile
-                MC_CUDA(cudaFuncSetAttribute(classify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hist));
+            if (hist > 32 * 1024) allow_shared((const void *)classify_kernel);  // beside the static tile
             const int64_t tiles = (n + CLASSIFY_TILE - 1) / CLASSIFY_TILE;
             const int g = (int)std::min<int64_t>(tiles, (int64_t)sm_count() * (hist > 16 * 1024 ? 3 : 8));
             MC_LAUNCH("classify", s, classify_kernel<<<g, 256, hist, s>>>(c));
