@@ -902,7 +902,7 @@ __global__ void fill_ones_kernel(void *dst, int64_t n, int bytes)
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-static int64_t scan_tiles(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
+int64_t scan_tiles(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE; }
 
 // the scan with a caller-provided tile-sum buffer of m * scan_tiles(n) entries
 template <typename T>
@@ -921,6 +921,11 @@ static void inclusive_scan_buf(T *x, int64_t n, int64_t stride, int *err, T *ts,
 void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s, int m)
 {
     if (n > 0) inclusive_scan_buf<u128>(x, n, n, err, scratch.get<u128>((size_t)scan_tiles(n) * m), s, m);
+}
+
+void inclusive_scan_u64(uint64_t *x, int64_t n, int64_t stride, int *err, uint64_t *sums, cudaStream_t s, int m)
+{
+    inclusive_scan_buf<uint64_t>(x, n, stride, err, sums, s, m);
 }
 
 void inclusive_scan_u64(uint64_t *x, int64_t n, int64_t stride, int *err, Arena &scratch, cudaStream_t s, int m)

@@ -116,6 +116,9 @@ template <typename F> mc_status guarded(F &&f)
 // (or `stride` entries apart); overflow sets bit 0 of *err.
 void inclusive_scan_u128(u128 *x, int64_t n, int *err, Arena &scratch, cudaStream_t s, int m = 1);
 void inclusive_scan_u64(uint64_t *x, int64_t n, int64_t stride, int *err, Arena &scratch, cudaStream_t s, int m = 1);
+// the same with the caller's room for the tile sums, m * scan_tiles(n) entries
+void inclusive_scan_u64(uint64_t *x, int64_t n, int64_t stride, int *err, uint64_t *sums, cudaStream_t s, int m = 1);
+int64_t scan_tiles(int64_t n);
 // Bucket indexes (bstride entries apart) of m prefixes of n entries, and their
 // widths dD[m].
 void build_buckets(const u128 *prefix, int64_t n, int64_t nb, u128 *dD, uint32_t *start, cudaStream_t s, int m = 1,

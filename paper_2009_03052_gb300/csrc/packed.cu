@@ -152,15 +152,17 @@ static PackedView pack_level(mc_tables *t, const Rows &dense, int W, cudaStream_
     Arena scratch(true);
     scratch.alloc = t->arena.alloc;
     scratch.stream = s;
-    int *err = scratch.get<int>(1);
-    MC_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     PackedView p;
     p.width = (int)sizeof(CT);
     const int grid = grid_for(n * pack_lanes(W), 256);
     const int64_t stride = (n + 32) / 32 * 32;  // both offset arrays in one buffer
+    int *err = nullptr;
+    uint64_t *sums = nullptr;
     uint8_t *wid = nullptr;
     int64_t *off = nullptr;
-    auto arrays = [&] {
+    auto arrays = [&] {  // all that is requested before the synchronisation
+        if (!err) err = scratch.get<int>(1);
+        if (!sums) sums = scratch.get<uint64_t>((size_t)scan_tiles(n + 1) * 2);
         if (t->varlen && !wid) wid = t->arena.get<uint8_t>((size_t)n);
         off = t->arena.get<int64_t>(2 * (size_t)stride);
     };
@@ -171,9 +173,10 @@ static PackedView pack_level(mc_tables *t, const Rows &dense, int W, cudaStream_
         done();
         arrays();
     }
+    MC_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     int64_t *boff = off + stride;
     MC_LAUNCH("pack", s, pack_count_kernel<CT><<<grid, 256, 0, s>>>(dense, n, W, t->varlen ? 1 : 0, off, boff, wid));
-    inclusive_scan_u64((uint64_t *)off, n + 1, stride, err, scratch, s, 2);
+    inclusive_scan_u64((uint64_t *)off, n + 1, stride, err, sums, s, 2);
     int64_t tail[2] = {0, 0};
     int herr = 0;
     MC_CUDA(cudaMemcpyAsync(&tail[0], off + n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
