@@ -51,7 +51,10 @@ typedef enum {
 /* Device memory provider.  alloc returns device memory of at least `bytes`
  * bytes, aligned to 256 bytes, usable on `stream` (NULL on failure); free
  * releases it.  `ctx` is passed back unchanged and must outlive every handle
- * created with this allocator.  A NULL allocator means cudaMalloc/cudaFree. */
+ * created with this allocator.  A NULL allocator means cudaMalloc/cudaFree.
+ * Buffers of up to 128 KB are carved from 512 KB chunks (requested one by one
+ * when a chunk is refused): a graph, a table set and, with an allocator, each
+ * call's scratch take at least one. */
 typedef struct mc_allocator {
     void *(*alloc)(size_t bytes, void *ctx, void *stream);
     void (*free)(void *ptr, size_t bytes, void *ctx, void *stream);

@@ -1224,6 +1224,7 @@ extern "C" mc_status mc_estimate_counts(const mc_tables *t, const mc_estimate_pa
             const int64_t cap = bmax + (int64_t)nu * ahead;  // samples of one launch, at most
             int32_t *dcls = scratch.get<int32_t>((size_t)cap);
             SampleSeg *dseg = scratch.get<SampleSeg>((size_t)nu);
+            unsigned long long *next = batch_counter(scratch, s);  // of every launch in turn
             // the part table, then the class ids of one launch
             const size_t seg_bytes = ((size_t)nu * sizeof(SampleSeg) + 255) & ~(size_t)255;
             char *pin = (char *)pinned_scratch(seg_bytes + (size_t)cap * sizeof(int32_t));
@@ -1323,7 +1324,8 @@ extern "C" mc_status mc_estimate_counts(const mc_tables *t, const mc_estimate_pa
                 a.ncls = ncls;
                 a.err = err;
                 a.bytes = bytes = sample_byte_counter(scratch, s);
-                a.next = batch_counter(scratch, s);
+                a.next = next;
+                MC_CUDA(cudaMemsetAsync(next, 0, sizeof(*next), s));
                 launch_sampler(t, a, &split, s);
                 MC_CUDA(cudaMemcpyAsync(hcls, dcls, (size_t)total * 4, cudaMemcpyDeviceToHost, s));
                 MC_CUDA(cudaEventRecord(done.e, s));

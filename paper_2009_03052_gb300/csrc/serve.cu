@@ -58,32 +58,75 @@ namespace mc {
 
 int64_t bucket_count(int64_t n);
 
+// What an arena takes for the buffers added, as Arena::get does: small ones
+// are carved from chunks (`carves`), each chunk but the last filled up to one
+// small buffer.
+struct ArenaCharge {
+    bool carves;
+    size_t plain = 0, small = 0;
+    void add(size_t bytes)
+    {
+        bytes = (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
+        (carves && bytes <= Arena::SMALL ? small : plain) += bytes;
+    }
+    size_t total() const
+    {
+        return plain + (small ? Arena::CHUNK * (1 + small / (Arena::CHUNK - Arena::SMALL)) : 0);
+    }
+};
+
 // Device bytes a request allocates while it runs (outputs, scratch, and any
 // root or star index it creates on first use), from the request and the
-// tables it reads: what admission charges it.
+// tables it reads: what admission charges it.  The scratch of a call carves
+// small buffers only from a caller's allocator, the handles' own arenas always.
 static size_t request_memory(const mc_tables *t, const mc_request &r)
 {
     const int64_t n = t->g->n;
-    const size_t scan = (size_t)((n + 4095) / 4096 + 1) * 16;            // scan tile sums
-    const size_t index = (size_t)n * 16 + (size_t)(bucket_count(n) + 1) * 4 + scan + 64;  // prefix + buckets
-    const size_t small = 4096;                                            // flags, counters
+    const bool custom = t->arena.alloc.custom;
+    const size_t scan = (size_t)scan_tiles(n) * 16, prefix = (size_t)n * 16,
+                 bucket = (size_t)(bucket_count(n) + 1) * 4;
+    ArenaCharge call{custom};  // the call's scratch
+    auto flags = [](ArenaCharge &c) {  // error flags, counters, bucket widths
+        for (int i = 0; i < 4; ++i) c.add(64);
+    };
+    auto index = [&](ArenaCharge &c) {  // a root index of the call's own
+        c.add(prefix);
+        c.add(bucket);
+        c.add(scan);
+        c.add(16);
+    };
+    // an index made on first use: kept by the handle, scratch of its own
+    auto first_use = [&](bool kept_custom) {
+        ArenaCharge kept{true}, scratch{kept_custom};
+        kept.add(prefix);
+        kept.add(bucket);
+        scratch.add(scan);
+        flags(scratch);
+        return kept.total() + scratch.total();
+    };
+    flags(call);
     if (r.kind == MC_REQ_SAMPLE) {
-        size_t m = (size_t)std::max<int64_t>(r.count, 1) * ((size_t)r.h + 1) * 4 + small;
-        if (r.unrooted_shape >= 0 || !t->prefix[r.h]) m += index;  // a shape's index is per call
-        return m;
+        size_t m = (size_t)std::max<int64_t>(r.count, 1) * ((size_t)r.h + 1) * 4 + 512;
+        if (r.unrooted_shape >= 0) index(call);  // a shape's index is per call
+        else if (!t->prefix[r.h]) m += first_use(custom);
+        return m + call.total();
     }
     const mc_estimate_params &p = r.est;
     const int h = p.h;
     const int ncls = mc_num_classes(h);
     const size_t cls = (size_t)std::max(ncls, 1) * 8;
-    size_t m = small + 3 * cls;                                           // histogram, sigma, estimates
-    auto split = [&](int64_t samples) {                                   // nodes and parents of split sampling
+    size_t m = 0;
+    for (int i = 0; i < 3; ++i) call.add(cls);  // histogram, sigma, estimates
+    auto split = [&](int64_t samples, bool grown) {  // nodes and parents of split sampling
         int64_t cap = 1;
         while (cap < samples && cap < SPLIT_CHUNK) cap *= 2;
-        return (size_t)cap * ((size_t)h + 1) * 4;
+        for (; cap >= 1; cap = grown ? cap / 2 : 0) {
+            call.add((size_t)cap * h * 4);
+            call.add((size_t)cap * 4);
+        }
     };
-    if (p.mode != MC_EST_AGS) m += split(p.samples);
-    if (!t->prefix[h]) m += index;
+    if (p.mode != MC_EST_AGS) split(p.samples, false);
+    if (!t->prefix[h]) m += first_use(custom);
     if (p.mode == MC_EST_AGS) {
         // a root index per treelet shape it samples from (at most all of
         // them), one shape-total pass, and the class ids and part table of
@@ -91,11 +134,17 @@ static size_t request_memory(const mc_tables *t, const mc_request &r)
         const int nu = mc_num_unrooted(h);
         const int64_t bmax = p.batch > 0 ? p.batch : (int64_t)1 << 22;
         const int64_t ahead = std::min<int64_t>(bmax, 4096);
-        m += (size_t)std::max(nu, 1) * index + index + (size_t)(bmax + (int64_t)nu * ahead) * 4 +
-             (size_t)nu * 128 + 2 * split(bmax + (int64_t)nu * ahead);  // (grown by doubling)
+        for (int j = 0; j <= std::max(nu, 1); ++j) index(call);
+        call.add((size_t)(bmax + (int64_t)nu * ahead) * 4);
+        call.add((size_t)nu * 128);
+        split(bmax + (int64_t)nu * ahead, true);  // grown by doubling
     }
-    if (p.star_samples > 0 && !t->g->star_prefix[h]) m += index + cls;
-    return m;
+    if (p.star_samples > 0) {
+        call.add(cls);
+        call.add(64);
+        if (!t->g->star_prefix[h]) m += first_use(t->g->arena.alloc.custom);
+    }
+    return m + call.total();
 }
 
 // Free device memory now (0 if the query fails).
