@@ -207,21 +207,28 @@ mc_status mc_tables_status(const mc_tables *t, void *stream);
  * level have a few schedules (lanes per node, rows in flight, registers per
  * thread) that compute identical tables.  mc_build_tables times
  * every candidate once for each new (kernel, k, count width, level, degree
- * bucket) key and keeps the fastest; the degree bucket is floor(log2 n),
- * floor(2 log2(nnz / n)) and floor(log2(max degree + 1)).  mc_rebuild_tables
+ * bucket, layout) key and keeps the fastest; the degree bucket is floor(log2 n),
+ * floor(2 log2(nnz / n)) and floor(log2(max degree + 1)), the layout a number
+ * for the widths the counts are kept in and the merge's program.  mc_rebuild_tables
  * never tunes (it may be captured): it uses the choices made so far.
  *   mode 0: never tune (choices loaded or made earlier, else the first
  *           schedule); 1 (default): tune keys not seen yet; 2: tune every key
  *           once more in this process.
  *   cache_file (may be NULL: unchanged; "": stop appending): load its
  *   choices now and append every new one to it; the MC_AUTOTUNE_CACHE
- *   environment variable does the same at the first build.  One line per key: kind k bits h logn logdeg loghub choice.
+ *   environment variable does the same at the first build.  One line per key:
+ *   kind k bits h logn logdeg loghub choice layout set.  Lines of another set
+ *   of schedules and unknown schedules are skipped; lines that end at the
+ *   choice (set unknown) hold where nothing is tuned: in mode 0 and in
+ *   rebuilds of keys not tuned yet.
  * mc_autotune_choice: the schedule chosen so far for kernel kind (0 the
  * neighbour sums, schedules 0..6; 1 the merge, schedules 0..5) at level h
  * of tables with k colours and count_bits counts on graphs of n nodes, nnz
- * adjacency entries and largest degree max_degree (mc_graph_info), or -1.
- * mc_autotune_set: fix that choice (MC_E_INVALID for an unknown kind or
- * schedule); builds use it and do not tune it again (in mode 1). */
+ * adjacency entries and largest degree max_degree (mc_graph_info), the last
+ * one if there are several layouts, or -1.
+ * mc_autotune_set: fix that choice for every layout (MC_E_INVALID for an unknown
+ * kind or schedule); builds use it (the first schedule where a layout does not
+ * have it) and do not tune it again (in mode 1). */
 mc_status mc_autotune(int mode, const char *cache_file);
 int mc_autotune_choice(int kind, int k, int count_bits, int h, int64_t n, int64_t nnz, int64_t max_degree);
 mc_status mc_autotune_set(int kind, int k, int count_bits, int h, int64_t n, int64_t nnz, int64_t max_degree,

@@ -1160,25 +1160,41 @@ static bool launch_merge(const MergeTileArgs &ta, const MergePairs &Q, int h, in
 
 // ---------------------------------------------------------------------------
 // Autotuner: the schedule of each (kernel, k, count width, level, graph
-// shape) is chosen by timing every candidate once on the first build that
-// meets it (the candidates compute identical tables, so which one runs does
-// not change any result).  The graph's shape is reduced to a degree bucket:
-// log2 n, log2 of the average degree in half steps, log2 of the largest
-// degree.  Choices can be loaded from and appended to a cache file
-// (mc_autotune, or the MC_AUTOTUNE_CACHE environment variable).
+// shape, layout) is chosen by timing every candidate once on the first build
+// that meets it (the candidates compute identical tables, so which one runs
+// does not change any result).  The graph's shape is reduced to a degree
+// bucket: log2 n, log2 of the average degree in half steps, log2 of the largest
+// degree.  The layout is what else decides which candidate is best, or whether
+// it exists: the bytes of the first-plane counts, the node order and, at level
+// k, the merge program.  Choices can be loaded from and appended to a cache file
+// (mc_autotune, or the MC_AUTOTUNE_CACHE environment variable); a line names
+// the set of schedules that it was chosen from (TUNE_SET, counted up whenever a
+// schedule number changes its meaning), and only the present set's are used as
+// they are.
 // ---------------------------------------------------------------------------
 namespace {
+constexpr int TUNE_SET = 2;
 struct TuneKey {
     int kind, k, bits, h, logn, logdeg, loghub;
+    int layout = -1;  // -1: of any layout (pinned choices, lines without one)
     bool operator<(const TuneKey &o) const
     {
-        return std::tie(kind, k, bits, h, logn, logdeg, loghub) <
-               std::tie(o.kind, o.k, o.bits, o.h, o.logn, o.logdeg, o.loghub);
+        return std::tie(kind, k, bits, h, logn, logdeg, loghub, layout) <
+               std::tie(o.kind, o.k, o.bits, o.h, o.logn, o.logdeg, o.loghub, o.layout);
+    }
+    TuneKey any() const
+    {
+        TuneKey x = *this;
+        x.layout = -1;
+        return x;
     }
 };
 struct TuneState {
     std::mutex mu;
-    std::map<TuneKey, int> choice;
+    std::map<TuneKey, int> choice;  // timed here or by another process
+    std::map<TuneKey, int> pinned;  // by mc_autotune_set
+    std::map<TuneKey, int> hint;    // file lines without a set: used where tuning is off
+    std::map<TuneKey, int> latest;  // the last of these per key of any layout
     std::set<TuneKey> retuned;  // mode 2: keys tuned again in this process
     int mode = 1;               // 0 never tune, 1 tune unknown keys, 2 tune every key once more
     std::string file;
@@ -1190,15 +1206,29 @@ TuneState &tune_state()
     return st;
 }
 
+int candidates(int kind) { return kind == 0 ? GATHER_CANDIDATES : MERGE_CANDIDATES; }
+
 void tune_load_file_locked(TuneState &st, const std::string &path)
 {
     FILE *f = std::fopen(path.c_str(), "r");
     if (!f) return;
-    TuneKey k{};
-    int v = 0;
-    while (std::fscanf(f, "%d %d %d %d %d %d %d %d", &k.kind, &k.k, &k.bits, &k.h, &k.logn, &k.logdeg, &k.loghub,
-                       &v) == 8)
-        st.choice[k] = v;
+    char line[256];
+    while (std::fgets(line, sizeof(line), f)) {
+        TuneKey k{};
+        int v = 0, layout = -1, set = 0;
+        const int got = std::sscanf(line, "%d %d %d %d %d %d %d %d %d %d", &k.kind, &k.k, &k.bits, &k.h, &k.logn,
+                                    &k.logdeg, &k.loghub, &v, &layout, &set);
+        if ((k.kind != 0 && k.kind != 1) || v < 0 || v >= candidates(k.kind)) continue;
+        if (got == 8) {
+            st.hint[k.any()] = v;
+        } else if (got == 10 && set == TUNE_SET && layout >= 0) {
+            k.layout = layout;
+            st.choice[k] = v;
+        } else {
+            continue;
+        }
+        st.latest[k.any()] = v;
+    }
     std::fclose(f);
 }
 
@@ -1223,20 +1253,52 @@ static TuneKey tune_key(int kind, int k, int count_bits, int h, int64_t n, int64
                    ilog2((double)max_degree + 1)};
 }
 
+// The key of a build's kernel of level h.  Widths grow with the level, so those
+// of a merge's operands follow from the first level of 8-byte counts.
+static TuneKey tune_key(int kind, const mc_tables *t, int h)
+{
+    TuneKey key = tune_key(kind, t->k, t->bits, h, t->g->n, t->g->nnz, t->g->max_degree);
+    if (kind == 0) {
+        key.layout = (t->Nc[h] == 8) | (t->Ns[h] == 8) << 1;
+    } else {
+        int first = 1;
+        while (first <= h && t->Nc[first] == 4) ++first;
+        key.layout = first | (t->g->order != nullptr) << 4 | (t->skip_round && h == t->k) << 5 |
+                     (t->zero_root && h == t->k) << 6;
+    }
+    return key;
+}
+
 // Run `launch(candidate)` for the tuned candidate of `key`; when tuning is
-// allowed and the key is new (or mode 2), time every candidate first.
+// allowed and the key is new (or mode 2, or the stored candidate is refused),
+// time every candidate first.
 template <typename F>
 static void run_tuned(TuneKey key, int ncand, bool allow, cudaStream_t s, F &&launch)
 {
     TuneState &st = tune_state();
     int v = -1;
-    bool tune = false;
+    bool tune = false, stored = false;
     {
         std::lock_guard<std::mutex> lock(st.mu);
         tune_env_locked(st);
-        auto it = st.choice.find(key);
-        if (it != st.choice.end()) v = it->second;
-        tune = allow && st.mode > 0 && (v < 0 || (st.mode == 2 && !st.retuned.count(key)));
+        allow = allow && st.mode > 0;
+        auto find = [&](const std::map<TuneKey, int> &m, const TuneKey &k) {
+            auto it = m.find(k);
+            if (it == m.end()) return false;
+            v = it->second;
+            return true;
+        };
+        stored = find(st.choice, key);
+        if (!stored && !find(st.pinned, key.any())) {
+            tune = allow;
+            if (!tune) find(st.hint, key.any());
+        }
+        tune = tune || (allow && st.mode == 2 && !st.retuned.count(key));
+    }
+    if (!tune && v >= 0) {
+        if (launch(v)) return;
+        v = -1;
+        tune = allow && stored;
     }
     if (tune) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -1271,11 +1333,12 @@ static void run_tuned(TuneKey key, int ncand, bool allow, cudaStream_t s, F &&la
         v = bv < 0 ? 0 : bv;
         std::lock_guard<std::mutex> lock(st.mu);
         st.choice[key] = v;
+        st.latest[key.any()] = v;
         st.retuned.insert(key);
         if (!st.file.empty()) {
             if (FILE *f = std::fopen(st.file.c_str(), "a")) {
-                std::fprintf(f, "%d %d %d %d %d %d %d %d\n", key.kind, key.k, key.bits, key.h, key.logn, key.logdeg,
-                             key.loghub, v);
+                std::fprintf(f, "%d %d %d %d %d %d %d %d %d %d\n", key.kind, key.k, key.bits, key.h, key.logn,
+                             key.logdeg, key.loghub, v, key.layout, TUNE_SET);
                 std::fclose(f);
             }
         }
@@ -1328,7 +1391,7 @@ template <typename CT> static void build_levels(mc_tables *t, int *err, cudaStre
         if (g->order)
             MC_LAUNCH("zero_rows", s, zero_rows_kernel<<<grid_for((n - g->n_do) * 32, 256), 256, 0, s>>>(
                                           ta.out, g->order + g->n_do, n - g->n_do));
-        const TuneKey mkey = tune_key(1, k, (int)sizeof(CT) * 8, h, n, g->nnz, g->max_degree);
+        const TuneKey mkey = tune_key(1, t, h);
         run_tuned(mkey, MERGE_CANDIDATES, allow_tune, s, [&](int c) { return launch_merge<CT>(ta, programs(k, t->skip_round).pairs[h], h, c, s); });
         if (h <= k - 1) {
             GatherArgs ga{};
@@ -1353,7 +1416,7 @@ template <typename CT> static void build_levels(mc_tables *t, int *err, cudaStre
             ga.err = err;
             ga.sched = g->sched;
             ga.n_small = g->n_small;
-            const TuneKey gkey = tune_key(0, k, (int)sizeof(CT) * 8, h, n, g->nnz, g->max_degree);
+            const TuneKey gkey = tune_key(0, t, h);
             const int rh = shape_catalog().r[h];
             run_tuned(gkey, GATHER_CANDIDATES, allow_tune, s, [&](int c) { return launch_gather<CT>(ga, rh, h, c, s); });
             if (g->n_hubs) {
@@ -2067,8 +2130,8 @@ extern "C" int mc_autotune_choice(int kind, int k, int count_bits, int h, int64_
     TuneState &st = tune_state();
     std::lock_guard<std::mutex> lock(st.mu);
     tune_env_locked(st);
-    auto it = st.choice.find(key);
-    return it == st.choice.end() ? -1 : it->second;
+    auto it = st.latest.find(key);
+    return it == st.latest.end() ? -1 : it->second;
 }
 
 extern "C" mc_status mc_autotune_set(int kind, int k, int count_bits, int h, int64_t n, int64_t nnz,
@@ -2076,11 +2139,13 @@ extern "C" mc_status mc_autotune_set(int kind, int k, int count_bits, int h, int
 {
     return guarded([&] {
         MC_REQUIRE(kind == 0 || kind == 1, "kind must be 0 (neighbour sums) or 1 (merge)");
-        MC_REQUIRE(choice >= 0 && choice < (kind == 0 ? GATHER_CANDIDATES : MERGE_CANDIDATES), "no such schedule");
+        MC_REQUIRE(choice >= 0 && choice < candidates(kind), "no such schedule");
         const TuneKey key = tune_key(kind, k, count_bits, h, n, nnz, max_degree);
         TuneState &st = tune_state();
         std::lock_guard<std::mutex> lock(st.mu);
         tune_env_locked(st);
-        st.choice[key] = choice;
+        for (auto it = st.choice.lower_bound(key); it != st.choice.end() && !(key < it->first.any());)
+            it = st.choice.erase(it);  // every layout's
+        st.pinned[key] = st.latest[key] = choice;
     });
 }
