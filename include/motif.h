@@ -251,7 +251,7 @@ mc_status mc_table_nonzeros(const mc_tables *t, int h, int which, int64_t *count
 
 /* Copy a whole level (n * row_entries * entry_bytes bytes) into dst (host or
  * device as dst_on_device says; dst needs no alignment).  Level 1 of c is all
- * ones and is produced on the fly.  Uses up to 64 MB of scratch unless dst is
+ * ones and is produced on the fly.  Uses up to 256 MB of scratch unless dst is
  * memory of the current device aligned to a count; without it, copies are put
  * together on the host (packed tables: a whole dense level of scratch, else
  * MC_E_NOMEM).  Synchronises `stream`. */

@@ -2094,12 +2094,15 @@ extern "C" mc_status mc_read_table(const mc_tables *t, int h, int which, void *d
         MC_REQUIRE(dst_bytes >= bytes, "dst too small");
         cudaStream_t s = (cudaStream_t)stream;
         if (bytes == 0) return;
-        const bool ones = which == 0 && h == 1;
+        const bool ones = which == 0 && h == 1, dense = !ones && !t->packed;
+        const Rows x = t->rows(h, which);
         const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
         Arena scratch(true);
         scratch.alloc = t->arena.alloc;
         scratch.stream = s;
-        if (dst_on_device && stores_counts(dst, cb)) {
+        if (dense && x.N == (int)cb) {  // the first plane is the rows as they are
+            MC_CUDA(cudaMemcpyAsync(dst, x.p0, bytes, kind, s));
+        } else if (dst_on_device && stores_counts(dst, cb)) {
             if (ones)
                 MC_LAUNCH("fill_ones", s, fill_ones_kernel<<<grid_for(n, 256), 256, 0, s>>>(dst, n, (int)cb));
             else if (t->packed)
@@ -2123,9 +2126,30 @@ extern "C" mc_status mc_read_table(const mc_tables *t, int h, int which, void *d
             void *tmp = scratch.get<uint8_t>(bytes);
             launch_unpack(t, h, which, tmp, s);
             MC_CUDA(cudaMemcpyAsync(dst, tmp, bytes, kind, s));
-        } else {  // through a scratch buffer of some rows, without one from the planes as they are
+        } else if (!dst_on_device && bytes <= 256 * 1024 && !(t->wide_levels & x.bit)) {
+            // a small level: its first plane copied and widened here, without
+            // scratch and a launch (0.020 against 0.027 ms for a 1k-node graph)
+            std::vector<uint8_t> low((size_t)(n * x.s0));
+            MC_CUDA(cudaMemcpyAsync(low.data(), x.p0, low.size(), cudaMemcpyDeviceToHost, s));
+            MC_CUDA(cudaStreamSynchronize(s));
+            uint8_t *at = (uint8_t *)dst;
+            auto widen_rows = [&](auto from) {
+                for (int64_t v = 0; v < n; ++v)
+                    for (int e = 0; e < x.W; ++e, at += cb) {
+                        std::memcpy(&from, low.data() + v * x.s0 + e * sizeof(from), sizeof(from));
+                        const uint64_t y[2] = {from, 0};
+                        if (cb == 8) std::memcpy(at, y, 8);
+                        else std::memcpy(at, y, 16);
+                    }
+            };
+            if (x.N == 4) widen_rows((uint32_t)0);
+            else widen_rows((uint64_t)0);
+        } else {
+            // through a scratch buffer of up to 256 MB (each further copy into host
+            // pages not touched before costs some 0.5 ms beside its bytes), without
+            // one from the planes as they are
             const int64_t row = W * (int64_t)cb;
-            const int64_t step = std::max<int64_t>(1, std::min<int64_t>(n, ((int64_t)64 << 20) / row));
+            const int64_t step = std::max<int64_t>(1, std::min<int64_t>(n, ((int64_t)256 << 20) / row));
             void *tmp = nullptr;
             std::vector<uint8_t> host;
             try {

@@ -57,3 +57,20 @@ def test_any_address(M, monkeypatch, bits, kw):
                 assert np.array_equal(_device_read(M, T, h, which, off), want), (which, h, off)
         finally:
             al.closed = False
+
+
+@pytest.mark.parametrize("bits", [64, 128])
+@pytest.mark.parametrize("make", [lambda: synth.er_1k(), lambda: synth.star(500), lambda: synth.chung_lu(9000, 40000, 2.4, seed=1)])
+def test_host_at_any_address(M, bits, make):
+    # small levels are widened on the host, the others on the device
+    g, k = make(), 5
+    T = M.Tables(M.Graph.from_csr(g), synth.balanced_colors(g.n, k, 3), k, bits)
+    for which, h in ((0, 1), (0, 2), (0, 4), (0, 5), (1, 1), (1, 3), (1, 4)):
+        want = _device_read(M, T, h, which, 0)
+        W, b = T.layout(h, which)
+        for off in (0, 8, 1):
+            buf = np.full(want.size + 64, 0xA5, np.uint8)
+            M._check(M.load().mc_read_table(T.handle, h, which, C.c_void_p(buf.ctypes.data + off), want.size, 0,
+                                            M._stream_ptr()))
+            assert np.array_equal(buf[off:off + want.size], want), (which, h, off)
+            assert (buf[:off] == 0xA5).all() and (buf[off + want.size:] == 0xA5).all()
