@@ -519,6 +519,7 @@ static void fill_sample_args(SampleArgs &a, const mc_tables *t, int h)
         a.R_[i] = cat.r[i];
     }
     a.levels = t->wide_levels;
+    a.wide = t->wide;
     a.k = t->k;
     a.h = h;
     for (int i = 0; i <= MAXK + 1; ++i) a.first[i] = cat.first[std::min(i, MAXK + 1)];
@@ -701,18 +702,19 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, SplitScratch *spli
     // instantiation of its own, so other launches carry none of its work; else
     // split sampling if it has the memory.  The latency mode at full size is
     // twice as slow.
+    // Rows below level h that carry upper parts:
+    const uint32_t below = ((1u << a.h) - 1u) & ~3u;
+    const bool wide = !t->packed && t->bits == 128 && (a.levels & (below | below << 16 | 2u << 16));
     SampleMode mode = SampleMode::Lanes;
     if (a.count <= (int64_t)sm_count() * (a.h >= 5 ? 64 : 32)) mode = SampleMode::Warps;
     else if (!t->packed && a.count <= (int64_t)sm_count() * 256) mode = SampleMode::Latency;
     else if (a.bytes && !t->packed) mode = SampleMode::Counted;
-    else if (split && split->room(!a.nodes, !a.classes, std::min(a.count, a.nodes && a.classes ? a.count : SPLIT_CHUNK), a.h))
+    else if (split &&
+             split->room(!a.nodes, !a.classes, std::min(a.count, a.nodes && a.classes ? a.count : SPLIT_CHUNK), a.h))
         mode = SampleMode::Split;
     if (mode != SampleMode::Counted) a.bytes = nullptr;
-    // rows below level h that carry upper parts
-    const uint32_t below = ((1u << a.h) - 1u) & ~3u;
-    const bool wide = mode == SampleMode::Split && !t->packed && t->bits == 128 && (a.levels & (below | below << 16 | 2u << 16));
-    auto kern = t->packed ? sample_kernel_packed(mode, t->bits, narrow)
-                          : sample_kernel_dense(wide ? SampleMode::SplitWide : mode, t->bits, narrow);
+    const int in_line = !wide ? 0 : a.count > (int64_t)sm_count() * 2 * SAMPLE_BLOCK ? 3 : 4;  // one wave: 2 blocks per SM
+    auto kern = t->packed ? sample_kernel_packed(mode, t->bits, narrow) : sample_kernel_dense(mode, t->bits, narrow, in_line);
     const int block = mode == SampleMode::Warps ? 256 : mode == SampleMode::Latency ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
     const size_t hist = a.hist ? (size_t)a.ncls * sizeof(uint32_t) : 0;
     const size_t smem = (mode == SampleMode::Warps ? 0 : (size_t)SAMPLE_WORDS * block * sizeof(uint32_t)) +

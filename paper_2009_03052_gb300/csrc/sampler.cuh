@@ -53,6 +53,7 @@ struct SampleArgs {
     const int32_t *coff;
     int64_t n;
     Rows c[MAXK + 1], S[MAXK + 1];  // the levels of dense tables
+    const uint32_t *wide;       // per node, the levels at which its row is wide
     uint32_t levels;            // the levels that have wide rows
     PackedView pc[MAXK + 1], ps[MAXK + 1];  // the levels of packed (succinct) tables
     const void *Sp[MAXK + 1];   // per level: inclusive prefix of each hub's chunk sums
@@ -97,6 +98,7 @@ struct SampleSmem {
     uint8_t pair[32];                   // per bit of the adjacency word: i | j << 4
     uint2 shape[MAX_SHAPES];            // size | local id << 8 | beta << 16; T' | T'' << 8
     uint4 level[2][MAXK + 1];           // c, S: first-plane base, row stride, N | has wide rows << 8
+    uint4 upper[2][MAXK + 1];           // their second planes: base, row stride, counts per row
     int r[MAXK + 1];                    // rooted shapes per size
 };
 
@@ -112,6 +114,8 @@ template <int T> __device__ __forceinline__ void fill_sample_smem(const SampleAr
         const Rows &r = i > MAXK ? a.S[l] : a.c[l];
         sm.level[i / (MAXK + 1)][l] = make_uint4((uint32_t)(uint64_t)r.p0, (uint32_t)((uint64_t)r.p0 >> 32), (uint32_t)r.s0,
                                                  (uint32_t)r.N | ((a.levels & r.bit) ? 256u : 0u));
+        sm.upper[i / (MAXK + 1)][l] = make_uint4((uint32_t)(uint64_t)r.p1, (uint32_t)((uint64_t)r.p1 >> 32), (uint32_t)r.s1,
+                                                 (uint32_t)r.W);
         if (i <= MAXK) sm.r[l] = a.R_[l];
     }
     const int h = a.h, P = h * (h - 1) / 2;
@@ -120,29 +124,44 @@ template <int T> __device__ __forceinline__ void fill_sample_smem(const SampleAr
 }
 
 // Row x of level h of c (which = 0) or S (1): entry get(idx) of dense rows, or
-// (PK) by a binary search of the packed row's keys.
+// (PK) by a binary search of the packed row's keys.  full(idx) adds the upper
+// part of a row that is wide, in line, so that the items of a scan are in flight
+// together.  (Reading the upper part before the row is known to be wide, for a
+// shorter chain of loads, was slower at every launch size: 20k samples of R-MAT
+// 22, k = 7, 0.444 against 0.409 ms, 1M 3.13 against 2.56.)
 template <typename CT, bool PK> struct RowRef {
     const SampleArgs &a;
+    const SampleSmem &sm;
     const uint8_t *low;
     int64_t x;
     int h, N, which;
     bool wide;
-    __device__ __forceinline__ RowRef(const SampleArgs &a_, const SampleSmem &sm, int which_, int h_, int64_t x_)
-        : a(a_), low(nullptr), x(x_), h(h_), N(8), which(which_), wide(false)
+    __device__ __forceinline__ RowRef(const SampleArgs &a_, const SampleSmem &sm_, int which_, int h_, int64_t x_)
+        : a(a_), sm(sm_), low(nullptr), x(x_), h(h_), N(8), which(which_), wide(false)
     {
         if constexpr (!PK) {
             const uint4 l = sm.level[which][h];
             low = (const uint8_t *)(((uint64_t)l.y << 32) | l.x) + x * (uint64_t)l.z;
             N = (int)(l.w & 255u);
-            if (l.w >> 8) wide = (rows().wide[x] & rows().bit) != 0;
+            if (l.w >> 8) wide = (a.wide[x] >> (which ? 16 + h : h)) & 1u;
         }
     }
-    __device__ __forceinline__ const Rows &rows() const { return which ? a.S[h] : a.c[h]; }
     // entry idx of a row that is not wide
     __device__ __forceinline__ CT get(int idx) const
     {
         if constexpr (PK) return (CT)packed_get(which ? a.ps[h] : a.pc[h], x, idx);
         else return row_low_any<CT>(low, N, idx);
+    }
+    __device__ __forceinline__ CT rest(int idx) const
+    {
+        const uint4 u = sm.upper[which][h];
+        return row_rest<CT>((const uint8_t *)(((uint64_t)u.y << 32) | u.x) + x * (uint64_t)u.z, (int)u.w, N, idx);
+    }
+    __device__ __forceinline__ CT full(int idx) const
+    {
+        CT v = row_low_any<CT>(low, N, idx);
+        if (wide) v |= rest(idx);
+        return v;
     }
 };
 
@@ -151,15 +170,6 @@ template <typename CT, bool PK> struct RowRef {
 template <typename CT> __device__ __noinline__ CT entry_wide(const SampleArgs &a, int which, int h, int64_t x, int idx)
 {
     return entry_at<CT>(which ? a.S[h] : a.c[h], x, idx);
-}
-
-// The same of a row that is (`wide`) or is not wide, in line, so that the
-// items of a scan are in flight together.
-template <typename CT> __device__ __forceinline__ CT entry_full(const Rows &r, int64_t x, bool wide, int idx)
-{
-    CT v = row_low_any<CT>(r.low(x), r.N, idx);
-    if (wide) v |= row_rest<CT>(r.high(x), r.W, r.N, idx);
-    return v;
 }
 
 __device__ __forceinline__ uint64_t quotient(uint64_t a, uint64_t b) { return a / b; }
@@ -284,22 +294,24 @@ __device__ __forceinline__ int64_t first_true(int64_t lo, int64_t hi, P pred, F 
 // that the searches of the classification neither hold the sampler's registers
 // nor wait in the divergence of its warps (1M samples at k = 5: 0.75 + 0.16 ms
 // against 1.08 in one kernel; the code before both 1.11).
-// WD (split sampling from 128-bit tables with wide rows below level h): counts
-// above 64 bits carry most of the weight, so most samples pass through wide
-// rows; their entries are read in line, low and upper parts and the wide words
-// of 3 neighbours in flight, where the other kernels call entry_wide one at a
-// time (ms for 1M / 10M samples of R-MAT 22, k = 7: 2.71 / 24.6; by calls 3.25 /
-// 31.6; whole 16-byte counts 2.91 / 27.8; 2 in flight 2.70 / 23.6 but 0.88
-// against 0.85 for 200k, 4: 2.95 / 27.9).  Tables with wide rows at level h only
-// stay with the calls: 4.03 against 4.38 for 1M samples of Chung-Lu 2M, k = 8.
+// WD > 0 (128-bit dense tables with wide rows below level h): counts above 64 bits
+// carry most of the weight, so most samples pass through wide rows; their entries
+// are read in line, low and upper parts and the wide words of WD neighbours in
+// flight, where the other kernels call entry_wide one at a time.  R-MAT 22, k = 7,
+// ms with estimates (by calls / in line / whole 16-byte counts): 10M samples 31.6
+// / 22.6 / 27.9, 1M 3.25 / 2.56 / 2.92, all split; 100k 0.58 / 0.518 / 0.516; 20k
+// (latency mode) 0.465 / 0.413 / 0.413; without split scratch 1M 4.03 / 3.42 /
+// 3.11.  WD: 3 where split sampling fills the GPU more than once (10M: 4 in flight
+// 23.5), else 4 (100k: 3 in flight 0.569; latency mode: 8 0.455, 16 0.485; without
+// split scratch 1M: 3 3.66, 5 3.71).
 constexpr int SAMPLE_WORDS = 3 * MAXK;  // shared words per thread
 constexpr int SAMPLE_BLOCK = 512, SAMPLE_BLOCK_LAT = 64;
 
-template <typename CT, typename V, bool PK, bool LAT, bool CNT, bool SPLIT, bool WD = false>
+template <typename CT, typename V, bool PK, bool LAT, bool CNT, bool SPLIT, int WD = 0>
 __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1 : (sizeof(CT) == 16 && !PK ? 2 : 3))
     sample_kernel(const __grid_constant__ SampleArgs a)
 {
-    constexpr int NW = LAT ? 16 : WD ? 3 : sizeof(CT) == 16 && !PK ? 4 : 2;  // items of a scan in flight
+    constexpr int NW = WD ? WD : LAT ? 16 : sizeof(CT) == 16 && !PK ? 4 : 2;  // items of a scan in flight
     constexpr int NQ = LAT ? 8 : 4;   // adjacency searches in flight
     constexpr int KS = LAT ? 8 : 1;   // probes per round of the root and hub chunk searches
     constexpr int T = LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
@@ -387,11 +399,10 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                         return al ? (V)at((e - sh * Bc) * Rh + sh) : (V)0;
                     }, bf);
                 };
-                const int found = !PK && row.wide ? scan([&](int i) {
-                    if constexpr (CB == 16) return entry_full<CT>(a.c[h], v, true, i);
-                    else return entry_wide<CT>(a, 0, h, v, i);
-                })
-                                                  : scan([&](int i) { return row.get(i); });
+                int found;
+                if (!PK && CB == 16 && sm.level[0][h].w >> 8) found = scan([&](int i) { return row.full(i); });
+                else if (!PK && row.wide) found = scan([&](int i) { return entry_wide<CT>(a, 0, h, v, i); });
+                else found = scan([&](int i) { return row.get(i); });
                 if (found < 0) { ok = false; bad = true; }
                 else {
                     const int cv = a.colors[v];
@@ -438,7 +449,8 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                 V Y = 0;
                 const RowRef<CT, PK> rg(a, sm, 0, hg, x);
                 const int ig = sm.crank[rest] * sm.r[hg] + (int)(sg.x >> 8 & 255u);
-                const V W = (V)(sg.x >> 16 & 255u) * (V)(!PK && rg.wide ? entry_wide<CT>(a, 0, hg, x, ig) : rg.get(ig));
+                const V W = (V)(sg.x >> 16 & 255u) *
+                            (V)(WD ? rg.full(ig) : !PK && rg.wide ? entry_wide<CT>(a, 0, hg, x, ig) : rg.get(ig));
                 if (!draw_below(a.seed, index, step, W, Y)) { ok = false; bad = true; }
                 if (ok) {
                     // block of C'' (ascending mask), weights c(T'_{C\C''}, x) S(T'', C'', x)
@@ -448,7 +460,7 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                     for (int i = 1; i <= hb; ++i) nsub = nsub * (nr - hb + i) / i;
                     const int Ra = sm.r[ha], Rb = sm.r[hb];
                     const RowRef<CT, PK> ra(a, sm, 0, ha, x), rb_(a, sm, 1, hb, x);
-                    const bool wide = !PK && (ra.wide || rb_.wide);
+                    const bool wide = WD ? true : !PK && (ra.wide || rb_.wide);
                     auto index_a = [&](unsigned c2) { return sm.crank[rest & ~c2] * Ra + la; };
                     V before;
                     auto scan = [&](auto at_a, auto at_b) {
@@ -460,11 +472,11 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                     };
                     const int blk = wide ? scan(
                                                [&](int i) {
-                                                   if constexpr (WD) return entry_full<CT>(a.c[ha], x, ra.wide, i);
+                                                   if constexpr (WD > 0) return ra.full(i);
                                                    else return entry_wide<CT>(a, 0, ha, x, i);
                                                },
                                                [&](int i) {
-                                                   if constexpr (WD) return entry_full<CT>(a.S[hb], x, rb_.wide, i);
+                                                   if constexpr (WD > 0) return rb_.full(i);
                                                    else return entry_wide<CT>(a, 1, hb, x, i);
                                                })
                                          : scan([&](int i) { return ra.get(i); }, [&](int i) { return rb_.get(i); });
@@ -473,6 +485,7 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                         const unsigned c2 = select_bits(sm.unrank[hb][blk], pos);
                         C2 = insert_colour_gap(c2, cx);
                         const V x1 = ha == 1 ? (V)1
+                                     : WD    ? (V)ra.full(index_a(c2))
                                              : (V)(wide ? entry_wide<CT>(a, 0, ha, x, index_a(c2)) : ra.get(index_a(c2)));
                         q = (CT)quotient(Y - before, x1);  // < S(T'', C'', x): fits CT
                         sidx = sm.crank[c2] * Rb + lb;
@@ -554,16 +567,19 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                                 MC_COUNT(5, 5);  // contiguous edge colours and ids
                                 if (in) MC_COUNT(CB, 32);  // the neighbour's row entry
                                 y[i] = in ? row_low_any<CT>(p0 + id[i] * (uint64_t)lv.z, N, index_of(ci[i])) : (CT)0;
-                                if constexpr (WD) ww[i] = in && lv.w >> 8 ? a.c[hb].wide[id[i]] & a.c[hb].bit : 0u;
+                                if constexpr (WD > 0) ww[i] = in && lv.w >> 8 ? (a.wide[id[i]] >> hb) & 1u : 0u;
                             }
-                            if constexpr (WD) {
+                            if constexpr (WD > 0) {
+                                const uint4 uv = sm.upper[0][hb];
+                                const uint8_t *p1 = (const uint8_t *)(((uint64_t)uv.y << 32) | uv.x);
                                 uint32_t any = 0;
 #pragma unroll
                                 for (int i = 0; i < NW; ++i) any |= ww[i];
                                 if (any) {
 #pragma unroll
                                     for (int i = 0; i < NW; ++i)
-                                        if (ww[i]) y[i] |= row_rest<CT>(a.c[hb].high(id[i]), a.c[hb].W, N, index_of(ci[i]));
+                                        if (ww[i])
+                                            y[i] |= row_rest<CT>(p1 + id[i] * (uint64_t)uv.z, (int)uv.w, N, index_of(ci[i]));
                                 }
                             }
 #pragma unroll
@@ -1197,11 +1213,12 @@ static __global__ void __launch_bounds__(256) classify_kernel(const __grid_const
 }
 
 typedef void (*SampleKernel)(SampleArgs);
-enum class SampleMode { Lanes, Latency, Counted, Split, Warps, SplitWide };
+enum class SampleMode { Lanes, Latency, Counted, Split, Warps };
 // The kernel for tables of bits-bit counts with 64-bit descent arithmetic
-// (narrow) or 128-bit, dense (sampler_dense.cu; all modes) or packed
+// (narrow) or 128-bit, dense (sampler_dense.cu; all modes; `wide`, 128-bit counts
+// only: rows below level h are wide, 3 or 4 of their items in flight) or packed
 // (sampler_packed.cu: Lanes, Split, Warps).
-SampleKernel sample_kernel_dense(SampleMode mode, int bits, bool narrow);
+SampleKernel sample_kernel_dense(SampleMode mode, int bits, bool narrow, int wide);
 SampleKernel sample_kernel_packed(SampleMode mode, int bits, bool narrow);
 
 }  // namespace mc
