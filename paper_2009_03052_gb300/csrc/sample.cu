@@ -700,16 +700,23 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, SplitScratch *spli
     // the latency mode (dense tables, blocks of 64 spread over more SMs) for
     // launches that leave most SMs idle; byte counting (profiling) runs an
     // instantiation of its own, so other launches carry none of its work; else
-    // split sampling if it has the memory.  The latency mode at full size is
-    // twice as slow.
+    // split sampling, if it has the memory, where it pays for its second launch:
+    // from four waves of 3 blocks of 512 per SM on (sample_kernel / split, ms with
+    // estimates: 400k samples 0.496 / 0.512, 1M 1.012 / 1.002, 10M 8.44 / 8.32 at
+    // k = 5; 0.727 / 0.742, 1.555 / 1.564, 15.1 / 14.1 at k = 6; 100k of a 1k-node
+    // graph, k = 4, 0.146 / 0.165), for h >= 7 (15 and 21 pairs to test per
+    // sample) and with wide rows read in line from one wave on (200k at k = 7,
+    // R-MAT 19 and 22: 0.647 / 0.623 and 0.92 / 0.79).  The latency mode at full
+    // size is twice as slow.
     // Rows below level h that carry upper parts:
     const uint32_t below = ((1u << a.h) - 1u) & ~3u;
     const bool wide = !t->packed && t->bits == 128 && (a.levels & (below | below << 16 | 2u << 16));
+    const bool many = a.h >= 7 || wide || a.count >= (int64_t)sm_count() * 4 * 1536;
     SampleMode mode = SampleMode::Lanes;
     if (a.count <= (int64_t)sm_count() * (a.h >= 5 ? 64 : 32)) mode = SampleMode::Warps;
     else if (!t->packed && a.count <= (int64_t)sm_count() * 256) mode = SampleMode::Latency;
     else if (a.bytes && !t->packed) mode = SampleMode::Counted;
-    else if (split &&
+    else if (many && split &&
              split->room(!a.nodes, !a.classes, std::min(a.count, a.nodes && a.classes ? a.count : SPLIT_CHUNK), a.h))
         mode = SampleMode::Split;
     if (mode != SampleMode::Counted) a.bytes = nullptr;
