@@ -2100,15 +2100,15 @@ extern "C" mc_status mc_read_table(const mc_tables *t, int h, int which, void *d
         Arena scratch(true);
         scratch.alloc = t->arena.alloc;
         scratch.stream = s;
-        if (dense && x.N == (int)cb) {  // the first plane is the rows as they are
-            MC_CUDA(cudaMemcpyAsync(dst, x.p0, bytes, kind, s));
-        } else if (dst_on_device && stores_counts(dst, cb)) {
+        if (dst_on_device && stores_counts(dst, cb)) {
             if (ones)
                 MC_LAUNCH("fill_ones", s, fill_ones_kernel<<<grid_for(n, 256), 256, 0, s>>>(dst, n, (int)cb));
             else if (t->packed)
                 launch_unpack(t, h, which, dst, s);
             else
                 launch_expand(t, h, which, 0, n, dst, s);
+        } else if (dense && x.N == (int)cb) {  // the first plane is the rows as they are
+            MC_CUDA(cudaMemcpyAsync(dst, x.p0, bytes, kind, s));
         } else if (ones) {
             std::vector<uint8_t> one;
             uint8_t *at = (uint8_t *)dst;
