@@ -71,16 +71,33 @@ def geometry(k: int):
     return Wc, Ws
 
 
-def algorithmic_bytes(name: str, n: int, nnz: int, k: int, B: int):
+def plane_widths(degrees, k: int):
+    """Bytes of the first-plane counts of c_h and S_h (the library's rule: 4
+    where a level's largest count is expected below 2^30, from the largest
+    degree and the sum of squared degrees per adjacency entry; else 8)."""
+    d = np.asarray(degrees, dtype=np.float64)
+    star = math.log2(max(float(d.max(initial=0)) / k, 1.0))
+    walk = math.log2(max(float((d * d).sum()) / max(float(d.sum()), 1.0) / k, 1e-3))
+
+    def width(h):
+        trees = (h - 1) * walk + math.log2(math.factorial(h - 1))
+        return 4 if h <= 2 or ((h - 1) * star <= 30 and trees <= 30) else 8
+    return {h: width(h) for h in range(1, k + 1)}, {h: 4 if h == 1 else width(h + 1) for h in range(1, k)}
+
+
+def algorithmic_bytes(name: str, n: int, nnz: int, k: int, B: int, planes=None):
     """Compulsory DRAM bytes of one launch of a build kernel (each input row
-    read once, each output row written once, plus the CSR it walks)."""
+    read once, each output row written once, plus the CSR it walks), for rows
+    of B-byte counts or, with `planes` (plane_widths), of the first planes the
+    kernels read and write."""
     Wc, Ws = geometry(k)
+    Nc, Ns = planes if planes else ({h: B for h in Wc}, {h: B for h in Ws})
     csr = 8 * (n + 1) + 4 * nnz + n
     if name == "gather_h1":
-        return csr + n * (k - 1) * B
+        return csr + n * (k - 1) * Ns[1]
     if name.startswith("gather_h"):
         h = int(name[len("gather_h"):])
-        return n * Wc[h] * B + n * Ws[h] * B + csr
+        return n * Wc[h] * Nc[h] + n * Ws[h] * Ns[h] + csr
     if name.startswith("merge_h"):
         import paper_2009_03052_gb300 as M
         h = int(name[len("merge_h"):])
@@ -97,9 +114,51 @@ def algorithmic_bytes(name: str, n: int, nnz: int, k: int, B: int):
             h2 = end // 2
             used1.add(h - h2)
             used2.add(h2)
-        rd = sum(Wc[x] for x in used1 if x > 1) + sum(Ws[x] for x in used2)
-        return n * (rd + Wc[h]) * B
+        rd = sum(Wc[x] * Nc[x] for x in used1 if x > 1) + sum(Ws[x] * Ns[x] for x in used2)
+        return n * (rd + Wc[h] * Nc[h])
     return None
+
+
+def kernel_roofline(nm: str, prof: dict, counted: dict, hbm_peak: float, peak_source: str, compulsory, traffic):
+    """A kernel's bytes over its time in the timed steps, against the copy peak.
+    prof: name -> (ms, launches) of the timed steps; counted: name -> (ms,
+    launches, bytes) of the counted step; compulsory: the build kernels' bytes
+    per launch (None: unknown).  The counting sampler classifies too, so its
+    bytes are set against the time of both kernels of split sampling."""
+    ms, cnt = prof[nm]
+    kernel, item = nm, None
+    _, ccnt, citems = counted.get(nm, (0.0, 0, 0))
+    sectors = counted.get(nm + " sectors", (0.0, 0, 0))[2]
+    if sectors > 0 and ccnt > 0:
+        # the sector model of the sampler's bytes (32 B per random access:
+        # root-search probes, each scanned neighbour's row entry, chunk-
+        # and adjacency-search probes; contiguous runs by their bytes),
+        # per launch of the counting step
+        by = sectors / ccnt
+        src = ("counted by the kernel, 32-byte sector model: 32 B per random access, "
+               "contiguous runs by their bytes (one extra counted step)")
+        item = int(citems / ccnt)
+        if nm == "sample" and "classify" in prof:
+            ms += prof["classify"][0]
+            kernel = "sample + classify"
+    else:
+        by = compulsory
+        src = "compulsory bytes (each first-plane row read once, written once, plus the CSR)"
+    if by is None:
+        return None
+    achieved = by / (ms / cnt / 1e3) / 1e9
+    out = {"kernel": kernel, "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm_peak,
+           "unit": "GB/s", "frac": round(achieved / hbm_peak, 4),
+           "traffic": traffic, "algorithmic_bytes": int(by),
+           "bytes_model": src, "peak_source": peak_source, "avg_launch_ms": round(ms / cnt, 4)}
+    if item is not None:  # the bytes of the data items themselves
+        out["item_bytes"] = item
+        out["item_frac"] = round(item / (ms / cnt / 1e3) / 1e9 / hbm_peak, 4)
+    if traffic:  # the DRAM bytes of the ncu capture over this run's launch time
+        dram = traffic / (ms / cnt / 1e3) / 1e9
+        out["dram_gbs"] = round(dram, 1)
+        out["dram_frac"] = round(dram / hbm_peak, 4)
+    return out
 
 
 # ---------------------------------------------------------------------------
@@ -346,39 +405,12 @@ def run_gpu(args, rank: int, world: int, local_rank: int):
         hbm_peak, peak_src = float(peaks["hbm_gbs"]), "measured"
     else:
         hbm_peak, peak_src = 6800.0, "fallback"
+    planes = plane_widths(np.diff(graph.row_ptr), k)
+
     def roofline(nm):
-        ms, cnt = prof[nm]
-        item = None
-        cms, ccnt, citems = counted.get(nm, (0.0, 0, 0))
-        sectors = counted.get(nm + " sectors", (0.0, 0, 0))[2]
-        if sectors > 0 and ccnt > 0:
-            # the sector model of the sampler's bytes (32 B per random access:
-            # root-search probes, each scanned neighbour's row entry, chunk-
-            # and adjacency-search probes; contiguous runs by their bytes),
-            # per launch of the counting step
-            by = sectors / ccnt
-            src = ("counted by the kernel, 32-byte sector model: 32 B per random access, "
-                   "contiguous runs by their bytes (one extra counted step)")
-            item = int(citems / ccnt)
-        else:
-            by = algorithmic_bytes(nm, n, nnz, k, BITS // 8)
-            src = "compulsory bytes (each row read once, written once, plus the CSR)"
-        if by is None:
-            return None
-        achieved = by / (ms / cnt / 1e3) / 1e9
-        traffic = traffic_of(wname, nm, schedules.get(nm))
-        out = {"kernel": nm, "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm_peak,
-               "unit": "GB/s", "frac": round(achieved / hbm_peak, 4),
-               "traffic": traffic, "algorithmic_bytes": int(by),
-               "bytes_model": src, "peak_source": peak_src, "avg_launch_ms": round(ms / cnt, 4)}
-        if item is not None:  # the bytes of the data items themselves
-            out["item_bytes"] = item
-            out["item_frac"] = round(item / (ms / cnt / 1e3) / 1e9 / hbm_peak, 4)
-        if traffic:  # the DRAM bytes of the ncu capture over this run's launch time
-            dram = traffic / (ms / cnt / 1e3) / 1e9
-            out["dram_gbs"] = round(dram, 1)
-            out["dram_frac"] = round(dram / hbm_peak, 4)
-        return out
+        return kernel_roofline(nm, prof, counted, hbm_peak, peak_src,
+                               algorithmic_bytes(nm, n, nnz, k, BITS // 8, planes),
+                               traffic_of(wname, nm, schedules.get(nm)))
 
     top = max(prof.items(), key=lambda x: x[1][0])[0] if prof else None
     roof = roofline(top) if top else None
@@ -811,16 +843,10 @@ def run_serve(args):
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch, from
 # one ncu capture of the named kernel on the named workload (the summaries in
 # profiles/), with a hash of the kernel's source file when it was captured:
-# the figure is reported only while that source is unchanged.
-TRAFFIC: dict = {
-    # profiles/sample_kernel_chung_lu_1m_k5.md
-    ("chung_lu_1m_k5", "sample"): (2_766_753_792, "ddde42efec355d4f"),
-    # profiles/gather_kernel_chung_lu_1m_k5.md, under schedules 6, 4, 4
-    ("chung_lu_1m_k5", "gather_h2"): (548_702_208, "887df3f50aaa2286", 6),
-    ("chung_lu_1m_k5", "gather_h3"): (1_256_040_192, "887df3f50aaa2286", 4),
-    ("chung_lu_1m_k5", "gather_h4"): (1_108_238_080, "887df3f50aaa2286", 4),
-}
-KERNEL_SOURCE = {"sample": "sample.cu", "gather": "gather.cuh", "merge": "build.cu"}
+# the figure is reported only while that source is unchanged.  Entries:
+# (workload, kernel): (bytes, hash[, schedule]).
+TRAFFIC: dict = {}
+KERNEL_SOURCE = {"sample": "sampler.cuh", "classify": "sampler.cuh", "gather": "gather.cuh", "merge": "build.cu"}
 
 
 def source_hash(kernel: str) -> str:

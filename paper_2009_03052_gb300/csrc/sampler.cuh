@@ -152,6 +152,8 @@ template <typename CT, bool PK> struct RowRef {
         if constexpr (PK) return (CT)packed_get(which ? a.ps[h] : a.pc[h], x, idx);
         else return row_low_any<CT>(low, N, idx);
     }
+    // of one entry (byte counting)
+    __device__ __forceinline__ int bytes() const { return wide ? (int)sizeof(CT) : N; }
     __device__ __forceinline__ CT rest(int idx) const
     {
         const uint4 u = sm.upper[which][h];
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                     return lane_first_exceeding<NW, V>(a.Wc[h], rem, [&](int e) -> V {
                         const int sh = e / Bc;
                         const bool al = sh < 64 ? (allow0 >> sh) & 1 : (allow1 >> (sh - 64)) & 1;
-                        MC_COUNT(al ? CB : 0, al ? CB : 0);  // one contiguous row
+                        MC_COUNT(al ? row.bytes() : 0, al ? row.bytes() : 0);  // one contiguous row
                         return al ? (V)at((e - sh * Bc) * Rh + sh) : (V)0;
                     }, bf);
                 };
@@ -440,7 +442,6 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                 const int hg = (int)(sg.x & 255u), ha = (int)(sa & 255u), la = (int)(sa >> 8 & 255u);
                 hb = (int)(sb & 255u);
                 lb = (int)(sb >> 8 & 255u);
-                MC_COUNT(16 + 4 + CB, 96);  // row offsets, first chunk, c(T_C, x)
                 e0 = a.row_ptr[x];
                 deg = a.row_ptr[x + 1] - e0;
                 chunk0 = a.node_chunk0[x];
@@ -448,6 +449,7 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                 const unsigned rest = drop_colour(C & ~(1u << cx), cx);
                 V Y = 0;
                 const RowRef<CT, PK> rg(a, sm, 0, hg, x);
+                MC_COUNT(16 + 4 + rg.bytes(), 96);  // row offsets, first chunk, c(T_C, x)
                 const int ig = sm.crank[rest] * sm.r[hg] + (int)(sg.x >> 8 & 255u);
                 const V W = (V)(sg.x >> 16 & 255u) *
                             (V)(WD ? rg.full(ig) : !PK && rg.wide ? entry_wide<CT>(a, 0, hg, x, ig) : rg.get(ig));
@@ -466,7 +468,7 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                     auto scan = [&](auto at_a, auto at_b) {
                         return lane_first_exceeding<NW, V>(nsub, Y, [&](int i) -> V {
                             const unsigned c2 = select_bits(sm.unrank[hb][i], pos);
-                            MC_COUNT(2 * CB, 64);
+                            MC_COUNT((ha == 1 ? 0 : ra.bytes()) + rb_.bytes(), ha == 1 ? 32 : 64);
                             return (ha == 1 ? (V)1 : (V)at_a(index_a(c2))) * (V)at_b(sm.crank[c2] * Rb + lb);
                         }, before);
                     };
@@ -541,6 +543,8 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                     } else if (!WD && sm.level[0][hb].w >> 8) {  // the level has wide rows
                         r = lane_first_exceeding<NW, CT>((int)len, q, [&](int i) -> CT {
                             const int ci = cols[i];
+                            MC_COUNT(5, 5);  // contiguous edge colours and ids
+                            if ((C2 >> ci) & 1u) MC_COUNT((int)(sm.level[0][hb].w & 255u) + 4, 64);  // entry, wide word
                             return ((C2 >> ci) & 1u) ? entry_wide<CT>(a, 0, hb, ids[i], index_of(ci)) : (CT)0;
                         }, bn);
                     } else {
@@ -565,7 +569,7 @@ __global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1
                             for (int i = 0; i < NW; ++i) {
                                 const bool in = b + i < n && ((C2 >> ci[i]) & 1u);
                                 MC_COUNT(5, 5);  // contiguous edge colours and ids
-                                if (in) MC_COUNT(CB, 32);  // the neighbour's row entry
+                                if (in) MC_COUNT(N, 32);  // the neighbour's row entry
                                 y[i] = in ? row_low_any<CT>(p0 + id[i] * (uint64_t)lv.z, N, index_of(ci[i])) : (CT)0;
                                 if constexpr (WD > 0) ww[i] = in && lv.w >> 8 ? (a.wide[id[i]] >> hb) & 1u : 0u;
                             }
