@@ -126,9 +126,10 @@ __global__ void __launch_bounds__(256) hub_reduce_kernel(CT *__restrict__ partia
 // one node (tid mod TN) and takes every (threads / TN)-th output, so the
 // threads that share an output run one program and read one entry of
 // neighbouring rows: no divergence, no bank conflicts, and every lower row
-// crosses the memory bus once.  Bound by instruction issue (60%, a third of
-// it the integer multiplies) at 36% of the warps, which shared memory allows;
-// staging the next pair while one is computed needs more of it and was slower
+// crosses the memory bus once.  Bound by latency at the few warps that shared
+// memory allows (30 - 36%): issue slots are idle 38 - 46% of the time, and the
+// stalls are fixed-latency waits, staging and barriers, in that order.  Staging
+// the next pair while one is computed needs more shared memory and was slower
 // (k = 7 levels 6 / 7: 4.8 / 5.5 against 3.9 / 4.8 ms), two nodes per thread
 // gave nothing.  Against a thread per (node, output) reading whole counts
 // through L1, ms per level 5 / 6 / 7 on R-MAT 22, k = 7, 128-bit counts: 10.6 /
@@ -142,7 +143,7 @@ __global__ void __launch_bounds__(256) hub_reduce_kernel(CT *__restrict__ partia
 // the rest of such a row is zeroed when the tile leaves.
 struct TilePair {
     int h1, h2;         // sizes of T' and T''
-    int wa, wb;         // row widths of c_{h1} (0 for h1 = 1: implicit) and S_{h2}
+    int wa;             // row width of c_{h1} (0 for h1 = 1: implicit)
     int ca, cb;         // 8-byte pieces of their first planes
     int sa, sb;         // strides in shared memory (odd), in 8-byte pieces
     uint32_t ma, mb;    // ceil(2^32 / pieces): division by the row's pieces
@@ -1098,7 +1099,6 @@ static bool plan_merge_tile(MergeTileArgs &ta, const MergePairs &Q, int shift, s
         P.h1 = Q.h1[p];
         P.h2 = Q.h2[p];
         P.wa = P.h1 == 1 ? 0 : ta.c[P.h1].W;
-        P.wb = ta.S[P.h2].W;
         P.ca = P.wa ? ta.c[P.h1].s0 / 8 : 0;
         P.cb = ta.S[P.h2].s0 / 8;
         P.sa = P.wa ? P.ca | 1 : 0;
@@ -1343,7 +1343,7 @@ static void run_tuned(TuneKey key, int ncand, bool allow, cudaStream_t s, F &&la
             }
         }
     }
-    if (v < 0 || !launch(v)) launch(0);
+    if ((v < 0 || !launch(v)) && !launch(0)) throw Error(MC_E_INTERNAL, "no schedule runs this level");
 }
 
 template <typename CT> static void build_levels(mc_tables *t, int *err, cudaStream_t s, bool allow_tune)

@@ -291,7 +291,6 @@ static void *pinned_scratch(size_t bytes)
 }
 
 // A CUDA event, released with its scope.
-
 struct EventHandle {
     cudaEvent_t e = nullptr;
     EventHandle() { MC_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming)); }
@@ -300,16 +299,15 @@ struct EventHandle {
     EventHandle &operator=(const EventHandle &) = delete;
 };
 
-// Up to NQ adjacency tests at once (binary search of the shorter list),
+// Up to four adjacency tests at once (binary search of the shorter list),
 // advancing all searches one level per round so their loads overlap.
-template <int NQ = 4, bool CNT = false>
 __device__ __forceinline__ void adjacent4(const int64_t *row_ptr, const uint32_t *col, const uint32_t *qa,
-                                          const uint32_t *qb, int nq, bool *out, uint64_t &rb, uint64_t &rs)
+                                          const uint32_t *qb, int nq, bool *out)
 {
-    int64_t lo[NQ], hi[NQ], end[NQ];
-    uint32_t key[NQ];
+    int64_t lo[4], hi[4], end[4];
+    uint32_t key[4];
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) {
+    for (int i = 0; i < 4; ++i) {
         if (i < nq) {
             uint32_t x = qa[i], y = qb[i];
             const int64_t dx = row_ptr[x + 1] - row_ptr[x], dy = row_ptr[y + 1] - row_ptr[y];
@@ -318,7 +316,6 @@ __device__ __forceinline__ void adjacent4(const int64_t *row_ptr, const uint32_t
             hi[i] = row_ptr[x + 1];
             end[i] = hi[i];
             key[i] = y;
-            MC_COUNT(32 + 4, 64 + 32);  // both degrees, the final probe
         } else {
             lo[i] = hi[i] = end[i] = 0;
             key[i] = 0;
@@ -328,16 +325,15 @@ __device__ __forceinline__ void adjacent4(const int64_t *row_ptr, const uint32_t
     while (more) {
         more = false;
 #pragma unroll
-        for (int i = 0; i < NQ; ++i)
+        for (int i = 0; i < 4; ++i)
             if (lo[i] < hi[i]) {
                 const int64_t mid = (lo[i] + hi[i]) >> 1;
                 if (col[mid] < key[i]) lo[i] = mid + 1; else hi[i] = mid;
-                MC_COUNT(4, 32);
                 more |= lo[i] < hi[i];
             }
     }
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) out[i] = i < nq && lo[i] < end[i] && col[lo[i]] == key[i];
+    for (int i = 0; i < 4; ++i) out[i] = i < nq && lo[i] < end[i] && col[lo[i]] == key[i];
 }
 
 // Uniform estimator (Section 2.2): g_i = ((t * hits_i) / (sigma_i * N)) * (1/p),
@@ -462,21 +458,20 @@ __global__ void __launch_bounds__(256) star_kernel(const __grid_constant__ StarA
         // four searches in flight
         uint32_t word = 0, qa[4], qb[4];
         int qp[4], nq = 0;
-        uint64_t rb = 0, rs = 0;
         for (int x = 0; x < h; ++x)
             for (int y = x + 1; y < h; ++y) {
                 if (nd[x] == c || nd[y] == c) { word |= 1u << pair_pos(h, x, y); continue; }
                 qa[nq] = nd[x]; qb[nq] = nd[y]; qp[nq] = pair_pos(h, x, y); ++nq;
                 if (nq == 4) {
                     bool r4[4];
-                    adjacent4(a.row_ptr, a.col, qa, qb, nq, r4, rb, rs);
+                    adjacent4(a.row_ptr, a.col, qa, qb, nq, r4);
                     for (int q = 0; q < nq; ++q) if (r4[q]) word |= 1u << qp[q];
                     nq = 0;
                 }
             }
         if (nq) {
             bool r4[4];
-            adjacent4(a.row_ptr, a.col, qa, qb, nq, r4, rb, rs);
+            adjacent4(a.row_ptr, a.col, qa, qb, nq, r4);
             for (int q = 0; q < nq; ++q) if (r4[q]) word |= 1u << qp[q];
         }
         const int cls = a.lut[word];
