@@ -596,11 +596,17 @@ extern "C" mc_status mc_load_graph(int64_t n, int64_t nnz, const int64_t *row_pt
             // the merges skip neighbourless nodes when at least an eighth are
             // (below that, reading 4 bytes per node for the list and losing
             // the runs of consecutive rows costs what the skipped rows give)
-            if ((int64_t)hh[0] * 8 >= n) {
-                g->order = g->arena.get<uint32_t>((size_t)n);
+            uint32_t *order = nullptr;
+            unsigned *dc = nullptr;
+            if ((int64_t)hh[0] * 8 >= n) try {
+                order = g->arena.get<uint32_t>((size_t)n);
+                dc = scratch.get<unsigned>(2);
+            } catch (const Error &) {  // no room: the merges take all nodes
+            }
+            if (order && dc) {
+                g->order = order;
                 g->n_do = n - hh[0];
                 oc[1] = (unsigned)g->n_do;
-                unsigned *dc = scratch.get<unsigned>(2);
                 MC_CUDA(cudaMemcpyAsync(dc, oc, sizeof(oc), cudaMemcpyHostToDevice, s));
                 MC_LAUNCH("active_order", s, active_order_kernel<<<grid_for(n, 256), 256, 0, s>>>(g->row_ptr, n, dc,
                                                                                                   g->order));
