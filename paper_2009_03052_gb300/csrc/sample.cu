@@ -1140,6 +1140,7 @@ extern "C" mc_status mc_estimate_counts(const mc_tables *t, const mc_estimate_pa
             MC_REQUIRE(p->star_samples >= 0, "star_samples must be >= 0");
             MC_REQUIRE(p->star_samples == 0 || (p->node_lo <= 0 && (p->node_hi <= 0 || p->node_hi == t->g->n)),
                        "star samples cover the whole graph: no node range with star_samples");
+            ensure_star_index(t->g, h, s);  // before split sampling takes what memory is left
         }
         if (p->mode == MC_EST_UNIFORM) {
             MC_REQUIRE(p->samples > 0, "uniform estimation needs samples > 0");

@@ -1,5 +1,6 @@
 """Memory that only makes calls faster is done without when it is refused: the
-list of nodes with neighbours."""
+list of nodes with neighbours, and the scratch of split sampling, which never
+takes what the call needs after it."""
 import threading
 
 import numpy as np
@@ -69,3 +70,18 @@ def test_graph_without_the_node_list(M, monkeypatch):
     T = M.Tables(G, colors, k, 64)
     for h in range(1, k + 1):
         assert np.array_equal(T.read(h), want.read(h)) and T.total(h) == want.total(h)
+
+
+def test_star_samples_beside_split_scratch(M, monkeypatch):
+    g, k, n = synth.chung_lu(200_000, 600_000, 2.5, seed=3), 5, 1 << 20
+    colors = synth.balanced_colors(g.n, k, 1)
+    M.sigma(k)
+    want = M.Tables(M.Graph.from_csr(g), colors, k, 64, skip_round=True).estimate(k, 7, n, star_samples=1000)
+    al = Limited(M)
+    monkeypatch.setattr(M, "torch_allocator", lambda: al)
+    T = M.Tables(M.Graph.from_csr(g), colors, k, 64, skip_round=True)
+    # room for the split scratch (4 (h + 1) bytes per sample), not for the star index on top of it
+    al.limit = al.held + 4 * (k + 1) * n + (2 << 20)
+    got = T.estimate(k, 7, n, star_samples=1000)
+    al.limit = None
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
