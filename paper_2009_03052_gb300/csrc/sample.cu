@@ -692,7 +692,7 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, SplitScratch *spli
     // 256 per SM), four when h >= 5 (longer chains: us lane / warp at 4500 and
     // 10000 samples 40 / 39 and 40 / 76 at k = 4, 159 / 63 and 159 / 126 at
     // k = 5, 289 / 100 and 292 / 216 at k = 7, 373 / 105 and 375 / 236 at k = 8);
-    // the latency mode (dense tables, blocks of 64 spread over more SMs) for
+    // the latency mode (blocks of 64 spread over more SMs) for
     // launches that leave most SMs idle; byte counting (profiling) runs an
     // instantiation of its own, so other launches carry none of its work; else
     // split sampling, if it has the memory, where it pays for its second launch:
@@ -709,14 +709,15 @@ static void launch_sampler(const mc_tables *t, SampleArgs &a, SplitScratch *spli
     const bool many = a.h >= 7 || wide || a.count >= (int64_t)sm_count() * 4 * 1536;
     SampleMode mode = SampleMode::Lanes;
     if (a.count <= (int64_t)sm_count() * (a.h >= 5 ? 64 : 32)) mode = SampleMode::Warps;
-    else if (!t->packed && a.count <= (int64_t)sm_count() * 256) mode = SampleMode::Latency;
+    else if (a.count <= (int64_t)sm_count() * 256) mode = SampleMode::Latency;
     else if (a.bytes && !t->packed) mode = SampleMode::Counted;
     else if (many && split &&
              split->room(!a.nodes, !a.classes, std::min(a.count, a.nodes && a.classes ? a.count : SPLIT_CHUNK), a.h))
         mode = SampleMode::Split;
     if (mode != SampleMode::Counted) a.bytes = nullptr;
-    const int in_line = !wide ? 0 : a.count > (int64_t)sm_count() * 2 * SAMPLE_BLOCK ? 3 : 4;  // one wave: 2 blocks per SM
-    auto kern = t->packed ? sample_kernel_packed(mode, t->bits, narrow) : sample_kernel_dense(mode, t->bits, narrow, in_line);
+    const bool few = a.count <= (int64_t)sm_count() * 2 * SAMPLE_BLOCK;  // one wave at 2 blocks per SM
+    auto kern = t->packed ? sample_kernel_packed(mode, t->bits, narrow, few)
+                          : sample_kernel_dense(mode, t->bits, narrow, !wide ? 0 : few ? 4 : 3);
     const int block = mode == SampleMode::Warps ? 256 : mode == SampleMode::Latency ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
     const size_t hist = a.hist ? (size_t)a.ncls * sizeof(uint32_t) : 0;
     const size_t smem = (mode == SampleMode::Warps ? 0 : (size_t)SAMPLE_WORDS * block * sizeof(uint32_t)) +

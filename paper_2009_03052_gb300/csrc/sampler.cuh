@@ -290,8 +290,12 @@ __device__ __forceinline__ int64_t first_true(int64_t lo, int64_t hi, P pred, F 
 // samples of Chung-Lu 1M, k = 5; 4: 0.88, 1: 0.82, 3: 0.80), 4 for 128-bit
 // counts in dense tables (12.9 ms for the adaptive run; 2: 13.6, 8: 19.9).
 // LAT (launches too small to fill the GPU): no register cap, 16 items of a scan
-// and 8 adjacency searches in flight per lane, so each sample's chain of
-// dependent loads is shorter.  The samples are the same in both modes.  SPLIT:
+// (4 of packed rows, each a search of its own) and 8 adjacency searches in flight
+// per lane, so each sample's chain of dependent loads is shorter.  FEW (packed
+// rows, launches of at most 2 blocks per SM): registers for 2 blocks, the third
+// would not run.  Packed rows, k = 6, Chung-Lu 200k, 128 bits, ms with estimates:
+// 20k samples 0.744 in the latency mode, 0.880 without either (0.777 with the
+// state in local memory), 100k 0.772 with FEW, 0.870 without (0.769).  The samples are the same in both modes.  SPLIT:
 // the nodes and their parents go to memory and classify_kernel takes over, so
 // that the searches of the classification neither hold the sampler's registers
 // nor wait in the divergence of its warps (1M samples at k = 5: 0.75 + 0.16 ms
@@ -309,11 +313,11 @@ __device__ __forceinline__ int64_t first_true(int64_t lo, int64_t hi, P pred, F 
 constexpr int SAMPLE_WORDS = 3 * MAXK;  // shared words per thread
 constexpr int SAMPLE_BLOCK = 512, SAMPLE_BLOCK_LAT = 64;
 
-template <typename CT, typename V, bool PK, bool LAT, bool CNT, bool SPLIT, int WD = 0>
-__global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1 : (sizeof(CT) == 16 && !PK ? 2 : 3))
+template <typename CT, typename V, bool PK, bool LAT, bool CNT, bool SPLIT, int WD = 0, bool FEW = false>
+__global__ void __launch_bounds__(LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK, LAT ? 1 : ((sizeof(CT) == 16 && !PK) || FEW ? 2 : 3))
     sample_kernel(const __grid_constant__ SampleArgs a)
 {
-    constexpr int NW = WD ? WD : LAT ? 16 : sizeof(CT) == 16 && !PK ? 4 : 2;  // items of a scan in flight
+    constexpr int NW = WD ? WD : LAT ? (PK ? 4 : 16) : sizeof(CT) == 16 && !PK ? 4 : 2;  // items of a scan in flight
     constexpr int NQ = LAT ? 8 : 4;   // adjacency searches in flight
     constexpr int KS = LAT ? 8 : 1;   // probes per round of the root and hub chunk searches
     constexpr int T = LAT ? SAMPLE_BLOCK_LAT : SAMPLE_BLOCK;
@@ -1221,8 +1225,8 @@ enum class SampleMode { Lanes, Latency, Counted, Split, Warps };
 // The kernel for tables of bits-bit counts with 64-bit descent arithmetic
 // (narrow) or 128-bit, dense (sampler_dense.cu; all modes; `wide`, 128-bit counts
 // only: rows below level h are wide, 3 or 4 of their items in flight) or packed
-// (sampler_packed.cu: Lanes, Split, Warps).
+// (sampler_packed.cu; all but Counted; `few`: at most 2 blocks per SM).
 SampleKernel sample_kernel_dense(SampleMode mode, int bits, bool narrow, int wide);
-SampleKernel sample_kernel_packed(SampleMode mode, int bits, bool narrow);
+SampleKernel sample_kernel_packed(SampleMode mode, int bits, bool narrow, bool few);
 
 }  // namespace mc

@@ -1,6 +1,6 @@
 """Requests on either side of the sizes where sampling and classification split
-into two kernels (h <= 6: four waves of lanes, h >= 7: past the latency mode)
-give the samples and hits of small requests at the same indices, from dense and
+into two kernels (h <= 6: four waves of lanes, h >= 7: past the latency mode),
+and in the latency mode, give the samples and hits of small requests at the same indices, from dense and
 packed tables."""
 import numpy as np
 import pytest
@@ -20,7 +20,7 @@ def M():
     return M
 
 
-@pytest.mark.parametrize("k,bits,kw", [(4, 64, {}), (6, 128, {}), (6, 64, {"varlen": True}), (7, 128, {})])
+@pytest.mark.parametrize("k,bits,kw", [(4, 64, {}), (6, 128, {}), (6, 64, {"varlen": True}), (7, 128, {}), (7, 128, {"succinct": True})])
 def test_both_sides_of_the_split(M, k, bits, kw):
     import torch
     waves = torch.cuda.get_device_properties(0).multi_processor_count * 4 * 1536
@@ -28,7 +28,7 @@ def test_both_sides_of_the_split(M, k, bits, kw):
     G = M.Graph.from_csr(g)
     T = M.Tables(G, M.color(G, k, 2), k, bits, **kw)
     M.sigma(k)
-    for n in (50_000, waves - 1, waves, waves + 77):
+    for n in (20_000, 50_000, waves - 1, waves, waves + 77):
         got = [x.cpu().numpy() for x in T.sample(k, 21, 5, n)]
         for at in (0, n - 400):
             for x, y in zip(got, T.sample(k, 21, 5 + at, 400)):
