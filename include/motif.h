@@ -269,6 +269,7 @@ mc_status mc_read_table(const mc_tables *t, int h, int which, void *dst, size_t 
  * nodes ascending), roots uint32[count], shapes int32[count] (rooted shape
  * id), classes int32[count] (id of the induced h-node graphlet: rank of its
  * canonical adjacency word among those of all connected h-node graphs).
+ * Without nodes or classes, large calls take scratch as mc_estimate_counts does.
  * MC_E_INVALID when no such treelet exists. */
 mc_status mc_sample(const mc_tables *t, int h, int32_t unrooted_shape, uint64_t seed,
                     uint64_t first_index, int64_t count, uint32_t *nodes, uint32_t *roots,
@@ -341,7 +342,10 @@ typedef struct {
 
 /* est: host double[N_h], the estimated number of induced copies of each
  * h-node graphlet in G; hits: host uint64[N_h], samples per graphlet;
- * stats: host, may be NULL.  N_h = mc_num_classes(h).  Synchronises.  AGS
+ * stats: host, may be NULL.  N_h = mc_num_classes(h).  Synchronises.  Large
+ * launches take scratch for their samples' nodes, 4 (h + 1) bytes per sample of a
+ * launch of at most 2^22 (151 MB at h = 8; AGS grows it by doubling), and do
+ * without it, more slowly, when it is refused.  AGS
  * page-locks a host buffer of about 4 (B + 4096 U) bytes (B = batch, or 2^22
  * when automatic; U = mc_num_unrooted(h)) that the calling thread keeps for
  * its later calls and frees when it exits. */

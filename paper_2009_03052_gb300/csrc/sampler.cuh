@@ -295,11 +295,13 @@ __device__ __forceinline__ int64_t first_true(int64_t lo, int64_t hi, P pred, F 
 // rows, launches of at most 2 blocks per SM): registers for 2 blocks, the third
 // would not run.  Packed rows, k = 6, Chung-Lu 200k, 128 bits, ms with estimates:
 // 20k samples 0.744 in the latency mode, 0.880 without either (0.777 with the
-// state in local memory), 100k 0.772 with FEW, 0.870 without (0.769).  The samples are the same in both modes.  SPLIT:
-// the nodes and their parents go to memory and classify_kernel takes over, so
-// that the searches of the classification neither hold the sampler's registers
-// nor wait in the divergence of its warps (1M samples at k = 5: 0.75 + 0.16 ms
-// against 1.08 in one kernel; the code before both 1.11).
+// state in local memory), 100k 0.772 with FEW, 0.870 without (0.769).  The samples
+// are the same in every mode.  SPLIT: the nodes and their parents go to memory and
+// classify_kernel takes over, so that the searches of the classification neither
+// hold the sampler's registers nor wait in the divergence of its warps (ms with
+// estimates, split / one kernel: 10M samples at k = 6 14.1 / 15.1, 1M at k = 7,
+// R-MAT 19, 1.99 / 2.20, 1M at k = 5 1.00 / 1.01; with the state in local memory
+// 1.21).
 // WD > 0 (128-bit dense tables with wide rows below level h): counts above 64 bits
 // carry most of the weight, so most samples pass through wide rows; their entries
 // are read in line, low and upper parts and the wide words of WD neighbours in
