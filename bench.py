@@ -845,7 +845,14 @@ def run_serve(args):
 # profiles/), with a hash of the kernel's source file when it was captured:
 # the figure is reported only while that source is unchanged.  Entries:
 # (workload, kernel): (bytes, hash[, schedule]).
-TRAFFIC: dict = {}
+TRAFFIC: dict = {
+    # profiles/sample_kernel_chung_lu_1m_k5.md: sample_kernel (split) and classify_kernel
+    ("chung_lu_1m_k5", "sample"): (1_855_826_000, "3df130a07b48cb78"),
+    # profiles/gather_kernel_chung_lu_1m_k5.md, under schedules 6, 0, 3
+    ("chung_lu_1m_k5", "gather_h2"): (275_516_000, "d80c94faf71a2e17", 6),
+    ("chung_lu_1m_k5", "gather_h3"): (554_230_000, "d80c94faf71a2e17", 0),
+    ("chung_lu_1m_k5", "gather_h4"): (984_188_000, "d80c94faf71a2e17", 3),
+}
 KERNEL_SOURCE = {"sample": "sampler.cuh", "classify": "sampler.cuh", "gather": "gather.cuh", "merge": "build.cu"}
 
 

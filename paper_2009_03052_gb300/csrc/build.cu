@@ -133,9 +133,9 @@ __global__ void __launch_bounds__(256) hub_reduce_kernel(CT *__restrict__ partia
 // (k = 7 levels 6 / 7: 4.8 / 5.5 against 3.9 / 4.8 ms), two nodes per thread
 // gave nothing.  Against a thread per (node, output) reading whole counts
 // through L1, ms per level 5 / 6 / 7 on R-MAT 22, k = 7, 128-bit counts: 10.6 /
-// 15.0 / 12.5 before, 2.8 / 3.9 / 4.8 now; levels 6 / 7 / 8 on Chung-Lu 2M,
-// k = 8: 20.8 / 27.8 / 21.1 before, 10.9 / 14.3 / 11.9 now; level 5 / 6 on a
-// 994k-node grid, k = 6, 64-bit counts: 0.69 / 0.47 before, 0.30 / 0.25 now.
+// 15.0 / 12.5 before, 2.95 / 4.05 / 4.5 now; levels 6 / 7 / 8 on Chung-Lu 2M,
+// k = 8: 20.8 / 27.8 / 21.1 before, 10.8 / 14.6 / 12.4 now; level 5 / 6 on a
+// 994k-node grid, k = 6, 64-bit counts: 0.69 / 0.47 before, 0.34 / 0.26 now.
 // Rows are read and written by their first planes (common.cuh): operands of 4
 // or 8 bytes, with products of 64 to 128 bits.  A node with a wide row among a
 // pair's operands reads that pair's operands from memory instead, in full;
